@@ -31,12 +31,19 @@
 #include "nfd_sm100.cuh"
 
 template <int BN> struct GemmCfg {
-    // ring deep enough that one CTA owns an SM; the wide tiles (passes of several frames) keep about the same
-    // number of bytes in flight with fewer, larger stages
-    static constexpr int STAGES = BN <= 32 ? 7 : (BN <= 128 ? 6 : (BN <= 192 ? 4 : 3));
+    // A ring stage holds KU k-blocks of 64 elements.  A stage costs the producer about 280 clocks of barrier
+    // operations and 40 per TMA instruction whatever its size, an SM takes in up to 120 bytes per clock: with
+    // one 64-element block per stage the producer's own instructions set the pace (128 + 64 rows: 380 clocks per
+    // block, 65 bytes per clock), with two the SM's intake does (220 clocks per block).  A 256-wide tile
+    // brings 48 KB per block, which is enough for a stage.
+    static constexpr int KU = BN <= 192 ? 2 : 1;
+    // ring deep enough that one CTA owns an SM
+    static constexpr int STAGES = BN <= 64 ? 4 : (BN <= 128 ? 3 : (BN <= 192 ? 2 : 3));
     static constexpr int A_BYTES = 128 * 128;                  // 128 rows x 64 bf16
     static constexpr int B_BYTES = BN * 128;
-    static constexpr int RING_BYTES = STAGES * (A_BYTES + B_BYTES);
+    static constexpr int KB_BYTES = A_BYTES + B_BYTES;
+    static constexpr int ST_BYTES = KU * KB_BYTES;             // a stage: KU A blocks, then KU B blocks
+    static constexpr int RING_BYTES = STAGES * ST_BYTES;
     static constexpr int SROW = BN + 4;                        // staging row stride (floats)
     static constexpr int STAGE_BYTES = 128 * SROW * 4;         // partial accumulator tile; reuses the ring
     static constexpr int TMEM_COLS = BN <= 32 ? 32 : (BN <= 64 ? 64 : (BN <= 128 ? 128 : 256));
@@ -48,6 +55,7 @@ template <int BN> struct GemmCfg {
     static constexpr int EPI_THREADS = 256;
     static constexpr int MAX_S = 4;                            // largest cluster split
     static constexpr int MIN_CTAS = 1;
+    static_assert(SMEM <= 232448, "shared memory of a CTA");
     static_assert(STAGE_BYTES <= RING_BYTES, "staging tile must fit the operand ring");
 };
 
@@ -74,7 +82,6 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
     const int split = blockIdx.x % S, n_tile = blockIdx.x / S;
     const int m0 = blockIdx.y * 128, n0 = n_tile * BN;
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    uint8_t *sA = smem, *sB = smem + G::STAGES * G::A_BYTES;
     float *stage = reinterpret_cast<float *>(smem);          // reuses the ring once the UMMAs are done
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + G::RING_BYTES);
     const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + G::STAGES),
@@ -120,31 +127,73 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
     int uv_f0 = 0;                                           // first frame of the tile (folded LayerNorm)
     if constexpr (Epi::kRowStats) uv_f0 = m0 / epi.ln.T;
 
+    const int nst = (nkb + G::KU - 1) / G::KU;               // ring stages of this CTA's K range
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
+            const uint32_t ring = smem_u32(smem);
+            // the k-blocks of stage st: KU, fewer in the last one
+            auto load_b = [&](int st, int s) {
+                const int n = nkb - st * G::KU < G::KU ? nkb - st * G::KU : G::KU;
+                mbar_expect_tx(full0 + 8 * s, (uint32_t)n * G::KB_BYTES);
+#pragma unroll
+                for (int u = 0; u < G::KU; ++u)
+                    if (u < n)
+                        tma_load_2d(ring + s * G::ST_BYTES + G::KU * G::A_BYTES + u * G::B_BYTES, &tmB, full0 + 8 * s,
+                                    (kb0 + st * G::KU + u) * 64, n0);
+            };
+            auto load_a = [&](int st, int s) {
+                const int n = nkb - st * G::KU < G::KU ? nkb - st * G::KU : G::KU;
+#pragma unroll
+                for (int u = 0; u < G::KU; ++u)
+                    if (u < n)
+                        tma_load_2d(ring + s * G::ST_BYTES + u * G::A_BYTES, &tmA, full0 + 8 * s,
+                                    (kb0 + st * G::KU + u) * 64, m0);
+            };
             // weights never depend on the previous kernel: fill the ring's weight halves first
-            const int pre = nkb < G::STAGES ? nkb : G::STAGES;
-            for (int kb = 0; kb < pre; ++kb) {
-                mbar_expect_tx(full0 + 8 * kb, G::A_BYTES + G::B_BYTES);
-                tma_load_2d(smem_u32(sB + kb * G::B_BYTES), &tmB, full0 + 8 * kb, (kb0 + kb) * 64, n0);
-            }
+            const int pre = nst < G::STAGES ? nst : G::STAGES;
+            for (int st = 0; st < pre; ++st) load_b(st, st);
             // test switch (see nfd_sm100.cuh): leave out the last stage, so that the wait for it runs out
             const int skip_last = *reinterpret_cast<volatile int *>(status + 2);
             pdl_wait();
             NFD_TRACE_MARK(TRK_OTHER + 1);
-            for (int kb = 0; kb < pre; ++kb) {
-                if (skip_last && kb == nkb - 1) continue;      // its weight half has landed; the stage stays incomplete
-                tma_load_2d(smem_u32(sA + kb * G::A_BYTES), &tmA, full0 + 8 * kb, (kb0 + kb) * 64, m0);
+            for (int st = 0; st < pre; ++st) {
+                if (skip_last && st == nst - 1) continue;      // its weight half has landed; the stage stays incomplete
+                load_a(st, st);
             }
-            for (int kb = pre; kb < nkb; ++kb) {
-                if (skip_last && kb == nkb - 1) break;
-                const int s = kb % G::STAGES;
-                if (!mbar_wait(empty0 + 8 * s, ((kb / G::STAGES) - 1) & 1, status)) break;
-                mbar_expect_tx(full0 + 8 * s, G::A_BYTES + G::B_BYTES);
-                tma_load_2d(smem_u32(sA + s * G::A_BYTES), &tmA, full0 + 8 * s, (kb0 + kb) * 64, m0);
-                tma_load_2d(smem_u32(sB + s * G::B_BYTES), &tmB, full0 + 8 * s, (kb0 + kb) * 64, n0);
+            for (int st = pre; st < nst; ++st) {
+                if (skip_last && st == nst - 1) break;
+                const int s = st % G::STAGES;
+                if (!mbar_wait(empty0 + 8 * s, ((st / G::STAGES) - 1) & 1, status)) break;
+                load_b(st, s);
+                load_a(st, s);
             }
-        } else if (lane == 1) {
+        }
+    } else if (warp == 1) {
+        if (elect_one()) {
+            pdl_launch();
+            constexpr uint32_t idesc = umma_idesc_bf16(128, BN);
+            const uint32_t ring = smem_u32(smem);
+            for (int st = 0; st < nst; ++st) {
+                const int s = st % G::STAGES;
+                if (!mbar_wait(full0 + 8 * s, (st / G::STAGES) & 1, status)) break;
+                tc_fence_after();
+                if (st == 0) NFD_TRACE_MARK_T(TRK_OTHER + 5, 32);
+                if (st == nst - 1) NFD_TRACE_MARK_T(TRK_OTHER + 6, 32);
+#pragma unroll
+                for (int u = 0; u < G::KU; ++u) {
+                    if (u > 0 && st * G::KU + u >= nkb) break;
+                    const uint64_t ad = umma_desc_k128(ring + s * G::ST_BYTES + u * G::A_BYTES);
+                    const uint64_t bd = umma_desc_k128(ring + s * G::ST_BYTES + G::KU * G::A_BYTES + u * G::B_BYTES);
+#pragma unroll
+                    for (int k4 = 0; k4 < 4; ++k4)
+                        umma_bf16_ss(tmem_base, ad + 2 * k4, bd + 2 * k4, idesc, (st | u | k4) != 0);
+                }
+                umma_commit(empty0 + 8 * s);
+            }
+            umma_commit(accf);          // arrives when every UMMA above has completed
+        }
+    } else {
+        if (warp == 2 && elect_one()) {
             // this CTA's slice of the next GEMM's weights, towards L2 in 8 KiB pieces, and whatever the
             // epilogue functor knows the next kernel will read
             const unsigned long long n_cta = (unsigned long long)gridDim.x * gridDim.y;
@@ -159,26 +208,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
                 bulk_prefetch_l2(reinterpret_cast<const uint8_t *>(pf.ptr) + b, (uint32_t)n);
             }
         }
-    } else if (warp == 1) {
-        if (lane == 0) {
-            pdl_launch();
-            constexpr uint32_t idesc = umma_idesc_bf16(128, BN);
-            for (int kb = 0; kb < nkb; ++kb) {
-                const int s = kb % G::STAGES;
-                if (!mbar_wait(full0 + 8 * s, (kb / G::STAGES) & 1, status)) break;
-                tc_fence_after();
-                if (kb == 0) NFD_TRACE_MARK_T(TRK_OTHER + 5, 32);
-                if (kb == nkb - 1) NFD_TRACE_MARK_T(TRK_OTHER + 6, 32);
-                const uint64_t ad = umma_desc_k128(smem_u32(sA + s * G::A_BYTES));
-                const uint64_t bd = umma_desc_k128(smem_u32(sB + s * G::B_BYTES));
-#pragma unroll
-                for (int k4 = 0; k4 < 4; ++k4)
-                    umma_bf16_ss(tmem_base, ad + 2 * k4, bd + 2 * k4, idesc, (kb | k4) != 0);
-                umma_commit(empty0 + 8 * s);
-            }
-            umma_commit(accf);          // arrives when every UMMA above has completed
-        }
-    } else {
+        __syncwarp();
         pdl_wait();
         // side inputs of the first items (bias, gate, residual, rotary table), fetched while the UMMAs run
 #pragma unroll
