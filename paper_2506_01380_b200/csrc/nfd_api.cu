@@ -508,7 +508,7 @@ static int tune_gemms(nfd_ctx *c) {
         p.nf = nf;
         for (int j = 0; j < nf; ++j) {
             p.fr[j].stream = 0, p.fr[j].frame = j, p.fr[j].win_first = 0, p.fr[j].cond_row = 0, p.fr[j].first_new = 0;
-            p.fr[j].src = 0, p.fr[j].src_index = j, p.fr[j].out_index = -1;
+            p.fr[j].src = 0, p.fr[j].src_index = j, p.fr[j].out_index = -1, p.fr[j].win_slot = 0;
         }
         k_set_params<<<1, 256, 0, c->st>>>(p, c->d_sp, c->lim, c->d_status);
         CK(cudaGetLastError());
@@ -701,6 +701,7 @@ static int build_pass_frames(nfd_ctx *c, const std::vector<PassFrame> &fr, int k
         f.stream = pf.stream;
         f.frame = pf.frame;
         f.win_first = pf.frame - g.ctx_frames > 0 ? pf.frame - g.ctx_frames : 0;
+        f.win_slot = f.win_first % c->D.R;
         f.cond_row = row;
         f.first_new = pf.first_new;
         f.src = pf.src, f.src_index = pf.src_index, f.out_index = pf.out_index;
@@ -793,7 +794,7 @@ int nfd_create(nfd_ctx **out, const nfd_weights *w, const nfd_cfg *cfg, void *cu
     D.R = cfg->ctx_frames + 2 * cfg->max_spec, D.W = cfg->ctx_frames, D.n_streams = cfg->n_streams;
     D.norm = cfg->norm, D.eps = cfg->norm_eps, D.t_scale = cfg->t_scale;
     D.page_elems = (size_t)D.H * D.T * D.dh;
-    c->lim.n_streams = cfg->n_streams, c->lim.W = cfg->ctx_frames, c->lim.n_slots = NFD_COND_SLOTS;
+    c->lim.n_streams = cfg->n_streams, c->lim.W = cfg->ctx_frames, c->lim.R = D.R, c->lim.n_slots = NFD_COND_SLOTS;
     c->lim.n_actions = cfg->n_actions, c->lim.max_frames = NFD_MAX_PASS_FRAMES;
     c->lim.pend_slots = cfg->n_streams * cfg->max_spec;
     c->n_committed.assign(cfg->n_streams, 0);
@@ -1293,6 +1294,7 @@ int nfd_attention(nfd_ctx *c, const void *q, const void *k, const void *v, int n
         p.fr[j].stream = 0;
         p.fr[j].frame = n_kv - n_q + j;
         p.fr[j].win_first = p.fr[j].frame - window > 0 ? p.fr[j].frame - window : 0;
+        p.fr[j].win_slot = p.fr[j].win_first % D.R;
         p.fr[j].first_new = n_kv - n_q;
     }
     c->cls = CLS_PARAMS;
@@ -1538,10 +1540,11 @@ extern "C" int nfd_attention_noalloc(const void *q, const void *k_pages, const v
         p.fr[j].stream = 0;
         p.fr[j].frame = n_kv_frames - n_q_frames + j;
         p.fr[j].win_first = p.fr[j].frame - window > 0 ? p.fr[j].frame - window : 0;
+        p.fr[j].win_slot = p.fr[j].win_first % D.R;
         p.fr[j].first_new = n_kv_frames - n_q_frames;
     }
     DescLimits lim;
-    lim.n_streams = 1, lim.W = window, lim.n_slots = 1, lim.n_actions = 1, lim.max_frames = NFD_MAX_PASS_FRAMES;
+    lim.n_streams = 1, lim.W = window, lim.R = D.R, lim.n_slots = 1, lim.n_actions = 1, lim.max_frames = NFD_MAX_PASS_FRAMES;
     lim.pend_slots = 1;
     // the descriptor is rewritten in full on every call; nothing of the previous call survives
     k_set_params<<<1, 256, 0, st>>>(p, d_sp, lim, d_stat);

@@ -24,13 +24,27 @@ struct FastState {
     int n_sm = 148;
     size_t a_rows = 0;     // rows of every activation buffer (NFD_MAX_PASS_FRAMES * T)
     AttnPlan plan;         // KB == 0: tensor-core attention not available for this shape
-    float *part_o = nullptr;           // per-split states of the attention kernel: [query tile][split] x PARK_BYTES
+    float *part_o = nullptr;           // per-split states of the attention kernel: [query tile][split] x ATTN_STATE_BYTES
     unsigned int *attn_counters = nullptr;   // one per (frame, head, query tile); zero between launches
-    size_t cache_rows = 0;
+    size_t cache_pages = 0;            // (stream, layer, ring slot, head) pages of T rows
     std::map<std::tuple<const void *, int, int, int>, CUtensorMap> maps;   // (ptr, rows, cols, box_rows)
     int force_BN = 0, force_S = 0;     // set while candidates are being timed
     int slots[5] = {0, 0, 0, 0, 0};    // CTAs of a GEMM that can be resident at once, by cluster size (1, 2, 4)
 };
+
+// Key block, blocks per page and query tiles for pages of T tokens: the block that walks a page in the least time, a
+// block costing its columns (padded ones included) plus a fixed part of about 24 columns (barriers and hand-overs).
+static void attn_blocks(AttnPlan &pl, int T) {
+    const int kbs[4] = {128, 112, 96, 64};
+    for (int kb : kbs) {
+        const int bpf = (T + kb - 1) / kb;
+        if (!pl.KB || bpf * (kb + 24) < pl.BPF * (pl.KB + 24)) pl.KB = kb, pl.BPF = bpf;
+    }
+    pl.QT = (T + 127) / 128;
+}
+static void attn_divisors(AttnPlan &pl, int H) {
+    pl.split_div.set(pl.MAXSPLIT), pl.qt_div.set(pl.QT), pl.h_div.set(H), pl.ch_div.set(pl.CH), pl.bpf_div.set(pl.BPF);
+}
 
 static int fast_create(FastState &fs, const Dims &D, bool bf16_mode, cudaStream_t st, int *d_status) {
     (void)st;
@@ -52,14 +66,11 @@ static int fast_create(FastState &fs, const Dims &D, bool bf16_mode, cudaStream_
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&fs.n_sm, cudaDevAttrMultiProcessorCount, dev);
     fs.ready = true;
-    // attention plan: head_dim 64, key blocks that divide the tokens per frame
+    // attention plan: any number of tokens per frame, head dimension 64 or 32
     AttnPlan pl;
-    const int KB = D.T % 128 == 0 ? 128 : (D.T % 112 == 0 ? 112 : (D.T % 64 == 0 ? 64 : 0));
-    fs.cache_rows = (size_t)D.n_streams * D.L * D.R * D.H * D.T;
-    if (D.dh == 64 && KB && D.H * D.T >= 128 && fs.cache_rows < 0x7fffffffull) {
-        pl.KB = KB;
-        pl.BPF = D.T / KB;
-        pl.QT = (D.T + 127) / 128;
+    fs.cache_pages = (size_t)D.n_streams * D.L * D.R * D.H;
+    if ((D.dh == 64 || D.dh == 32) && fs.cache_pages < 0x7fffffffull) {
+        attn_blocks(pl, D.T);
         // split the longest window (a frame sees at most W + 1 pages) so that streams x heads x query tiles x
         // splits fills the SMs once: a context made for several streams is run with batched passes, which bring
         // enough (frame, head, query tile) items by themselves, and long unsplit key ranges amortise the
@@ -70,13 +81,14 @@ static int fast_create(FastState &fs, const Dims &D, bool bf16_mode, cudaStream_
         pl.MAXSPLIT = ((D.W + 1) * pl.BPF + pl.CH - 1) / pl.CH;
         if (pl.MAXSPLIT > 1) {
             const size_t tiles = (size_t)NFD_MAX_PASS_FRAMES * D.H * pl.QT;
-            if (cudaMalloc((void **)&fs.part_o, tiles * pl.MAXSPLIT * (size_t)AttnCfg<64>::PARK_BYTES) != cudaSuccess ||
+            if (cudaMalloc((void **)&fs.part_o, tiles * pl.MAXSPLIT * (size_t)ATTN_STATE_BYTES) != cudaSuccess ||
                 cudaMalloc((void **)&fs.attn_counters, tiles * sizeof(unsigned int)) != cudaSuccess ||
                 cudaMemset(fs.attn_counters, 0, tiles * sizeof(unsigned int)) != cudaSuccess) {
                 cudaGetLastError();
                 return NFD_E_NOMEM;
             }
         }
+        attn_divisors(pl, D.H);
         fs.plan = pl;
     }
     return NFD_OK;
@@ -109,6 +121,23 @@ static const CUtensorMap *get_map_2d(FastState &fs, const void *ptr, int rows, i
         return nullptr;
     }
     return &fs.maps.emplace(key, m).first->second;
+}
+
+// 3D bf16 tensor map [pages][rows][cols] for the attention operands: box = 1 page x box_rows x 64 columns, 128-byte
+// swizzle.  Rows beyond a page's end and, for head dimension 32, columns beyond the row's end read as zero.
+static bool encode_map_3d(PFN_encodeTiled encode, CUtensorMap *m, const void *ptr, size_t pages, int rows, int cols,
+                          int box_rows) {
+    cuuint64_t gdim[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)pages};
+    cuuint64_t gstr[2] = {(cuuint64_t)cols * 2, (cuuint64_t)cols * 2 * rows};
+    cuuint32_t box[3] = {64, (cuuint32_t)box_rows, 1};
+    cuuint32_t estr[3] = {1, 1, 1};
+    CUresult r = encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(ptr), gdim, gstr, box, estr,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS)
+        fprintf(stderr, "libnfd: cuTensorMapEncodeTiled failed (%d) for [%zu x %d x %d] box %d\n", (int)r, pages, rows,
+                cols, box_rows);
+    return r == CUDA_SUCCESS;
 }
 
 // ---------------------------------------------------------------------------
@@ -298,14 +327,16 @@ static int launch_attn_tc(FastState &fs, cudaStream_t st, const StepParams *sp, 
         }
         attr_set = true;
     }
-    const CUtensorMap *mq = get_map_2d(fs, q, D.H * nf * D.T, 64, 128);
-    const CUtensorMap *mk = get_map_2d(fs, kc, (int)fs.cache_rows, 64, KB);
-    const CUtensorMap *mv = get_map_2d(fs, vc, (int)fs.cache_rows, 64, KB);
-    if (!mq || !mk || !mv) return 0;
+    CUtensorMap mq, mk, mv;
+    if (!encode_map_3d(fs.encode, &mq, q, D.H, nf * D.T, D.dh, 128) ||
+        !encode_map_3d(fs.encode, &mk, kc, fs.cache_pages, D.T, D.dh, KB) ||
+        !encode_map_3d(fs.encode, &mv, vc, fs.cache_pages, D.T, D.dh, KB))
+        return 0;
     const AttnPlan &pl = fs.plan;
-    dim3 grid(pl.MAXSPLIT, pl.QT, nf * D.H);
-    cudaError_t e = launch_pdl(kern, grid, dim3(A::THREADS), (size_t)A::SMEM, st, 1, *mq, *mk, *mv, sp, D, layer, pl, out,
-                               fs.part_o, fs.attn_counters, fs.d_status);
+    const int n_items = pl.MAXSPLIT * pl.QT * D.H * nf;
+    dim3 grid(n_items < fs.n_sm ? n_items : fs.n_sm);
+    cudaError_t e = launch_pdl(kern, grid, dim3(A::THREADS), (size_t)A::SMEM, st, 1, mq, mk, mv, sp, D, layer, pl, n_items,
+                               out, fs.part_o, fs.attn_counters, fs.d_status);
     if (e != cudaSuccess) {
         fprintf(stderr, "libnfd: tensor-core attention launch failed: %s\n", cudaGetErrorString(e));
         cudaGetLastError();
@@ -324,6 +355,7 @@ static int fast_attention(bool enabled, FastState &fs, cudaStream_t st, const St
         if (!enabled || !fs.ready || fs.plan.KB == 0) return 0;
         if (fs.plan.KB == 128) return launch_attn_tc<128>(fs, st, sp, D, nf, layer, q, kc, vc, out);
         if (fs.plan.KB == 112) return launch_attn_tc<112>(fs, st, sp, D, nf, layer, q, kc, vc, out);
+        if (fs.plan.KB == 96) return launch_attn_tc<96>(fs, st, sp, D, nf, layer, q, kc, vc, out);
         return launch_attn_tc<64>(fs, st, sp, D, nf, layer, q, kc, vc, out);
     }
 }

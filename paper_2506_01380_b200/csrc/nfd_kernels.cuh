@@ -16,7 +16,7 @@
 // output -- so that nothing downstream leaves its buffers; the caller learns of
 // it from nfd_status and must treat the cache as lost.
 struct DescLimits {
-    int n_streams, W, n_slots, n_actions, max_frames, pend_slots;
+    int n_streams, W, R, n_slots, n_actions, max_frames, pend_slots;
 };
 // It does not release its dependents early: a kernel that starts after this one
 // may read the descriptor before its own wait on the predecessor grid.
@@ -31,7 +31,7 @@ __global__ void k_set_params(StepParams p, StepParams *dst, DescLimits lim, int 
     if (t < NFD_MAX_PASS_FRAMES && t < p.nf) {
         const FrameDesc &f = p.fr[t];
         bad = bad || f.stream < 0 || f.stream >= lim.n_streams || f.frame < 0 || f.win_first < 0 ||
-              f.win_first > f.frame || f.frame - f.win_first > lim.W || f.first_new < 0 || f.first_new > f.frame ||
+              f.win_first > f.frame || f.frame - f.win_first > lim.W || f.win_slot != f.win_first % lim.R || f.first_new < 0 || f.first_new > f.frame ||
               f.cond_row < 0 || f.cond_row >= lim.n_slots || f.src < 0 || f.src > 1 || f.src_index < 0 ||
               f.src_index >= (f.src ? lim.pend_slots : lim.max_frames) || f.out_index < -1 ||
               f.out_index >= lim.max_frames;
@@ -60,7 +60,7 @@ __global__ void k_set_params(StepParams p, StepParams *dst, DescLimits lim, int 
         if (t < NFD_MAX_PASS_FRAMES) {
             FrameDesc f;
             f.stream = 0, f.frame = t, f.win_first = t, f.cond_row = 0, f.first_new = 0;
-            f.src = 0, f.src_index = 0, f.out_index = -1;
+            f.src = 0, f.src_index = 0, f.out_index = -1, f.win_slot = t % lim.R;
             dst->fr[t] = f;
         }
     }
