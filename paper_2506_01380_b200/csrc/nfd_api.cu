@@ -315,16 +315,15 @@ template <typename TS> static void launch_attention(nfd_ctx *c, int nf, int laye
         c->launches += n_fast;
         return;
     }
-    long long warps = (long long)nf * D.T * D.H;
-    int grid = (int)((warps + 3) / 4);
+    const dim3 grid((D.T + ATTN_ROWS_Q - 1) / ATTN_ROWS_Q, D.H, nf);
     if (D.dh == 32)
-        PLAUNCH(c, (k_attn_simple<TS, 32>), grid, 128, 0, (const StepParams *)c->d_sp, D, layer, (const TS *)c->qbuf,
+        PLAUNCH(c, (k_attn_rows<TS, 32>), grid, 256, 0, (const StepParams *)c->d_sp, D, layer, (const TS *)c->qbuf,
                 (const TS *)c->kc, (const TS *)c->vc, (TS *)c->abuf);
     else if (D.dh == 64)
-        PLAUNCH(c, (k_attn_simple<TS, 64>), grid, 128, 0, (const StepParams *)c->d_sp, D, layer, (const TS *)c->qbuf,
+        PLAUNCH(c, (k_attn_rows<TS, 64>), grid, 256, 0, (const StepParams *)c->d_sp, D, layer, (const TS *)c->qbuf,
                 (const TS *)c->kc, (const TS *)c->vc, (TS *)c->abuf);
     else
-        PLAUNCH(c, (k_attn_simple<TS, 128>), grid, 128, 0, (const StepParams *)c->d_sp, D, layer, (const TS *)c->qbuf,
+        PLAUNCH(c, (k_attn_rows<TS, 128>), grid, 256, 0, (const StepParams *)c->d_sp, D, layer, (const TS *)c->qbuf,
                 (const TS *)c->kc, (const TS *)c->vc, (TS *)c->abuf);
 }
 
@@ -1479,19 +1478,40 @@ static void *g_noalloc_dev_ptr[NFD_NOALLOC_MAX_DEVICES] = {nullptr};
 template <typename TS>
 static int noalloc_launch(cudaStream_t st, const StepParams *d_sp, const Dims &D, int n_q, const void *q,
                           const void *k_pages, const void *v_pages, void *out) {
-    const long long warps = (long long)n_q * D.T * D.H;
-    const int grid = (int)((warps + 3) / 4);
+    const dim3 grid((D.T + ATTN_ROWS_Q - 1) / ATTN_ROWS_Q, D.H, n_q);
     if (D.dh == 32)
-        k_attn_simple<TS, 32><<<grid, 128, 0, st>>>(d_sp, D, 0, (const TS *)q, (const TS *)k_pages,
-                                                    (const TS *)v_pages, (TS *)out);
+        k_attn_rows<TS, 32><<<grid, 256, 0, st>>>(d_sp, D, 0, (const TS *)q, (const TS *)k_pages, (const TS *)v_pages, (TS *)out);
     else if (D.dh == 64)
-        k_attn_simple<TS, 64><<<grid, 128, 0, st>>>(d_sp, D, 0, (const TS *)q, (const TS *)k_pages,
-                                                    (const TS *)v_pages, (TS *)out);
+        k_attn_rows<TS, 64><<<grid, 256, 0, st>>>(d_sp, D, 0, (const TS *)q, (const TS *)k_pages, (const TS *)v_pages, (TS *)out);
     else
-        k_attn_simple<TS, 128><<<grid, 128, 0, st>>>(d_sp, D, 0, (const TS *)q, (const TS *)k_pages,
-                                                     (const TS *)v_pages, (TS *)out);
+        k_attn_rows<TS, 128><<<grid, 256, 0, st>>>(d_sp, D, 0, (const TS *)q, (const TS *)k_pages, (const TS *)v_pages, (TS *)out);
     CK(cudaGetLastError());
     return NFD_OK;
+}
+
+// The tensor-core kernel on the caller's pages, key ranges unsplit (a split would need memory for its states).
+// Returns false where it does not handle the case.
+static bool noalloc_launch_tc(int dev, cudaStream_t st, const StepParams *d_sp, int *d_stat, const Dims &D, int n_q,
+                              const void *q, const void *k_pages, const void *v_pages, void *out) {
+    static PFN_encodeTiled enc[NFD_NOALLOC_MAX_DEVICES];
+    static int n_sm[NFD_NOALLOC_MAX_DEVICES];
+    if (D.dh != 64 && D.dh != 32) return false;
+    if (!enc[dev]) {
+        // looked up once per device, like the array's address
+        PFN_encodeTiled e = get_encode_fn();
+        if (!e || cudaDeviceGetAttribute(&n_sm[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        enc[dev] = e;
+    }
+    AttnPlan pl;
+    attn_blocks(pl, D.T);
+    pl.CH = (D.W + 1) * pl.BPF, pl.MAXSPLIT = 1;
+    const long long n_items = (long long)pl.QT * D.H * n_q;
+    if (!attn_divisors(pl, D.H, n_items, D.W)) return false;
+    return launch_attn_plan(enc[dev], n_sm[dev], st, d_sp, D, n_q, 0, pl, (size_t)D.R * D.H, (const bf16 *)q,
+                            (const bf16 *)k_pages, (const bf16 *)v_pages, (bf16 *)out, nullptr, nullptr, d_stat) != 0;
 }
 
 extern "C" int nfd_attention_noalloc(const void *q, const void *k_pages, const void *v_pages, int dtype, int n_heads,
@@ -1530,7 +1550,8 @@ extern "C" int nfd_attention_noalloc(const void *q, const void *k_pages, const v
     Dims D;
     memset(&D, 0, sizeof(D));
     D.L = 1, D.H = n_heads, D.dh = head_dim, D.d = n_heads * head_dim, D.T = tokens_per_frame;
-    D.R = n_kv_frames, D.W = window, D.n_streams = 1;
+    // (a window beyond the pages is the pages)
+    D.R = n_kv_frames, D.W = window < n_kv_frames ? window : n_kv_frames, D.n_streams = 1;
     D.page_elems = (size_t)n_heads * tokens_per_frame * head_dim;
     StepParams p;
     memset(&p, 0, sizeof(p));
@@ -1549,6 +1570,8 @@ extern "C" int nfd_attention_noalloc(const void *q, const void *k_pages, const v
     // the descriptor is rewritten in full on every call; nothing of the previous call survives
     k_set_params<<<1, 256, 0, st>>>(p, d_sp, lim, d_stat);
     CK(cudaGetLastError());
+    if (dtype == NFD_DTYPE_BF16 && noalloc_launch_tc(dev, st, d_sp, d_stat, D, n_q_frames, q, k_pages, v_pages, out))
+        return NFD_OK;
     if (dtype == NFD_DTYPE_BF16) return noalloc_launch<bf16>(st, d_sp, D, n_q_frames, q, k_pages, v_pages, out);
     return noalloc_launch<float>(st, d_sp, D, n_q_frames, q, k_pages, v_pages, out);
 }

@@ -42,8 +42,22 @@ static void attn_blocks(AttnPlan &pl, int T) {
     }
     pl.QT = (T + 127) / 128;
 }
-static void attn_divisors(AttnPlan &pl, int H) {
+// The plan's divisors; false where a dividend is too large for them (n * d has to stay below 2^32).
+static bool attn_divisors(AttnPlan &pl, int H, long long n_items, int W) {
     pl.split_div.set(pl.MAXSPLIT), pl.qt_div.set(pl.QT), pl.h_div.set(H), pl.ch_div.set(pl.CH), pl.bpf_div.set(pl.BPF);
+    const long long nb = ((long long)W + 1) * pl.BPF + pl.CH, big = 0x100000000ll;
+    const int d_item = pl.QT > H ? (pl.QT > pl.MAXSPLIT ? pl.QT : pl.MAXSPLIT) : (H > pl.MAXSPLIT ? H : pl.MAXSPLIT);
+    return n_items < 0x7fffffffll && n_items * d_item < big && nb < 0x7fffffffll && nb * (pl.CH > pl.BPF ? pl.CH : pl.BPF) < big;
+}
+static PFN_encodeTiled get_encode_fn() {
+    void *fn = nullptr;
+    cudaDriverEntryPointQueryResult qres;
+    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres) != cudaSuccess || !fn ||
+        qres != cudaDriverEntryPointSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    return (PFN_encodeTiled)fn;
 }
 
 static int fast_create(FastState &fs, const Dims &D, bool bf16_mode, cudaStream_t st, int *d_status) {
@@ -52,16 +66,12 @@ static int fast_create(FastState &fs, const Dims &D, bool bf16_mode, cudaStream_
     fs.d_status = d_status;
     fs.a_rows = (size_t)NFD_MAX_PASS_FRAMES * D.T;
     if (!bf16_mode) return NFD_OK;
-    void *fn = nullptr;
-    cudaDriverEntryPointQueryResult qres;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres) != cudaSuccess || !fn ||
-        qres != cudaDriverEntryPointSuccess) {
+    fs.encode = get_encode_fn();
+    if (!fs.encode) {
         // no silent change of path: without tensor maps a bf16 context would run the plain validation kernels
-        cudaGetLastError();
         fprintf(stderr, "libnfd: the driver does not provide cuTensorMapEncodeTiled; a bf16 context needs it\n");
         return NFD_E_CUDA;
     }
-    fs.encode = (PFN_encodeTiled)fn;
     int dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&fs.n_sm, cudaDevAttrMultiProcessorCount, dev);
@@ -79,17 +89,18 @@ static int fast_create(FastState &fs, const Dims &D, bool bf16_mode, cudaStream_
         const int target = fs.n_sm / items_per_pass > 1 ? fs.n_sm / items_per_pass : 1;
         pl.CH = ((D.W + 1) * pl.BPF + target - 1) / target;
         pl.MAXSPLIT = ((D.W + 1) * pl.BPF + pl.CH - 1) / pl.CH;
-        if (pl.MAXSPLIT > 1) {
-            const size_t tiles = (size_t)NFD_MAX_PASS_FRAMES * D.H * pl.QT;
-            if (cudaMalloc((void **)&fs.part_o, tiles * pl.MAXSPLIT * (size_t)ATTN_STATE_BYTES) != cudaSuccess ||
-                cudaMalloc((void **)&fs.attn_counters, tiles * sizeof(unsigned int)) != cudaSuccess ||
-                cudaMemset(fs.attn_counters, 0, tiles * sizeof(unsigned int)) != cudaSuccess) {
-                cudaGetLastError();
-                return NFD_E_NOMEM;
+        if (attn_divisors(pl, D.H, (long long)NFD_MAX_PASS_FRAMES * D.H * pl.QT * pl.MAXSPLIT, D.W)) {
+            if (pl.MAXSPLIT > 1) {
+                const size_t tiles = (size_t)NFD_MAX_PASS_FRAMES * D.H * pl.QT;
+                if (cudaMalloc((void **)&fs.part_o, tiles * pl.MAXSPLIT * (size_t)ATTN_STATE_BYTES) != cudaSuccess ||
+                    cudaMalloc((void **)&fs.attn_counters, tiles * sizeof(unsigned int)) != cudaSuccess ||
+                    cudaMemset(fs.attn_counters, 0, tiles * sizeof(unsigned int)) != cudaSuccess) {
+                    cudaGetLastError();
+                    return NFD_E_NOMEM;
+                }
             }
+            fs.plan = pl;
         }
-        attn_divisors(pl, D.H);
-        fs.plan = pl;
     }
     return NFD_OK;
 }
@@ -315,34 +326,41 @@ static bool fast_gemm(bool enabled, FastState &fs, cudaStream_t st, const TS *A,
 }
 
 template <int KB>
-static int launch_attn_tc(FastState &fs, cudaStream_t st, const StepParams *sp, const Dims &D, int nf, int layer,
-                          const bf16 *q, const bf16 *kc, const bf16 *vc, bf16 *out) {
+static int launch_attn_tc(PFN_encodeTiled encode, int n_sm, cudaStream_t st, const StepParams *sp, const Dims &D, int nf,
+                          int layer, const AttnPlan &pl, size_t pages, const bf16 *q, const bf16 *kc, const bf16 *vc,
+                          bf16 *out, float *part_o, unsigned int *counters, int *status) {
     using A = AttnCfg<KB>;
-    static bool attr_set = false;
     auto kern = k_attn_tc<KB>;
-    if (!attr_set) {
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, A::SMEM) != cudaSuccess) {
-            cudaGetLastError();
-            return 0;
-        }
-        attr_set = true;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, A::SMEM) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
     }
     CUtensorMap mq, mk, mv;
-    if (!encode_map_3d(fs.encode, &mq, q, D.H, nf * D.T, D.dh, 128) ||
-        !encode_map_3d(fs.encode, &mk, kc, fs.cache_pages, D.T, D.dh, KB) ||
-        !encode_map_3d(fs.encode, &mv, vc, fs.cache_pages, D.T, D.dh, KB))
+    if (!encode_map_3d(encode, &mq, q, D.H, nf * D.T, D.dh, 128) || !encode_map_3d(encode, &mk, kc, pages, D.T, D.dh, KB) ||
+        !encode_map_3d(encode, &mv, vc, pages, D.T, D.dh, KB))
         return 0;
-    const AttnPlan &pl = fs.plan;
     const int n_items = pl.MAXSPLIT * pl.QT * D.H * nf;
-    dim3 grid(n_items < fs.n_sm ? n_items : fs.n_sm);
+    dim3 grid(n_items < n_sm ? n_items : n_sm);
     cudaError_t e = launch_pdl(kern, grid, dim3(A::THREADS), (size_t)A::SMEM, st, 1, mq, mk, mv, sp, D, layer, pl, n_items,
-                               out, fs.part_o, fs.attn_counters, fs.d_status);
+                               out, part_o, counters, status);
     if (e != cudaSuccess) {
         fprintf(stderr, "libnfd: tensor-core attention launch failed: %s\n", cudaGetErrorString(e));
         cudaGetLastError();
         return 0;
     }
     return 1;
+}
+
+// Attention of a pass by plan `pl` over `pages` (stream, layer, ring slot, head) pages of K and V.
+static int launch_attn_plan(PFN_encodeTiled encode, int n_sm, cudaStream_t st, const StepParams *sp, const Dims &D, int nf,
+                            int layer, const AttnPlan &pl, size_t pages, const bf16 *q, const bf16 *kc, const bf16 *vc,
+                            bf16 *out, float *part_o, unsigned int *counters, int *status) {
+    switch (pl.KB) {
+        case 128: return launch_attn_tc<128>(encode, n_sm, st, sp, D, nf, layer, pl, pages, q, kc, vc, out, part_o, counters, status);
+        case 112: return launch_attn_tc<112>(encode, n_sm, st, sp, D, nf, layer, pl, pages, q, kc, vc, out, part_o, counters, status);
+        case 96: return launch_attn_tc<96>(encode, n_sm, st, sp, D, nf, layer, pl, pages, q, kc, vc, out, part_o, counters, status);
+        default: return launch_attn_tc<64>(encode, n_sm, st, sp, D, nf, layer, pl, pages, q, kc, vc, out, part_o, counters, status);
+    }
 }
 
 // Returns the number of kernels launched (0: not handled, use the plain kernel).
@@ -353,9 +371,7 @@ static int fast_attention(bool enabled, FastState &fs, cudaStream_t st, const St
         return 0;
     } else {
         if (!enabled || !fs.ready || fs.plan.KB == 0) return 0;
-        if (fs.plan.KB == 128) return launch_attn_tc<128>(fs, st, sp, D, nf, layer, q, kc, vc, out);
-        if (fs.plan.KB == 112) return launch_attn_tc<112>(fs, st, sp, D, nf, layer, q, kc, vc, out);
-        if (fs.plan.KB == 96) return launch_attn_tc<96>(fs, st, sp, D, nf, layer, q, kc, vc, out);
-        return launch_attn_tc<64>(fs, st, sp, D, nf, layer, q, kc, vc, out);
+        return launch_attn_plan(fs.encode, fs.n_sm, st, sp, D, nf, layer, fs.plan, fs.cache_pages, q, kc, vc, out, fs.part_o,
+                                fs.attn_counters, fs.d_status);
     }
 }

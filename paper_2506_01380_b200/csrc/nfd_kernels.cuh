@@ -1,6 +1,6 @@
 // Plain CUDA kernels of libnfd: conditioning, patch embedding, adaLN norm,
-// epilogue functors shared by every GEMM, a straightforward tiled GEMM and a
-// straightforward attention kernel (both used in fp32 validation mode and as
+// epilogue functors shared by every GEMM, a straightforward tiled GEMM and an
+// attention kernel on the fp32 pipes (both used in fp32 validation mode and as
 // the "fast = 0" path in bf16 mode), sampler glue, cache digest / read-out.
 #pragma once
 #include "nfd_common.cuh"
@@ -854,50 +854,137 @@ __global__ void __launch_bounds__(256) k_gemm_simple(const StepParams *sp, int T
 }
 
 // ---------------------------------------------------------------------------
-// Straightforward block-wise causal attention (Section 3.1): one warp per
-// (query token, head); keys are walked frame page by frame page over the
-// query frame's window, so the mask is a page range and never a matrix.
-// Lanes split the head dimension; online softmax in fp32.
+// Block-wise causal attention (Section 3.1) on the fp32 pipes: fp32 storage, bf16
+// with head dimension 128, and the "fast = 0" path.  A CTA takes 16 queries of one
+// (frame, head); its eight warps take the 32-key tiles of the query frame's window
+// in turn, page by page, so that the mask is a page range and never a matrix, each
+// with an online softmax of its own, merged at the end.
+// Bound by FMA and shared-memory issue: per tile and warp 2 x 16 x DH FMAs per lane
+// and a 16-byte shared-memory word for every four of them.  In S = Q K^T a lane owns a
+// key (its row comes straight from the page, the queries are shared-memory
+// broadcasts), in O += P V a lane owns DH/32 columns (V rows are read coalesced, P is
+// a broadcast); no sum over lanes is taken until the end, and the maximum over lanes
+// only where a tile raises it.  (One warp per query with a sum over lanes per key, as
+// it was: 139 us for 6 heads x 32, 2 x 77 queries, 462 keys in fp32.)
 // ---------------------------------------------------------------------------
+#define ATTN_ROWS_Q 16
 template <typename TS, int DH>
-__global__ void __launch_bounds__(128) k_attn_simple(const StepParams *sp, Dims D, int layer, const TS *q,
-                                                     const TS *kc, const TS *vc, TS *out) {
-    constexpr int R = DH / 32;
+__global__ void __launch_bounds__(256) k_attn_rows(const StepParams *sp, Dims D, int layer, const TS *q, const TS *kc,
+                                                   const TS *vc, TS *out) {
+    constexpr int R = DH / 32, NQ = ATTN_ROWS_Q, PS = NQ + 4, NV = WVec<TS>::N;
+    __shared__ __align__(16) float s_q[NQ][DH];
+    __shared__ __align__(16) float s_p[8][32 * PS];              // P of a tile: [key][query]; later O of a column slice
+    __shared__ float s_m[8][NQ], s_l[8][NQ];
     pdl_wait();
     pdl_launch();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int j = blockIdx.z, h = blockIdx.y, row0 = blockIdx.x * NQ;
     const int Nq = sp->nf * D.T;
-    const long long w = (long long)blockIdx.x * (blockDim.x >> 5) + warp;
-    if (w >= (long long)Nq * D.H) return;
-    const int m = (int)(w / D.H), h = (int)(w % D.H);
-    const FrameDesc fr = sp->fr[m / D.T];
-    float qv[R], acc[R];
+    const FrameDesc fr = sp->fr[j];
+    const float c = 1.4426950408889634f / sqrtf((float)DH);      // scores in the log2 domain
+    for (int i = threadIdx.x * NV; i < NQ * DH; i += 256 * NV) {
+        const int r = i / DH, e = i - r * DH;
+        float f[NV];
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-        qv[r] = to_f(q[((size_t)h * Nq + m) * DH + lane + 32 * r]);
-        acc[r] = 0.f;
+        for (int u = 0; u < NV; ++u) f[u] = 0.f;
+        if (row0 + r < D.T) WVec<TS>::load(q + ((size_t)h * Nq + j * D.T + row0 + r) * DH + e, f);
+#pragma unroll
+        for (int u = 0; u < NV; ++u) s_q[r][e + u] = f[u] * c;
     }
-    const float scale = rsqrtf((float)DH);
-    float mx = -INFINITY, l = 0.f;
-    for (int g = fr.win_first; g <= fr.frame; ++g) {
-        const size_t off = kv_page_offset(D, fr.stream, layer, g) + (size_t)h * D.T * DH;
-        const TS *kp = kc + off, *vp = vc + off;
-        for (int j = 0; j < D.T; ++j) {
-            float s = 0.f;
+    __syncthreads();
+    float O[NQ][R], m[NQ], l[NQ];                                // m the same in every lane, l a lane's own part
 #pragma unroll
-            for (int r = 0; r < R; ++r) s = fmaf(qv[r], to_f(kp[(size_t)j * DH + lane + 32 * r]), s);
-            s = warp_sum(s) * scale;
-            const float mn = fmaxf(mx, s);
-            const float corr = expf(mx - mn), p = expf(s - mn);
-            l = l * corr + p;
+    for (int i = 0; i < NQ; ++i) {
+        m[i] = -INFINITY, l[i] = 0.f;
 #pragma unroll
-            for (int r = 0; r < R; ++r) acc[r] = fmaf(p, to_f(vp[(size_t)j * DH + lane + 32 * r]), acc[r] * corr);
-            mx = mn;
+        for (int r = 0; r < R; ++r) O[i][r] = 0.f;
+    }
+    const int tpp = (D.T + 31) / 32, n_tiles = (fr.frame - fr.win_first + 1) * tpp;
+    float *pw = s_p[warp];
+    for (int t = warp; t < n_tiles; t += 8) {
+        const int pg = t / tpp, k0 = (t - pg * tpp) * 32, nk = min(32, D.T - k0);
+        const size_t off = kv_page_offset(D, fr.stream, layer, fr.win_first + pg) + ((size_t)h * D.T + k0) * DH;
+        const TS *krow = kc + off + (size_t)min(lane, nk - 1) * DH;
+        float s[NQ];
+#pragma unroll
+        for (int i = 0; i < NQ; ++i) s[i] = 0.f;
+#pragma unroll 2
+        for (int e = 0; e < DH; e += NV) {
+            float kf[NV];
+            WVec<TS>::load(krow + e, kf);
+#pragma unroll
+            for (int i = 0; i < NQ; ++i)
+#pragma unroll
+                for (int u = 0; u < NV; u += 4) {
+                    const float4 qv = *reinterpret_cast<const float4 *>(&s_q[i][e + u]);
+                    s[i] = fmaf(qv.x, kf[u], s[i]);
+                    s[i] = fmaf(qv.y, kf[u + 1], s[i]);
+                    s[i] = fmaf(qv.z, kf[u + 2], s[i]);
+                    s[i] = fmaf(qv.w, kf[u + 3], s[i]);
+                }
+        }
+        float p[NQ];
+#pragma unroll
+        for (int i = 0; i < NQ; ++i) {
+            if (lane >= nk) s[i] = -INFINITY;
+            if (__any_sync(0xffffffffu, s[i] > m[i])) {
+                const float mn = fmaxf(m[i], warp_max(s[i])), f = exp2f(m[i] - mn);
+                m[i] = mn, l[i] *= f;
+#pragma unroll
+                for (int r = 0; r < R; ++r) O[i][r] *= f;
+            }
+            p[i] = exp2f(s[i] - m[i]);
+            l[i] += p[i];
+        }
+        __syncwarp();                                            // the last tile's P has been read
+#pragma unroll
+        for (int i = 0; i < NQ; i += 4) *reinterpret_cast<float4 *>(pw + lane * PS + i) = make_float4(p[i], p[i + 1], p[i + 2], p[i + 3]);
+        __syncwarp();
+        const TS *vrow = vc + off + lane;
+#pragma unroll 4
+        for (int kk = 0; kk < nk; ++kk) {
+            float v[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) v[r] = to_f(vrow[(size_t)kk * DH + 32 * r]);
+#pragma unroll
+            for (int i = 0; i < NQ; i += 4) {
+                const float4 pv = *reinterpret_cast<const float4 *>(pw + kk * PS + i);
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    O[i][r] = fmaf(pv.x, v[r], O[i][r]), O[i + 1][r] = fmaf(pv.y, v[r], O[i + 1][r]);
+                    O[i + 2][r] = fmaf(pv.z, v[r], O[i + 2][r]), O[i + 3][r] = fmaf(pv.w, v[r], O[i + 3][r]);
+                }
+            }
         }
     }
-    const float inv = 1.0f / l;
+    // merge the warps' states, 32 columns at a time
 #pragma unroll
-    for (int r = 0; r < R; ++r) out[(size_t)m * D.d + h * DH + lane + 32 * r] = from_f<TS>(acc[r] * inv);
+    for (int i = 0; i < NQ; ++i) {
+        const float ls = warp_sum(l[i]);
+        if (lane == 0) s_m[warp][i] = m[i], s_l[warp][i] = ls;
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        __syncthreads();                                         // P (and the slice before) has been read
+#pragma unroll
+        for (int i = 0; i < NQ; ++i) pw[i * 32 + lane] = O[i][r];
+        __syncthreads();
+#pragma unroll
+        for (int i = warp; i < NQ; i += 8) {
+            float mx = s_m[0][i];
+#pragma unroll
+            for (int w = 1; w < 8; ++w) mx = fmaxf(mx, s_m[w][i]);
+            float num = 0.f, den = 0.f;
+#pragma unroll
+            for (int w = 0; w < 8; ++w) {
+                // (a warp without a tile has m = -inf and counts for nothing)
+                const float wgt = s_m[w][i] == -INFINITY ? 0.f : exp2f(s_m[w][i] - mx);
+                den = fmaf(s_l[w][i], wgt, den);
+                num = fmaf(s_p[w][i * 32 + lane], wgt, num);
+            }
+            if (row0 + i < D.T) out[(size_t)(j * D.T + row0 + i) * D.d + h * DH + 32 * r + lane] = from_f<TS>(num / den);
+        }
+    }
 }
 
 // ---------------------------------------------------------------------------

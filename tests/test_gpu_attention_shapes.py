@@ -51,3 +51,26 @@ def test_pages_and_tiles(hw, head_dim, heads, n_kv, n_q, window, rise):
     assert np.abs(got - ref).max() <= TOL_ABS
     assert np.linalg.norm(got - ref) / np.linalg.norm(ref) <= TOL_REL
     assert g.status() == 0
+
+
+@pytest.mark.parametrize("kind,heads,T,dh,n_kv,n_q,window", [
+    ("bf16", 3, 77, 32, 9, 2, 5), ("bf16", 5, 129, 64, 4, 2, 9), ("bf16", 16, 336, 64, 6, 4, 3),
+    ("bf16", 2, 33, 128, 5, 3, 2), ("fp32", 6, 77, 32, 9, 2, 5), ("fp32", 2, 16, 64, 1, 1, 0), ("fp32", 1, 1, 128, 3, 1, 2),
+    ("fp32", 3, 65, 128, 3, 2, 1)])
+def test_pages_of_the_caller(kind, heads, T, dh, n_kv, n_q, window):
+    """The allocation-free call: pages and query tiles that 16, 32 and the key block do not divide, windows longer
+    than the pages given.  fp32: sums of at most 700 products of order one, 1e-4 as in the other fp32 cases."""
+    import torch
+    from paper_2506_01380_b200 import nfd as N
+    tdt = torch.bfloat16 if kind == "bf16" else torch.float32
+    q, k, v = I.make_qkv(heads, dh, n_q * T, n_kv * T, seed=T + dh, bf16=kind == "bf16")
+    tq, tk, tv = [torch.as_tensor(a).cuda().to(tdt) for a in (q, k, v)]
+    pages = lambda x: x.view(heads, n_kv, T, dh).permute(1, 0, 2, 3).contiguous()
+    out = torch.full((n_q * T, heads * dh), float("nan"), device="cuda", dtype=tdt)
+    N.attention_noalloc(tq, pages(tk), pages(tv), n_q, window, out)
+    got = out.float().cpu().numpy().astype(np.float64)
+    ref = O.attention_block_causal(q, k, v, np.repeat(np.arange(n_kv - n_q, n_kv), T), np.repeat(np.arange(n_kv), T),
+                                   window).transpose(1, 0, 2).reshape(n_q * T, heads * dh)
+    tol = (TOL_ABS, TOL_REL) if kind == "bf16" else (1e-4, 1e-4)
+    assert np.all(np.isfinite(got))
+    assert np.abs(got - ref).max() <= tol[0] and np.linalg.norm(got - ref) / np.linalg.norm(ref) <= tol[1]
