@@ -443,6 +443,7 @@ static int tune_gemms(nfd_ctx *c) {
     const size_t mod_row = (size_t)D.L * 6 * d, uv_row = (size_t)D.L * (3 * d + D.n1);
     struct Kind { int tc, N, K; };
     const Kind kinds[4] = {{TC_QKV, 3 * d, d}, {TC_RES, d, d}, {TC_GELU, D.n1, d}, {TC_RES, d, D.dm}};
+    const int forms[4] = {FORM_QKV, FORM_RES, FORM_MLP, FORM_RES};
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
@@ -490,7 +491,7 @@ static int tune_gemms(nfd_ctx *c) {
         return ok;
     };
     const int nfs[] = {1, 2, 3, 4, 5, 6, 8, 12, 16, 24, 32};
-    const int widths[] = {32, 64, 96, 128, 192, 256};
+    const int widths[] = {32, 64, 96, 128};
     bool touched = false;
     // the largest pass this context can build: per stream a speculation plus the deferred frames of the last one
     const int nf_max = D.n_streams * 2 * c->cfg.max_spec;
@@ -498,8 +499,13 @@ static int tune_gemms(nfd_ctx *c) {
         if (nf > NFD_MAX_PASS_FRAMES || nf > nf_max) break;
         const int M = nf * T;
         bool need = false;
-        for (const Kind &k : kinds)
-            if (!g_tuned_BN.count(std::make_tuple(k.tc + (k.K > 2048 ? 10 : 0), k.N, k.K, fs.n_sm, M))) need = true;
+        for (int ki = 0; ki < 4; ++ki) {
+            const Kind &k = kinds[ki];
+            const int kk = k.tc + (k.K > 2048 ? 10 : 0);
+            if (!g_tuned_BN.count(std::make_tuple(kk, k.N, k.K, fs.n_sm, M)) &&
+                (!g_tuned_S.count(std::make_tuple(kk, k.N, k.K, fs.n_sm)) || !plan_gemm(fs, M, k.N, k.K, k.tc, forms[ki]).p))
+                need = true;
+        }
         if (!need) continue;
         // a pass descriptor for nf scratch frames of stream 0
         StepParams &p = c->h_sp;
@@ -523,7 +529,10 @@ static int tune_gemms(nfd_ctx *c) {
             const int nkb = (k.K + 63) / 64;
             // the cost model's plan is the incumbent: another one must beat it by 3 % (timing noise must not
             // flip plans between processes without need)
-            const GemmPlan model = plan_gemm(fs, M, k.N, k.K, k.tc);
+            // (k_gemm_p goes by its own rule and is not timed; the split of a one-frame pass is found on k_gemm_tc)
+            GemmPlan model = plan_gemm(fs, M, k.N, k.K, k.tc, forms[ki]);
+            if (model.p && !s_open) continue;
+            if (model.p) model = GemmPlan{128, model.S, false};
             float t_best = 1e30f;
             GemmPlan best = model;
             if (!time_of(ki, M, model.BN, model.S, &t_best)) t_best = 1e30f;
@@ -533,13 +542,12 @@ static int tune_gemms(nfd_ctx *c) {
                 if (S > 1 && nkb / S < 2) continue;
                 for (int BN : widths) {
                     if (BN > 32 && BN > k.N) continue;
-                    if (nf == 1 && BN > 128) continue;
                     if (BN == model.BN && S == model.S) continue;
                     const long long ctas = (long long)((M + 127) / 128) * ((k.N + BN - 1) / BN) * S;
                     if (ctas > 3LL * fs.n_sm) continue;          // hopeless: several waves
                     float t;
                     const bool ok_t = time_of(ki, M, BN, S, &t);
-                    if (ok_t && t < t_best) t_best = t, best = GemmPlan{BN, S};
+                    if (ok_t && t < t_best) t_best = t, best = GemmPlan{BN, S, false};
                 }
             }
             if (s_open) g_tuned_S[skey] = best.S;

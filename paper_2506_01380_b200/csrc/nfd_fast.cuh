@@ -9,6 +9,7 @@
 
 #include "nfd_sm100.cuh"
 #include "nfd_gemm_tc.cuh"
+#include "nfd_gemm_p.cuh"
 #include "nfd_attn_tc.cuh"
 
 enum { TC_NONE = 0, TC_QKV = 1, TC_RES = 2, TC_GELU = 3 };
@@ -21,7 +22,7 @@ struct FastState {
     bool ready = false;
     PFN_encodeTiled encode = nullptr;
     int *d_status = nullptr;
-    int n_sm = 148;
+    int n_sm = 148, dh = 0;
     size_t a_rows = 0;     // rows of every activation buffer (NFD_MAX_PASS_FRAMES * T)
     AttnPlan plan;         // KB == 0: tensor-core attention not available for this shape
     float *part_o = nullptr;           // per-split states of the attention kernel: [query tile][split] x ATTN_STATE_BYTES
@@ -64,7 +65,7 @@ static int fast_create(FastState &fs, const Dims &D, bool bf16_mode, cudaStream_
     (void)st;
     fs.ready = false;
     fs.d_status = d_status;
-    fs.a_rows = (size_t)NFD_MAX_PASS_FRAMES * D.T;
+    fs.a_rows = (size_t)NFD_MAX_PASS_FRAMES * D.T, fs.dh = D.dh;
     if (!bf16_mode) return NFD_OK;
     fs.encode = get_encode_fn();
     if (!fs.encode) {
@@ -91,7 +92,9 @@ static int fast_create(FastState &fs, const Dims &D, bool bf16_mode, cudaStream_
         pl.MAXSPLIT = ((D.W + 1) * pl.BPF + pl.CH - 1) / pl.CH;
         if (attn_divisors(pl, D.H, (long long)NFD_MAX_PASS_FRAMES * D.H * pl.QT * pl.MAXSPLIT, D.W)) {
             if (pl.MAXSPLIT > 1) {
-                const size_t tiles = (size_t)NFD_MAX_PASS_FRAMES * D.H * pl.QT;
+                // (the largest pass of this context: per stream a speculation and the deferred frames of the last one)
+                const int nf_max = D.n_streams * (D.R - D.W);
+                const size_t tiles = (size_t)(nf_max < NFD_MAX_PASS_FRAMES ? nf_max : NFD_MAX_PASS_FRAMES) * D.H * pl.QT;
                 if (cudaMalloc((void **)&fs.part_o, tiles * pl.MAXSPLIT * (size_t)ATTN_STATE_BYTES) != cudaSuccess ||
                     cudaMalloc((void **)&fs.attn_counters, tiles * sizeof(unsigned int)) != cudaSuccess ||
                     cudaMemset(fs.attn_counters, 0, tiles * sizeof(unsigned int)) != cudaSuccess) {
@@ -180,7 +183,36 @@ static cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
 // ---------------------------------------------------------------------------
 struct GemmPlan {
     int BN, S;
+    bool p;        // k_gemm_p instead of k_gemm_tc
 };
+
+// Tile width of k_gemm_p for a GEMM [M x N x K] with a K split of S, or 0 where k_gemm_tc is the better one.  The line
+// lies where the row blocks times 128-wide column tiles fill the machine; measured on a 148-SM B200, k_gemm_tc -> k_gemm_p
+// in us with launch, for the projections into QKV and the MLP (K 768 to 1536): 72 tiles 12.9 -> 14.4, 96 tiles 14.9 ->
+// 14.8, 108 tiles 14.7 -> 13.0, 129 tiles 16.5 -> 14.6, 192 tiles 20.6 -> 16.9, 264 tiles 24 -> 19, 672 tiles 52 -> 32;
+// for those onto the residual stream (K 768 to 4096): 64 tiles 19.0 -> 23.0, 72 tiles 21 -> 28, 88 tiles 24.9 -> 23.0,
+// 112 tiles 18.8 -> 15.3, 126 tiles 20.8 -> 14.9, 168 tiles 47 -> 40.
+static int gemm_p_width(int n_sm, int form, int T, int dh, int M, int N, int K, int S) {
+    // a 128-row tile must not span more frames than the kernel keeps tables for; rotary rows of 64 floats at most
+    if (form == FORM_NONE || 127 / T + 2 > GemmPCfg<128, FORM_MLP>::MAX_FR || (form == FORM_QKV && dh > 64)) return 0;
+    const int mt = (M + 127) / 128, t128 = mt * ((N + 127) / 128);
+    if (form == FORM_RES) return t128 >= (88 * n_sm) / 148 ? 128 : 0;
+    if (t128 < (100 * n_sm) / 148) return 0;
+    if (S > 1) return 128;
+    // microseconds: a base and a wave, fitted to K = 768, 1024 and 1536 (within 2 us up to ten waves)
+    const float nkb = (float)((K + 63) / 64);
+    const int bns[3] = {128, 192, 256};
+    const float base[3] = {10.3f, 10.9f, 12.2f};
+    const float wave[3] = {nkb * 0.231f > 4.2f ? nkb * 0.231f : 4.2f, nkb * 0.25f + 1.4f, nkb * 0.4f};
+    int best = 128;
+    float t_best = 1e30f;
+    for (int i = 0; i < 3; ++i) {
+        const int tiles = mt * ((N + bns[i] - 1) / bns[i]);
+        const float t = base[i] + wave[i] * (float)((tiles + n_sm - 1) / n_sm);
+        if (t < t_best) t_best = t, best = bns[i];
+    }
+    return best;
+}
 // Plans found by timing (nfd_create), shared by every context of the process so that two contexts of the same
 // shape always sum in the same order: (kind, N, K, n_sm) -> S, and (kind, N, K, n_sm, M) -> BN.
 static std::map<std::tuple<int, int, int, int>, int> g_tuned_S;
@@ -210,13 +242,17 @@ template <typename Kern> static void query_gemm_slots(FastState &fs, Kern kern, 
     }
 }
 
-static GemmPlan plan_gemm(const FastState &fs, int M, int N, int K, int tc_kind) {
-    if (fs.force_BN) return {fs.force_BN, fs.force_S};
+static GemmPlan plan_gemm(const FastState &fs, int M, int N, int K, int tc_kind, int form) {
+    if (fs.force_BN) return {fs.force_BN, fs.force_S, false};
     const int kind_key = tc_kind + (K > 2048 ? 10 : 0);
     {
         auto is = g_tuned_S.find(std::make_tuple(kind_key, N, K, fs.n_sm));
         auto ib = g_tuned_BN.find(std::make_tuple(kind_key, N, K, fs.n_sm, M));
-        if (is != g_tuned_S.end() && ib != g_tuned_BN.end()) return {ib->second, is->second};
+        if (is != g_tuned_S.end()) {
+            const int bn_p = gemm_p_width(fs.n_sm, form, (int)(fs.a_rows / NFD_MAX_PASS_FRAMES), fs.dh, M, N, K, is->second);
+            if (bn_p) return {bn_p, is->second, true};
+            if (ib != g_tuned_BN.end()) return {ib->second, is->second, false};
+        }
     }
     // Cost in SM cycles, fitted to measurements on B200: an SM takes in operand tiles at about
     // 55 bytes per cycle whatever the ring depth; CTAs that share an SM share that rate.
@@ -257,14 +293,14 @@ static GemmPlan plan_gemm(const FastState &fs, int M, int N, int K, int tc_kind)
         auto is = g_tuned_S.find(std::make_tuple(kind_key, N, K, fs.n_sm));
         if (is != g_tuned_S.end()) S_best = is->second;
     }
-    GemmPlan best{32, S_best};
+    // the tile width follows M
+    if (const int bn_p = gemm_p_width(fs.n_sm, form, T, fs.dh, M, N, K, S_best)) return {bn_p, S_best, true};
+    GemmPlan best{32, S_best, false};
     best_cost = 1e30;
-    // the tile width follows M; passes of several frames may take the wide tiles
-    const int bnw[6] = {32, 64, 96, 128, 192, 256};
-    for (int bi = 0; bi < 6; ++bi) {
-        if (bnw[bi] > 32 && bnw[bi] > N) continue;
-        const double c = cost_of(M, bnw[bi], S_best);
-        if (c < best_cost) best_cost = c, best.BN = bnw[bi];
+    for (int bi = 0; bi < 4; ++bi) {
+        if (bns[bi] > 32 && bns[bi] > N) continue;
+        const double c = cost_of(M, bns[bi], S_best);
+        if (c < best_cost) best_cost = c, best.BN = bns[bi];
     }
     return best;
 }
@@ -304,6 +340,76 @@ static bool launch_gemm_tc(FastState &fs, cudaStream_t st, const bf16 *A, const 
     return launch_gemm_tc_sc<BN, Epi, 0>(fs, st, A, Wt, M, N, K, S, epi, pf);
 }
 
+// Tensor map [pages][rows][cols] (pages = 0: two dimensions) with boxes of 32 rows x box_cols, for the results and side
+// operands of k_gemm_p; the swizzle spans the box's row.
+static bool encode_map_box(const FastState &fs, CUtensorMap *m, const void *ptr, bool f32, size_t pages, int rows, int cols,
+                           int box_cols) {
+    const int es = f32 ? 4 : 2;
+    cuuint64_t gdim[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)pages};
+    cuuint64_t gstr[2] = {(cuuint64_t)cols * es, (cuuint64_t)cols * es * rows};
+    cuuint32_t box[3] = {(cuuint32_t)box_cols, 32, 1};
+    cuuint32_t estr[3] = {1, 1, 1};
+    const int bytes = box_cols * es;
+    CUresult r = fs.encode(m, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, pages ? 3 : 2,
+                           const_cast<void *>(ptr), gdim, gstr, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                           bytes == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : (bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B),
+                           CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) fprintf(stderr, "libnfd: cuTensorMapEncodeTiled failed (%d) for a box of 32 x %d\n", (int)r, box_cols);
+    return r == CUDA_SUCCESS;
+}
+static bool epi_maps(const FastState &fs, const EpiQKV<bf16> &e, int M, int, CUtensorMap *m) {
+    return encode_map_box(fs, m, e.q, false, e.D.H, M, e.D.dh, 32) &&
+           encode_map_box(fs, m + 1, e.kc, false, fs.cache_pages, e.D.T, e.D.dh, 32) &&
+           encode_map_box(fs, m + 2, e.vc, false, fs.cache_pages, e.D.T, e.D.dh, 32) &&
+           encode_map_box(fs, m + 3, e.rope_cs, true, 0, M, e.D.dh, 32);
+}
+static bool epi_maps(const FastState &fs, const EpiGateRes<bf16> &e, int M, int, CUtensorMap *m) {
+    return encode_map_box(fs, m, e.z, true, 0, M, e.D.d, 32) && (!e.a_out || encode_map_box(fs, m + 1, e.a_out, false, 0, M, e.D.d, 32));
+}
+static bool epi_maps(const FastState &fs, const EpiGelu<bf16> &e, int M, int N, CUtensorMap *m) {
+    return encode_map_box(fs, m, e.out, false, 0, M, e.act ? N / 2 : N, e.act ? 16 : 32);
+}
+
+template <int BN, typename Epi, bool SPLIT>
+static bool launch_gemm_p(FastState &fs, cudaStream_t st, const bf16 *A, const bf16 *Wt, int M, int N, int K, int S,
+                          Epi epi, L2Prefetch pf) {
+    using G = GemmPCfg<BN, Epi::kForm>;
+    static bool attr_set = false;
+    auto kern = k_gemm_p<BN, Epi, SPLIT>;
+    if (!attr_set) {
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        attr_set = true;
+    }
+    const CUtensorMap *ma = get_map_2d(fs, A, (int)fs.a_rows, K, 128);
+    const CUtensorMap *mb = get_map_2d(fs, Wt, N, K, BN);
+    CUtensorMap me[4];
+    memset(me, 0, sizeof(me));
+    if (!ma || !mb || !epi_maps(fs, epi, M, N, me)) return false;
+    const int tiles = ((M + 127) / 128) * ((N + BN - 1) / BN);
+    cudaError_t e = launch_pdl(kern, dim3(tiles < fs.n_sm ? tiles : fs.n_sm), dim3(G::THREADS), (size_t)G::SMEM, st, 1, *ma,
+                               *mb, me[0], me[1], me[2], me[3], M, N, K, S, epi, pf, (int)(fs.a_rows / NFD_MAX_PASS_FRAMES),
+                               fs.d_status);
+    if (e != cudaSuccess) {
+        fprintf(stderr, "libnfd: persistent GEMM launch failed (BN %d, S %d): %s\n", BN, S, cudaGetErrorString(e));
+        cudaGetLastError();
+        return false;
+    }
+    return true;
+}
+template <typename Epi>
+static bool launch_gemm_p_any(FastState &fs, cudaStream_t st, const bf16 *A, const bf16 *Wt, int M, int N, int K, int BN,
+                              int S, Epi epi, L2Prefetch pf) {
+    if (S > 1) return launch_gemm_p<128, Epi, true>(fs, st, A, Wt, M, N, K, S, epi, pf);
+    if constexpr (Epi::kForm != FORM_RES) {
+        if (BN == 256) return launch_gemm_p<256, Epi, false>(fs, st, A, Wt, M, N, K, S, epi, pf);
+        if (BN == 192) return launch_gemm_p<192, Epi, false>(fs, st, A, Wt, M, N, K, S, epi, pf);
+    }
+    return launch_gemm_p<128, Epi, false>(fs, st, A, Wt, M, N, K, S, epi, pf);
+}
+
 template <typename TS, typename Epi>
 static bool fast_gemm(bool enabled, FastState &fs, cudaStream_t st, const TS *A, const TS *Wt, int M, int N, int K,
                       Epi epi, int tc_kind, L2Prefetch pf) {
@@ -313,10 +419,11 @@ static bool fast_gemm(bool enabled, FastState &fs, cudaStream_t st, const TS *A,
         if (!enabled || !fs.ready) return false;
         if (K % 8 || K < 64 || N < 32 || (N & 7)) return false;
         if (((uintptr_t)A & 15) || ((uintptr_t)Wt & 15)) return false;
-        const GemmPlan pl = plan_gemm(fs, M, N, K, tc_kind);
+        const GemmPlan pl = plan_gemm(fs, M, N, K, tc_kind, Epi::kForm);
+        if constexpr (Epi::kForm != FORM_NONE) {
+            if (pl.p) return launch_gemm_p_any<Epi>(fs, st, A, Wt, M, N, K, pl.BN, pl.S, epi, pf);
+        }
         switch (pl.BN) {
-            case 256: return launch_gemm_tc<256, Epi>(fs, st, A, Wt, M, N, K, pl.S, epi, pf);
-            case 192: return launch_gemm_tc<192, Epi>(fs, st, A, Wt, M, N, K, pl.S, epi, pf);
             case 128: return launch_gemm_tc<128, Epi>(fs, st, A, Wt, M, N, K, pl.S, epi, pf);
             case 96: return launch_gemm_tc<96, Epi>(fs, st, A, Wt, M, N, K, pl.S, epi, pf);
             case 64: return launch_gemm_tc<64, Epi>(fs, st, A, Wt, M, N, K, pl.S, epi, pf);

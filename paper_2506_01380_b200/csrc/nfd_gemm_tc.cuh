@@ -34,11 +34,10 @@ template <int BN> struct GemmCfg {
     // A ring stage holds KU k-blocks of 64 elements.  A stage costs the producer about 280 clocks of barrier
     // operations and 40 per TMA instruction whatever its size, an SM takes in up to 120 bytes per clock: with
     // one 64-element block per stage the producer's own instructions set the pace (128 + 64 rows: 380 clocks per
-    // block, 65 bytes per clock), with two the SM's intake does (220 clocks per block).  A 256-wide tile
-    // brings 48 KB per block, which is enough for a stage.
-    static constexpr int KU = BN <= 192 ? 2 : 1;
+    // block, 65 bytes per clock), with two the SM's intake does (220 clocks per block).
+    static constexpr int KU = 2;
     // ring deep enough that one CTA owns an SM
-    static constexpr int STAGES = BN <= 64 ? 4 : (BN <= 128 ? 3 : (BN <= 192 ? 2 : 3));
+    static constexpr int STAGES = BN <= 64 ? 4 : 3;
     static constexpr int A_BYTES = 128 * 128;                  // 128 rows x 64 bf16
     static constexpr int B_BYTES = BN * 128;
     static constexpr int KB_BYTES = A_BYTES + B_BYTES;
@@ -46,7 +45,7 @@ template <int BN> struct GemmCfg {
     static constexpr int RING_BYTES = STAGES * ST_BYTES;
     static constexpr int SROW = BN + 4;                        // staging row stride (floats)
     static constexpr int STAGE_BYTES = 128 * SROW * 4;         // partial accumulator tile; reuses the ring
-    static constexpr int TMEM_COLS = BN <= 32 ? 32 : (BN <= 64 ? 64 : (BN <= 128 ? 128 : 256));
+    static constexpr int TMEM_COLS = BN <= 32 ? 32 : (BN <= 64 ? 64 : 128);
     static constexpr int UV_BYTES = LnFold::kMaxFrames * BN * 8;   // folded LayerNorm: (u, v) per frame and column
     static constexpr int TAB_BYTES = 128 * 16 + (BN / 8) * 32 + 128;   // epilogue row and column tables, row -> frame
     static constexpr int SMEM = RING_BYTES + 1024 /*align*/ + 256 /*barriers*/ + 1024 /*row statistics*/ + UV_BYTES +

@@ -502,6 +502,33 @@ __device__ __forceinline__ void ln_fold_apply(float *a, const float4 *uv, int st
         a[2 * i + 1] = fmaf(ms.y, fmaf(-ms.x, w.z, a[2 * i + 1]), w.w);
     }
 }
+// Pieces of the epilogues that k_gemm_tc (items of 8 columns) and k_gemm_p (rows of 32 columns) share.  Every
+// rounding is spelled out: a row's bits must not depend on which of the two kernels computed it.
+// (cos, sin) of two adjacent pairs applied to four columns
+__device__ __forceinline__ void rope4(float *a, const float4 &cs) {
+    const float r0 = fmaf(a[0], cs.x, -__fmul_rn(a[1], cs.y)), r1 = fmaf(a[0], cs.y, __fmul_rn(a[1], cs.x));
+    const float r2 = fmaf(a[2], cs.z, -__fmul_rn(a[3], cs.w)), r3 = fmaf(a[2], cs.w, __fmul_rn(a[3], cs.z));
+    a[0] = r0, a[1] = r1, a[2] = r2, a[3] = r3;
+}
+// (sum, sum of squares) of 4 values
+__device__ __forceinline__ float2 sums4(const float *z) {
+    auto q = [](float x, float y) { return fmaf(x, x, __fmul_rn(y, y)); };
+    return make_float2((z[0] + z[1]) + (z[2] + z[3]), q(z[0], z[1]) + q(z[2], z[3]));
+}
+__device__ __forceinline__ void gelu4(float *a) {
+#pragma unroll
+    for (int i = 0; i < 4; i += 2) {
+        const float2 g = gelu_erf_bf16_f2(make_float2(a[i], a[i + 1]));
+        a[i] = g.x, a[i + 1] = g.y;
+    }
+}
+// SiLU(gate) * up of two interleaved pairs, as a bf16 pair
+__device__ __forceinline__ uint32_t gated4(const float *a) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(__fmul_rn(silu_fast_f(a[0]), a[1]), __fmul_rn(silu_fast_f(a[2]), a[3]));
+    return *reinterpret_cast<const uint32_t *>(&h);
+}
+// Which epilogue k_gemm_p (nfd_gemm_p.cuh) runs for a functor.
+enum { FORM_NONE = 0, FORM_QKV, FORM_RES, FORM_MLP };
 __device__ __forceinline__ void bias_add(float *a, const uint4 &bits) {
     float b[8];
     unpack_bf16x8(bits, b);
@@ -590,21 +617,20 @@ template <typename TS> struct EpiQKV {
         else
             bias_add(a, s.bias);
         TS *dst;
-        if (which < 2) {
-            const float cv[4] = {s.c01.x, s.c01.z, s.c23.x, s.c23.z}, sv[4] = {s.c01.y, s.c01.w, s.c23.y, s.c23.w};
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const float r0 = a[2 * i] * cv[i] - a[2 * i + 1] * sv[i];
-                const float r1 = a[2 * i] * sv[i] + a[2 * i + 1] * cv[i];
-                a[2 * i] = r0;
-                a[2 * i + 1] = r1;
-            }
-        }
+        if (which < 2) rope4(a, s.c01), rope4(a + 4, s.c23);
         if (which == 0)
             dst = q + (row.q_off + col.q_off);
         else
             dst = ((which == 1) ? kc : vc) + (row.kv_off + col.kv_off);
         *reinterpret_cast<uint4 *>(dst) = pack_bf16x8(a);
+    }
+    // ---- k_gemm_p: a tile's table holds kTab values per frame and column ----
+    static constexpr int kForm = FORM_QKV, kTab = 2;           // u, v
+    __device__ __forceinline__ int cond_row(int fr) const { return sp->fr[fr].cond_row; }
+    __device__ __forceinline__ void tab(int row, int n, float *t) const {
+        // without the fold: mean 0, rstd 1, u 0 and the bias in the place of v
+        const float2 w = ln.on() ? ln.uv[(size_t)row * ln.row_stride + n] : make_float2(0.f, to_f(bias[n]));
+        t[0] = w.x, t[1] = w.y;
     }
     __device__ __forceinline__ void operator()(int m, int n, float a0, float a1) const {
         a0 += to_f(bias[n]);
@@ -674,33 +700,34 @@ template <typename TS> struct EpiGateRes {
                                           unsigned mask, const Row &, const Col &) const {
         float b[8];
         unpack_bf16x8(s.bias, b);
-        float4 z0 = s.z0, z1 = s.z1;
-        z0.x = fmaf(s.g0.x, a[0] + b[0], z0.x);
-        z0.y = fmaf(s.g0.y, a[1] + b[1], z0.y);
-        z0.z = fmaf(s.g0.z, a[2] + b[2], z0.z);
-        z0.w = fmaf(s.g0.w, a[3] + b[3], z0.w);
-        z1.x = fmaf(s.g1.x, a[4] + b[4], z1.x);
-        z1.y = fmaf(s.g1.y, a[5] + b[5], z1.y);
-        z1.z = fmaf(s.g1.z, a[6] + b[6], z1.z);
-        z1.w = fmaf(s.g1.w, a[7] + b[7], z1.w);
+        const float g[8] = {s.g0.x, s.g0.y, s.g0.z, s.g0.w, s.g1.x, s.g1.y, s.g1.z, s.g1.w};
+        float zn[8] = {s.z0.x, s.z0.y, s.z0.z, s.z0.w, s.z1.x, s.z1.y, s.z1.z, s.z1.w};
+#pragma unroll
+        for (int i = 0; i < 8; ++i) zn[i] = fmaf(g[i], a[i] + b[i], zn[i]);
         float4 *zp = reinterpret_cast<float4 *>(z + (size_t)m * D.d + n);
-        zp[0] = z0;
-        zp[1] = z1;
+        zp[0] = make_float4(zn[0], zn[1], zn[2], zn[3]);
+        zp[1] = make_float4(zn[4], zn[5], zn[6], zn[7]);
         if (stats) {
             if (a_out) {
-                float o[8] = {z0.x * (1.0f + s.s0.x), z0.y * (1.0f + s.s0.y), z0.z * (1.0f + s.s0.z),
-                              z0.w * (1.0f + s.s0.w), z1.x * (1.0f + s.s1.x), z1.y * (1.0f + s.s1.y),
-                              z1.z * (1.0f + s.s1.z), z1.w * (1.0f + s.s1.w)};
+                const float sc[8] = {s.s0.x, s.s0.y, s.s0.z, s.s0.w, s.s1.x, s.s1.y, s.s1.z, s.s1.w};
+                float o[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) o[i] = zn[i] * (1.0f + sc[i]);
                 *reinterpret_cast<uint4 *>(a_out + (size_t)m * D.d + n) = pack_bf16x8(o);
             }
             // the four lanes of a 32-column group hold the same row and are valid together
-            float s1 = ((z0.x + z0.y) + (z0.z + z0.w)) + ((z1.x + z1.y) + (z1.z + z1.w));
-            float s2 = ((z0.x * z0.x + z0.y * z0.y) + (z0.z * z0.z + z0.w * z0.w)) +
-                       ((z1.x * z1.x + z1.y * z1.y) + (z1.z * z1.z + z1.w * z1.w));
-            s1 += __shfl_xor_sync(mask, s1, 1), s2 += __shfl_xor_sync(mask, s2, 1);
-            s1 += __shfl_xor_sync(mask, s1, 2), s2 += __shfl_xor_sync(mask, s2, 2);
-            if ((n & 31) == 0) stats[(size_t)m * (D.d >> 5) + (n >> 5)] = make_float2(s1, s2);
+            const float2 ta = sums4(zn), tb = sums4(zn + 4);
+            float2 t = make_float2(ta.x + tb.x, ta.y + tb.y);
+            t.x += __shfl_xor_sync(mask, t.x, 1), t.y += __shfl_xor_sync(mask, t.y, 1);
+            t.x += __shfl_xor_sync(mask, t.x, 2), t.y += __shfl_xor_sync(mask, t.y, 2);
+            if ((n & 31) == 0) stats[(size_t)m * (D.d >> 5) + (n >> 5)] = t;
         }
+    }
+    static constexpr int kForm = FORM_RES, kTab = 3;           // k_gemm_p: bias, gate, 1 + scale_next
+    __device__ __forceinline__ int cond_row(int fr) const { return sp->fr[fr].cond_row; }
+    __device__ __forceinline__ void tab(int row, int n, float *t) const {
+        const size_t off = (size_t)row * row_stride + n;
+        t[0] = to_f(bias[n]), t[1] = gate[off], t[2] = a_out ? 1.0f + scale_next[off] : 0.f;
     }
     __device__ __forceinline__ void operator()(int m, int n, float a0, float a1) const {
         const int row = sp->fr[m / D.T].cond_row;
@@ -738,19 +765,17 @@ template <typename TS> struct EpiGelu {
         else
             bias_add(a, s.bias);
         if (act == 0) {
-#pragma unroll
-            for (int i = 0; i < 8; i += 2) {
-                const float2 g = gelu_erf_bf16_f2(make_float2(a[i], a[i + 1]));
-                a[i] = g.x, a[i + 1] = g.y;
-            }
+            gelu4(a), gelu4(a + 4);
             *reinterpret_cast<uint4 *>(out + (size_t)m * N + n) = pack_bf16x8(a);
         } else {
-            uint2 o;
-            __nv_bfloat162 *h = reinterpret_cast<__nv_bfloat162 *>(&o);
-            h[0] = __floats2bfloat162_rn(silu_fast_f(a[0]) * a[1], silu_fast_f(a[2]) * a[3]);
-            h[1] = __floats2bfloat162_rn(silu_fast_f(a[4]) * a[5], silu_fast_f(a[6]) * a[7]);
-            *reinterpret_cast<uint2 *>(out + (size_t)m * (N >> 1) + (n >> 1)) = o;
+            *reinterpret_cast<uint2 *>(out + (size_t)m * (N >> 1) + (n >> 1)) = make_uint2(gated4(a), gated4(a + 4));
         }
+    }
+    static constexpr int kForm = FORM_MLP, kTab = 2;           // k_gemm_p: u, v
+    __device__ __forceinline__ int cond_row(int fr) const { return ln.sp->fr[fr].cond_row; }
+    __device__ __forceinline__ void tab(int row, int n, float *t) const {
+        const float2 w = ln.on() ? ln.uv[(size_t)row * ln.row_stride + n] : make_float2(0.f, to_f(bias[n]));
+        t[0] = w.x, t[1] = w.y;
     }
     __device__ __forceinline__ void operator()(int m, int n, float a0, float a1) const {
         if (act) {
@@ -772,6 +797,7 @@ template <typename TS> struct EpiFinal {
     static constexpr int kBatch = 4;        // epilogue items a thread keeps in flight together
     static constexpr bool kRowStats = false;
     static constexpr bool kTables = false;
+    static constexpr int kForm = FORM_NONE;
     struct Row {};
     struct Col {};
     struct Side {
