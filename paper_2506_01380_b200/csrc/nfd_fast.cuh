@@ -449,7 +449,7 @@ static int launch_attn_tc(PFN_encodeTiled encode, int n_sm, cudaStream_t st, con
     const int n_items = pl.MAXSPLIT * pl.QT * D.H * nf;
     dim3 grid(n_items < n_sm ? n_items : n_sm);
     cudaError_t e = launch_pdl(kern, grid, dim3(A::THREADS), (size_t)A::SMEM, st, 1, mq, mk, mv, sp, D, layer, pl, n_items,
-                               out, part_o, counters, status);
+                               q, kc, vc, out, part_o, counters, status);
     if (e != cudaSuccess) {
         fprintf(stderr, "libnfd: tensor-core attention launch failed: %s\n", cudaGetErrorString(e));
         cudaGetLastError();
