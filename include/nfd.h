@@ -87,17 +87,12 @@ typedef struct {
 /* Create a context.  `cuda_stream` is a cudaStream_t (NULL = legacy default
  * stream).  Validates cfg (NFD_E_BADCFG), copies/repacks the weights, allocates
  * the cache: n_streams x n_layers x (W + 2 k_max) frame pages of K and of V.
- * In bf16 mode the first context of a shape in the process also times its GEMM
- * tile plans on scratch data (about half a second; the environment variable
- * NFD_NO_TUNE=1 skips it and keeps the built-in cost model's plans); the cache is
- * cleared afterwards.  The plan found fixes, among other things, over how many
- * thread blocks the K range of a projection is split, hence the order in which
- * its products are summed: all contexts of one process share the plans and give
- * bitwise equal results for equal inputs, two processes may differ in the last
- * bits (NFD_NO_TUNE=1 makes the plans, and with them the bits, the same
- * everywhere).  A bf16 context needs the driver's cuTensorMapEncodeTiled entry
- * point; without it the call fails with NFD_E_CUDA rather than run the plain
- * validation kernels unasked.  Synchronises the stream before returning. */
+ * The tile plans of the GEMMs, and with them the order in which products are
+ * summed, follow from the sizes in cfg alone: equal inputs give bitwise equal
+ * results in every context and every process on the same GPU model.
+ * A bf16 context needs the driver's cuTensorMapEncodeTiled entry point; without
+ * it the call fails with NFD_E_CUDA rather than run the plain validation kernels
+ * unasked.  Synchronises the stream before returning. */
 int nfd_create(nfd_ctx **out, const nfd_weights *w, const nfd_cfg *cfg, void *cuda_stream);
 int nfd_destroy(nfd_ctx *ctx);
 

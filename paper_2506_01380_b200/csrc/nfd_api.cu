@@ -284,12 +284,12 @@ static cudaError_t take_launch_err(nfd_ctx *c) {
 }
 
 template <typename TS, typename Epi>
-static void launch_gemm(nfd_ctx *c, const TS *A, const TS *Wt, int M, int N, int K, Epi epi, int tc_kind,
+static void launch_gemm(nfd_ctx *c, const TS *A, const TS *Wt, int M, int N, int K, Epi epi,
                         const void *next_w = nullptr, size_t next_elems = 0, bool folded = false) {
     prof_mark(c, false);
     // the next GEMM's weights, pulled towards L2 by this launch
     const L2Prefetch pf{next_w, next_w && c->l2_prefetch ? (unsigned long long)(next_elems * sizeof(TS)) & ~15ull : 0ull};
-    if (fast_gemm<TS, Epi>(c->fast && c->bf16_mode, c->fs, c->st, A, Wt, M, N, K, epi, tc_kind, pf)) {
+    if (fast_gemm<TS, Epi>(c->fast && c->bf16_mode, c->fs, c->st, A, Wt, M, N, K, epi, pf)) {
         prof_mark(c, true);
         c->launches++;
         return;
@@ -391,14 +391,14 @@ template <typename TS> static void enqueue_body(nfd_ctx *c, int nf, int kind) {
         EpiQKV<TS> eq{sp, (const TS *)c->b_qkv[l], (TS *)c->qbuf, (TS *)c->kc, (TS *)c->vc, c->d_rope, D, l,
                       c->rope_cs, M, lq, c->kv_prefetch ? 1 : 0};
         c->cls = CLS_GEMM_QKV;
-        launch_gemm<TS>(c, (const TS *)c->hbuf, (const TS *)c->w_qkv[l], M, 3 * d, d, eq, TC_QKV, c->w_o[l],
+        launch_gemm<TS>(c, (const TS *)c->hbuf, (const TS *)c->w_qkv[l], M, 3 * d, d, eq, c->w_o[l],
                         (size_t)d * d, fold);
         if (kind == 1 && l == L - 1) break;      // a commit only needs the K/V of every layer
         launch_attention<TS>(c, nf, l);
         EpiGateRes<TS> eo{sp, (const TS *)c->b_o[l], c->z, modl + 2 * d, mod_row, D,
                           fold ? (TS *)c->hbuf : (TS *)nullptr, modl + 4 * d, fold ? c->ln_stats : (float2 *)nullptr};
         c->cls = CLS_GEMM_O;
-        launch_gemm<TS>(c, (const TS *)c->abuf, (const TS *)c->w_o[l], M, d, d, eo, TC_RES, c->w_fc1[l],
+        launch_gemm<TS>(c, (const TS *)c->abuf, (const TS *)c->w_o[l], M, d, d, eo, c->w_fc1[l],
                         (size_t)d * D.n1, fold);
         if (!fold) {
             c->cls = CLS_ADALN;
@@ -407,14 +407,14 @@ template <typename TS> static void enqueue_body(nfd_ctx *c, int nf, int kind) {
         }
         EpiGelu<TS> eg{(const TS *)c->b_fc1[l], (TS *)c->mbuf, D.n1, D.act, lm};
         c->cls = CLS_GEMM_FC1;
-        launch_gemm<TS>(c, (const TS *)c->hbuf, (const TS *)c->w_fc1[l], M, D.n1, d, eg, TC_GELU, c->w_fc2[l],
+        launch_gemm<TS>(c, (const TS *)c->hbuf, (const TS *)c->w_fc1[l], M, D.n1, d, eg, c->w_fc2[l],
                         (size_t)d * D.dm, fold);
         // the last layer's output goes to the final adaLN kernel, which reads z itself
         const bool more = fold && l + 1 < L;
         EpiGateRes<TS> e2{sp, (const TS *)c->b_fc2[l], c->z, modl + 5 * d, mod_row, D,
                           more ? (TS *)c->hbuf : (TS *)nullptr, modl + 6 * d + d, more ? c->ln_stats : (float2 *)nullptr};
         c->cls = CLS_GEMM_FC2;
-        launch_gemm<TS>(c, (const TS *)c->mbuf, (const TS *)c->w_fc2[l], M, d, D.dm, e2, TC_RES,
+        launch_gemm<TS>(c, (const TS *)c->mbuf, (const TS *)c->w_fc2[l], M, d, D.dm, e2,
                         l + 1 < L ? c->w_qkv[l + 1] : nullptr, (size_t)3 * d * d, fold);
     }
     if (kind == 0) {
@@ -422,150 +422,8 @@ template <typename TS> static void enqueue_body(nfd_ctx *c, int nf, int kind) {
         PLAUNCH(c, (k_adaln<TS>), ln_grid, 128, 0, sp, D, (const float *)c->z, (TS *)c->hbuf, (const float *)c->fmod,
                 (size_t)2 * d, (size_t)0, (size_t)d);
         EpiFinal<TS> ef{sp, (const TS *)c->b_out, D};
-        launch_gemm<TS>(c, (const TS *)c->hbuf, (const TS *)c->w_out, M, D.P, d, ef, TC_NONE);
+        launch_gemm<TS>(c, (const TS *)c->hbuf, (const TS *)c->w_out, M, D.P, d, ef);
     }
-}
-
-// ---------------------------------------------------------------------------
-// Tile width and split of the four GEMMs of a block, found by timing at create.  For a pass of one frame
-// every (width, split) pair is timed and the best split is kept for good (the order in which the K range is
-// summed must not depend on the pass); for passes of more frames only the width is timed.  Results are kept
-// per process (nfd_fast.cuh), so a second context of the same shape does not time anything and sums in the
-// same order.  The timed launches run the real epilogues on scratch frames 0..nf-1 of stream 0 with whatever
-// the modulation tables hold; the caller clears the cache afterwards.
-// ---------------------------------------------------------------------------
-static int tune_gemms(nfd_ctx *c) {
-    const Dims &D = c->D;
-    const int d = D.d, T = D.T;
-    FastState &fs = c->fs;
-    if (!c->bf16_mode || !c->fast || !fs.ready || getenv("NFD_NO_TUNE")) return NFD_OK;
-    const bool fold = c->fold_active();
-    const size_t mod_row = (size_t)D.L * 6 * d, uv_row = (size_t)D.L * (3 * d + D.n1);
-    struct Kind { int tc, N, K; };
-    const Kind kinds[4] = {{TC_QKV, 3 * d, d}, {TC_RES, d, d}, {TC_GELU, D.n1, d}, {TC_RES, d, D.dm}};
-    const int forms[4] = {FORM_QKV, FORM_RES, FORM_MLP, FORM_RES};
-    cudaEvent_t e0, e1;
-    CK(cudaEventCreate(&e0));
-    CK(cudaEventCreate(&e1));
-    const StepParams *sp = c->d_sp;
-    auto launch = [&](int ki, int M) -> bool {        // one launch of GEMM `ki` of layer 0 with the forced plan
-        const L2Prefetch pf{nullptr, 0};
-        const float *modl = c->mod;
-        LnFold ln{nullptr, uv_row, c->ln_stats, d / 32, D.norm, D.eps, sp, T};
-        if (ki == 0) {
-            if (fold) ln.uv = c->uvtab;
-            EpiQKV<bf16> e{sp, (const bf16 *)c->b_qkv[0], (bf16 *)c->qbuf, (bf16 *)c->kc, (bf16 *)c->vc, c->d_rope, D, 0,
-                           c->rope_cs, M, ln};
-            return fast_gemm<bf16>(true, fs, c->st, (const bf16 *)c->hbuf, (const bf16 *)c->w_qkv[0], M, 3 * d, d, e, TC_QKV, pf);
-        }
-        if (ki == 1) {
-            EpiGateRes<bf16> e{sp, (const bf16 *)c->b_o[0], c->z, modl + 2 * d, mod_row, D,
-                               fold ? (bf16 *)c->hbuf : (bf16 *)nullptr, modl + 4 * d, fold ? c->ln_stats : (float2 *)nullptr};
-            return fast_gemm<bf16>(true, fs, c->st, (const bf16 *)c->abuf, (const bf16 *)c->w_o[0], M, d, d, e, TC_RES, pf);
-        }
-        if (ki == 2) {
-            if (fold) ln.uv = c->uvtab + 3 * d;
-            EpiGelu<bf16> e{(const bf16 *)c->b_fc1[0], (bf16 *)c->mbuf, D.n1, D.act, ln};
-            return fast_gemm<bf16>(true, fs, c->st, (const bf16 *)c->hbuf, (const bf16 *)c->w_fc1[0], M, D.n1, d, e, TC_GELU, pf);
-        }
-        EpiGateRes<bf16> e{sp, (const bf16 *)c->b_fc2[0], c->z, modl + 5 * d, mod_row, D,
-                           fold ? (bf16 *)c->hbuf : (bf16 *)nullptr, modl + 7 * d, fold ? c->ln_stats : (float2 *)nullptr};
-        return fast_gemm<bf16>(true, fs, c->st, (const bf16 *)c->mbuf, (const bf16 *)c->w_fc2[0], M, d, D.dm, e, TC_RES, pf);
-    };
-    auto time_of = [&](int ki, int M, int BN, int S, float *us) -> bool {
-        fs.force_BN = BN, fs.force_S = S;
-        bool ok = true;
-        for (int i = 0; i < 3 && ok; ++i) ok = launch(ki, M);
-        float best = 1e30f;
-        for (int rep = 0; rep < 3 && ok; ++rep) {
-            cudaEventRecord(e0, c->st);
-            for (int i = 0; i < 8 && ok; ++i) ok = launch(ki, M);
-            cudaEventRecord(e1, c->st);
-            if (cudaEventSynchronize(e1) != cudaSuccess) ok = false;
-            float ms = 0.f;
-            if (ok && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess && ms < best) best = ms;
-        }
-        fs.force_BN = fs.force_S = 0;
-        if (!ok) cudaGetLastError();
-        *us = best * 1000.f / 8.f;
-        return ok;
-    };
-    const int nfs[] = {1, 2, 3, 4, 5, 6, 8, 12, 16, 24, 32};
-    const int widths[] = {32, 64, 96, 128};
-    bool touched = false;
-    // the largest pass this context can build: per stream a speculation plus the deferred frames of the last one
-    const int nf_max = D.n_streams * 2 * c->cfg.max_spec;
-    for (int nf : nfs) {
-        if (nf > NFD_MAX_PASS_FRAMES || nf > nf_max) break;
-        const int M = nf * T;
-        bool need = false;
-        for (int ki = 0; ki < 4; ++ki) {
-            const Kind &k = kinds[ki];
-            const int kk = k.tc + (k.K > 2048 ? 10 : 0);
-            if (!g_tuned_BN.count(std::make_tuple(kk, k.N, k.K, fs.n_sm, M)) &&
-                (!g_tuned_S.count(std::make_tuple(kk, k.N, k.K, fs.n_sm)) || !plan_gemm(fs, M, k.N, k.K, k.tc, forms[ki]).p))
-                need = true;
-        }
-        if (!need) continue;
-        // a pass descriptor for nf scratch frames of stream 0
-        StepParams &p = c->h_sp;
-        memset(&p, 0, sizeof(p));
-        p.nf = nf;
-        for (int j = 0; j < nf; ++j) {
-            p.fr[j].stream = 0, p.fr[j].frame = j, p.fr[j].win_first = 0, p.fr[j].cond_row = 0, p.fr[j].first_new = 0;
-            p.fr[j].src = 0, p.fr[j].src_index = j, p.fr[j].out_index = -1, p.fr[j].win_slot = 0;
-        }
-        k_set_params<<<1, 256, 0, c->st>>>(p, c->d_sp, c->lim, c->d_status);
-        CK(cudaGetLastError());
-        touched = true;
-        for (int ki = 0; ki < 4; ++ki) {
-            const Kind &k = kinds[ki];
-            const int kk = k.tc + (k.K > 2048 ? 10 : 0);
-            const auto skey = std::make_tuple(kk, k.N, k.K, fs.n_sm);
-            const auto bkey = std::make_tuple(kk, k.N, k.K, fs.n_sm, M);
-            if (g_tuned_BN.count(bkey)) continue;
-            const bool s_open = !g_tuned_S.count(skey);
-            if (s_open && nf != 1) continue;                 // the split is decided by the one-frame pass
-            const int nkb = (k.K + 63) / 64;
-            // the cost model's plan is the incumbent: another one must beat it by 3 % (timing noise must not
-            // flip plans between processes without need)
-            // (k_gemm_p goes by its own rule and is not timed; the split of a one-frame pass is found on k_gemm_tc)
-            GemmPlan model = plan_gemm(fs, M, k.N, k.K, k.tc, forms[ki]);
-            if (model.p && !s_open) continue;
-            if (model.p) model = GemmPlan{128, model.S, false};
-            float t_best = 1e30f;
-            GemmPlan best = model;
-            if (!time_of(ki, M, model.BN, model.S, &t_best)) t_best = 1e30f;
-            t_best *= 0.97f;
-            for (int S = 1; S <= 4; S *= 2) {
-                if (!s_open && S != g_tuned_S[skey]) continue;
-                if (S > 1 && nkb / S < 2) continue;
-                for (int BN : widths) {
-                    if (BN > 32 && BN > k.N) continue;
-                    if (BN == model.BN && S == model.S) continue;
-                    const long long ctas = (long long)((M + 127) / 128) * ((k.N + BN - 1) / BN) * S;
-                    if (ctas > 3LL * fs.n_sm) continue;          // hopeless: several waves
-                    float t;
-                    const bool ok_t = time_of(ki, M, BN, S, &t);
-                    if (ok_t && t < t_best) t_best = t, best = GemmPlan{BN, S, false};
-                }
-            }
-            if (s_open) g_tuned_S[skey] = best.S;
-            g_tuned_BN[bkey] = best.BN;
-        }
-    }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    if (touched) {
-        // the timed epilogues wrote into scratch pages of stream 0 and into the activation buffers
-        const size_t cache_bytes = (size_t)D.n_streams * D.L * D.R * D.page_elems * c->esz;
-        CK(cudaMemsetAsync(c->kc, 0, cache_bytes, c->st));
-        CK(cudaMemsetAsync(c->vc, 0, cache_bytes, c->st));
-        CK(cudaMemsetAsync(c->d_status, 0, 16, c->st));
-        CK(cudaStreamSynchronize(c->st));
-        memset(&c->h_sp, 0, sizeof(c->h_sp));
-    }
-    return NFD_OK;
 }
 
 static void enqueue_body_any(nfd_ctx *c, int nf, int kind) {
@@ -878,15 +736,6 @@ int nfd_create(nfd_ctx **out, const nfd_weights *w, const nfd_cfg *cfg, void *cu
         }
     }
     if (rc == NFD_OK) rc = fast_create(c->fs, D, c->bf16_mode, c->st, c->d_status);
-    if (rc == NFD_OK && c->fs.ready) {
-        // how many CTAs of a GEMM fit at once, per cluster size (any instantiation: one CTA fills an SM)
-        auto kern = k_gemm_tc<96, EpiGateRes<bf16>, 0>;
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, GemmCfg<96>::SMEM) == cudaSuccess)
-            query_gemm_slots(c->fs, kern, GemmCfg<96>::SMEM, GemmCfg<96>::THREADS);
-        else
-            cudaGetLastError();
-    }
-    if (rc == NFD_OK) rc = tune_gemms(c);
     if (rc != NFD_OK) {
         nfd_destroy(c);
         return rc;

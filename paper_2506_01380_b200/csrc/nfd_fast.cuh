@@ -12,8 +12,6 @@
 #include "nfd_gemm_p.cuh"
 #include "nfd_attn_tc.cuh"
 
-enum { TC_NONE = 0, TC_QKV = 1, TC_RES = 2, TC_GELU = 3 };
-
 typedef CUresult (*PFN_encodeTiled)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
                                     const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
                                     CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -29,8 +27,6 @@ struct FastState {
     unsigned int *attn_counters = nullptr;   // one per (frame, head, query tile); zero between launches
     size_t cache_pages = 0;            // (stream, layer, ring slot, head) pages of T rows
     std::map<std::tuple<const void *, int, int, int>, CUtensorMap> maps;   // (ptr, rows, cols, box_rows)
-    int force_BN = 0, force_S = 0;     // set while candidates are being timed
-    int slots[5] = {0, 0, 0, 0, 0};    // CTAs of a GEMM that can be resident at once, by cluster size (1, 2, 4)
 };
 
 // Key block, blocks per page and query tiles for pages of T tokens: the block that walks a page in the least time, a
@@ -213,96 +209,35 @@ static int gemm_p_width(int n_sm, int form, int T, int dh, int M, int N, int K, 
     }
     return best;
 }
-// Plans found by timing (nfd_create), shared by every context of the process so that two contexts of the same
-// shape always sum in the same order: (kind, N, K, n_sm) -> S, and (kind, N, K, n_sm, M) -> BN.
-static std::map<std::tuple<int, int, int, int>, int> g_tuned_S;
-static std::map<std::tuple<int, int, int, int, int>, int> g_tuned_BN;
-
-// CTAs that can be resident at once: one per SM, less what clusters cannot use (a cluster lives inside one
-// GPC).  Asked of the runtime at create (on a 148-SM B200: 148 for clusters of 1 and 2, 132 for clusters of
-// 4); the fallback figures are those.
-static int gemm_slots(const FastState &fs, int S) {
-    if (S >= 1 && S <= 4 && fs.slots[S] > 0) return fs.slots[S];
-    if (S >= 4) return (fs.n_sm / 4 - 4) * 4;
-    return fs.n_sm;
-}
-template <typename Kern> static void query_gemm_slots(FastState &fs, Kern kern, int smem, int threads) {
-    for (int cs = 1; cs <= 4; cs *= 2) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(fs.n_sm / cs * cs), cfg.blockDim = dim3(threads), cfg.dynamicSmemBytes = (size_t)smem;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = cs, at[0].val.clusterDim.y = 1, at[0].val.clusterDim.z = 1;
-        cfg.attrs = at, cfg.numAttrs = 1;
-        int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess && n > 0)
-            fs.slots[cs] = n * cs < fs.n_sm ? n * cs : fs.n_sm;
-        else
-            cudaGetLastError();
-    }
-}
-
-static GemmPlan plan_gemm(const FastState &fs, int M, int N, int K, int tc_kind, int form) {
-    if (fs.force_BN) return {fs.force_BN, fs.force_S, false};
-    const int kind_key = tc_kind + (K > 2048 ? 10 : 0);
-    {
-        auto is = g_tuned_S.find(std::make_tuple(kind_key, N, K, fs.n_sm));
-        auto ib = g_tuned_BN.find(std::make_tuple(kind_key, N, K, fs.n_sm, M));
-        if (is != g_tuned_S.end()) {
-            const int bn_p = gemm_p_width(fs.n_sm, form, (int)(fs.a_rows / NFD_MAX_PASS_FRAMES), fs.dh, M, N, K, is->second);
-            if (bn_p) return {bn_p, is->second, true};
-            if (ib != g_tuned_BN.end()) return {ib->second, is->second, false};
-        }
-    }
-    // Cost in SM cycles, fitted to measurements on B200: an SM takes in operand tiles at about
-    // 55 bytes per cycle whatever the ring depth; CTAs that share an SM share that rate.
-    // The split S is chosen for a one-frame pass (M = tokens per frame) and then kept for every M:
-    // the order in which the K range is summed, and with it every bit of the result, must not
-    // depend on how many frames share a pass.  Only the tile width follows M.
-    const int nkb = (K + 63) / 64;
-    auto cost_of = [&](int m_rows, int BN, int S) {
-        const int mt = (m_rows + 127) / 128, nt = (N + BN - 1) / BN;
-        const long long ctas = (long long)mt * nt * S;
-        const int slots = gemm_slots(fs, S);
-        const double waves = (double)((ctas + slots - 1) / slots);
-        const double share = 1.0;
-        const double kb = (double)((nkb + S - 1) / S);
-        const double load = kb * (16384.0 + BN * 128.0) / 55.0 * share;
-        const double items = (128.0 / S) * (BN / 8.0) / 256.0;                 // epilogue items per thread
-        // with S > 1 every pair of items waits for the partials of the S - 1 other CTAs (distributed shared
-        // memory: a slow round trip per pair, longer the more peers are asked)
-        const double pairs = (double)(((int)(items + 0.999) + 1) / 2);
-        const double epi = 400.0 + items * 350.0 + (S - 1) * (pairs * 1000.0 + 300.0) + BN * 4.0;
-        const double fixed = 3200.0 + (S > 1 ? 500.0 : 0.0);
-        return waves * (fixed + load + epi);
-    };
+// CTAs of k_gemm_tc that can be resident at once: one per SM, less what clusters cannot use (a cluster lives inside one
+// GPC; on a 148-SM B200 cudaOccupancyMaxActiveClusters gives 148 CTAs for clusters of 1 and 2, 132 for clusters of 4).
+static int gemm_slots(int n_sm, int S) { return S >= 4 ? (n_sm / 4 - 4) * 4 : n_sm; }
+// The narrowest tile whose CTAs fit the machine at once, 0 if none does.
+static int gemm_tc_width(int n_sm, int M, int N, int S) {
     const int bns[4] = {32, 64, 96, 128};
-    const int T = (int)(fs.a_rows / NFD_MAX_PASS_FRAMES);
-    int S_best = 1;
-    double best_cost = 1e30;
-    for (int bi = 0; bi < 4; ++bi) {
-        if (bns[bi] > 32 && bns[bi] > N) continue;
-        for (int S = 1; S <= GemmCfg<64>::MAX_S; S *= 2) {
-            if (S > 1 && nkb / S < 2) break;
-            const double c = cost_of(T, bns[bi], S);
-            if (c < best_cost) best_cost = c, S_best = S;
-        }
+    for (int bn : bns) {
+        if (bn > 32 && bn > N) break;
+        if ((long long)((M + 127) / 128) * ((N + bn - 1) / bn) * S <= gemm_slots(n_sm, S)) return bn;
     }
-    {
-        // a split found by timing binds the model too (sizes of M that were not timed)
-        auto is = g_tuned_S.find(std::make_tuple(kind_key, N, K, fs.n_sm));
-        if (is != g_tuned_S.end()) S_best = is->second;
-    }
-    // the tile width follows M
-    if (const int bn_p = gemm_p_width(fs.n_sm, form, T, fs.dh, M, N, K, S_best)) return {bn_p, S_best, true};
-    GemmPlan best{32, S_best, false};
-    best_cost = 1e30;
-    for (int bi = 0; bi < 4; ++bi) {
-        if (bns[bi] > 32 && bns[bi] > N) continue;
-        const double c = cost_of(M, bns[bi], S_best);
-        if (c < best_cost) best_cost = c, best.BN = bns[bi];
-    }
-    return best;
+    return 0;
+}
+// K split and tile width of a GEMM [M x N x K].  The split is chosen for a one-frame pass (T rows) and kept for every M:
+// the order in which the K range is summed, and with it every bit of the result, must not depend on how many frames share
+// a pass.  The rules go by sizes alone, so that every process sums alike.  Measured on one B200 (us with launch), one
+// frame of 336 rows unless stated:
+//   split: K = 4096 onto 1024 columns: 1, 2, 4 -> 17.7, 15.6, 16.9 (two frames 20.5, 18.8, 23.5; 96 rows 17.0, 14.5,
+//     12.8); K = 2736: 15.9, 14.8, 15.6; K = 2048 onto 768: 12.8, 12.5, 14.3; K = 1024: 11.1, 12.8, 14.2.  Hence none
+//     below 40 blocks of 64; two CTAs to a tile above, four where there is a single row block.
+//   width: the narrowest that needs one wave (the CTAs that a wider tile saves stay idle, and its epilogue is longer):
+//     K = 1024 onto 1024 columns 32, 64, 96 wide 11.1, 12.8, 14.8; onto 3072 columns 64, 96, 128 wide 12.7, 14.8, 15.5;
+//     two frames, K = 4096 in two, 96, 128 wide (64 needs two waves) 18.8, 20.3, 25.1.
+static GemmPlan plan_gemm(const FastState &fs, int M, int N, int K, int form) {
+    const int T = (int)(fs.a_rows / NFD_MAX_PASS_FRAMES), nkb = (K + 63) / 64;
+    int S = nkb < 40 ? 1 : (T > 128 ? 2 : 4);
+    while (S > 1 && !gemm_tc_width(fs.n_sm, T, N, S)) S /= 2;
+    if (const int bn = gemm_p_width(fs.n_sm, form, T, fs.dh, M, N, K, S)) return {bn, S, true};
+    const int bn = gemm_tc_width(fs.n_sm, M, N, S);
+    return {bn ? bn : (N >= 128 ? 128 : 32), S, false};
 }
 
 template <int BN, typename Epi, int SC>
@@ -412,14 +347,14 @@ static bool launch_gemm_p_any(FastState &fs, cudaStream_t st, const bf16 *A, con
 
 template <typename TS, typename Epi>
 static bool fast_gemm(bool enabled, FastState &fs, cudaStream_t st, const TS *A, const TS *Wt, int M, int N, int K,
-                      Epi epi, int tc_kind, L2Prefetch pf) {
+                      Epi epi, L2Prefetch pf) {
     if constexpr (!std::is_same<TS, bf16>::value) {
         return false;
     } else {
         if (!enabled || !fs.ready) return false;
         if (K % 8 || K < 64 || N < 32 || (N & 7)) return false;
         if (((uintptr_t)A & 15) || ((uintptr_t)Wt & 15)) return false;
-        const GemmPlan pl = plan_gemm(fs, M, N, K, tc_kind, Epi::kForm);
+        const GemmPlan pl = plan_gemm(fs, M, N, K, Epi::kForm);
         if constexpr (Epi::kForm != FORM_NONE) {
             if (pl.p) return launch_gemm_p_any<Epi>(fs, st, A, Wt, M, N, K, pl.BN, pl.S, epi, pf);
         }
