@@ -17,11 +17,13 @@
 // exact to the same number of bits whatever its size, so that m only has to keep exp2 in range.  With no maximum to take
 // there is no state to rescale, and all softmax groups share one m and one O accumulator.  Should a block's sum of a
 // row pass 2^100 (scores rising by more than 69 nats over the first ones), the item is computed again on the plain path
-// (attn_item_plain).
+// (attn_item_plain).  No barrier joins the groups at the end of an item: m, found by the group of
+// the first block, and the sums go through shared memory and barriers of their own, two items deep, and the group of
+// an item's last block reads O and finishes the item while the others go on (groups 0 and 1 share a CTA's last item).
 //
 // Warps 0 and 3 = TMA producers (K, V), warp 1 = issuer of all products (and loader of Q), warps 4-15 = three softmax
-// groups of four warps; group g takes the key blocks b of an item with
-// b % 3 == g.  A softmax warp is a chain of tensor-memory loads, FMAs, exponentials and conversions: with two groups the
+// groups of four warps; group g takes the CTA's blocks n with
+// n % 3 == g.  A softmax warp is a chain of tensor-memory loads, FMAs, exponentials and conversions: with two groups the
 // schedulers issued in 42 % of the clocks.
 // S has NS accumulators in tensor memory, the CTA's n-th block using number n % NS (and a "P is stored" barrier of its
 // own: a warp of a group may be a whole block ahead of another).  S(n + NS) is issued right behind P V(n), which reads P(n)
@@ -31,19 +33,23 @@
 // ring of NS stages (free again when S(n) is complete, which the barrier of accumulator n % NS tells), V blocks through
 // one of NS (free when P V is complete); V(n) and K(n + NS), which the issuer needs at the same time, arrive on one barrier.
 //
-// What bounds it: the softmax warps (exponentials: 672 clocks per 128 x 112 block on the special-function unit), the
-// products take 490.
+// What bounds it: the softmax warps (exponentials: 672 clocks per 128 x 112 block on the special-function unit, 560
+// instructions a scheduler), the products take 490; a block takes about 1000.  Registers and code size count: spilled
+// registers are cold local memory, about 1 us on the path of a short item, and a cold code path costs as much.
 // Measured, 16 heads x 64 on one B200 (events around a launch): one frame of 336 tokens behind 16: 28.4 us with one thread
-// for all loads, one for all products and a maximum pass over S; 25.0 with the threads split and no maximum pass; 22.9
-// with three groups.  Four frames 88.8 -> 74 -> 64, eight frames behind 32 232 -> 188 -> 171 (715 TFLOP/s; issue slots
-// 59 %, special-function unit 66 %, tensor pipe 44 % active).  Pages of 220 tokens ran on the plain kernel, 1342 us; now 18.
+// for all loads, one for all products and a maximum pass over S; 25.0 with the threads split and no maximum pass; 23.0
+// with three groups; 22.5 with items that overlap and the issuer's loop in one copy.  Two frames 37.3 -> 35.2 by the
+// last step, four 88.8 -> 74 -> 66 -> 61, eight frames behind 32 232 -> 188 -> 178 -> 165 (738 TFLOP/s).  Pages of
+// 220 tokens ran on the plain kernel, 1342 us; now 18.
+// Tried and worse: sixteen softmax warps with half a row each (178 -> 201: the fixed part of a block doubles); four epilogue
+// warps beside the groups (96 registers a thread: four frames 60, but 2 us more on every short launch).
 //
 // The grid is persistent: a CTA takes items blockIdx.x, + gridDim.x, ...; producers and
-// issuers run ahead into the next item while the groups finish the last one.  A key range
+// issuer run ahead into the next item.  A key range
 // longer than CH blocks is split over several items; each publishes its
 // unnormalised (O, m, l) state in global memory, stored so that a warp writes and reads
-// whole lines, and the CTA that finishes last (a counter per query tile) reads the
-// others and merges the states in split order.  CH depends only on the configuration, so
+// whole lines, and the warp that finishes last (a counter per half of O and quadrant of a
+// query tile) reads the states and merges them in split order.  CH depends only on the configuration, so
 // a frame's result does not depend on which other frames share its pass.
 #pragma once
 #include "nfd_sm100.cuh"
@@ -57,15 +63,16 @@ struct AttnPlan {
     FastDiv split_div, qt_div, h_div, ch_div, bpf_div;      // by MAXSPLIT, QT, heads, CH, BPF
 };
 
-// A published state: [16 groups of 4 columns][128 rows] float4, then [128 rows] (m, l).
-#define ATTN_STATE_BYTES (128 * 64 * 4 + 128 * 8)
+// A published state: [16 groups of 4 columns][128 rows] float4, then [2 halves of O][128 rows] (m, l).
+#define ATTN_STATE_BYTES (128 * 64 * 4 + 2 * 128 * 8)
+#define ATTN_COUNTERS 8          // of a query tile: one per half of O and quadrant of its rows
 
 template <int KB> struct AttnCfg {
     static constexpr int NS = KB <= 112 ? 4 : 3;           // S accumulators = stages of the K and the V ring
     static constexpr int NGRP = 3;                         // softmax groups
     static constexpr int Q_BYTES = 128 * 128;              // two of them
     static constexpr int KV_BYTES = KB * 128;              // one K (or V) block
-    static constexpr int ML_BYTES = (1 + 2 * NGRP) * 128 * 4;   // m of every row; l of every row and group, two items
+    static constexpr int ML_BYTES = 2 * (1 + NGRP) * 128 * 4;   // m of every row, l of every row and group; two items
     static constexpr int SMEM = 2 * Q_BYTES + 2 * NS * KV_BYTES + ML_BYTES + 256 + 1024;
     static constexpr int TMEM_COLS = 512;
     static constexpr int S_STRIDE = KB <= 112 ? 112 : 128; // S accumulators from column 0, O at column 448
@@ -108,27 +115,6 @@ __device__ __forceinline__ float2 exp2_fma2(float s0, float s1, float ca, float 
     return make_float2(__int_as_float(__float_as_int(p.x) + (__float_as_int(t.x) << 23)),
                        __int_as_float(__float_as_int(p.y) + (__float_as_int(t.y) << 23)));
 }
-__device__ __forceinline__ void named_bar_sync(int id, int n_threads) {
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n_threads) : "memory");
-}
-__device__ __forceinline__ void named_bar_arrive(int id, int n_threads) {
-    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n_threads) : "memory");
-}
-// barrier that also tells whether any thread's v is true
-__device__ __forceinline__ bool named_bar_or(int id, int n_threads, bool v) {
-    uint32_t r;
-    asm volatile(
-        "{\n"
-        ".reg .pred p, q;\n"
-        "setp.ne.u32 p, %3, 0;\n"
-        "bar.red.or.pred q, %1, %2, p;\n"
-        "selp.u32 %0, 1, 0, q;\n"
-        "}\n"
-        : "=r"(r)
-        : "r"(id), "r"(n_threads), "r"((uint32_t)v)
-        : "memory");
-    return r != 0;
-}
 // add 1 with release and acquire semantics at device scope
 __device__ __forceinline__ unsigned int atomic_inc_acq_rel(unsigned int *p) {
     unsigned int v;
@@ -152,10 +138,18 @@ struct AttnItem {
         nb = min(nbt, b0 + pl.CH) - b0;
         if (nb < 0) nb = 0;
     }
+    // the first item at or after `item` (in steps of the grid) that has blocks; n_items or more: there is none
+    __device__ __forceinline__ int find(int item, int n_items, const StepParams *sp, const Dims &D, const AttnPlan &pl) {
+        for (; item < n_items; item += gridDim.x) {
+            set(item, sp, D, pl);
+            if (nb > 0) break;
+        }
+        return item;
+    }
 };
 
-// One row of an item without tensor cores (see the note on m at the top): columns c0 .. c0 + 31 of O relative to the row's
-// maximum, the maximum and the sum.  q: the row (dh values); kp, vp: the pages.
+// One row of an item without tensor cores (see the note on m at the top): columns c0 .. c0 + 31 of O relative to the
+// row's maximum, the maximum and the sum.  q: the row (dh values); kp, vp: the pages.
 static __device__ __noinline__ void attn_item_plain(const AttnItem &w, const Dims &D, const AttnPlan &pl,
                                                     int KB, int layer, const bf16 *q, const bf16 *kp, const bf16 *vp, float c,
                                                     int c0, float *O, float *m_out, float *l_out) {
@@ -180,6 +174,109 @@ static __device__ __noinline__ void attn_item_plain(const AttnItem &w, const Dim
     *m_out = m, *l_out = l;
 }
 
+// The end of an item for one warp: halves p0 .. p0 + np - 1 (32 columns each) of the 32 rows of its quadrant are read from
+// tensor memory and written out, or published; of the warps that hold a half of a tile's rows in its splits, the one that
+// finishes last merges them in split order.  (A counter per half and quadrant: no barrier of the CTA.)
+// m, l: reference and sum of this thread's row (an infinite sum: the row is computed again, see the note on m).
+template <int KB>
+static __device__ __forceinline__ void attn_finish(const AttnItem &w, int item, int p0, int np, uint32_t tO, uint32_t o_free, int trow, float m, float l,
+                                            float c, const StepParams *sp, const Dims &D, const AttnPlan &pl, int layer,
+                                            const bf16 *gq, const bf16 *gk, const bf16 *gv, bf16 *out, float *part_o,
+                                            unsigned int *counters) {
+    const int lane = threadIdx.x & 31, row = w.qt * 128 + trow;
+    const size_t item_q = ((size_t)w.j * D.H + w.h) * pl.QT + w.qt;
+    uint8_t *states = reinterpret_cast<uint8_t *>(part_o) + item_q * pl.MAXSPLIT * ATTN_STATE_BYTES;
+    auto o_at = [&](int p) { return (uint32_t)(p * 8 * 128 + trow) * 16; };
+    auto ml_at = [&](int p) { return 128 * 64 * 4 + (uint32_t)(p * 128 + trow) * 8; };
+    auto write_part = [&](int p, const float *O, float lt) {
+        if (row >= D.T || p * 32 >= D.dh) return;
+        const float inv = 1.0f / lt;
+        bf16 *o = out + (size_t)(w.j * D.T + row) * D.d + w.h * D.dh + p * 32;
+#pragma unroll
+        for (int e = 0; e < 32; e += 8) {
+            float t[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) t[u] = O[e + u] * inv;
+            *reinterpret_cast<uint4 *>(o + e) = pack_bf16x8(t);
+        }
+    };
+#pragma unroll 1
+    for (int p = p0; p < p0 + np; ++p) {
+        float O[32], mp = m, lp = l;
+        tmem_ld32(tO + 32 * p, reinterpret_cast<uint32_t *>(O));
+        tmem_ld_wait();
+        if (l == INFINITY) {
+            pdl_wait();                                    // this thread reads global memory itself
+            AttnItem wc;                                   // (looked up again: nothing of this path stays in registers)
+            wc.set(item, sp, D, pl);
+            float Oc[32], mc, lc;
+            attn_item_plain(wc, D, pl, KB, layer, gq + ((size_t)w.h * (size_t)(sp->nf * D.T) + w.j * D.T + min(row, D.T - 1)) * D.dh,
+                            gk, gv, c, 32 * p, Oc, &mc, &lc);
+            mp = mc, lp = lc;
+#pragma unroll
+            for (int e = 0; e < 32; ++e) O[e] = Oc[e];
+        }
+        __syncwarp();
+        if (w.nsplit == 1) {
+            write_part(p, O, lp);
+        } else {
+            uint8_t *st = states + (size_t)w.split * ATTN_STATE_BYTES;
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                *reinterpret_cast<float4 *>(st + o_at(p) + e * 2048) = make_float4(O[4 * e], O[4 * e + 1], O[4 * e + 2], O[4 * e + 3]);
+            *reinterpret_cast<float2 *>(st + ml_at(p)) = make_float2(mp, lp);
+        }
+    }
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0 && o_free) mbar_arrive(o_free);
+    if (w.nsplit == 1) return;
+    unsigned int last = 0;
+    if (lane < np) {
+        unsigned int *cnt = counters + item_q * ATTN_COUNTERS + (p0 + lane) * 4 + (trow >> 5);
+        last = atomic_inc_acq_rel(cnt) == (unsigned int)(w.nsplit - 1);
+        if (last) *cnt = 0;                                // ready for the next launch
+    }
+    last = __ballot_sync(0xffffffffu, last);
+#pragma unroll 1
+    for (int p = p0; p < p0 + np; ++p) {
+        if (!((last >> (p - p0)) & 1)) continue;
+        float O[32], lt = 0.f, mx = -INFINITY;
+#pragma unroll
+        for (int e = 0; e < 32; ++e) O[e] = 0.f;
+        // the loads of two states (its own is read back like the others) are in flight together
+#pragma unroll 1
+        for (int s0 = 0; s0 < w.nsplit; s0 += 1) {
+            float2 ml[1];
+            float4 v[1][8];
+#pragma unroll
+            for (int u = 0; u < 1; ++u) {
+                const uint8_t *st = states + (size_t)min(s0 + u, w.nsplit - 1) * ATTN_STATE_BYTES;
+                ml[u] = __ldcg(reinterpret_cast<const float2 *>(st + ml_at(p)));
+#pragma unroll
+                for (int e = 0; e < 8; ++e) v[u][e] = __ldcg(reinterpret_cast<const float4 *>(st + o_at(p) + e * 2048));
+            }
+            // (every rounding is spelled out: the bits must not depend on which CTA merges)
+#pragma unroll
+            for (int u = 0; u < 1; ++u) {
+                if (s0 + u >= w.nsplit) break;
+                const float mb = fmaxf(mx, ml[u].x);
+                const float fo = mx == mb ? 1.0f : ex2_approx(mx - mb), wgt = ex2_approx(ml[u].x - mb);
+                mx = mb;
+                lt = fmaf(ml[u].y, wgt, __fmul_rn(lt, fo));
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    O[4 * e] = fmaf(v[u][e].x, wgt, __fmul_rn(O[4 * e], fo));
+                    O[4 * e + 1] = fmaf(v[u][e].y, wgt, __fmul_rn(O[4 * e + 1], fo));
+                    O[4 * e + 2] = fmaf(v[u][e].z, wgt, __fmul_rn(O[4 * e + 2], fo));
+                    O[4 * e + 3] = fmaf(v[u][e].w, wgt, __fmul_rn(O[4 * e + 3], fo));
+                }
+            }
+        }
+        write_part(p, O, lt);
+    }
+}
+
 template <int KB>
 __global__ void __launch_bounds__(AttnCfg<KB>::THREADS, 1)
 k_attn_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
@@ -190,16 +287,15 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
     NFD_TRACE_T0();
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint8_t *sKV = smem + 2 * A::Q_BYTES;
-    float *s_m = reinterpret_cast<float *>(sKV + 2 * A::NS * A::KV_BYTES);      // [128]
-    float *s_l = s_m + 128;                                                           // [item parity][group][128]
+    float *s_m = reinterpret_cast<float *>(sKV + 2 * A::NS * A::KV_BYTES);      // [item parity][128]
+    float *s_l = s_m + 2 * 128;                                                       // [item parity][group][128]
     uint64_t *bars = reinterpret_cast<uint64_t *>(sKV + 2 * A::NS * A::KV_BYTES + A::ML_BYTES);
     // barriers: q_full[2] | q_empty[2] | o_free | k_first[NS] (K of blocks 0 .. NS-1) | s_full[NS] | p_full[NS] |
-    // kv_full[NS] (V(n) and K(n + NS)) | v_empty[NS]
+    // kv_full[NS] (V(n) and K(n + NS)) | v_empty[NS] | m_full[2] | l_full[2] | ml_empty[2]
     const uint32_t q_full = smem_u32(bars), q_empty = q_full + 16, o_free = q_empty + 16, k_first = o_free + 8,
                    s_full = k_first + 8 * A::NS, p_full = s_full + 8 * A::NS, kv_full = p_full + 8 * A::NS,
-                   v_empty = kv_full + 8 * A::NS;
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 5 + 5 * A::NS);
-    int *last_flag = reinterpret_cast<int *>(tmem_slot + 1);
+                   v_empty = kv_full + 8 * A::NS, m_full = v_empty + 8 * A::NS, l_full = m_full + 16, ml_empty = l_full + 16;
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 11 + 5 * A::NS);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // The first item's descriptor: its loads are in flight during the set-up.  (The pass descriptor was written by the
     // first kernel of the pass, which completed before this kernel's predecessor began.)
@@ -213,8 +309,11 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
         for (int s = 0; s < 2; ++s) {
             mbar_init(q_full + 8 * s, 1);
             mbar_init(q_empty + 8 * s, 1);
+            mbar_init(m_full + 8 * s, 4);                  // one arrival per warp of the group that finds m
+            mbar_init(l_full + 8 * s, 4 * A::NGRP);        // one per softmax warp
+            mbar_init(ml_empty + 8 * s, 4);                // one per warp of the group that finishes the item
         }
-        mbar_init(o_free, 8);                              // one arrival per warp that has read O
+        mbar_init(o_free, 4);                              // one arrival per warp that has read O
         for (int s = 0; s < A::NS; ++s) {
             mbar_init(k_first + 8 * s, 1);
             mbar_init(s_full + 8 * s, 1);
@@ -293,97 +392,92 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
             constexpr uint32_t idesc_s = umma_idesc_bf16(128, KB), idesc_pv = umma_idesc_bf16_bmn(128, 64);
             const uint32_t sQ = smem_u32(smem), sK = smem_u32(sKV), sV = sK + A::NS * A::KV_BYTES;
             bool ok = true;
-            // S runs NS blocks ahead of P V: items of their own for both
-            int item_s = blockIdx.x, it_s = -1, left_s = 0;            // item of S, how many before it, its blocks to come
-            int st_s = 0, lap_s = 0;
-            uint64_t qd = 0;
-            AttnItem ws = w0;
-            auto load_q = [&](int it) {                    // Q of item ws, the it-th of this CTA
-                const int qs = it & 1;
-                if (it >= 2) ok = ok && mbar_wait(q_empty + 8 * qs, ((it >> 1) - 1) & 1, status);
+            // S runs NS blocks ahead of P V: items of their own for both.  (One copy of the code for both the first S and the
+            // later ones: this thread's registers and instruction fetches are on every block's path.)
+            AttnItem ws = w0, w = w0;
+            int item_s = blockIdx.x, it_s = -1, left_s = 0;            // item whose Q was asked for last; items before S's; S to come
+            int item = blockIdx.x - gridDim.x, it = 0, left = 0;       // the same for P V
+            int st_s = 0, lap_s = 0, st = 0, lap = 0;
+            int ahead = A::NS;                             // S to issue before the first P V
+            auto load_q = [&](int qs) {                    // Q of item ws
                 mbar_expect_tx(q_full + 8 * qs, A::Q_BYTES);
                 tma_load_3d(sQ + qs * A::Q_BYTES, &tmQ, q_full + 8 * qs, 0, ws.j * D.T + ws.qt * 128, ws.h);
             };
-            // the next item with a block at or after item_s; its Q is asked for
-            auto next_item = [&]() {
-                while (item_s < n_items) {
-                    if (item_s != blockIdx.x) ws.set(item_s, sp, D, pl);
-                    if (ws.nb > 0) {
-                        load_q(it_s + 1);
-                        return;
-                    }
-                    item_s += gridDim.x;
-                }
-            };
-            auto issue_s = [&]() {                         // S of the next block, if there is one
-                if (left_s == 0) {
-                    if (item_s >= n_items) return;
-                    ++it_s, left_s = ws.nb;
-                    item_s += gridDim.x;
-                    qd = umma_desc_k128(sQ + (it_s & 1) * A::Q_BYTES);
-                    ok = ok && mbar_wait(q_full + 8 * (it_s & 1), (it_s >> 1) & 1, status);
-                    next_item();                           // Q of the item after it
-                }
-                // (K of later blocks has arrived together with V of the block NS back)
-                if (lap_s == 0) ok = ok && mbar_wait(k_first + 8 * st_s, 0, status);
-                if (!ok) return;
-                tc_fence_after();
-                const uint64_t kd = umma_desc_k128(sK + st_s * A::KV_BYTES);
-#pragma unroll
-                for (int k4 = 0; k4 < 4; ++k4)
-                    umma_bf16_ss(tmem + A::S_STRIDE * st_s, qd + 2 * k4, kd + 2 * k4, idesc_s, k4 != 0);
-                umma_commit(s_full + 8 * st_s);            // S is ready; K's stage is free
-                if (++st_s == A::NS) st_s = 0, ++lap_s;
-                if (--left_s == 0) umma_commit(q_empty + 8 * (it_s & 1));
-            };
             pdl_wait();
-            next_item();
-            for (int i = 0; i < A::NS && ok; ++i) issue_s();
-            int it = 0, st = 0, lap = 0;
-            AttnItem w = w0;
-            for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
-                if (item != blockIdx.x) w.set(item, sp, D, pl);
-                if (w.nb == 0) continue;
-                if (it > 0) ok = mbar_wait(o_free, (it - 1) & 1, status);      // O of the last item has been read
-                ++it;
-                for (int b = 0; b < w.nb && ok; ++b) {
-                    ok = mbar_wait(kv_full + 8 * st, lap & 1, status) && mbar_wait(p_full + 8 * st, lap & 1, status);
-                    if (!ok) break;
+            if (ws.nb == 0) item_s = ws.find(item_s + gridDim.x, n_items, sp, D, pl);
+            if (item_s < n_items) load_q(0);
+            while (ok) {
+                if (ahead > 0) {
+                    --ahead;
+                } else {
+                    uint32_t acc = 1;
+                    if (left == 0) {
+                        item = w.find(item + gridDim.x, n_items, sp, D, pl);
+                        if (item >= n_items) break;
+                        left = w.nb, acc = 0;
+                        if (it > 0 && !mbar_wait(o_free, (it - 1) & 1, status)) break;     // O of the last item has been read
+                        ++it;
+                    }
+                    if (!mbar_wait(kv_full + 8 * st, lap & 1, status) || !mbar_wait(p_full + 8 * st, lap & 1, status)) break;
                     tc_fence_after();
                     const uint64_t vd = umma_desc_k128(sV + st * A::KV_BYTES);
                     const uint32_t tP = tmem + A::S_STRIDE * st;
 #pragma unroll
                     for (int i = 0; i < KB / 16; ++i) {
                         // P: 16 keys = 8 columns of packed bf16 pairs; V: MN-major, 16 keys = 2 KiB per step
-                        umma_bf16_ts(tmem + A::TM_O, tP + 8 * i, vd + (uint64_t)(i * (2048 >> 4)), idesc_pv,
-                                     (uint32_t)(b != 0 || i != 0));
+                        umma_bf16_ts(tmem + A::TM_O, tP + 8 * i, vd + (uint64_t)(i * (2048 >> 4)), idesc_pv, i ? 1u : acc);
                     }
                     umma_commit(v_empty + 8 * st);         // P V(n) is complete: V's stage is free, O at rest
                     if (++st == A::NS) st = 0, ++lap;
-                    issue_s();                             // into the accumulator that P V(n) reads
+                    --left;
                 }
+                // S of the next block, if there is one, into the accumulator that P V(n) reads
+                if (left_s == 0) {
+                    if (item_s >= n_items) continue;
+                    ++it_s, left_s = ws.nb;
+                    ok = mbar_wait(q_full + 8 * (it_s & 1), (it_s >> 1) & 1, status);
+                    item_s = ws.find(item_s + gridDim.x, n_items, sp, D, pl);
+                    if (item_s < n_items) {                // Q of the item after it
+                        if (it_s >= 1) ok = ok && mbar_wait(q_empty + 8 * ((it_s + 1) & 1), ((it_s - 1) >> 1) & 1, status);
+                        load_q((it_s + 1) & 1);
+                    }
+                }
+                // (K of later blocks has arrived together with V of the block NS back)
+                if (lap_s == 0) ok = ok && mbar_wait(k_first + 8 * st_s, 0, status);
+                if (!ok) break;
+                tc_fence_after();
+                const uint64_t qd = umma_desc_k128(sQ + (it_s & 1) * A::Q_BYTES), kd = umma_desc_k128(sK + st_s * A::KV_BYTES);
+#pragma unroll
+                for (int k4 = 0; k4 < 4; ++k4)
+                    umma_bf16_ss(tmem + A::S_STRIDE * st_s, qd + 2 * k4, kd + 2 * k4, idesc_s, k4 != 0);
+                umma_commit(s_full + 8 * st_s);            // S is ready; K's stage is free
+                if (++st_s == A::NS) st_s = 0, ++lap_s;
+                if (--left_s == 0) umma_commit(q_empty + 8 * (it_s & 1));
             }
         }
     } else if (warp == 2) {
         // no work of its own (the softmax warps start at a multiple of four: a warp reads tensor-memory lanes 32 (warp % 4) ..)
     } else {
         // ---------------- softmax: one thread per query row, three groups ----------------
-        const int g = (warp - A::SM_WARP0) >> 2;           // group: blocks b with b % 3 == g
+        const int g = (warp - A::SM_WARP0) >> 2;           // group: blocks n with n % 3 == g
         const int quad = warp & 3;                         // tensor-memory lanes this warp may touch
         const int trow = quad * 32 + lane;
         const uint32_t lane_off = (uint32_t)(quad * 32) << 16;
         const float c = (1.0f / sqrtf((float)D.dh)) * 1.4426950408889634f;   // softmax scale in the log2 domain
         bool ok = true;
-        int n0 = 0, it = 0;
+        int n0 = 0, n03 = 0, it = 0;                       // the item's first block, that modulo 3, items before it
+        const uint32_t tO = tmem + A::TM_O + lane_off;
         AttnItem w = w0;
-        for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
-            if (item != blockIdx.x) w.set(item, sp, D, pl);
-            if (w.nb == 0) continue;
+        int item = blockIdx.x;
+        if (w.nb == 0) item = w.find(item + gridDim.x, n_items, sp, D, pl);
+        while (item < n_items) {
+            const int ip = it & 1, iph = (it >> 1) & 1;    // item parity: which m and l, phase of their barriers
+            const int r = g >= n03 ? g - n03 : g - n03 + A::NGRP;      // this group's blocks: b % 3 == r
             float m_run = 0.f, l_run = 0.f, l_top = 0.f;   // l_top: the largest sum of a block
-            int kb = w.b0 + g;                             // block of the page, for the mask of its last block
+            int kb = w.b0 + r;                             // block of the page, for the mask of its last block
             kb -= pl.bpf_div.div(kb) * pl.BPF;
-            for (int b = g; b < w.nb || b == g; b += A::NGRP) {
-                // (a group without a block still takes part in the hand-over of m)
+            for (int b = r; b < w.nb || b == r; b += A::NGRP) {
+                // (a group without a block still takes part in the hand-over of m and l)
                 const bool some = b < w.nb;
                 const int n = n0 + b, st = n % A::NS;
                 const uint32_t tS = tmem + A::S_STRIDE * st + lane_off;
@@ -418,22 +512,26 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
                         tmem_st_wait();
                     }
                 }
-                if (b == g) {
-                    // m of the item: the largest of the first 16 scores of the row, found by group 0 for all
-                    if (g == 0) {
+                if (b == r) {
+                    // m of the item: the largest of the first 16 scores of the row, found by the group of block 0 for all
+                    if (r == 0) {
                         NFD_TRACE_MARK_T(TRK_OTHER + 11, 128);
-                        uint32_t r[16];
-                        tmem_ld16(tS, r);
+                        if (it >= 2) ok = ok && mbar_wait(ml_empty + 8 * ip, iph ^ 1, status);   // item it - 2 is done with
+                        __syncwarp();
+                        uint32_t x[16];
+                        tmem_ld16(tS, x);
                         tmem_ld_wait();
                         float mx = -INFINITY;
 #pragma unroll
-                        for (int e = 0; e < 16; ++e) mx = fmaxf(mx, __uint_as_float(r[e]));
+                        for (int e = 0; e < 16; ++e) mx = fmaxf(mx, __uint_as_float(x[e]));
                         m_run = mx * c;
-                        s_m[trow] = m_run;
-                        named_bar_arrive(2, 32 * 4 * A::NGRP);
+                        s_m[ip * 128 + trow] = m_run;
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(m_full + 8 * ip);
                     } else {
-                        named_bar_sync(2, 32 * 4 * A::NGRP);
-                        m_run = s_m[trow];
+                        ok = ok && mbar_wait(m_full + 8 * ip, iph, status);
+                        m_run = s_m[ip * 128 + trow];
+                        __syncwarp();
                     }
                     if (!some) break;
                 }
@@ -474,105 +572,33 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
                 if (lane == 0) mbar_arrive(p_full + 8 * st);
             }
             NFD_TRACE_MARK_T(TRK_OTHER + 12, 128);
-            // ---- the groups' sums; then groups 0 and 1 finish 32 columns of O each ----
-            float *sl = s_l + (it & 1) * A::NGRP * 128;
-            sl[g * 128 + trow] = l_run;
-            const bool redo = named_bar_or(1, 32 * 4 * A::NGRP, l_top > 1.2676506e30f /* 2^100 */);
+            // the group's sum; infinite: the item's row is to be computed again
+            s_l[(ip * A::NGRP + r) * 128 + trow] = l_top > 1.2676506e30f /* 2^100 */ ? INFINITY : l_run;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(l_full + 8 * ip);
             const int bl = n0 + w.nb - 1;                  // the item's last block
             n0 += w.nb, ++it;
-            if (g == 2) continue;
-            float O[32], m_cta = m_run, l_cta = (sl[trow] + sl[128 + trow]) + sl[256 + trow];
-            ok = ok && mbar_wait(v_empty + 8 * (bl % A::NS), (bl / A::NS) & 1, status);
-            __syncwarp();
-            tc_fence_after();
-            tmem_ld32(tmem + A::TM_O + 32 * g + lane_off, reinterpret_cast<uint32_t *>(O));
-            tmem_ld_wait();
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(o_free);
-            if (redo) {
-                pdl_wait();                                // this thread reads global memory itself
-                const int row = min(w.qt * 128 + trow, D.T - 1);
-                const AttnItem wc = w;                     // (copies: only what is on this path may live in memory)
-                float Oc[32], mc, lc;
-                attn_item_plain(wc, D, pl, KB, layer, gq + ((size_t)w.h * (size_t)(sp->nf * D.T) + w.j * D.T + row) * D.dh, gk, gv,
-                                c, 32 * g, Oc, &mc, &lc);
-                m_cta = mc, l_cta = lc;
-#pragma unroll
-                for (int e = 0; e < 32; ++e) O[e] = Oc[e];
+            const int gl = (n03 + w.nb - 1) % A::NGRP;     // the group of that block
+            n03 = gl + 1 == A::NGRP ? 0 : gl + 1;
+            const int cur = item;
+            AttnItem wn;
+            item = wn.find(item + gridDim.x, n_items, sp, D, pl);
+            // The group of the last block finishes the item while the others are on the next one; groups 0 and 1 share the
+            // CTA's last item.
+            const bool fin = item >= n_items;
+            if (fin ? g < 2 : g == gl) {
+                ok = ok && mbar_wait(l_full + 8 * ip, iph, status);
+                const float *sl = s_l + ip * A::NGRP * 128 + trow;
+                const float m = s_m[ip * 128 + trow], l = (sl[0] + sl[128]) + sl[256];
+                __syncwarp();
+                if (!fin && lane == 0) mbar_arrive(ml_empty + 8 * ip);
+                ok = ok && mbar_wait(v_empty + 8 * (bl % A::NS), (bl / A::NS) & 1, status);
+                __syncwarp();
+                tc_fence_after();
+                attn_finish<KB>(w, cur, fin ? g : 0, fin ? 1 : 2, tO, fin ? 0u : o_free, trow, m, l, c, sp, D, pl, layer, gq, gk, gv,
+                                out, part_o, counters);
             }
-            NFD_TRACE_MARK_T(TRK_OTHER + 13, 128);
-            bool write_out = true;
-            float l_tot = l_cta;
-            if (w.nsplit > 1) {
-                // ---- publish this item's state; the CTA that finishes last merges the splits in split order ----
-                const size_t item_q = ((size_t)w.j * D.H + w.h) * pl.QT + w.qt;
-                uint8_t *states = reinterpret_cast<uint8_t *>(part_o) + item_q * pl.MAXSPLIT * ATTN_STATE_BYTES;
-                {
-                    uint8_t *st = states + (size_t)w.split * ATTN_STATE_BYTES;
-                    float4 *so = reinterpret_cast<float4 *>(st) + g * 8 * 128 + trow;
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) so[e * 128] = make_float4(O[4 * e], O[4 * e + 1], O[4 * e + 2], O[4 * e + 3]);
-                    if (g == 0) reinterpret_cast<float2 *>(st + 128 * 64 * 4)[trow] = make_float2(m_cta, l_cta);
-                }
-                named_bar_sync(3, 256);
-                if (threadIdx.x == 32 * A::SM_WARP0) {
-                    const unsigned int prev = atomic_inc_acq_rel(counters + item_q);
-                    const int last = prev == (unsigned int)(w.nsplit - 1);
-                    if (last) counters[item_q] = 0;        // ready for the next launch
-                    *last_flag = last;
-                }
-                NFD_TRACE_MARK_T(TRK_OTHER + 14, 128);
-                named_bar_sync(3, 256);
-                write_out = *last_flag != 0;
-                if (write_out) {
-                    float acc[32], l = 0.f, mx = -INFINITY;
-#pragma unroll
-                    for (int e = 0; e < 32; ++e) acc[e] = 0.f;
-#pragma unroll 1
-                    for (int sidx = 0; sidx < w.nsplit; ++sidx) {
-                        float2 ml = make_float2(m_cta, l_cta);
-                        float4 v[8];
-                        if (sidx == w.split) {
-#pragma unroll
-                            for (int e = 0; e < 8; ++e) v[e] = make_float4(O[4 * e], O[4 * e + 1], O[4 * e + 2], O[4 * e + 3]);
-                        } else {
-                            const uint8_t *st = states + (size_t)sidx * ATTN_STATE_BYTES;
-                            const float4 *so = reinterpret_cast<const float4 *>(st) + g * 8 * 128 + trow;
-                            ml = __ldcg(reinterpret_cast<const float2 *>(st + 128 * 64 * 4) + trow);
-#pragma unroll
-                            for (int e = 0; e < 8; ++e) v[e] = __ldcg(so + e * 128);
-                        }
-                        // (every rounding is spelled out: the bits must not depend on which CTA merges)
-                        const float mb = fmaxf(mx, ml.x);
-                        const float fo = mx == mb ? 1.0f : ex2_approx(mx - mb), wgt = ex2_approx(ml.x - mb);
-                        mx = mb;
-                        l = fmaf(ml.y, wgt, __fmul_rn(l, fo));
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) {
-                            acc[4 * e] = fmaf(v[e].x, wgt, __fmul_rn(acc[4 * e], fo));
-                            acc[4 * e + 1] = fmaf(v[e].y, wgt, __fmul_rn(acc[4 * e + 1], fo));
-                            acc[4 * e + 2] = fmaf(v[e].z, wgt, __fmul_rn(acc[4 * e + 2], fo));
-                            acc[4 * e + 3] = fmaf(v[e].w, wgt, __fmul_rn(acc[4 * e + 3], fo));
-                        }
-                    }
-                    l_tot = l;
-#pragma unroll
-                    for (int e = 0; e < 32; ++e) O[e] = acc[e];
-                }
-            }
-            const int row = w.qt * 128 + trow;
-            if (write_out && row < D.T && g * 32 < D.dh) {
-                const float inv = 1.0f / l_tot;
-                bf16 *o = out + (size_t)(w.j * D.T + row) * D.d + w.h * D.dh + g * 32;
-#pragma unroll
-                for (int e = 0; e < 32; e += 8) {
-                    float t[8];
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) t[u] = O[e + u] * inv;
-                    *reinterpret_cast<uint4 *>(o + e) = pack_bf16x8(t);
-                }
-            }
+            w = wn;
         }
     }
     NFD_TRACE_MARK_T(TRK_OTHER + 16, 128);

@@ -24,7 +24,7 @@ struct FastState {
     size_t a_rows = 0;     // rows of every activation buffer (NFD_MAX_PASS_FRAMES * T)
     AttnPlan plan;         // KB == 0: tensor-core attention not available for this shape
     float *part_o = nullptr;           // per-split states of the attention kernel: [query tile][split] x ATTN_STATE_BYTES
-    unsigned int *attn_counters = nullptr;   // one per (frame, head, query tile); zero between launches
+    unsigned int *attn_counters = nullptr;   // ATTN_COUNTERS per (frame, head, query tile); zero between launches
     size_t cache_pages = 0;            // (stream, layer, ring slot, head) pages of T rows
     std::map<std::tuple<const void *, int, int, int>, CUtensorMap> maps;   // (ptr, rows, cols, box_rows)
 };
@@ -92,8 +92,8 @@ static int fast_create(FastState &fs, const Dims &D, bool bf16_mode, cudaStream_
                 const int nf_max = D.n_streams * (D.R - D.W);
                 const size_t tiles = (size_t)(nf_max < NFD_MAX_PASS_FRAMES ? nf_max : NFD_MAX_PASS_FRAMES) * D.H * pl.QT;
                 if (cudaMalloc((void **)&fs.part_o, tiles * pl.MAXSPLIT * (size_t)ATTN_STATE_BYTES) != cudaSuccess ||
-                    cudaMalloc((void **)&fs.attn_counters, tiles * sizeof(unsigned int)) != cudaSuccess ||
-                    cudaMemset(fs.attn_counters, 0, tiles * sizeof(unsigned int)) != cudaSuccess) {
+                    cudaMalloc((void **)&fs.attn_counters, tiles * ATTN_COUNTERS * sizeof(unsigned int)) != cudaSuccess ||
+                    cudaMemset(fs.attn_counters, 0, tiles * ATTN_COUNTERS * sizeof(unsigned int)) != cudaSuccess) {
                     cudaGetLastError();
                     return NFD_E_NOMEM;
                 }
