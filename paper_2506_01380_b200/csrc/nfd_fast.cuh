@@ -192,7 +192,14 @@ static int gemm_p_width(int n_sm, int form, int T, int dh, int M, int N, int K, 
     // a 128-row tile must not span more frames than the kernel keeps tables for; rotary rows of 64 floats at most
     if (form == FORM_NONE || 127 / T + 2 > GemmPCfg<128, FORM_MLP>::MAX_FR || (form == FORM_QKV && dh > 64)) return 0;
     const int mt = (M + 127) / 128, t128 = mt * ((N + 127) / 128);
-    if (form == FORM_RES) return t128 >= (88 * n_sm) / 148 ? 128 : 0;
+    if (form == FORM_RES) {
+        if (t128 < (88 * n_sm) / 148) return 0;
+        // 96 columns unless they need a wave more.  128 -> 96 wide, us with launch, K = 4096: 88 -> 121 tiles 27.8 -> 23.4,
+        // 152 -> 209 38.5 -> 36.2, 168 -> 231 40.9 -> 36.3 (K = 1024: 23.0 -> 20.9); a wave more: 112 -> 154 27.9 -> 33.4,
+        // 252 -> 336 48.6 -> 54.8
+        const int t96 = mt * ((N + 95) / 96);
+        return (t96 + n_sm - 1) / n_sm <= (t128 + n_sm - 1) / n_sm ? 96 : 128;
+    }
     if (t128 < (100 * n_sm) / 148) return 0;
     if (S > 1) return 128;
     // microseconds: a base and a wave, fitted to K = 768, 1024 and 1536 (within 2 us up to ten waves)
@@ -337,6 +344,10 @@ static bool launch_gemm_p(FastState &fs, cudaStream_t st, const bf16 *A, const b
 template <typename Epi>
 static bool launch_gemm_p_any(FastState &fs, cudaStream_t st, const bf16 *A, const bf16 *Wt, int M, int N, int K, int BN,
                               int S, Epi epi, L2Prefetch pf) {
+    if constexpr (Epi::kForm == FORM_RES) {
+        if (BN == 96) return S > 1 ? launch_gemm_p<96, Epi, true>(fs, st, A, Wt, M, N, K, S, epi, pf)
+                                   : launch_gemm_p<96, Epi, false>(fs, st, A, Wt, M, N, K, S, epi, pf);
+    }
     if (S > 1) return launch_gemm_p<128, Epi, true>(fs, st, A, Wt, M, N, K, S, epi, pf);
     if constexpr (Epi::kForm != FORM_RES) {
         if (BN == 256) return launch_gemm_p<256, Epi, false>(fs, st, A, Wt, M, N, K, S, epi, pf);

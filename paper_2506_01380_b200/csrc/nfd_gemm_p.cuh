@@ -19,8 +19,8 @@
 // segment order in registers), so that a row's bits are those of k_gemm_tc.
 //
 // Warps 0 and 2 = TMA producers (activations, weights: one thread for both took 369 clocks per 64-element k-block), warp 1
-// = tensor-memory allocation and UMMA issue, warp 3 = tables (and L2 prefetch of the next GEMM's weights), warps 4-11
-// = epilogue (two per tensor-memory lane quadrant, each half of the columns).
+// = tensor-memory allocation and UMMA issue, warp 3 = tables (and L2 prefetch of the next GEMM's weights), warps 4 and up
+// = epilogue (two per tensor-memory lane quadrant, three for 96 columns, which share the columns).
 #pragma once
 #include "nfd_gemm_tc.cuh"
 
@@ -28,10 +28,11 @@ template <int BN, int FORM> struct GemmPCfg {
     static constexpr int A_BYTES = 128 * 128, B_BYTES = BN * 128, ST_BYTES = A_BYTES + B_BYTES;
     // a stage (64 elements of K) comes back about 1200 clocks after it was asked for: the ring holds about what the
     // products use in that time
-    static constexpr int STAGES = BN <= 128 ? (FORM == FORM_MLP ? 5 : 4) : (BN <= 192 && FORM == FORM_MLP ? 4 : 3);
+    static constexpr int STAGES = BN <= 96 ? 5 : (BN <= 128 ? (FORM == FORM_MLP ? 5 : 4) : (BN <= 192 && FORM == FORM_MLP ? 4 : 3));
     static constexpr int RING_BYTES = STAGES * ST_BYTES;
-    static constexpr int EPI_WARP0 = 4, EPI_WARPS = 8;
-    static constexpr int HC = BN / 2, NG = HC / 32;            // columns and 32-column groups per epilogue warp
+    static constexpr int PARTS = BN == 96 ? 3 : 2;             // epilogue warps per tensor-memory lane quadrant
+    static constexpr int EPI_WARP0 = 4, EPI_WARPS = 4 * PARTS;
+    static constexpr int HC = BN / PARTS, NG = HC / 32;        // columns and 32-column groups per epilogue warp
     // side operands: the tile's rows of the rotary table (two halves of 32 floats), or of the residual stream
     static constexpr int SIDE_BYTES = FORM == FORM_QKV ? 2 * 128 * 128 : (FORM == FORM_RES ? 128 * BN * 4 : 0);
     static constexpr int NOUT = FORM == FORM_RES ? 1 : 2;      // result boxes of 32 x 32 bf16 per warp
@@ -210,7 +211,7 @@ k_gemm_p(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
         }
     } else {
         // ---------------- epilogue: one thread per row ----------------
-        const int quad = warp & 3, half = (warp - G::EPI_WARP0) >> 2, ew = warp - G::EPI_WARP0;
+        const int quad = warp & 3, part = (warp - G::EPI_WARP0) >> 2, ew = warp - G::EPI_WARP0;
         const uint32_t lane_off = (uint32_t)(quad * 32) << 16;
         float2 *stat = s_stat + ew * 32;                       // of this warp's rows
         uint8_t *outb = s_out + ew * G::NOUT * 2048;
@@ -222,12 +223,12 @@ k_gemm_p(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
         pdl_wait();
         for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++it) {
             const int tb = it & 1;
-            const int mt = t / n_nt, m0 = mt * 128, n0 = (t - mt * n_nt) * BN + half * G::HC;
+            const int mt = t / n_nt, m0 = mt * 128, n0 = (t - mt * n_nt) * BN + part * G::HC;
             const int mw = m0 + quad * 32, m = mw + lane;      // the warp's first row, this thread's row
             const int f0 = m0 / T, b1 = (f0 + 1) * T, b2 = b1 + T;     // first rows of the tile's second and third frame
             const bool valid = m < M;
             const int fo = valid ? (m >= b1) + (m >= b2) : 0;  // frame of the row, relative to f0
-            const float *tab = s_tab + (size_t)tb * (G::TAB_BYTES / 4) + fo * BN + half * G::HC;
+            const float *tab = s_tab + (size_t)tb * (G::TAB_BYTES / 4) + fo * BN + part * G::HC;
             // side operands of this tile
             if constexpr (FORM == FORM_RES) {
                 if (lane == 0) {
@@ -238,9 +239,9 @@ k_gemm_p(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
                 }
             }
             if constexpr (FORM == FORM_QKV) {
-                // the rotary rows of a quadrant are shared by its two warps: one loads them when both are done with the last
-                if (it > 0) asm volatile("bar.sync %0, 64;" ::"r"(1 + quad) : "memory");
-                if (half == 0 && lane == 0) {
+                // the rotary rows of a quadrant are shared by its warps: one loads them when all are done with the last
+                if (it > 0) asm volatile("bar.sync %0, %1;" ::"r"(1 + quad), "n"(32 * G::PARTS) : "memory");
+                if (part == 0 && lane == 0) {
                     const int nb = epi.D.dh > 32 ? 2 : 1;
                     mbar_expect_tx(sidebar, nb * 4096);
                     for (int h = 0; h < nb; ++h) tma_load_2d(smem_u32(s_side) + (quad * 2 + h) * 4096, &tm3, sidebar, 32 * h, mw);
@@ -315,7 +316,7 @@ k_gemm_p(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
 #pragma unroll 1
                 for (int sg = 0; sg < S; ++sg) {
                     wait_acc();
-                    const uint32_t ta = tmem_base + (ab & 1) * G::ACC_STRIDE + lane_off + half * G::HC;
+                    const uint32_t ta = tmem_base + (ab & 1) * G::ACC_STRIDE + lane_off + part * G::HC;
 #pragma unroll
                     for (int c = 0; c < G::HC; c += 16) {
                         uint32_t r[16];
@@ -339,7 +340,7 @@ k_gemm_p(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
             ok = ok && mbar_wait(tab_full + 8 * tb, (it >> 1) & 1, status);
             if (FORM != FORM_MLP) ok = ok && mbar_wait(sidebar, it & 1, status);
             ok = __all_sync(0xffffffffu, ok);
-            const uint32_t ta = tmem_base + (ab & 1) * G::ACC_STRIDE + lane_off + half * G::HC;
+            const uint32_t ta = tmem_base + (ab & 1) * G::ACC_STRIDE + lane_off + part * G::HC;
 #pragma unroll 1
             for (int g = 0; g < G::NG; ++g) {
                 const int n = n0 + 32 * g;                     // columns n .. n + 31

@@ -14,6 +14,7 @@ pytestmark = pytest.mark.gpu
     ((48, 28), 4, 2, 0, 3072, 12, 1),       # 2688 rows: several tiles per CTA, residual projections too
     ((48, 28), 4, 2, 1, 2730, 12, 1),       # gated, output columns that no tile divides
     ((48, 28), 4, 2, 0, 2052, 12, 0),       # stand-alone LayerNorm: plain bias
+    ((48, 28), 3, 2, 0, 3072, 12, 1),       # 2016 rows: residual projections 96 wide, K split and not
     ((40, 22), 4, 3, 0, 3072, 12, 1),       # 220 tokens: frames end inside tiles and inside a warp's 32 rows
     ((16, 16), 8, 4, 1, 2048, 12, 1),       # 64 tokens: three frames in a tile
     ((46, 30), 4, 2, 0, 3072, 24, 1),       # 345 tokens, head dimension 32
