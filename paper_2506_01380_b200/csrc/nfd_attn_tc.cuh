@@ -33,14 +33,17 @@
 // ring of NS stages (free again when S(n) is complete, which the barrier of accumulator n % NS tells), V blocks through
 // one of NS (free when P V is complete); V(n) and K(n + NS), which the issuer needs at the same time, arrive on one barrier.
 //
-// What bounds it: the softmax warps (exponentials: 672 clocks per 128 x 112 block on the special-function unit, 560
-// instructions a scheduler), the products take 490; a block takes about 1000.  Registers and code size count: spilled
+// What bounds it: the softmax warps (exponentials: 896 clocks per 128 x 112 block on the special-function unit), the
+// products take 490; a block takes about 1100.  Registers and code size count: spilled
 // registers are cold local memory, about 1 us on the path of a short item, and a cold code path costs as much.
 // Measured, 16 heads x 64 on one B200 (events around a launch): one frame of 336 tokens behind 16: 28.4 us with one thread
 // for all loads, one for all products and a maximum pass over S; 25.0 with the threads split and no maximum pass; 23.0
 // with three groups; 22.5 with items that overlap and the issuer's loop in one copy.  Two frames 37.3 -> 35.2 by the
 // last step, four 88.8 -> 74 -> 66 -> 61, eight frames behind 32 232 -> 188 -> 178 -> 165 (738 TFLOP/s).  Pages of
 // 220 tokens ran on the plain kernel, 1342 us; now 18.
+// Every exponential is the special-function unit's.  (Two pairs of eight by a polynomial on the FMA pipe took 22.5, 35.3,
+// 61.9 and 165 us where this takes 23.0, 37.3, 64.2 and 181; its range reduction saturated, which turns the score NaN into
+// a probability of nought, and its exponentials were good to 1e-5.)
 // Tried and worse: sixteen softmax warps with half a row each (178 -> 201: the fixed part of a block doubles); four epilogue
 // warps beside the groups (96 registers a thread: four frames 60, but 2 us more on every short launch).
 //
@@ -93,28 +96,6 @@ __device__ __forceinline__ float ex2_approx(float x) {
     return y;
 }
 
-// 2^y for two values y = S c - m on the FMA pipe: 2^n 2^f with n = round(y), f in [-1/2, 1/2], and 2^f by a
-// polynomial of degree 4 fitted for equal relative error (2.7e-6; the result is rounded to bf16, 2e-3, afterwards).
-// y is brought into [-125, 127] by the saturation of an FMA that maps this range to [0, 1]: ca = c / 252,
-// cb = (125 - m) / 252.
-#define EXP2_RANGE 252.0f
-#define EXP2_LOW 125.0f
-__device__ __forceinline__ float2 exp2_fma2(float s0, float s1, float ca, float cb) {
-    const float M = 12582912.0f;                           // 1.5 * 2^23: adding it rounds to an integer
-    auto k2 = [](float v) { return make_float2(v, v); };
-    float2 z;
-    asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(z.x) : "f"(s0), "f"(ca), "f"(cb));
-    asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(z.y) : "f"(s1), "f"(ca), "f"(cb));
-    const float2 t = ffma2(z, k2(EXP2_RANGE), k2(M - EXP2_LOW));     // M + n
-    const float2 n = fadd2(t, k2(EXP2_LOW - M));                     // n + 125
-    const float2 f = ffma2(z, k2(EXP2_RANGE), make_float2(-n.x, -n.y));
-    float2 p = ffma2(k2(0.009570100344717503f), f, k2(0.05591785907745361f));
-    p = ffma2(p, f, k2(0.240247443318367f));
-    p = ffma2(p, f, k2(0.6931217908859253f));
-    p = ffma2(p, f, k2(0.9999992847442627f));
-    return make_float2(__int_as_float(__float_as_int(p.x) + (__float_as_int(t.x) << 23)),
-                       __int_as_float(__float_as_int(p.y) + (__float_as_int(t.y) << 23)));
-}
 // add 1 with release and acquire semantics at device scope
 __device__ __forceinline__ unsigned int atomic_inc_acq_rel(unsigned int *p) {
     unsigned int v;
@@ -537,7 +518,6 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
                 }
                 // One pass over S, 16 columns at a time with the next load in flight: p = exp2(S c - m), written as packed
                 // bf16 pairs over columns of S that have been read already (keys k .. k+15 go to columns k/2 .. k/2+7).
-                const float c252 = c * (1.0f / EXP2_RANGE), b252 = (EXP2_LOW - m_run) * (1.0f / EXP2_RANGE);
                 float2 ls2[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
                 uint32_t sa[16], sb[16];
                 tmem_ld16(tS, sa);
@@ -550,13 +530,8 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
 #pragma unroll
                     for (int u = 0; u < 8; ++u) {
                         const float s0 = __uint_as_float(cur[2 * u]), s1 = __uint_as_float(cur[2 * u + 1]);
-                        float2 p;
-                        if (u == 3 || u == 7) {                   // on the FMA pipe
-                            p = exp2_fma2(s0, s1, c252, b252);
-                        } else {
-                            const float2 y = ffma2(make_float2(s0, s1), make_float2(c, c), make_float2(-m_run, -m_run));
-                            p = make_float2(ex2_approx(y.x), ex2_approx(y.y));
-                        }
+                        const float2 y = ffma2(make_float2(s0, s1), make_float2(c, c), make_float2(-m_run, -m_run));
+                        const float2 p = make_float2(ex2_approx(y.x), ex2_approx(y.y));
                         ls2[u & 3] = fadd2(ls2[u & 3], p);
                         const __nv_bfloat162 hp = __floats2bfloat162_rn(p.x, p.y);
                         pk[u] = *reinterpret_cast<const uint32_t *>(&hp);
