@@ -212,7 +212,8 @@ int nfd_attention(nfd_ctx *ctx, const void *q, const void *k, const void *v, int
  * call, so nothing needs clearing, but two calls whose kernels overlap on the
  * GPU (different streams) race on it -- serialise them.
  * Runs on `cuda_stream` (a cudaStream_t): bf16 with head_dim 64 or 32 on the tensor-core kernel, everything else on
- * the fp32 pipes. */
+ * the fp32 pipes.  Scores and sums are fp32 in both; the tensor-core kernel multiplies V by probabilities that are
+ * within 2^-17 of their fp32 value, so that a bf16 result has the error of its own rounding. */
 int nfd_attention_noalloc(const void *q, const void *k_pages, const void *v_pages, int dtype, int n_heads,
                           int head_dim, int tokens_per_frame, int n_q_frames, int n_kv_frames, int window,
                           void *out, void *cuda_stream);

@@ -8,11 +8,15 @@
 //     S  = Q K^T          UMMA 128 x KB x 64, operands in shared memory (TMA),
 //                         accumulator in tensor memory
 //     P  = exp2(S*c - m)  one thread per query row: TMEM -> registers, running
-//                         sum, bf16 P written back to tensor memory over
-//                         the first half of the S columns it came from
-//     O += P V            UMMA 128 x 64 x KB, P read from tensor memory, V used
+//                         sum, P written back to tensor memory as the sum of two
+//                         bf16 numbers, over the S columns it came from
+//     O += P V            two UMMAs 128 x 64 x KB, P read from tensor memory, V used
 //                         straight from its page (MN-major B operand in shared
 //                         memory), accumulated in tensor memory
+// The second number of P keeps what rounding to bf16 leaves (2^-17 of P at most is lost), so that the error of the result
+// is that of its own rounding to bf16: 1.66e-3 (2-norm) for normal data, as with fp32 probabilities.  With the first
+// number alone it was 2.33e-3 whatever the data; the product doubles and a block takes about 200 clocks more (16 heads
+// x 64, 336 tokens: one frame 23.0 -> 25.0 us, two 37.3 -> 40.9, four 64.2 -> 70.7, eight streams 181 -> 210).
 // The reference m of a row is the largest of the first 16 scores of the item and is never changed: a probability is
 // exact to the same number of bits whatever its size, so that m only has to keep exp2 in range.  With no maximum to take
 // there is no state to rescale, and all softmax groups share one m and one O accumulator.  Should a block's sum of a
@@ -33,8 +37,8 @@
 // ring of NS stages (free again when S(n) is complete, which the barrier of accumulator n % NS tells), V blocks through
 // one of NS (free when P V is complete); V(n) and K(n + NS), which the issuer needs at the same time, arrive on one barrier.
 //
-// What bounds it: the softmax warps (exponentials: 896 clocks per 128 x 112 block on the special-function unit), the
-// products take 490; a block takes about 1100.  Registers and code size count: spilled
+// What bounds it: the softmax warps (exponentials: 896 clocks per 128 x 112 block on the special-function unit) and the
+// turn of an accumulator, S -> softmax -> P V; the products take 700; a block takes about 1300.  Registers and code size count: spilled
 // registers are cold local memory, about 1 us on the path of a short item, and a cold code path costs as much.
 // Measured, 16 heads x 64 on one B200 (events around a launch): one frame of 336 tokens behind 16: 28.4 us with one thread
 // for all loads, one for all products and a maximum pass over S; 25.0 with the threads split and no maximum pass; 23.0
@@ -96,6 +100,24 @@ __device__ __forceinline__ float ex2_approx(float x) {
     return y;
 }
 
+// p as a sum of two bf16 numbers: hi = p rounded, lo = what that leaves, rounded (2^-17 of p at most is lost), as
+// packed pairs.  The subtraction takes hi as it is packed (fma with a bf16 factor).
+__device__ __forceinline__ void bf16_split2(float2 p, uint32_t &hi, uint32_t &lo) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(p.x, p.y);
+    hi = *reinterpret_cast<const uint32_t *>(&h);
+    float2 d;
+    asm("{\n"
+        ".reg .b16 a, b, m1;\n"
+        "mov.b32 {a, b}, %2;\n"
+        "mov.b16 m1, 0xBF80;\n"                            // -1
+        "fma.rn.f32.bf16 %0, a, m1, %3;\n"
+        "fma.rn.f32.bf16 %1, b, m1, %4;\n"
+        "}\n"
+        : "=f"(d.x), "=f"(d.y)
+        : "r"(hi), "f"(p.x), "f"(p.y));
+    const __nv_bfloat162 l = __floats2bfloat162_rn(d.x, d.y);
+    lo = *reinterpret_cast<const uint32_t *>(&l);
+}
 // add 1 with release and acquire semantics at device scope
 __device__ __forceinline__ unsigned int atomic_inc_acq_rel(unsigned int *p) {
     unsigned int v;
@@ -405,8 +427,10 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
                     const uint32_t tP = tmem + A::S_STRIDE * st;
 #pragma unroll
                     for (int i = 0; i < KB / 16; ++i) {
-                        // P: 16 keys = 8 columns of packed bf16 pairs; V: MN-major, 16 keys = 2 KiB per step
-                        umma_bf16_ts(tmem + A::TM_O, tP + 8 * i, vd + (uint64_t)(i * (2048 >> 4)), idesc_pv, i ? 1u : acc);
+                        // P: 16 keys = 8 columns of packed bf16 pairs, and 8 of what they leave; V: MN-major, 16 keys = 2 KiB
+                        const uint64_t vi = vd + (uint64_t)(i * (2048 >> 4));
+                        umma_bf16_ts(tmem + A::TM_O, tP + 16 * i, vi, idesc_pv, i ? 1u : acc);
+                        umma_bf16_ts(tmem + A::TM_O, tP + 16 * i + 8, vi, idesc_pv, 1u);
                     }
                     umma_commit(v_empty + 8 * st);         // P V(n) is complete: V's stage is free, O at rest
                     if (++st == A::NS) st = 0, ++lap;
@@ -516,8 +540,8 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
                     }
                     if (!some) break;
                 }
-                // One pass over S, 16 columns at a time with the next load in flight: p = exp2(S c - m), written as packed
-                // bf16 pairs over columns of S that have been read already (keys k .. k+15 go to columns k/2 .. k/2+7).
+                // One pass over S, 16 columns at a time with the next load in flight: p = exp2(S c - m), written as two packed
+                // bf16 pairs over the columns it came from (keys k .. k+15: the first numbers go to columns k .. k+7).
                 float2 ls2[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
                 uint32_t sa[16], sb[16];
                 tmem_ld16(tS, sa);
@@ -526,17 +550,16 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
                     uint32_t *cur = ((cc >> 4) & 1) ? sb : sa, *nxt = ((cc >> 4) & 1) ? sa : sb;
                     tmem_ld_wait();
                     if (cc + 16 < KB) tmem_ld16(tS + cc + 16, nxt);
-                    uint32_t pk[8];
+                    uint32_t pk[16];
 #pragma unroll
                     for (int u = 0; u < 8; ++u) {
                         const float s0 = __uint_as_float(cur[2 * u]), s1 = __uint_as_float(cur[2 * u + 1]);
                         const float2 y = ffma2(make_float2(s0, s1), make_float2(c, c), make_float2(-m_run, -m_run));
                         const float2 p = make_float2(ex2_approx(y.x), ex2_approx(y.y));
                         ls2[u & 3] = fadd2(ls2[u & 3], p);
-                        const __nv_bfloat162 hp = __floats2bfloat162_rn(p.x, p.y);
-                        pk[u] = *reinterpret_cast<const uint32_t *>(&hp);
+                        bf16_split2(p, pk[u], pk[8 + u]);
                     }
-                    tmem_st8(tS + (cc >> 1), pk);
+                    tmem_st16(tS + cc, pk);
                 }
                 const float ls = ((ls2[0].x + ls2[0].y) + (ls2[1].x + ls2[1].y)) + ((ls2[2].x + ls2[2].y) + (ls2[3].x + ls2[3].y));
                 l_run += ls;
