@@ -1366,7 +1366,7 @@ static bool noalloc_launch_tc(int dev, cudaStream_t st, const StepParams *d_sp, 
     attn_blocks(pl, D.T);
     pl.CH = (D.W + 1) * pl.BPF, pl.MAXSPLIT = 1;
     const long long n_items = (long long)pl.QT * D.H * n_q;
-    if (!attn_divisors(pl, D.H, n_items, D.W)) return false;
+    if (!attn_divisors(pl, D.H, n_items, D.W, n_sm[dev])) return false;
     return launch_attn_plan(enc[dev], n_sm[dev], st, d_sp, D, n_q, 0, pl, (size_t)D.R * D.H, (const bf16 *)q,
                             (const bf16 *)k_pages, (const bf16 *)v_pages, (bf16 *)out, nullptr, nullptr, d_stat) != 0;
 }

@@ -20,10 +20,12 @@
 // The reference m of a row is the largest of the first 16 scores of the item and is never changed: a probability is
 // exact to the same number of bits whatever its size, so that m only has to keep exp2 in range.  With no maximum to take
 // there is no state to rescale, and all softmax groups share one m and one O accumulator.  Should a block's sum of a
-// row pass 2^100 (scores rising by more than 69 nats over the first ones), the item is computed again on the plain path
-// (attn_item_plain).  No barrier joins the groups at the end of an item: m, found by the group of
-// the first block, and the sums go through shared memory and barriers of their own, two items deep, and the group of
-// an item's last block reads O and finishes the item while the others go on (groups 0 and 1 share a CTA's last item).
+// row pass 2^100 (scores rising by more than 69 nats over the first ones), all of its first scores be -inf, or O leave fp32,
+// the item is walked twice more when the CTA is through with its items: once for the true maxima of its rows and once with
+// these as m (attn_again).  No data takes more than three times as long, and no wait is any longer.
+// No barrier joins the groups at the end of an item: m, found by the group of the first block, and the sums go through shared
+// memory and barriers of their own, two items deep, and the group of an item's last block reads O and finishes the item while
+// the others go on (groups 0 and 1 share a CTA's last item).
 //
 // Warps 0 and 3 = TMA producers (K, V), warp 1 = issuer of all products (and loader of Q), warps 4-15 = three softmax
 // groups of four warps; group g takes the CTA's blocks n with
@@ -73,14 +75,19 @@ struct AttnPlan {
 // A published state: [16 groups of 4 columns][128 rows] float4, then [2 halves of O][128 rows] (m, l).
 #define ATTN_STATE_BYTES (128 * 64 * 4 + 2 * 128 * 8)
 #define ATTN_COUNTERS 8          // of a query tile: one per half of O and quadrant of its rows
+#define ATTN_CTA_ITEMS 2048      // items of a CTA, at most: each has a byte of shared memory (see attn_finish)
+// Flags that are read when all roles are through: an item is marked, a wait has run out.  (In registers, with a vote at the
+// end, they cost two frames 39.6 -> 41.5 us.)
+#define ATTN_MARKED 1u
+#define ATTN_EXPIRED 2u
 
 template <int KB> struct AttnCfg {
     static constexpr int NS = KB <= 112 ? 4 : 3;           // S accumulators = stages of the K and the V ring
     static constexpr int NGRP = 3;                         // softmax groups
     static constexpr int Q_BYTES = 128 * 128;              // two of them
     static constexpr int KV_BYTES = KB * 128;              // one K (or V) block
-    static constexpr int ML_BYTES = 2 * (1 + NGRP) * 128 * 4;   // m of every row, l of every row and group; two items
-    static constexpr int SMEM = 2 * Q_BYTES + 2 * NS * KV_BYTES + ML_BYTES + 256 + 1024;
+    static constexpr int ML_BYTES = (2 * (1 + NGRP) + 1) * 128 * 4;   // m of every row, l of every row and group, two items; maxima
+    static constexpr int SMEM = 2 * Q_BYTES + 2 * NS * KV_BYTES + ML_BYTES + 8 + ATTN_CTA_ITEMS + 256 + 1024;
     static constexpr int TMEM_COLS = 512;
     static constexpr int S_STRIDE = KB <= 112 ? 112 : 128; // S accumulators from column 0, O at column 448
     static constexpr int TM_O = 448;
@@ -141,9 +148,9 @@ struct AttnItem {
         nb = min(nbt, b0 + pl.CH) - b0;
         if (nb < 0) nb = 0;
     }
-    // the first item at or after `item` (in steps of the grid) that has blocks; n_items or more: there is none
-    __device__ __forceinline__ int find(int item, int n_items, const StepParams *sp, const Dims &D, const AttnPlan &pl) {
-        for (; item < n_items; item += gridDim.x) {
+    // the first item at or after `item` (in steps of the grid) that has blocks; `end` or more: there is none
+    __device__ __forceinline__ int find(int item, int end, const StepParams *sp, const Dims &D, const AttnPlan &pl) {
+        for (; item < end; item += gridDim.x) {
             set(item, sp, D, pl);
             if (nb > 0) break;
         }
@@ -151,41 +158,15 @@ struct AttnItem {
     }
 };
 
-// One row of an item without tensor cores (see the note on m at the top): columns c0 .. c0 + 31 of O relative to the
-// row's maximum, the maximum and the sum.  q: the row (dh values); kp, vp: the pages.
-static __device__ __noinline__ void attn_item_plain(const AttnItem &w, const Dims &D, const AttnPlan &pl,
-                                                    int KB, int layer, const bf16 *q, const bf16 *kp, const bf16 *vp, float c,
-                                                    int c0, float *O, float *m_out, float *l_out) {
-    float m = -INFINITY, l = 0.f;
-    for (int e = 0; e < 32; ++e) O[e] = 0.f;
-    const int dh = D.dh;
-    for (int b = w.b0; b < w.b0 + w.nb; ++b) {
-        const int f = b / pl.BPF, k0 = (b - f * pl.BPF) * KB, k1 = min(k0 + KB, D.T);
-        const size_t off = kv_page_offset(D, w.fr.stream, layer, w.fr.win_first + f) + (size_t)w.h * D.T * dh;
-        for (int key = k0; key < k1; ++key) {
-            const bf16 *kr = kp + off + (size_t)key * dh, *vr = vp + off + (size_t)key * dh;
-            float s = 0.f;
-            for (int e = 0; e < dh; ++e) s = fmaf(to_f(q[e]), to_f(kr[e]), s);
-            s *= c;
-            const float mn = fmaxf(m, s), fo = m == mn ? 1.0f : ex2_approx(m - mn), p = ex2_approx(s - mn);
-            l = fmaf(l, fo, p), m = mn;
-            const float pb = to_f(__float2bfloat16_rn(p));
-            for (int e = 0; e < 32; ++e)
-                if (c0 + e < dh) O[e] = fmaf(pb, to_f(vr[c0 + e]), O[e] * fo);
-        }
-    }
-    *m_out = m, *l_out = l;
-}
-
 // The end of an item for one warp: halves p0 .. p0 + np - 1 (32 columns each) of the 32 rows of its quadrant are read from
 // tensor memory and written out, or published; of the warps that hold a half of a tile's rows in its splits, the one that
 // finishes last merges them in split order.  (A counter per half and quadrant: no barrier of the CTA.)
-// m, l: reference and sum of this thread's row (an infinite sum: the row is computed again, see the note on m).
-template <int KB>
-static __device__ __forceinline__ void attn_finish(const AttnItem &w, int item, int p0, int np, uint32_t tO, uint32_t o_free, int trow, float m, float l,
-                                            float c, const StepParams *sp, const Dims &D, const AttnPlan &pl, int layer,
-                                            const bf16 *gq, const bf16 *gk, const bf16 *gv, bf16 *out, float *part_o,
-                                            unsigned int *counters) {
+// m, l: reference and sum of this thread's row.  With `redo` (see AttnShared; a byte per item, a bit per half and
+// quadrant; this is item `num`) a half whose l or O has left fp32 is left alone and marked there; without it, `mask` tells
+// which halves to take.
+static __device__ __forceinline__ void attn_finish(const AttnItem &w, int p0, int np, int mask, uint32_t tO, uint32_t o_free,
+                                                   int trow, float m, float l, const Dims &D, const AttnPlan &pl, bf16 *out,
+                                                   float *part_o, unsigned int *counters, uint32_t *redo, int num) {
     const int lane = threadIdx.x & 31, row = w.qt * 128 + trow;
     const size_t item_q = ((size_t)w.j * D.H + w.h) * pl.QT + w.qt;
     uint8_t *states = reinterpret_cast<uint8_t *>(part_o) + item_q * pl.MAXSPLIT * ATTN_STATE_BYTES;
@@ -205,29 +186,31 @@ static __device__ __forceinline__ void attn_finish(const AttnItem &w, int item, 
     };
 #pragma unroll 1
     for (int p = p0; p < p0 + np; ++p) {
-        float O[32], mp = m, lp = l;
+        float O[32];
         tmem_ld32(tO + 32 * p, reinterpret_cast<uint32_t *>(O));
         tmem_ld_wait();
-        if (l == INFINITY) {
-            pdl_wait();                                    // this thread reads global memory itself
-            AttnItem wc;                                   // (looked up again: nothing of this path stays in registers)
-            wc.set(item, sp, D, pl);
-            float Oc[32], mc, lc;
-            attn_item_plain(wc, D, pl, KB, layer, gq + ((size_t)w.h * (size_t)(sp->nf * D.T) + w.j * D.T + min(row, D.T - 1)) * D.dh,
-                            gk, gv, c, 32 * p, Oc, &mc, &lc);
-            mp = mc, lp = lc;
+        if (redo) {
+            float2 x = make_float2(0.f, 0.f);              // NaN if an element of O is infinite or NaN
 #pragma unroll
-            for (int e = 0; e < 32; ++e) O[e] = Oc[e];
+            for (int e = 0; e < 32; e += 2) x = ffma2(make_float2(O[e], O[e + 1]), make_float2(0.f, 0.f), x);
+            // (rows beyond the frame's are another frame's or nothing, and not looked at)
+            if (__any_sync(0xffffffffu, row < D.T && (l == INFINITY || x.x != x.x || x.y != x.y))) {
+                mask &= ~(1 << p);
+                if (lane == 0) {
+                    atomicOr(redo, ATTN_MARKED);
+                    atomicOr(redo + 2 + (num >> 2), 1u << (8 * (num & 3) + 4 * p + (trow >> 5)));
+                }
+            }
         }
-        __syncwarp();
+        if (!((mask >> p) & 1)) continue;
         if (w.nsplit == 1) {
-            write_part(p, O, lp);
+            write_part(p, O, l);
         } else {
             uint8_t *st = states + (size_t)w.split * ATTN_STATE_BYTES;
 #pragma unroll
             for (int e = 0; e < 8; ++e)
                 *reinterpret_cast<float4 *>(st + o_at(p) + e * 2048) = make_float4(O[4 * e], O[4 * e + 1], O[4 * e + 2], O[4 * e + 3]);
-            *reinterpret_cast<float2 *>(st + ml_at(p)) = make_float2(mp, lp);
+            *reinterpret_cast<float2 *>(st + ml_at(p)) = make_float2(m, l);
         }
     }
     tc_fence_before();
@@ -235,7 +218,7 @@ static __device__ __forceinline__ void attn_finish(const AttnItem &w, int item, 
     if (lane == 0 && o_free) mbar_arrive(o_free);
     if (w.nsplit == 1) return;
     unsigned int last = 0;
-    if (lane < np) {
+    if (lane < np && ((mask >> (p0 + lane)) & 1)) {
         unsigned int *cnt = counters + item_q * ATTN_COUNTERS + (p0 + lane) * 4 + (trow >> 5);
         last = atomic_inc_acq_rel(cnt) == (unsigned int)(w.nsplit - 1);
         if (last) *cnt = 0;                                // ready for the next launch
@@ -264,7 +247,8 @@ static __device__ __forceinline__ void attn_finish(const AttnItem &w, int item, 
             for (int u = 0; u < 1; ++u) {
                 if (s0 + u >= w.nsplit) break;
                 const float mb = fmaxf(mx, ml[u].x);
-                const float fo = mx == mb ? 1.0f : ex2_approx(mx - mb), wgt = ex2_approx(ml[u].x - mb);
+                // (a state with nothing but scores of -inf has m = -inf and counts for nothing)
+                const float fo = mx == mb ? 1.0f : ex2_approx(mx - mb), wgt = ml[u].x == -INFINITY ? 0.f : ex2_approx(ml[u].x - mb);
                 mx = mb;
                 lt = fmaf(ml[u].y, wgt, __fmul_rn(lt, fo));
 #pragma unroll
@@ -280,64 +264,74 @@ static __device__ __forceinline__ void attn_finish(const AttnItem &w, int item, 
     }
 }
 
-template <int KB>
-__global__ void __launch_bounds__(AttnCfg<KB>::THREADS, 1)
-k_attn_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
-          const __grid_constant__ CUtensorMap tmV, const StepParams *sp, const __grid_constant__ Dims D, int layer,
-          const __grid_constant__ AttnPlan pl, int n_items, const bf16 *gq, const bf16 *gk, const bf16 *gv, bf16 *out, float *part_o, unsigned int *counters, int *status) {
+// The shared memory of a CTA, and its tensor memory.
+template <int KB> struct AttnShared {
     using A = AttnCfg<KB>;
-    extern __shared__ uint8_t smem_raw[];
-    NFD_TRACE_T0();
-    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    uint8_t *sKV = smem + 2 * A::Q_BYTES;
-    float *s_m = reinterpret_cast<float *>(sKV + 2 * A::NS * A::KV_BYTES);      // [item parity][128]
-    float *s_l = s_m + 2 * 128;                                                       // [item parity][group][128]
-    uint64_t *bars = reinterpret_cast<uint64_t *>(sKV + 2 * A::NS * A::KV_BYTES + A::ML_BYTES);
-    // barriers: q_full[2] | q_empty[2] | o_free | k_first[NS] (K of blocks 0 .. NS-1) | s_full[NS] | p_full[NS] |
-    // kv_full[NS] (V(n) and K(n + NS)) | v_empty[NS] | m_full[2] | l_full[2] | ml_empty[2]
-    const uint32_t q_full = smem_u32(bars), q_empty = q_full + 16, o_free = q_empty + 16, k_first = o_free + 8,
-                   s_full = k_first + 8 * A::NS, p_full = s_full + 8 * A::NS, kv_full = p_full + 8 * A::NS,
-                   v_empty = kv_full + 8 * A::NS, m_full = v_empty + 8 * A::NS, l_full = m_full + 16, ml_empty = l_full + 16;
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 11 + 5 * A::NS);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // The first item's descriptor: its loads are in flight during the set-up.  (The pass descriptor was written by the
-    // first kernel of the pass, which completed before this kernel's predecessor began.)
-    AttnItem w0;
-    w0.set(blockIdx.x, sp, D, pl);
-
-    if (warp == 0 && lane == 0) {
-        tma_prefetch_desc(&tmQ);
-        tma_prefetch_desc(&tmK);
-        tma_prefetch_desc(&tmV);
+    uint32_t q, kv, bars, tmem;
+    float *m, *l, *mx;       // [item parity][128], [item parity][group][128], [128] true maxima (times c)
+    uint32_t *redo;          // flags (below), nothing, and a byte per item (see attn_finish)
+    __device__ __forceinline__ uint32_t *tmem_slot() const { return redo + 2 + ATTN_CTA_ITEMS / 4 + 2 * (11 + 5 * A::NS); }
+    __device__ __forceinline__ AttnShared(uint8_t *raw) {
+        uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~(uintptr_t)1023);
+        q = smem_u32(smem), kv = q + 2 * A::Q_BYTES, tmem = 0;
+        m = reinterpret_cast<float *>(smem + 2 * A::Q_BYTES + 2 * A::NS * A::KV_BYTES), l = m + 2 * 128;
+        mx = l + 2 * A::NGRP * 128, redo = reinterpret_cast<uint32_t *>(mx + 128);
+        bars = smem_u32(redo + 2 + ATTN_CTA_ITEMS / 4);
+    }
+    // barriers (K of blocks 0 .. NS-1 arrives on k_first, V(n) and K(n + NS) on kv_full)
+    __device__ __forceinline__ uint32_t q_full() const { return bars; }
+    __device__ __forceinline__ uint32_t q_empty() const { return bars + 16; }
+    __device__ __forceinline__ uint32_t m_full() const { return bars + 32; }
+    __device__ __forceinline__ uint32_t l_full() const { return bars + 48; }
+    __device__ __forceinline__ uint32_t ml_empty() const { return bars + 64; }
+    __device__ __forceinline__ uint32_t o_free() const { return bars + 80; }
+    __device__ __forceinline__ uint32_t k_first() const { return bars + 88; }
+    __device__ __forceinline__ uint32_t s_full() const { return k_first() + 8 * A::NS; }
+    __device__ __forceinline__ uint32_t p_full() const { return s_full() + 8 * A::NS; }
+    __device__ __forceinline__ uint32_t kv_full() const { return p_full() + 8 * A::NS; }
+    __device__ __forceinline__ uint32_t v_empty() const { return kv_full() + 8 * A::NS; }
+    __device__ __forceinline__ void init_bars() const {
         for (int s = 0; s < 2; ++s) {
-            mbar_init(q_full + 8 * s, 1);
-            mbar_init(q_empty + 8 * s, 1);
-            mbar_init(m_full + 8 * s, 4);                  // one arrival per warp of the group that finds m
-            mbar_init(l_full + 8 * s, 4 * A::NGRP);        // one per softmax warp
-            mbar_init(ml_empty + 8 * s, 4);                // one per warp of the group that finishes the item
+            mbar_init(q_full() + 8 * s, 1);
+            mbar_init(q_empty() + 8 * s, 1);
+            mbar_init(m_full() + 8 * s, 4);                // one arrival per warp of the group that finds m
+            mbar_init(l_full() + 8 * s, 4 * A::NGRP);      // one per softmax warp
+            mbar_init(ml_empty() + 8 * s, 4);              // one per warp of the group that finishes the item
         }
-        mbar_init(o_free, 4);                              // one arrival per warp that has read O
+        mbar_init(o_free(), 4);                            // one arrival per warp that has read O
         for (int s = 0; s < A::NS; ++s) {
-            mbar_init(k_first + 8 * s, 1);
-            mbar_init(s_full + 8 * s, 1);
-            mbar_init(p_full + 8 * s, 4);                  // one arrival per softmax warp of the group
-        }
-        for (int s = 0; s < A::NS; ++s) {
-            mbar_init(kv_full + 8 * s, 2);                 // one arrival per producer
-            mbar_init(v_empty + 8 * s, 1);
+            mbar_init(k_first() + 8 * s, 1);
+            mbar_init(s_full() + 8 * s, 1);
+            mbar_init(p_full() + 8 * s, 4);                // one arrival per softmax warp of the group
+            mbar_init(kv_full() + 8 * s, 2);               // one arrival per producer
+            mbar_init(v_empty() + 8 * s, 1);
         }
         fence_mbar_init();
     }
-    if (warp == 1) {
-        tmem_alloc(smem_u32(tmem_slot), A::TMEM_COLS);
-        tmem_relinquish();
+    __device__ __forceinline__ void inval_bars() const {
+        for (int i = 0; i < 11 + 5 * A::NS; ++i) mbar_inval(bars + 8 * i);
     }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
+};
 
-    // Blocks are numbered through the CTA's items (n): ring stages, accumulators and barrier phases follow n.
+// What a walk through items is for: the results, with m from the first scores; the true maxima of an item's rows (S alone
+// counts: P and O are not looked at); the results with these as m.
+enum { RD_FIRST, RD_MAX, RD_AGAIN };
+
+// The CTA's items first, first + gridDim.x, ... below end (w0 is the first one); `num`: number of the item in sh.redo, not for
+// RD_FIRST.
+template <int KB>
+__device__ __forceinline__ void attn_items(const AttnShared<KB> &sh, const CUtensorMap &tmQ, const CUtensorMap &tmK,
+                                           const CUtensorMap &tmV, const StepParams *sp, const Dims &D, int layer, const AttnPlan &pl,
+                                           const AttnItem &w0, int first, int end, int mode, int num, bf16 *out, float *part_o,
+                                           unsigned int *counters, int *status) {
+    using A = AttnCfg<KB>;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t q_full = sh.q_full(), q_empty = sh.q_empty(), o_free = sh.o_free(), k_first = sh.k_first(), s_full = sh.s_full(),
+                   p_full = sh.p_full(), kv_full = sh.kv_full(), v_empty = sh.v_empty(), m_full = sh.m_full(), l_full = sh.l_full(),
+                   ml_empty = sh.ml_empty(), tmem = sh.tmem;
+    float *s_m = sh.m, *s_l = sh.l;
+    bool ok = true;
+    // Blocks are numbered through the items (n): ring stages, accumulators and barrier phases follow n.
     if (warp == 0 || warp == 3) {
         // ---------------- TMA producers: K (warp 0), V (warp 3) ----------------
         // The two loops are kept short and free of divisions: as one thread with a division per block they took
@@ -345,14 +339,14 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
         // and this thread, not the softmax, set the pace of the whole kernel.
         if (elect_one()) {
             const bool is_k = warp == 0;
-            const uint32_t ring = smem_u32(sKV) + (is_k ? 0 : A::NS * A::KV_BYTES);
+            const uint32_t ring = sh.kv + (is_k ? 0 : A::NS * A::KV_BYTES);
             const CUtensorMap *tm = is_k ? &tmK : &tmV;
             const uint32_t empty = is_k ? s_full : v_empty;
-            bool waited = false, ok = true;
+            bool waited = false;
             int st = 0, lap = 0;                           // ring stage of the next block, how often the ring was filled
             AttnItem w = w0;
-            for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
-                if (item != blockIdx.x) w.set(item, sp, D, pl);
+            for (int item = first; item < end && ok; item += gridDim.x) {
+                if (item != first) w.set(item, sp, D, pl);
                 const int f = pl.bpf_div.div(w.b0);
                 int kb = w.b0 - f * pl.BPF;
                 int left = w.fr.first_new - (w.fr.win_first + f);      // frames until the pages that this pass writes
@@ -387,19 +381,19 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
                     if (ok) mbar_arrive(kv_full + 8 * (x % A::NS));
                 }
             }
+            if (!ok) atomicOr(sh.redo, ATTN_EXPIRED);
         }
     } else if (warp == 1) {
         // ---------------- issuer of S = Q K^T and O += P V, loader of Q ----------------
         if (elect_one()) {
             pdl_launch();
             constexpr uint32_t idesc_s = umma_idesc_bf16(128, KB), idesc_pv = umma_idesc_bf16_bmn(128, 64);
-            const uint32_t sQ = smem_u32(smem), sK = smem_u32(sKV), sV = sK + A::NS * A::KV_BYTES;
-            bool ok = true;
+            const uint32_t sQ = sh.q, sK = sh.kv, sV = sK + A::NS * A::KV_BYTES;
             // S runs NS blocks ahead of P V: items of their own for both.  (One copy of the code for both the first S and the
             // later ones: this thread's registers and instruction fetches are on every block's path.)
             AttnItem ws = w0, w = w0;
-            int item_s = blockIdx.x, it_s = -1, left_s = 0;            // item whose Q was asked for last; items before S's; S to come
-            int item = blockIdx.x - gridDim.x, it = 0, left = 0;       // the same for P V
+            int item_s = first, it_s = -1, left_s = 0;            // item whose Q was asked for last; items before S's; S to come
+            int item = first - gridDim.x, it = 0, left = 0;            // the same for P V
             int st_s = 0, lap_s = 0, st = 0, lap = 0;
             int ahead = A::NS;                             // S to issue before the first P V
             auto load_q = [&](int qs) {                    // Q of item ws
@@ -407,21 +401,22 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
                 tma_load_3d(sQ + qs * A::Q_BYTES, &tmQ, q_full + 8 * qs, 0, ws.j * D.T + ws.qt * 128, ws.h);
             };
             pdl_wait();
-            if (ws.nb == 0) item_s = ws.find(item_s + gridDim.x, n_items, sp, D, pl);
-            if (item_s < n_items) load_q(0);
+            if (ws.nb == 0) item_s = ws.find(item_s + gridDim.x, end, sp, D, pl);
+            if (item_s < end) load_q(0);
             while (ok) {
                 if (ahead > 0) {
                     --ahead;
                 } else {
                     uint32_t acc = 1;
                     if (left == 0) {
-                        item = w.find(item + gridDim.x, n_items, sp, D, pl);
-                        if (item >= n_items) break;
+                        item = w.find(item + gridDim.x, end, sp, D, pl);
+                        if (item >= end) break;
                         left = w.nb, acc = 0;
-                        if (it > 0 && !mbar_wait(o_free, (it - 1) & 1, status)) break;     // O of the last item has been read
+                        if (it > 0) ok = mbar_wait(o_free, (it - 1) & 1, status);          // O of the last item has been read
                         ++it;
                     }
-                    if (!mbar_wait(kv_full + 8 * st, lap & 1, status) || !mbar_wait(p_full + 8 * st, lap & 1, status)) break;
+                    ok = ok && mbar_wait(kv_full + 8 * st, lap & 1, status) && mbar_wait(p_full + 8 * st, lap & 1, status);
+                    if (!ok) break;
                     tc_fence_after();
                     const uint64_t vd = umma_desc_k128(sV + st * A::KV_BYTES);
                     const uint32_t tP = tmem + A::S_STRIDE * st;
@@ -438,11 +433,11 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
                 }
                 // S of the next block, if there is one, into the accumulator that P V(n) reads
                 if (left_s == 0) {
-                    if (item_s >= n_items) continue;
+                    if (item_s >= end) continue;
                     ++it_s, left_s = ws.nb;
                     ok = mbar_wait(q_full + 8 * (it_s & 1), (it_s >> 1) & 1, status);
-                    item_s = ws.find(item_s + gridDim.x, n_items, sp, D, pl);
-                    if (item_s < n_items) {                // Q of the item after it
+                    item_s = ws.find(item_s + gridDim.x, end, sp, D, pl);
+                    if (item_s < end) {                    // Q of the item after it
                         if (it_s >= 1) ok = ok && mbar_wait(q_empty + 8 * ((it_s + 1) & 1), ((it_s - 1) >> 1) & 1, status);
                         load_q((it_s + 1) & 1);
                     }
@@ -459,6 +454,12 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
                 if (++st_s == A::NS) st_s = 0, ++lap_s;
                 if (--left_s == 0) umma_commit(q_empty + 8 * (it_s & 1));
             }
+            // completions that nobody has waited for yet: none may arrive when the barriers are set up anew
+            const int n = lap * A::NS + st;
+            for (int x = n > A::NS ? n - A::NS : 0; x < n; ++x)
+                ok = ok && mbar_wait(v_empty + 8 * (x % A::NS), (x / A::NS) & 1, status);
+            for (int i = it_s > 0 ? it_s - 1 : 0; i <= it_s; ++i) ok = ok && mbar_wait(q_empty + 8 * (i & 1), (i >> 1) & 1, status);
+            if (!ok) atomicOr(sh.redo, ATTN_EXPIRED);
         }
     } else if (warp == 2) {
         // no work of its own (the softmax warps start at a multiple of four: a warp reads tensor-memory lanes 32 (warp % 4) ..)
@@ -469,16 +470,15 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
         const int trow = quad * 32 + lane;
         const uint32_t lane_off = (uint32_t)(quad * 32) << 16;
         const float c = (1.0f / sqrtf((float)D.dh)) * 1.4426950408889634f;   // softmax scale in the log2 domain
-        bool ok = true;
         int n0 = 0, n03 = 0, it = 0;                       // the item's first block, that modulo 3, items before it
         const uint32_t tO = tmem + A::TM_O + lane_off;
         AttnItem w = w0;
-        int item = blockIdx.x;
-        if (w.nb == 0) item = w.find(item + gridDim.x, n_items, sp, D, pl);
-        while (item < n_items) {
+        int item = first;
+        if (w.nb == 0) item = w.find(item + gridDim.x, end, sp, D, pl);
+        while (item < end) {
             const int ip = it & 1, iph = (it >> 1) & 1;    // item parity: which m and l, phase of their barriers
             const int r = g >= n03 ? g - n03 : g - n03 + A::NGRP;      // this group's blocks: b % 3 == r
-            float m_run = 0.f, l_run = 0.f, l_top = 0.f;   // l_top: the largest sum of a block
+            float m_run = 0.f, l_run = mode == RD_MAX ? -INFINITY : 0.f, l_top = 0.f;      // l_top: the largest sum of a block
             int kb = w.b0 + r;                             // block of the page, for the mask of its last block
             kb -= pl.bpf_div.div(kb) * pl.BPF;
             for (int b = r; b < w.nb || b == r; b += A::NGRP) {
@@ -529,7 +529,7 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
                         float mx = -INFINITY;
 #pragma unroll
                         for (int e = 0; e < 16; ++e) mx = fmaxf(mx, __uint_as_float(x[e]));
-                        m_run = mx * c;
+                        m_run = mode == RD_AGAIN ? sh.mx[trow] : mx * c;
                         s_m[ip * 128 + trow] = m_run;
                         __syncwarp();
                         if (lane == 0) mbar_arrive(m_full + 8 * ip);
@@ -539,6 +539,20 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
                         __syncwarp();
                     }
                     if (!some) break;
+                }
+                if (mode == RD_MAX) {                      // l_run: the largest score
+#pragma unroll 1
+                    for (int cc = 0; cc < KB; cc += 16) {
+                        uint32_t x[16];
+                        tmem_ld16(tS + cc, x);
+                        tmem_ld_wait();
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) l_run = fmaxf(l_run, __uint_as_float(x[e]));
+                    }
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(p_full + 8 * st);
+                    continue;
                 }
                 // One pass over S, 16 columns at a time with the next load in flight: p = exp2(S c - m), written as two packed
                 // bf16 pairs over the columns it came from (keys k .. k+15: the first numbers go to columns k .. k+7).
@@ -571,37 +585,112 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
             }
             NFD_TRACE_MARK_T(TRK_OTHER + 12, 128);
             // the group's sum; infinite: the item's row is to be computed again
-            s_l[(ip * A::NGRP + r) * 128 + trow] = l_top > 1.2676506e30f /* 2^100 */ ? INFINITY : l_run;
+            s_l[(ip * A::NGRP + r) * 128 + trow] =
+                mode == RD_FIRST && (l_top > 1.2676506e30f /* 2^100 */ || m_run == -INFINITY) ? INFINITY : l_run;
             __syncwarp();
             if (lane == 0) mbar_arrive(l_full + 8 * ip);
             const int bl = n0 + w.nb - 1;                  // the item's last block
             n0 += w.nb, ++it;
             const int gl = (n03 + w.nb - 1) % A::NGRP;     // the group of that block
             n03 = gl + 1 == A::NGRP ? 0 : gl + 1;
-            const int cur = item;
             AttnItem wn;
-            item = wn.find(item + gridDim.x, n_items, sp, D, pl);
+            item = wn.find(item + gridDim.x, end, sp, D, pl);
             // The group of the last block finishes the item while the others are on the next one; groups 0 and 1 share the
             // CTA's last item.
-            const bool fin = item >= n_items;
+            const bool fin = item >= end;
             if (fin ? g < 2 : g == gl) {
                 ok = ok && mbar_wait(l_full + 8 * ip, iph, status);
                 const float *sl = s_l + ip * A::NGRP * 128 + trow;
-                const float m = s_m[ip * 128 + trow], l = (sl[0] + sl[128]) + sl[256];
+                const float l = (sl[0] + sl[128]) + sl[256];
+                float m = s_m[ip * 128 + trow];
+                // the maxima of the rows; a row without any counts from 0 (and its sum is 0)
+                if (mode == RD_MAX && g == 0) {
+                    const float mx = fmaxf(fmaxf(sl[0], sl[128]), sl[256]) * c;
+                    sh.mx[trow] = mx == -INFINITY ? 0.f : mx;
+                }
                 __syncwarp();
                 if (!fin && lane == 0) mbar_arrive(ml_empty + 8 * ip);
                 ok = ok && mbar_wait(v_empty + 8 * (bl % A::NS), (bl / A::NS) & 1, status);
                 __syncwarp();
                 tc_fence_after();
-                attn_finish<KB>(w, cur, fin ? g : 0, fin ? 1 : 2, tO, fin ? 0u : o_free, trow, m, l, c, sp, D, pl, layer, gq, gk, gv,
-                                out, part_o, counters);
+                if (mode != RD_MAX) {
+                    int mask = 3;
+                    if (mode == RD_AGAIN) {
+                        const uint32_t marks = sh.redo[2 + (num >> 2)] >> (8 * (num & 3) + quad);
+                        mask = (marks & 1) | ((marks >> 3) & 2);
+                        if (l == 0.f) m = -INFINITY;
+                    }
+                    attn_finish(w, fin ? g : 0, fin ? 1 : 2, mask, tO, fin ? 0u : o_free, trow, m, l, D, pl, out,
+                                part_o, counters, mode == RD_FIRST ? sh.redo : nullptr, it - 1);
+                }
             }
             w = wn;
         }
+        if (!ok && lane == 0) atomicOr(sh.redo, ATTN_EXPIRED);
     }
+}
+
+// The items with marked rows once more, each twice.  Not inlined: the first walk's code is as if this were not there.
+template <int KB>
+static __device__ __noinline__ void attn_again(const AttnShared<KB> sh, const CUtensorMap &tmQ, const CUtensorMap &tmK,
+                                               const CUtensorMap &tmV, const StepParams *sp, const Dims &D, int layer,
+                                               const AttnPlan &pl, int n_items, bf16 *out, float *part_o, unsigned int *counters,
+                                               int *status) {
+    AttnItem w;
+    int num = 0;                                           // items with blocks so far
+    for (int item = blockIdx.x; (item = w.find(item, n_items, sp, D, pl)) < n_items; item += gridDim.x, ++num) {
+        if (!((sh.redo[2 + (num >> 2)] >> (8 * (num & 3))) & 255)) continue;
+#pragma unroll 1
+        for (int mode = RD_MAX; mode <= RD_AGAIN; ++mode) {
+            // (every completion of the last walk has been waited for)
+            if (threadIdx.x == 0) sh.inval_bars(), sh.init_bars();
+            __syncthreads();
+            tc_fence_after();
+            attn_items<KB>(sh, tmQ, tmK, tmV, sp, D, layer, pl, w, item, item + 1, mode, num, out, part_o, counters, status);
+            tc_fence_before();
+            __syncthreads();
+            if (sh.redo[0] & ATTN_EXPIRED) return;
+        }
+    }
+}
+
+template <int KB>
+__global__ void __launch_bounds__(AttnCfg<KB>::THREADS, 1)
+k_attn_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
+          const __grid_constant__ CUtensorMap tmV, const StepParams *sp, const __grid_constant__ Dims D, int layer,
+          const __grid_constant__ AttnPlan pl, int n_items, bf16 *out, float *part_o, unsigned int *counters, int *status) {
+    using A = AttnCfg<KB>;
+    extern __shared__ uint8_t smem_raw[];
+    NFD_TRACE_T0();
+    AttnShared<KB> sh(smem_raw);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // The first item's descriptor: its loads are in flight during the set-up.  (The pass descriptor was written by the
+    // first kernel of the pass, which completed before this kernel's predecessor began.)
+    AttnItem w0;
+    w0.set(blockIdx.x, sp, D, pl);
+
+    if (warp == 0 && lane == 0) {
+        tma_prefetch_desc(&tmQ);
+        tma_prefetch_desc(&tmK);
+        tma_prefetch_desc(&tmV);
+        sh.init_bars();
+    }
+    for (int i = threadIdx.x; i < 2 + ATTN_CTA_ITEMS / 4; i += A::THREADS) sh.redo[i] = 0;
+    if (warp == 1) {
+        tmem_alloc(smem_u32(sh.tmem_slot()), A::TMEM_COLS);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    sh.tmem = *sh.tmem_slot();
+
+    attn_items<KB>(sh, tmQ, tmK, tmV, sp, D, layer, pl, w0, blockIdx.x, n_items, RD_FIRST, 0, out, part_o, counters, status);
     NFD_TRACE_MARK_T(TRK_OTHER + 16, 128);
     tc_fence_before();
     __syncthreads();
-    if (warp == 1) tmem_dealloc(tmem, A::TMEM_COLS);
+    if (sh.redo[0] == ATTN_MARKED)
+        attn_again<KB>(sh, tmQ, tmK, tmV, sp, D, layer, pl, n_items, out, part_o, counters, status);
+    if (warp == 1) tmem_dealloc(sh.tmem, A::TMEM_COLS);
     NFD_TRACE_END(TRK_ATTN);
 }

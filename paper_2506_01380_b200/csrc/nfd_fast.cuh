@@ -39,12 +39,13 @@ static void attn_blocks(AttnPlan &pl, int T) {
     }
     pl.QT = (T + 127) / 128;
 }
-// The plan's divisors; false where a dividend is too large for them (n * d has to stay below 2^32).
-static bool attn_divisors(AttnPlan &pl, int H, long long n_items, int W) {
+// The plan's divisors; false where a dividend is too large for them (n * d has to stay below 2^32) or a CTA would get more
+// items than it keeps account of.
+static bool attn_divisors(AttnPlan &pl, int H, long long n_items, int W, int n_sm) {
     pl.split_div.set(pl.MAXSPLIT), pl.qt_div.set(pl.QT), pl.h_div.set(H), pl.ch_div.set(pl.CH), pl.bpf_div.set(pl.BPF);
     const long long nb = ((long long)W + 1) * pl.BPF + pl.CH, big = 0x100000000ll;
     const int d_item = pl.QT > H ? (pl.QT > pl.MAXSPLIT ? pl.QT : pl.MAXSPLIT) : (H > pl.MAXSPLIT ? H : pl.MAXSPLIT);
-    return n_items < 0x7fffffffll && n_items * d_item < big && nb < 0x7fffffffll && nb * (pl.CH > pl.BPF ? pl.CH : pl.BPF) < big;
+    return n_items <= (long long)ATTN_CTA_ITEMS * n_sm && n_items * d_item < big && nb < 0x7fffffffll && nb * (pl.CH > pl.BPF ? pl.CH : pl.BPF) < big;
 }
 static PFN_encodeTiled get_encode_fn() {
     void *fn = nullptr;
@@ -86,7 +87,7 @@ static int fast_create(FastState &fs, const Dims &D, bool bf16_mode, cudaStream_
         const int target = fs.n_sm / items_per_pass > 1 ? fs.n_sm / items_per_pass : 1;
         pl.CH = ((D.W + 1) * pl.BPF + target - 1) / target;
         pl.MAXSPLIT = ((D.W + 1) * pl.BPF + pl.CH - 1) / pl.CH;
-        if (attn_divisors(pl, D.H, (long long)NFD_MAX_PASS_FRAMES * D.H * pl.QT * pl.MAXSPLIT, D.W)) {
+        if (attn_divisors(pl, D.H, (long long)NFD_MAX_PASS_FRAMES * D.H * pl.QT * pl.MAXSPLIT, D.W, fs.n_sm)) {
             if (pl.MAXSPLIT > 1) {
                 // (the largest pass of this context: per stream a speculation and the deferred frames of the last one)
                 const int nf_max = D.n_streams * (D.R - D.W);
@@ -395,7 +396,7 @@ static int launch_attn_tc(PFN_encodeTiled encode, int n_sm, cudaStream_t st, con
     const int n_items = pl.MAXSPLIT * pl.QT * D.H * nf;
     dim3 grid(n_items < n_sm ? n_items : n_sm);
     cudaError_t e = launch_pdl(kern, grid, dim3(A::THREADS), (size_t)A::SMEM, st, 1, mq, mk, mv, sp, D, layer, pl, n_items,
-                               q, kc, vc, out, part_o, counters, status);
+                               out, part_o, counters, status);
     if (e != cudaSuccess) {
         fprintf(stderr, "libnfd: tensor-core attention launch failed: %s\n", cudaGetErrorString(e));
         cudaGetLastError();

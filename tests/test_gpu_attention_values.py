@@ -1,5 +1,6 @@
 """Attention on values that a fast softmax can get wrong: NaN in a key, at every place that a key can have among the
-columns that one thread takes together; and how exact its probabilities are, for flat and for peaked rows."""
+columns that one thread takes together; how exact its probabilities are, for flat and for peaked rows; scores that rise
+beyond what the first ones are a reference for, and scores of -inf."""
 import pytest
 
 from paper_2506_01380_b200 import inputs as I
@@ -71,3 +72,83 @@ def test_bf16_result_is_as_exact_as_its_own_rounding(heads, dh, T, n_kv, n_q, wi
         rows = lambda x: x.permute(1, 0, 2, 3).reshape(heads, n_kv * T, dh).contiguous()
         assert _rel(g.attention(q, rows(k), rows(v), n_q, n_kv, window), ref) <= limit
         assert g.status() == 0
+
+
+def _rising(heads, dh, T, n_kv, n_q, seed, nats, v_scale=1.0):
+    """Scores that rise by `nats` from the first page to the last, evenly: q has 8 in one column, and k there what it takes.
+    The first rows of q take no part in it."""
+    import torch
+    q, k, v, out = _pages(heads, dh, T, n_kv, n_q, seed)
+    q[:, :, 3] = 8
+    q[:, :5, 3] = 0
+    k[..., 3] = (torch.arange(n_kv, device="cuda") * (nats * dh ** 0.5 / 8 / max(n_kv - 1, 1))).view(n_kv, 1, 1).to(k.dtype)
+    return q, k, v * v_scale, out
+
+
+# Every item is walked again (the rise passes 2^100 over the item's first scores); a bf16 result within its own rounding.
+@pytest.mark.parametrize("heads,T,streams,n_kv,n_q,window", [
+    (16, 336, 8, 33, 8, 32),         # unsplit long windows, several items per CTA
+    (16, 336, 1, 17, 1, 16),         # split windows
+    (16, 220, 1, 17, 4, 16),         # pages that no block divides, several items per CTA
+    (2, 64, 1, 40, 2, 39),           # one block per page
+])
+def test_scores_that_rise_beyond_the_reference(heads, T, streams, n_kv, n_q, window):
+    import torch
+    from paper_2506_01380_b200 import nfd as N
+    q, k, v, out = _rising(heads, 64, T, n_kv, n_q, seed=T, nats=40 * n_kv)
+    ref = _exact(q, k, v, n_q, window)
+    limit = 1.02 * _rel(ref.to(torch.bfloat16), ref)
+    cfg = I.make_cfg("nfd310m", n_layers=1, d_model=heads * 64, n_heads=heads, d_mlp=256, latent_h=T // 2, latent_w=8,
+                     ctx_frames=window, max_spec=8, n_streams=streams)
+    g = N.NFD(cfg, I.make_weights(cfg, 0))
+    rows = lambda x: x.permute(1, 0, 2, 3).reshape(heads, n_kv * T, 64).contiguous()
+    one = g.attention(q, rows(k), rows(v), n_q, n_kv, window)
+    assert _rel(one, ref) <= limit
+    assert torch.equal(one, g.attention(q, None, None, n_q, n_kv, window))
+    # a frame alone and with others
+    last = g.attention(q[:, -T:].contiguous(), None, None, 1, n_kv, window)
+    assert torch.equal(last, one[-T:])
+    assert g.status() == 0
+    assert _rel(N.attention_noalloc(q, k, v, n_q, window, out), ref) <= limit
+
+
+def test_rising_scores_over_a_long_window():
+    """The same with 1200 frames in the window of the allocation-free call, one CTA to a query tile."""
+    import torch
+    from paper_2506_01380_b200 import nfd as N
+    heads, T, n_kv = 2, 336, 1201
+    q, k, v, out = _rising(heads, 64, T, n_kv, 1, seed=1, nats=400)
+    got = N.attention_noalloc(q, k, v, 1, n_kv, out)
+    ref = torch.cat([_exact(q[h:h + 1], k[:, h:h + 1], v[:, h:h + 1], 1, n_kv) for h in range(heads)], dim=1)
+    assert _rel(got, ref) <= 1.02 * _rel(ref.to(torch.bfloat16), ref)
+
+
+def test_sums_that_leave_fp32_before_the_guard_of_the_scores():
+    """Scores rise by 60 nats only, but with values of 2^80 the unnormalised sums pass 2^127."""
+    import torch
+    from paper_2506_01380_b200 import nfd as N
+    q, k, v, out = _rising(4, 64, 220, 12, 2, seed=2, nats=60, v_scale=2.0 ** 80)
+    got = N.attention_noalloc(q, k, v, 2, 11, out)
+    ref = _exact(q, k, v, 2, 11)
+    assert _rel(got, ref) <= 1.02 * _rel(ref.to(torch.bfloat16), ref)
+
+
+@pytest.mark.parametrize("pages", [0, 3])
+def test_scores_of_minus_infinity_count_for_nothing(pages):
+    """The first 16 keys, or all keys of the first pages (more than a split takes), at -inf."""
+    import torch
+    from paper_2506_01380_b200 import nfd as N
+    heads, T, n_kv, window = 16, 336, 17, 16
+    q, k, v, out = _pages(heads, 64, T, n_kv, 1, seed=9)
+    q[:, :, 0] = 1
+    if pages:
+        k[:pages, :, :, 0] = float("-inf")
+    else:
+        k[0, :, :16, 0] = float("-inf")
+    ref = _exact(q, k, v, 1, window)
+    limit = 1.02 * _rel(ref.to(torch.bfloat16), ref)
+    cfg = I.make_cfg("nfd310m", n_layers=1, ctx_frames=window)
+    g = N.NFD(cfg, I.make_weights(cfg, 0))
+    rows = lambda x: x.permute(1, 0, 2, 3).reshape(heads, n_kv * T, 64).contiguous()
+    assert _rel(g.attention(q, rows(k), rows(v), 1, n_kv, window), ref) <= limit
+    assert _rel(N.attention_noalloc(q, k, v, 1, window, out), ref) <= limit
