@@ -409,13 +409,18 @@ k_gemm_p(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
                             else tma_store_3d(which == 1 ? &tm1 : &tm2, smem_u32(box), e, mw - (f0 + fa) * T, pg + head);
                             bulk_commit();
                         }
-                    } else if (valid) {
+                    } else {
                         // the warp's rows belong to two frames, hence two pages
-                        const int pg = fo == 0 ? page[0] : (fo == 1 ? page[1] : page[2]);
-                        uint4 *dst = reinterpret_cast<uint4 *>((which == 1 ? epi.kc : epi.vc) +
-                                                               ((size_t)(pg + head) * T + (m - (f0 + fo) * T)) * epi.D.dh + e);
+                        if (valid) {
+                            const int pg = fo == 0 ? page[0] : (fo == 1 ? page[1] : page[2]);
+                            uint4 *dst = reinterpret_cast<uint4 *>((which == 1 ? epi.kc : epi.vc) +
+                                                                   ((size_t)(pg + head) * T + (m - (f0 + fo) * T)) * epi.D.dh + e);
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) dst[c] = pack_bf16x8(a + 8 * c);
+                            for (int c = 0; c < 4; ++c) dst[c] = pack_bf16x8(a + 8 * c);
+                        }
+                        // No box was used and no store is under way from one: the next group takes this one, whose last
+                        // store has read it.  (The other one's may not have.)
+                        continue;
                     }
                 }
                 if constexpr (FORM == FORM_RES) {

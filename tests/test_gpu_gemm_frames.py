@@ -20,11 +20,23 @@ pytestmark = pytest.mark.gpu
     ((46, 30), 4, 2, 0, 3072, 24, 1),       # 345 tokens, head dimension 32
 ])
 def test_batched_pass_equals_single_frames(hw, streams, k, act, dm, heads, fuse_ln):
+    _batched_equals_single(768, hw, streams, k, act, dm, heads, fuse_ln)
+
+
+@pytest.mark.parametrize("streams,k", [(5, 1), (3, 2)])
+def test_tiles_of_three_groups_per_warp(streams, k):
+    """1680 and 2016 rows onto 3072 columns: tiles 192 wide, of which a warp has three groups of 32, several tiles per CTA;
+    warps whose rows belong to two frames store K and V themselves and Q through the two result boxes.  Repeated, for a
+    store from a box that is overwritten too early is a matter of time."""
+    _batched_equals_single(1024, (48, 28), streams, k, 0, 1024, 16, 1, passes=40)
+
+
+def _batched_equals_single(d, hw, streams, k, act, dm, heads, fuse_ln, passes=1):
     import torch
     from paper_2506_01380_b200.nfd import NFD
-    dh = 768 // heads
+    dh = d // heads
     rope = dict(rope_t=16, rope_h=24, rope_w=24) if dh == 64 else dict(rope_t=8, rope_h=12, rope_w=12)
-    cfg = I.make_cfg("nfd310m", n_layers=2, d_model=768, n_heads=heads, head_dim=dh, d_mlp=dm, act=act, latent_h=hw[0],
+    cfg = I.make_cfg("nfd310m", n_layers=2, d_model=d, n_heads=heads, head_dim=dh, d_mlp=dm, act=act, latent_h=hw[0],
                      latent_w=hw[1], ctx_frames=3, n_streams=streams, **rope)
     g = NFD(cfg, I.make_weights(cfg, 1, "stress"))
     g.set_option("fuse_ln", fuse_ln)
@@ -38,10 +50,11 @@ def test_batched_pass_equals_single_frames(hw, streams, k, act, dm, heads, fuse_
     one = torch.stack([torch.cat([g.denoise_step(x[s, j:j + 1].contiguous(), 0.6, acts[s], stream=s, offset=j) for j in range(k)])
                        for s in range(streams)])
     ref = [[g.kv_read(l, g.kv_state(s)[0] + j, stream=s) for l in (0, 1) for j in range(k)] for s in range(streams)]
-    both = g.denoise_step_batched(list(range(streams)), x, [0.6] * streams, acts)
-    assert torch.isfinite(both).all() and torch.equal(both, one)
-    for s in range(streams):
-        new = [g.kv_read(l, g.kv_state(s)[0] + j, stream=s) for l in (0, 1) for j in range(k)]
-        for a, b in zip(new, ref[s]):
-            assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1])
+    for _ in range(passes):
+        both = g.denoise_step_batched(list(range(streams)), x, [0.6] * streams, acts)
+        assert torch.isfinite(both).all() and torch.equal(both, one)
+        for s in range(streams):
+            new = [g.kv_read(l, g.kv_state(s)[0] + j, stream=s) for l in (0, 1) for j in range(k)]
+            for a, b in zip(new, ref[s]):
+                assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1])
     assert g.status() == 0
