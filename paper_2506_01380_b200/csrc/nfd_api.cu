@@ -304,11 +304,12 @@ static void launch_gemm(nfd_ctx *c, const TS *A, const TS *Wt, int M, int N, int
     PLAUNCH(c, (k_gemm_simple<TS, Epi>), grid, 256, 0, (const StepParams *)c->d_sp, c->D.T, A, Wt, N, K, epi);
 }
 
-template <typename TS> static void launch_attention(nfd_ctx *c, int nf, int layer) {
+// `early`: see launch_attn_plan; set inside a pass, where the QKV projection comes before.
+template <typename TS> static void launch_attention(nfd_ctx *c, int nf, int layer, bool early) {
     const Dims &D = c->D;
     c->cls = CLS_ATTN;
     prof_mark(c, false);
-    const int n_fast = fast_attention<TS>(c->fast && c->bf16_mode, c->fs, c->st, c->d_sp, D, nf, layer,
+    const int n_fast = fast_attention<TS>(c->fast && c->bf16_mode, early, c->fs, c->st, c->d_sp, D, nf, layer,
                                           (const TS *)c->qbuf, (const TS *)c->kc, (const TS *)c->vc, (TS *)c->abuf);
     if (n_fast > 0) {
         prof_mark(c, true);
@@ -394,7 +395,7 @@ template <typename TS> static void enqueue_body(nfd_ctx *c, int nf, int kind) {
         launch_gemm<TS>(c, (const TS *)c->hbuf, (const TS *)c->w_qkv[l], M, 3 * d, d, eq, c->w_o[l],
                         (size_t)d * d, fold);
         if (kind == 1 && l == L - 1) break;      // a commit only needs the K/V of every layer
-        launch_attention<TS>(c, nf, l);
+        launch_attention<TS>(c, nf, l, true);
         EpiGateRes<TS> eo{sp, (const TS *)c->b_o[l], c->z, modl + 2 * d, mod_row, D,
                           fold ? (TS *)c->hbuf : (TS *)nullptr, modl + 4 * d, fold ? c->ln_stats : (float2 *)nullptr};
         c->cls = CLS_GEMM_O;
@@ -1155,10 +1156,11 @@ int nfd_attention(nfd_ctx *c, const void *q, const void *k, const void *v, int n
     }
     c->cls = CLS_PARAMS;
     PLAUNCH(c, k_set_params, 1, 256, 0, p, c->d_sp, c->lim, c->d_status);
+    // (k_set_params is the predecessor here: attention starts when it has ended)
     if (c->bf16_mode)
-        launch_attention<bf16>(c, n_q, 0);
+        launch_attention<bf16>(c, n_q, 0, false);
     else
-        launch_attention<float>(c, n_q, 0);
+        launch_attention<float>(c, n_q, 0, false);
     CK(take_launch_err(c));
     CK(cudaMemcpyAsync(out, c->abuf, qbytes, cudaMemcpyDeviceToDevice, c->st));
     return NFD_OK;
@@ -1367,7 +1369,7 @@ static bool noalloc_launch_tc(int dev, cudaStream_t st, const StepParams *d_sp, 
     pl.CH = (D.W + 1) * pl.BPF, pl.MAXSPLIT = 1;
     const long long n_items = (long long)pl.QT * D.H * n_q;
     if (!attn_divisors(pl, D.H, n_items, D.W, n_sm[dev])) return false;
-    return launch_attn_plan(enc[dev], n_sm[dev], st, d_sp, D, n_q, 0, pl, (size_t)D.R * D.H, (const bf16 *)q,
+    return launch_attn_plan(false, enc[dev], n_sm[dev], st, d_sp, D, n_q, 0, pl, (size_t)D.R * D.H, (const bf16 *)q,
                             (const bf16 *)k_pages, (const bf16 *)v_pages, (bf16 *)out, nullptr, nullptr, d_stat) != 0;
 }
 

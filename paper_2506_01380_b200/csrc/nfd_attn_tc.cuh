@@ -664,8 +664,9 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
     NFD_TRACE_T0();
     AttnShared<KB> sh(smem_raw);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // The first item's descriptor: its loads are in flight during the set-up.  (The pass descriptor was written by the
-    // first kernel of the pass, which completed before this kernel's predecessor began.)
+    // The first item's descriptor: its loads are in flight during the set-up.  (In a pass the descriptor was written by the
+    // first kernel, for whose end the kernels between have waited; where its writer is this kernel's predecessor, the launch
+    // is in plain stream order.)
     AttnItem w0;
     w0.set(blockIdx.x, sp, D, pl);
 

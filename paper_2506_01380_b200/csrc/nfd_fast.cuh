@@ -152,20 +152,22 @@ static bool encode_map_3d(PFN_encodeTiled encode, CUtensorMap *m, const void *pt
 }
 
 // ---------------------------------------------------------------------------
-// Kernel launch with programmatic stream serialisation (and an optional cluster
-// along x).  Works the same under stream capture.
+// Kernel launch, with programmatic stream serialisation where `early` is set (the kernel may start while its
+// predecessor runs) and with an optional cluster along x.  Works the same under stream capture.
 // ---------------------------------------------------------------------------
 template <typename... KArgs, typename... Args>
-static cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                              int cluster_x, Args &&...args) {
+static cudaError_t launch_kernel(bool early, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                                 int cluster_x, Args &&...args) {
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = grid, cfg.blockDim = block, cfg.dynamicSmemBytes = smem, cfg.stream = st;
     cudaLaunchAttribute attr[2];
     int na = 0;
-    attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[na].val.programmaticStreamSerializationAllowed = 1;
-    ++na;
+    if (early) {
+        attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[na].val.programmaticStreamSerializationAllowed = 1;
+        ++na;
+    }
     if (cluster_x > 1) {
         attr[na].id = cudaLaunchAttributeClusterDimension;
         attr[na].val.clusterDim.x = (unsigned)cluster_x, attr[na].val.clusterDim.y = 1, attr[na].val.clusterDim.z = 1;
@@ -173,6 +175,11 @@ static cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
     }
     cfg.attrs = attr, cfg.numAttrs = (unsigned)na;
     return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
+}
+template <typename... KArgs, typename... Args>
+static cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                              int cluster_x, Args &&...args) {
+    return launch_kernel(true, kern, grid, block, smem, st, cluster_x, std::forward<Args>(args)...);
 }
 
 // ---------------------------------------------------------------------------
@@ -380,7 +387,7 @@ static bool fast_gemm(bool enabled, FastState &fs, cudaStream_t st, const TS *A,
 }
 
 template <int KB>
-static int launch_attn_tc(PFN_encodeTiled encode, int n_sm, cudaStream_t st, const StepParams *sp, const Dims &D, int nf,
+static int launch_attn_tc(bool early, PFN_encodeTiled encode, int n_sm, cudaStream_t st, const StepParams *sp, const Dims &D, int nf,
                           int layer, const AttnPlan &pl, size_t pages, const bf16 *q, const bf16 *kc, const bf16 *vc,
                           bf16 *out, float *part_o, unsigned int *counters, int *status) {
     using A = AttnCfg<KB>;
@@ -395,8 +402,8 @@ static int launch_attn_tc(PFN_encodeTiled encode, int n_sm, cudaStream_t st, con
         return 0;
     const int n_items = pl.MAXSPLIT * pl.QT * D.H * nf;
     dim3 grid(n_items < n_sm ? n_items : n_sm);
-    cudaError_t e = launch_pdl(kern, grid, dim3(A::THREADS), (size_t)A::SMEM, st, 1, mq, mk, mv, sp, D, layer, pl, n_items,
-                               out, part_o, counters, status);
+    cudaError_t e = launch_kernel(early, kern, grid, dim3(A::THREADS), (size_t)A::SMEM, st, 1, mq, mk, mv, sp, D, layer, pl, n_items,
+                                  out, part_o, counters, status);
     if (e != cudaSuccess) {
         fprintf(stderr, "libnfd: tensor-core attention launch failed: %s\n", cudaGetErrorString(e));
         cudaGetLastError();
@@ -405,27 +412,29 @@ static int launch_attn_tc(PFN_encodeTiled encode, int n_sm, cudaStream_t st, con
     return 1;
 }
 
-// Attention of a pass by plan `pl` over `pages` (stream, layer, ring slot, head) pages of K and V.
-static int launch_attn_plan(PFN_encodeTiled encode, int n_sm, cudaStream_t st, const StepParams *sp, const Dims &D, int nf,
+// Attention of a pass by plan `pl` over `pages` (stream, layer, ring slot, head) pages of K and V.  `early`: the kernel may
+// start before its predecessor ends.  It reads the pass descriptor, and pages that the pass does not write, without waiting
+// for the predecessor: that must not be the kernel that writes them.
+static int launch_attn_plan(bool early, PFN_encodeTiled encode, int n_sm, cudaStream_t st, const StepParams *sp, const Dims &D, int nf,
                             int layer, const AttnPlan &pl, size_t pages, const bf16 *q, const bf16 *kc, const bf16 *vc,
                             bf16 *out, float *part_o, unsigned int *counters, int *status) {
     switch (pl.KB) {
-        case 128: return launch_attn_tc<128>(encode, n_sm, st, sp, D, nf, layer, pl, pages, q, kc, vc, out, part_o, counters, status);
-        case 112: return launch_attn_tc<112>(encode, n_sm, st, sp, D, nf, layer, pl, pages, q, kc, vc, out, part_o, counters, status);
-        case 96: return launch_attn_tc<96>(encode, n_sm, st, sp, D, nf, layer, pl, pages, q, kc, vc, out, part_o, counters, status);
-        default: return launch_attn_tc<64>(encode, n_sm, st, sp, D, nf, layer, pl, pages, q, kc, vc, out, part_o, counters, status);
+        case 128: return launch_attn_tc<128>(early, encode, n_sm, st, sp, D, nf, layer, pl, pages, q, kc, vc, out, part_o, counters, status);
+        case 112: return launch_attn_tc<112>(early, encode, n_sm, st, sp, D, nf, layer, pl, pages, q, kc, vc, out, part_o, counters, status);
+        case 96: return launch_attn_tc<96>(early, encode, n_sm, st, sp, D, nf, layer, pl, pages, q, kc, vc, out, part_o, counters, status);
+        default: return launch_attn_tc<64>(early, encode, n_sm, st, sp, D, nf, layer, pl, pages, q, kc, vc, out, part_o, counters, status);
     }
 }
 
 // Returns the number of kernels launched (0: not handled, use the plain kernel).
 template <typename TS>
-static int fast_attention(bool enabled, FastState &fs, cudaStream_t st, const StepParams *sp, const Dims &D, int nf,
+static int fast_attention(bool enabled, bool early, FastState &fs, cudaStream_t st, const StepParams *sp, const Dims &D, int nf,
                           int layer, const TS *q, const TS *kc, const TS *vc, TS *out) {
     if constexpr (!std::is_same<TS, bf16>::value) {
         return 0;
     } else {
         if (!enabled || !fs.ready || fs.plan.KB == 0) return 0;
-        return launch_attn_plan(fs.encode, fs.n_sm, st, sp, D, nf, layer, fs.plan, fs.cache_pages, q, kc, vc, out, fs.part_o,
+        return launch_attn_plan(early, fs.encode, fs.n_sm, st, sp, D, nf, layer, fs.plan, fs.cache_pages, q, kc, vc, out, fs.part_o,
                                 fs.attn_counters, fs.d_status);
     }
 }
