@@ -224,6 +224,8 @@ static __device__ __forceinline__ void attn_finish(const AttnItem &w, int p0, in
         if (last) *cnt = 0;                                // ready for the next launch
     }
     last = __ballot_sync(0xffffffffu, last);
+    // the ballot orders control only: this hands what the counting lanes have acquired to the lanes that read the states
+    __syncwarp();
 #pragma unroll 1
     for (int p = p0; p < p0 + np; ++p) {
         if (!((last >> (p - p0)) & 1)) continue;
