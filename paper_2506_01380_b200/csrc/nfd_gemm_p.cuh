@@ -229,9 +229,9 @@ k_gemm_p(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
             const bool valid = m < M;
             const int fo = valid ? (m >= b1) + (m >= b2) : 0;  // frame of the row, relative to f0
             const float *tab = s_tab + (size_t)tb * (G::TAB_BYTES / 4) + fo * BN + part * G::HC;
-            // side operands of this tile
+            // side operands of this tile (no copy is begun after a wait has run out)
             if constexpr (FORM == FORM_RES) {
-                if (lane == 0) {
+                if (lane == 0 && ok) {
                     bulk_wait_read<0>();                       // the last tile's stores have read the buffers
                     mbar_expect_tx(sidebar, G::NG * 4096);
                     for (int g = 0; g < G::NG; ++g)
@@ -241,7 +241,7 @@ k_gemm_p(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
             if constexpr (FORM == FORM_QKV) {
                 // the rotary rows of a quadrant are shared by its warps: one loads them when all are done with the last
                 if (it > 0) asm volatile("bar.sync %0, %1;" ::"r"(1 + quad), "n"(32 * G::PARTS) : "memory");
-                if (part == 0 && lane == 0) {
+                if (part == 0 && lane == 0 && ok) {
                     const int nb = epi.D.dh > 32 ? 2 : 1;
                     mbar_expect_tx(sidebar, nb * 4096);
                     for (int h = 0; h < nb; ++h) tma_load_2d(smem_u32(s_side) + (quad * 2 + h) * 4096, &tm3, sidebar, 32 * h, mw);

@@ -85,3 +85,33 @@ def test_expired_wait_surfaces_as_timeout_and_context_survives(name):
     v1, v2 = a.denoise_step(x, 0.5, 1), b.denoise_step(x, 0.5, 1)
     assert torch.equal(v1, v2), "the context must compute as before once the switch is off"
     _same_generation(cfg, a, b, torch, 9)
+
+
+def _late(g):
+    g.set_option("test_wait_limit_us", 200)
+    g.set_option("test_skip_stage", 1)
+
+
+def _in_time(g):
+    g.set_option("test_skip_stage", 0)
+    g.set_option("test_wait_limit_us", 0)
+    g.set_option("clear_status", 1)
+
+
+def test_expired_wait_in_the_persistent_gemm():
+    """A batched pass of 2688 rows: every projection, residual ones too, runs in the persistent kernel."""
+    import torch
+    from paper_2506_01380_b200.nfd import NFD
+    cfg = I.make_cfg("nfd310m", n_layers=2, d_model=768, n_heads=12, d_mlp=3072, ctx_frames=2, n_streams=4)
+    g = NFD(cfg, I.make_weights(cfg, 1, "stress"))
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(1)
+    x = torch.randn(4, 2, *I.frame_shape(cfg), generator=gen, device="cuda")
+    one = lambda: g.denoise_step_batched([0, 1, 2, 3], x, [0.6] * 4, [1, 2, 3, 4])
+    ref = one()
+    _late(g)
+    one()
+    assert g.status() == E_TIMEOUT
+    _in_time(g)
+    assert g.status() == 0
+    assert torch.equal(one(), ref) and g.status() == 0
