@@ -179,7 +179,8 @@ int nfd_kv_read(nfd_ctx *ctx, int stream, int layer, int frame, float *k_out, fl
  * key sequence and sees key frames max(0, that - window) .. that.  out: dev,
  * storage type, [n_q_frames*T, n_heads*head_dim].  The data are first copied
  * into cache pages of batch slot 0 (which is reset), then the same attention
- * kernel the forward pass uses runs on them.
+ * kernel the forward pass uses runs on them.  (A wait that runs out in it leaves
+ * NaN in the rows concerned, and NFD_E_TIMEOUT in the status latch.)
  * n_kv_frames <= W + 2 k_max, n_q_frames <= k_max, window <= W. */
 int nfd_attention(nfd_ctx *ctx, const void *q, const void *k, const void *v, int n_q_frames, int n_kv_frames,
                   int window, void *out);
@@ -213,7 +214,9 @@ int nfd_attention(nfd_ctx *ctx, const void *q, const void *k, const void *v, int
  * GPU (different streams) race on it -- serialise them.
  * Runs on `cuda_stream` (a cudaStream_t): bf16 with head_dim 64 or 32 on the tensor-core kernel, everything else on
  * the fp32 pipes.  Scores and sums are fp32 in both; the tensor-core kernel multiplies V by probabilities that are
- * within 2^-17 of their fp32 value, so that a bf16 result has the error of its own rounding. */
+ * within 2^-17 of their fp32 value, so that a bf16 result has the error of its own rounding.
+ * Should a device-side wait of the tensor-core kernel run out (there is no context whose nfd_status would tell), the
+ * rows concerned are NaN. */
 int nfd_attention_noalloc(const void *q, const void *k_pages, const void *v_pages, int dtype, int n_heads,
                           int head_dim, int tokens_per_frame, int n_q_frames, int n_kv_frames, int window,
                           void *out, void *cuda_stream);
@@ -310,7 +313,8 @@ int nfd_warm_modulation(nfd_ctx *ctx);
  * size the runtime refuses, so the call returns NFD_E_CUDA; "test_corrupt_desc"
  * 1: the next pass descriptor names a batch slot that does not exist, which the
  * pass's first kernel must catch (NFD_E_DEVICE); "test_skip_stage" 1/0: the TMA
- * producer of every tensor-core GEMM leaves out its last pipeline stage, so that
+ * producer of every tensor-core GEMM leaves out its last pipeline stage (that of
+ * nfd_attention all of K), so that
  * the consumer's wait for it expires (NFD_E_TIMEOUT); "test_wait_limit_us" n:
  * bounded waits give up after n microseconds instead of 0.4 s (0 = default).
  * Returns NFD_E_RANGE for unknown names. */

@@ -305,11 +305,11 @@ static void launch_gemm(nfd_ctx *c, const TS *A, const TS *Wt, int M, int N, int
 }
 
 // `early`: see launch_attn_plan; set inside a pass, where the QKV projection comes before.
-template <typename TS> static void launch_attention(nfd_ctx *c, int nf, int layer, bool early) {
+template <typename TS> static void launch_attention(nfd_ctx *c, int nf, int layer, bool early, int test_skip = 0) {
     const Dims &D = c->D;
     c->cls = CLS_ATTN;
     prof_mark(c, false);
-    const int n_fast = fast_attention<TS>(c->fast && c->bf16_mode, early, c->fs, c->st, c->d_sp, D, nf, layer,
+    const int n_fast = fast_attention<TS>(c->fast && c->bf16_mode, early, test_skip, c->fs, c->st, c->d_sp, D, nf, layer,
                                           (const TS *)c->qbuf, (const TS *)c->kc, (const TS *)c->vc, (TS *)c->abuf);
     if (n_fast > 0) {
         prof_mark(c, true);
@@ -1158,7 +1158,7 @@ int nfd_attention(nfd_ctx *c, const void *q, const void *k, const void *v, int n
     PLAUNCH(c, k_set_params, 1, 256, 0, p, c->d_sp, c->lim, c->d_status);
     // (k_set_params is the predecessor here: attention starts when it has ended)
     if (c->bf16_mode)
-        launch_attention<bf16>(c, n_q, 0, false);
+        launch_attention<bf16>(c, n_q, 0, false, c->test_words[2]);
     else
         launch_attention<float>(c, n_q, 0, false);
     CK(take_launch_err(c));
@@ -1369,7 +1369,7 @@ static bool noalloc_launch_tc(int dev, cudaStream_t st, const StepParams *d_sp, 
     pl.CH = (D.W + 1) * pl.BPF, pl.MAXSPLIT = 1;
     const long long n_items = (long long)pl.QT * D.H * n_q;
     if (!attn_divisors(pl, D.H, n_items, D.W, n_sm[dev])) return false;
-    return launch_attn_plan(false, enc[dev], n_sm[dev], st, d_sp, D, n_q, 0, pl, (size_t)D.R * D.H, (const bf16 *)q,
+    return launch_attn_plan(false, 0, enc[dev], n_sm[dev], st, d_sp, D, n_q, 0, pl, (size_t)D.R * D.H, (const bf16 *)q,
                             (const bf16 *)k_pages, (const bf16 *)v_pages, (bf16 *)out, nullptr, nullptr, d_stat) != 0;
 }
 

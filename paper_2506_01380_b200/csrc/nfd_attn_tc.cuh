@@ -325,7 +325,7 @@ template <int KB>
 __device__ __forceinline__ void attn_items(const AttnShared<KB> &sh, const CUtensorMap &tmQ, const CUtensorMap &tmK,
                                            const CUtensorMap &tmV, const StepParams *sp, const Dims &D, int layer, const AttnPlan &pl,
                                            const AttnItem &w0, int first, int end, int mode, int num, bf16 *out, float *part_o,
-                                           unsigned int *counters, int *status) {
+                                           unsigned int *counters, int *status, int test_skip) {
     using A = AttnCfg<KB>;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t q_full = sh.q_full(), q_empty = sh.q_empty(), o_free = sh.o_free(), k_first = sh.k_first(), s_full = sh.s_full(),
@@ -345,6 +345,7 @@ __device__ __forceinline__ void attn_items(const AttnShared<KB> &sh, const CUten
             const CUtensorMap *tm = is_k ? &tmK : &tmV;
             const uint32_t empty = is_k ? s_full : v_empty;
             bool waited = false;
+            if (is_k && test_skip) ok = false;             // test switch: no K comes, and every wait behind it runs out
             int st = 0, lap = 0;                           // ring stage of the next block, how often the ring was filled
             AttnItem w = w0;
             for (int item = first; item < end && ok; item += gridDim.x) {
@@ -439,9 +440,9 @@ __device__ __forceinline__ void attn_items(const AttnShared<KB> &sh, const CUten
                     ++it_s, left_s = ws.nb;
                     ok = mbar_wait(q_full + 8 * (it_s & 1), (it_s >> 1) & 1, status);
                     item_s = ws.find(item_s + gridDim.x, end, sp, D, pl);
-                    if (item_s < end) {                    // Q of the item after it
+                    if (ok && item_s < end) {              // Q of the item after it
                         if (it_s >= 1) ok = ok && mbar_wait(q_empty + 8 * ((it_s + 1) & 1), ((it_s - 1) >> 1) & 1, status);
-                        load_q((it_s + 1) & 1);
+                        if (ok) load_q((it_s + 1) & 1);    // (no copy is begun after a wait has run out)
                     }
                 }
                 // (K of later blocks has arrived together with V of the block NS back)
@@ -603,7 +604,7 @@ __device__ __forceinline__ void attn_items(const AttnShared<KB> &sh, const CUten
             if (fin ? g < 2 : g == gl) {
                 ok = ok && mbar_wait(l_full + 8 * ip, iph, status);
                 const float *sl = s_l + ip * A::NGRP * 128 + trow;
-                const float l = (sl[0] + sl[128]) + sl[256];
+                float l = (sl[0] + sl[128]) + sl[256];
                 float m = s_m[ip * 128 + trow];
                 // the maxima of the rows; a row without any counts from 0 (and its sum is 0)
                 if (mode == RD_MAX && g == 0) {
@@ -615,15 +616,17 @@ __device__ __forceinline__ void attn_items(const AttnShared<KB> &sh, const CUten
                 ok = ok && mbar_wait(v_empty + 8 * (bl % A::NS), (bl / A::NS) & 1, status);
                 __syncwarp();
                 tc_fence_after();
+                ok = __all_sync(0xffffffffu, ok);
                 if (mode != RD_MAX) {
                     int mask = 3;
+                    if (!ok) l = NAN;                      // a wait has run out: the result says so
                     if (mode == RD_AGAIN) {
                         const uint32_t marks = sh.redo[2 + (num >> 2)] >> (8 * (num & 3) + quad);
                         mask = (marks & 1) | ((marks >> 3) & 2);
                         if (l == 0.f) m = -INFINITY;
                     }
                     attn_finish(w, fin ? g : 0, fin ? 1 : 2, mask, tO, fin ? 0u : o_free, trow, m, l, D, pl, out,
-                                part_o, counters, mode == RD_FIRST ? sh.redo : nullptr, it - 1);
+                                part_o, counters, mode == RD_FIRST && ok ? sh.redo : nullptr, it - 1);
                 }
             }
             w = wn;
@@ -633,26 +636,34 @@ __device__ __forceinline__ void attn_items(const AttnShared<KB> &sh, const CUten
 }
 
 // The items with marked rows once more, each twice.  Not inlined: the first walk's code is as if this were not there.
+// After a wait that has run out the marked rows are NaN (and counted: the tile's other splits may be waited for).
 template <int KB>
 static __device__ __noinline__ void attn_again(const AttnShared<KB> sh, const CUtensorMap &tmQ, const CUtensorMap &tmK,
                                                const CUtensorMap &tmV, const StepParams *sp, const Dims &D, int layer,
                                                const AttnPlan &pl, int n_items, bf16 *out, float *part_o, unsigned int *counters,
                                                int *status) {
+    using A = AttnCfg<KB>;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = (warp - A::SM_WARP0) >> 2, quad = warp & 3;
     AttnItem w;
     int num = 0;                                           // items with blocks so far
     for (int item = blockIdx.x; (item = w.find(item, n_items, sp, D, pl)) < n_items; item += gridDim.x, ++num) {
-        if (!((sh.redo[2 + (num >> 2)] >> (8 * (num & 3))) & 255)) continue;
+        const uint32_t marks = (sh.redo[2 + (num >> 2)] >> (8 * (num & 3))) & 255;
+        if (!marks) continue;
+        int mode = RD_MAX;
 #pragma unroll 1
-        for (int mode = RD_MAX; mode <= RD_AGAIN; ++mode) {
+        for (; mode <= RD_AGAIN && !(sh.redo[0] & ATTN_EXPIRED); ++mode) {
             // (every completion of the last walk has been waited for)
             if (threadIdx.x == 0) sh.inval_bars(), sh.init_bars();
             __syncthreads();
             tc_fence_after();
-            attn_items<KB>(sh, tmQ, tmK, tmV, sp, D, layer, pl, w, item, item + 1, mode, num, out, part_o, counters, status);
+            attn_items<KB>(sh, tmQ, tmK, tmV, sp, D, layer, pl, w, item, item + 1, mode, num, out, part_o, counters, status, 0);
             tc_fence_before();
             __syncthreads();
-            if (sh.redo[0] & ATTN_EXPIRED) return;
         }
+        // (the second walk writes its rows in any case)
+        if (mode <= RD_AGAIN && warp >= A::SM_WARP0 && g < 2)
+            attn_finish(w, g, 1, (marks >> quad & 1) | (marks >> quad >> 3 & 2), sh.tmem + A::TM_O + ((uint32_t)(quad * 32) << 16), 0u,
+                        quad * 32 + lane, 0.f, NAN, D, pl, out, part_o, counters, nullptr, 0);
     }
 }
 
@@ -660,7 +671,8 @@ template <int KB>
 __global__ void __launch_bounds__(AttnCfg<KB>::THREADS, 1)
 k_attn_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
           const __grid_constant__ CUtensorMap tmV, const StepParams *sp, const __grid_constant__ Dims D, int layer,
-          const __grid_constant__ AttnPlan pl, int n_items, bf16 *out, float *part_o, unsigned int *counters, int *status) {
+          const __grid_constant__ AttnPlan pl, int n_items, bf16 *out, float *part_o, unsigned int *counters, int *status,
+          int test_skip) {
     using A = AttnCfg<KB>;
     extern __shared__ uint8_t smem_raw[];
     NFD_TRACE_T0();
@@ -688,11 +700,12 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
     tc_fence_after();
     sh.tmem = *sh.tmem_slot();
 
-    attn_items<KB>(sh, tmQ, tmK, tmV, sp, D, layer, pl, w0, blockIdx.x, n_items, RD_FIRST, 0, out, part_o, counters, status);
+    attn_items<KB>(sh, tmQ, tmK, tmV, sp, D, layer, pl, w0, blockIdx.x, n_items, RD_FIRST, 0, out, part_o, counters, status,
+                   test_skip);
     NFD_TRACE_MARK_T(TRK_OTHER + 16, 128);
     tc_fence_before();
     __syncthreads();
-    if (sh.redo[0] == ATTN_MARKED)
+    if (sh.redo[0] & ATTN_MARKED)
         attn_again<KB>(sh, tmQ, tmK, tmV, sp, D, layer, pl, n_items, out, part_o, counters, status);
     if (warp == 1) tmem_dealloc(sh.tmem, A::TMEM_COLS);
     NFD_TRACE_END(TRK_ATTN);

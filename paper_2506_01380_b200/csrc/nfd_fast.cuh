@@ -387,7 +387,7 @@ static bool fast_gemm(bool enabled, FastState &fs, cudaStream_t st, const TS *A,
 }
 
 template <int KB>
-static int launch_attn_tc(bool early, PFN_encodeTiled encode, int n_sm, cudaStream_t st, const StepParams *sp, const Dims &D, int nf,
+static int launch_attn_tc(bool early, int test_skip, PFN_encodeTiled encode, int n_sm, cudaStream_t st, const StepParams *sp, const Dims &D, int nf,
                           int layer, const AttnPlan &pl, size_t pages, const bf16 *q, const bf16 *kc, const bf16 *vc,
                           bf16 *out, float *part_o, unsigned int *counters, int *status) {
     using A = AttnCfg<KB>;
@@ -403,7 +403,7 @@ static int launch_attn_tc(bool early, PFN_encodeTiled encode, int n_sm, cudaStre
     const int n_items = pl.MAXSPLIT * pl.QT * D.H * nf;
     dim3 grid(n_items < n_sm ? n_items : n_sm);
     cudaError_t e = launch_kernel(early, kern, grid, dim3(A::THREADS), (size_t)A::SMEM, st, 1, mq, mk, mv, sp, D, layer, pl, n_items,
-                                  out, part_o, counters, status);
+                                  out, part_o, counters, status, test_skip);
     if (e != cudaSuccess) {
         fprintf(stderr, "libnfd: tensor-core attention launch failed: %s\n", cudaGetErrorString(e));
         cudaGetLastError();
@@ -414,27 +414,27 @@ static int launch_attn_tc(bool early, PFN_encodeTiled encode, int n_sm, cudaStre
 
 // Attention of a pass by plan `pl` over `pages` (stream, layer, ring slot, head) pages of K and V.  `early`: the kernel may
 // start before its predecessor ends.  It reads the pass descriptor, and pages that the pass does not write, without waiting
-// for the predecessor: that must not be the kernel that writes them.
-static int launch_attn_plan(bool early, PFN_encodeTiled encode, int n_sm, cudaStream_t st, const StepParams *sp, const Dims &D, int nf,
+// for the predecessor: that must not be the kernel that writes them.  `test_skip`: the test switch of nfd_sm100.cuh.
+static int launch_attn_plan(bool early, int test_skip, PFN_encodeTiled encode, int n_sm, cudaStream_t st, const StepParams *sp, const Dims &D, int nf,
                             int layer, const AttnPlan &pl, size_t pages, const bf16 *q, const bf16 *kc, const bf16 *vc,
                             bf16 *out, float *part_o, unsigned int *counters, int *status) {
     switch (pl.KB) {
-        case 128: return launch_attn_tc<128>(early, encode, n_sm, st, sp, D, nf, layer, pl, pages, q, kc, vc, out, part_o, counters, status);
-        case 112: return launch_attn_tc<112>(early, encode, n_sm, st, sp, D, nf, layer, pl, pages, q, kc, vc, out, part_o, counters, status);
-        case 96: return launch_attn_tc<96>(early, encode, n_sm, st, sp, D, nf, layer, pl, pages, q, kc, vc, out, part_o, counters, status);
-        default: return launch_attn_tc<64>(early, encode, n_sm, st, sp, D, nf, layer, pl, pages, q, kc, vc, out, part_o, counters, status);
+        case 128: return launch_attn_tc<128>(early, test_skip, encode, n_sm, st, sp, D, nf, layer, pl, pages, q, kc, vc, out, part_o, counters, status);
+        case 112: return launch_attn_tc<112>(early, test_skip, encode, n_sm, st, sp, D, nf, layer, pl, pages, q, kc, vc, out, part_o, counters, status);
+        case 96: return launch_attn_tc<96>(early, test_skip, encode, n_sm, st, sp, D, nf, layer, pl, pages, q, kc, vc, out, part_o, counters, status);
+        default: return launch_attn_tc<64>(early, test_skip, encode, n_sm, st, sp, D, nf, layer, pl, pages, q, kc, vc, out, part_o, counters, status);
     }
 }
 
 // Returns the number of kernels launched (0: not handled, use the plain kernel).
 template <typename TS>
-static int fast_attention(bool enabled, bool early, FastState &fs, cudaStream_t st, const StepParams *sp, const Dims &D, int nf,
+static int fast_attention(bool enabled, bool early, int test_skip, FastState &fs, cudaStream_t st, const StepParams *sp, const Dims &D, int nf,
                           int layer, const TS *q, const TS *kc, const TS *vc, TS *out) {
     if constexpr (!std::is_same<TS, bf16>::value) {
         return 0;
     } else {
         if (!enabled || !fs.ready || fs.plan.KB == 0) return 0;
-        return launch_attn_plan(early, fs.encode, fs.n_sm, st, sp, D, nf, layer, fs.plan, fs.cache_pages, q, kc, vc, out, fs.part_o,
+        return launch_attn_plan(early, test_skip, fs.encode, fs.n_sm, st, sp, D, nf, layer, fs.plan, fs.cache_pages, q, kc, vc, out, fs.part_o,
                                 fs.attn_counters, fs.d_status);
     }
 }

@@ -9,7 +9,8 @@
 // default when it is not 0, [2] a test switch: when it is not 0 the GEMM's TMA
 // producer leaves out its last ring stage, so that the consumer's wait for it
 // runs out (used to show that an expired wait surfaces through nfd_status and
-// leaves the context usable), [3] unused.
+// leaves the context usable; nfd_attention hands it to its kernel, whose K then
+// does not come), [3] unused.
 #pragma once
 #include <cuda.h>
 #include "nfd_common.cuh"

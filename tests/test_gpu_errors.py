@@ -115,3 +115,21 @@ def test_expired_wait_in_the_persistent_gemm():
     _in_time(g)
     assert g.status() == 0
     assert torch.equal(one(), ref) and g.status() == 0
+
+
+@pytest.mark.parametrize("streams,n_q", [(1, 1), (8, 4)])
+def test_expired_wait_in_attention_leaves_nan(streams, n_q):
+    """K does not come: the rows are NaN and not what the accumulators happened to hold, with split windows (whose counters
+    must be at rest afterwards) and unsplit ones, several items per CTA."""
+    import torch
+    from paper_2506_01380_b200.nfd import NFD
+    cfg = I.make_cfg("nfd310m", n_layers=1, ctx_frames=16, n_streams=streams)
+    g = NFD(cfg, I.make_weights(cfg, 0))
+    q, k, v = [torch.as_tensor(a).cuda().bfloat16() for a in I.make_qkv(16, 64, n_q * 336, 20 * 336, seed=5)]
+    ref = g.attention(q, k, v, n_q, 20, 16)
+    assert torch.isfinite(ref).all()
+    _late(g)
+    assert torch.isnan(g.attention(q, k, v, n_q, 20, 16)).all()
+    assert g.status() == E_TIMEOUT
+    _in_time(g)
+    assert torch.equal(g.attention(q, k, v, n_q, 20, 16), ref) and g.status() == 0
