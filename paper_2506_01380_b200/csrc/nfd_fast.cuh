@@ -182,6 +182,14 @@ static cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
     return launch_kernel(true, kern, grid, block, smem, st, cluster_x, std::forward<Args>(args)...);
 }
 
+// More than 48 KB of shared memory for a kernel, on the current device.  Asked for before every launch: the limit belongs to
+// a device, and a process may have contexts on several.
+template <typename... KArgs> static bool allow_smem(void (*kern)(KArgs...), int bytes) {
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess) return true;
+    cudaGetLastError();
+    return false;
+}
+
 // ---------------------------------------------------------------------------
 // Tile width BN and cluster split S of a GEMM [M x N x K].
 // ---------------------------------------------------------------------------
@@ -259,15 +267,8 @@ template <int BN, typename Epi, int SC>
 static bool launch_gemm_tc_sc(FastState &fs, cudaStream_t st, const bf16 *A, const bf16 *Wt, int M, int N, int K, int S,
                               Epi epi, L2Prefetch pf) {
     using G = GemmCfg<BN>;
-    static bool attr_set = false;
     auto kern = k_gemm_tc<BN, Epi, SC>;
-    if (!attr_set) {
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM) != cudaSuccess) {
-            cudaGetLastError();
-            return false;
-        }
-        attr_set = true;
-    }
+    if (!allow_smem(kern, G::SMEM)) return false;
     const CUtensorMap *ma = get_map_2d(fs, A, (int)fs.a_rows, K, 128);
     const CUtensorMap *mb = get_map_2d(fs, Wt, N, K, BN);
     if (!ma || !mb) return false;
@@ -324,15 +325,8 @@ template <int BN, typename Epi, bool SPLIT>
 static bool launch_gemm_p(FastState &fs, cudaStream_t st, const bf16 *A, const bf16 *Wt, int M, int N, int K, int S,
                           Epi epi, L2Prefetch pf) {
     using G = GemmPCfg<BN, Epi::kForm>;
-    static bool attr_set = false;
     auto kern = k_gemm_p<BN, Epi, SPLIT>;
-    if (!attr_set) {
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM) != cudaSuccess) {
-            cudaGetLastError();
-            return false;
-        }
-        attr_set = true;
-    }
+    if (!allow_smem(kern, G::SMEM)) return false;
     const CUtensorMap *ma = get_map_2d(fs, A, (int)fs.a_rows, K, 128);
     const CUtensorMap *mb = get_map_2d(fs, Wt, N, K, BN);
     CUtensorMap me[4];
@@ -392,10 +386,7 @@ static int launch_attn_tc(bool early, int test_skip, PFN_encodeTiled encode, int
                           bf16 *out, float *part_o, unsigned int *counters, int *status) {
     using A = AttnCfg<KB>;
     auto kern = k_attn_tc<KB>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, A::SMEM) != cudaSuccess) {
-        cudaGetLastError();
-        return 0;
-    }
+    if (!allow_smem(kern, A::SMEM)) return 0;
     CUtensorMap mq, mk, mv;
     if (!encode_map_3d(encode, &mq, q, D.H, nf * D.T, D.dh, 128) || !encode_map_3d(encode, &mk, kc, pages, D.T, D.dh, KB) ||
         !encode_map_3d(encode, &mv, vc, pages, D.T, D.dh, KB))
