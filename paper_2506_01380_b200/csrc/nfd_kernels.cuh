@@ -959,7 +959,8 @@ __global__ void __launch_bounds__(256) k_attn_rows(const StepParams *sp, Dims D,
 #pragma unroll
                 for (int r = 0; r < R; ++r) O[i][r] *= f;
             }
-            p[i] = exp2f(s[i] - m[i]);
+            // (a score of -inf counts for nothing, also while there is no other: -inf - -inf is NaN)
+            p[i] = s[i] == -INFINITY ? 0.f : exp2f(s[i] - m[i]);
             l[i] += p[i];
         }
         __syncwarp();                                            // the last tile's P has been read

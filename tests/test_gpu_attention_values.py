@@ -152,3 +152,17 @@ def test_scores_of_minus_infinity_count_for_nothing(pages):
     rows = lambda x: x.permute(1, 0, 2, 3).reshape(heads, n_kv * T, 64).contiguous()
     assert _rel(g.attention(q, rows(k), rows(v), 1, n_kv, window), ref) <= limit
     assert _rel(N.attention_noalloc(q, k, v, 1, window, out), ref) <= limit
+
+
+@pytest.mark.parametrize("dtype,dh,tol", [("fp32", 64, 1e-5), ("bf16", 128, 4e-3)])
+def test_tiles_of_minus_infinity_on_the_fp32_pipes(dtype, dh, tol):
+    """A warp's whole first tile of 32 keys at -inf, with finite ones after it.  fp32: sums of some hundred products of order
+    one; bf16: half a unit in the last place of the result."""
+    import torch
+    from paper_2506_01380_b200 import nfd as N
+    T, n_kv = 336, 3
+    q, k, v, out = _pages(4, dh, T, n_kv, 1, seed=4, dtype=dtype)
+    q[:, :, 0] = 1
+    k[0, :, 64:130, 0] = float("-inf")
+    k[0, :, 200:270, 0] = float("-inf")
+    assert _rel(N.attention_noalloc(q, k, v, 1, 2, out), _exact(q, k, v, 1, 2)) <= tol
