@@ -2,6 +2,7 @@
 #pragma once
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
+#include <float.h>
 #include <stdint.h>
 #include "nfd.h"
 

@@ -921,7 +921,8 @@ __global__ void __launch_bounds__(256) k_attn_rows(const StepParams *sp, Dims D,
     float O[NQ][R], m[NQ], l[NQ];                                // m the same in every lane, l a lane's own part
 #pragma unroll
     for (int i = 0; i < NQ; ++i) {
-        m[i] = -INFINITY, l[i] = 0.f;
+        // (the lowest number and not -inf: scores of -inf count for nothing while there is no other, -inf - -inf is NaN)
+        m[i] = -FLT_MAX, l[i] = 0.f;
 #pragma unroll
         for (int r = 0; r < R; ++r) O[i][r] = 0.f;
     }
@@ -959,8 +960,7 @@ __global__ void __launch_bounds__(256) k_attn_rows(const StepParams *sp, Dims D,
 #pragma unroll
                 for (int r = 0; r < R; ++r) O[i][r] *= f;
             }
-            // (a score of -inf counts for nothing, also while there is no other: -inf - -inf is NaN)
-            p[i] = s[i] == -INFINITY ? 0.f : exp2f(s[i] - m[i]);
+            p[i] = exp2f(s[i] - m[i]);
             l[i] += p[i];
         }
         __syncwarp();                                            // the last tile's P has been read
@@ -1004,8 +1004,7 @@ __global__ void __launch_bounds__(256) k_attn_rows(const StepParams *sp, Dims D,
             float num = 0.f, den = 0.f;
 #pragma unroll
             for (int w = 0; w < 8; ++w) {
-                // (a warp without a tile has m = -inf and counts for nothing)
-                const float wgt = s_m[w][i] == -INFINITY ? 0.f : exp2f(s_m[w][i] - mx);
+                const float wgt = exp2f(s_m[w][i] - mx);          // (nought for a warp without a tile)
                 den = fmaf(s_l[w][i], wgt, den);
                 num = fmaf(s_p[w][i * 32 + lane], wgt, num);
             }
