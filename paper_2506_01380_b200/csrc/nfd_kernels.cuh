@@ -926,12 +926,16 @@ __global__ void __launch_bounds__(256) k_attn_rows(const StepParams *sp, Dims D,
 #pragma unroll
         for (int r = 0; r < R; ++r) O[i][r] = 0.f;
     }
-    const int tpp = (D.T + 31) / 32, n_tiles = (fr.frame - fr.win_first + 1) * tpp;
+    // a tile: 32 keys of a page, or as many whole pages as have no more than 32
+    const int n_pages = fr.frame - fr.win_first + 1, tpp = (D.T + 31) / 32, ppt = D.T < 32 ? 32 / D.T : 1;
+    const int n_tiles = (n_pages + ppt - 1) / ppt * tpp;
     float *pw = s_p[warp];
     for (int t = warp; t < n_tiles; t += 8) {
-        const int pg = t / tpp, k0 = (t - pg * tpp) * 32, nk = min(32, D.T - k0);
-        const size_t off = kv_page_offset(D, fr.stream, layer, fr.win_first + pg) + ((size_t)h * D.T + k0) * DH;
-        const TS *krow = kc + off + (size_t)min(lane, nk - 1) * DH;
+        const int pg = t / tpp * ppt, k0 = t % tpp * 32;
+        const int np = min(ppt, n_pages - pg), per = min(32, D.T - k0), nk = np * per;      // pages, keys of each, keys
+        auto page_at = [&](int i) { return kv_page_offset(D, fr.stream, layer, fr.win_first + pg + i) + ((size_t)h * D.T + k0) * DH; };
+        const int key = min(lane, nk - 1), kp = key / per;
+        const TS *krow = kc + page_at(kp) + (size_t)(key - kp * per) * DH;
         float s[NQ];
 #pragma unroll
         for (int i = 0; i < NQ; ++i) s[i] = 0.f;
@@ -967,19 +971,22 @@ __global__ void __launch_bounds__(256) k_attn_rows(const StepParams *sp, Dims D,
 #pragma unroll
         for (int i = 0; i < NQ; i += 4) *reinterpret_cast<float4 *>(pw + lane * PS + i) = make_float4(p[i], p[i + 1], p[i + 2], p[i + 3]);
         __syncwarp();
-        const TS *vrow = vc + off + lane;
+        for (int x = 0; x < np; ++x) {
+            const TS *vrow = vc + page_at(x) + lane;
+            const float *px = pw + x * per * PS;
 #pragma unroll 4
-        for (int kk = 0; kk < nk; ++kk) {
-            float v[R];
+            for (int kk = 0; kk < per; ++kk) {
+                float v[R];
 #pragma unroll
-            for (int r = 0; r < R; ++r) v[r] = to_f(vrow[(size_t)kk * DH + 32 * r]);
+                for (int r = 0; r < R; ++r) v[r] = to_f(vrow[(size_t)kk * DH + 32 * r]);
 #pragma unroll
-            for (int i = 0; i < NQ; i += 4) {
-                const float4 pv = *reinterpret_cast<const float4 *>(pw + kk * PS + i);
+                for (int i = 0; i < NQ; i += 4) {
+                    const float4 pv = *reinterpret_cast<const float4 *>(px + kk * PS + i);
 #pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    O[i][r] = fmaf(pv.x, v[r], O[i][r]), O[i + 1][r] = fmaf(pv.y, v[r], O[i + 1][r]);
-                    O[i + 2][r] = fmaf(pv.z, v[r], O[i + 2][r]), O[i + 3][r] = fmaf(pv.w, v[r], O[i + 3][r]);
+                    for (int r = 0; r < R; ++r) {
+                        O[i][r] = fmaf(pv.x, v[r], O[i][r]), O[i + 1][r] = fmaf(pv.y, v[r], O[i + 1][r]);
+                        O[i + 2][r] = fmaf(pv.z, v[r], O[i + 2][r]), O[i + 3][r] = fmaf(pv.w, v[r], O[i + 3][r]);
+                    }
                 }
             }
         }

@@ -166,3 +166,13 @@ def test_tiles_of_minus_infinity_on_the_fp32_pipes(dtype, dh, tol):
     k[0, :, 64:130, 0] = float("-inf")
     k[0, :, 200:270, 0] = float("-inf")
     assert _rel(N.attention_noalloc(q, k, v, 1, 2, out), _exact(q, k, v, 1, 2)) <= tol
+
+
+@pytest.mark.parametrize("T", [1, 2, 3, 5, 15, 16, 17, 31, 32, 33])
+@pytest.mark.parametrize("dtype,dh,tol", [("fp32", 64, 1e-5), ("bf16", 128, 4e-3)])
+def test_small_pages_on_the_fp32_pipes(T, dtype, dh, tol):
+    """Several pages to a tile of 32 keys, the last tile with fewer; the tolerances of the case above."""
+    from paper_2506_01380_b200 import nfd as N
+    q, k, v, out = _pages(3, dh, T, 37, 2, seed=T, dtype=dtype)
+    for window in (36, 5, 0):
+        assert _rel(N.attention_noalloc(q, k, v, 2, window, out), _exact(q, k, v, 2, window)) <= tol
