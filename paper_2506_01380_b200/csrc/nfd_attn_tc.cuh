@@ -39,17 +39,18 @@
 // ring of NS stages (free again when S(n) is complete, which the barrier of accumulator n % NS tells), V blocks through
 // one of NS (free when P V is complete); V(n) and K(n + NS), which the issuer needs at the same time, arrive on one barrier.
 //
-// What bounds it: the softmax warps (exponentials: 896 clocks per 128 x 112 block on the special-function unit) and the
-// turn of an accumulator, S -> softmax -> P V; the products take 700; a block takes about 1300.  Registers and code size count: spilled
-// registers are cold local memory, about 1 us on the path of a short item, and a cold code path costs as much.
-// Measured, 16 heads x 64 on one B200 (events around a launch): one frame of 336 tokens behind 16: 28.4 us with one thread
-// for all loads, one for all products and a maximum pass over S; 25.0 with the threads split and no maximum pass; 23.0
-// with three groups; 22.5 with items that overlap and the issuer's loop in one copy.  Two frames 37.3 -> 35.2 by the
-// last step, four 88.8 -> 74 -> 66 -> 61, eight frames behind 32 232 -> 188 -> 178 -> 165 (738 TFLOP/s).  Pages of
-// 220 tokens ran on the plain kernel, 1342 us; now 18.
-// Every exponential is the special-function unit's.  (Two pairs of eight by a polynomial on the FMA pipe took 22.5, 35.3,
-// 61.9 and 165 us where this takes 23.0, 37.3, 64.2 and 181; its range reduction saturated, which turns the score NaN into
-// a probability of nought, and its exponentials were good to 1e-5.)
+// What bounds it: the turn of an accumulator, S -> softmax -> P V, and in it the softmax warps (exponentials: 896 clocks per
+// 128 x 112 block on the special-function unit) and the one issuer (18 products, 29 to 60 clocks each, and their barriers); a
+// block takes about 1300 clocks.  Registers and code size count: spilled registers are cold local memory, about 1 us on the
+// path of a short item, and a cold code path costs as much.
+// Measured, 16 heads x 64 on one B200 (events around a launch), one, two and four frames of 336 tokens behind 16 and eight
+// streams behind 32: 25.0, 40.8, 71.8, 210 us (580 TFLOP/s).  How it came there, with P rounded to bf16 and a quarter of the
+// exponentials by a polynomial on the FMA pipe: one frame 28.4 with one thread for all loads, one for all products and a
+// maximum pass over S; 25.0 with the threads split and no maximum pass; 23.0 with three groups; 22.5 with items that overlap
+// and the issuer's loop in one copy (then 35.2, 61 and 165 for the others).  The polynomial's range reduction saturated,
+// which gave the score NaN a probability of nought; with every exponential the special-function unit's 23.0, 37.3, 64.2, 181.
+// With P as two numbers the polynomial gains nothing (24.9, 39.4, 69.5, 210 with an eighth of the exponentials, 25.0, 39.9,
+// 70.2, 207 without).  Pages of 220 tokens behind nine frames: 17 us (plain kernel: 800).
 // Tried and worse: sixteen softmax warps with half a row each (178 -> 201: the fixed part of a block doubles); four epilogue
 // warps beside the groups (96 registers a thread: four frames 60, but 2 us more on every short launch).
 //
@@ -232,34 +233,26 @@ static __device__ __forceinline__ void attn_finish(const AttnItem &w, int p0, in
         float O[32], lt = 0.f, mx = -INFINITY;
 #pragma unroll
         for (int e = 0; e < 32; ++e) O[e] = 0.f;
-        // the loads of two states (its own is read back like the others) are in flight together
+        // (its own state is read back like the others)
 #pragma unroll 1
-        for (int s0 = 0; s0 < w.nsplit; s0 += 1) {
-            float2 ml[1];
-            float4 v[1][8];
+        for (int sp = 0; sp < w.nsplit; ++sp) {
+            const uint8_t *st = states + (size_t)sp * ATTN_STATE_BYTES;
+            const float2 ml = __ldcg(reinterpret_cast<const float2 *>(st + ml_at(p)));
+            float4 v[8];
 #pragma unroll
-            for (int u = 0; u < 1; ++u) {
-                const uint8_t *st = states + (size_t)min(s0 + u, w.nsplit - 1) * ATTN_STATE_BYTES;
-                ml[u] = __ldcg(reinterpret_cast<const float2 *>(st + ml_at(p)));
+            for (int e = 0; e < 8; ++e) v[e] = __ldcg(reinterpret_cast<const float4 *>(st + o_at(p) + e * 2048));
+            // every rounding is spelled out: the bits must not depend on which CTA merges
+            const float mb = fmaxf(mx, ml.x);
+            // (a state with nothing but scores of -inf has m = -inf and counts for nothing)
+            const float fo = mx == mb ? 1.0f : ex2_approx(mx - mb), wgt = ml.x == -INFINITY ? 0.f : ex2_approx(ml.x - mb);
+            mx = mb;
+            lt = fmaf(ml.y, wgt, __fmul_rn(lt, fo));
 #pragma unroll
-                for (int e = 0; e < 8; ++e) v[u][e] = __ldcg(reinterpret_cast<const float4 *>(st + o_at(p) + e * 2048));
-            }
-            // (every rounding is spelled out: the bits must not depend on which CTA merges)
-#pragma unroll
-            for (int u = 0; u < 1; ++u) {
-                if (s0 + u >= w.nsplit) break;
-                const float mb = fmaxf(mx, ml[u].x);
-                // (a state with nothing but scores of -inf has m = -inf and counts for nothing)
-                const float fo = mx == mb ? 1.0f : ex2_approx(mx - mb), wgt = ml[u].x == -INFINITY ? 0.f : ex2_approx(ml[u].x - mb);
-                mx = mb;
-                lt = fmaf(ml[u].y, wgt, __fmul_rn(lt, fo));
-#pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    O[4 * e] = fmaf(v[u][e].x, wgt, __fmul_rn(O[4 * e], fo));
-                    O[4 * e + 1] = fmaf(v[u][e].y, wgt, __fmul_rn(O[4 * e + 1], fo));
-                    O[4 * e + 2] = fmaf(v[u][e].z, wgt, __fmul_rn(O[4 * e + 2], fo));
-                    O[4 * e + 3] = fmaf(v[u][e].w, wgt, __fmul_rn(O[4 * e + 3], fo));
-                }
+            for (int e = 0; e < 8; ++e) {
+                O[4 * e] = fmaf(v[e].x, wgt, __fmul_rn(O[4 * e], fo));
+                O[4 * e + 1] = fmaf(v[e].y, wgt, __fmul_rn(O[4 * e + 1], fo));
+                O[4 * e + 2] = fmaf(v[e].z, wgt, __fmul_rn(O[4 * e + 2], fo));
+                O[4 * e + 3] = fmaf(v[e].w, wgt, __fmul_rn(O[4 * e + 3], fo));
             }
         }
         write_part(p, O, lt);

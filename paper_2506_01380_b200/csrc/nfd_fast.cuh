@@ -201,17 +201,22 @@ struct GemmPlan {
 // Tile width of k_gemm_p for a GEMM [M x N x K] with a K split of S, or 0 where k_gemm_tc is the better one.  The line
 // lies where the row blocks times 128-wide column tiles fill the machine; measured on a 148-SM B200, k_gemm_tc -> k_gemm_p
 // in us with launch, for the projections into QKV and the MLP (K 768 to 1536): 72 tiles 12.9 -> 14.4, 96 tiles 14.9 ->
-// 14.8, 108 tiles 14.7 -> 13.0, 129 tiles 16.5 -> 14.6, 192 tiles 20.6 -> 16.9, 264 tiles 24 -> 19, 672 tiles 52 -> 32;
-// for those onto the residual stream (K 768 to 4096): 64 tiles 19.0 -> 23.0, 72 tiles 21 -> 28, 88 tiles 24.9 -> 23.0,
-// 112 tiles 18.8 -> 15.3, 126 tiles 20.8 -> 14.9, 168 tiles 47 -> 40.
+// 14.8, 108 tiles 14.7 -> 13.0, 129 tiles 16.5 -> 14.6, 192 tiles 20.6 -> 16.9, 264 tiles 24 -> 19, 672 tiles 52 -> 32.
+// For those onto the residual stream, out of attention / out of the MLP, k_gemm_tc -> k_gemm_p 96 wide, 128 wide (the rule
+// below takes the former or the latter), frames of 336 rows: hidden 1024, MLP 4096: 48 tiles of 128 columns 13.6 / 18.8 ->
+// 14.7 / 23.1, 14.8 / 26.9; 64 tiles 14.5 / 20.8 -> 14.7 / 23.2, 15.1 / 27.0; 88 tiles 15.8 / 34.1 -> 14.7 / 23.6, 15.2 /
+// 27.5; 112 tiles 18.8 / 34.3 -> 17.1 / 33.9, 15.5 / 27.7; 168 tiles 29.5 / 48.4 -> 20.1 / 37.4, 20.9 / 40.0.  Hidden 1536,
+// MLP 4096: 72 tiles 17.0 / 21.6 -> 16.9 / 23.9, 18.8 / 28.0; 96 tiles 20.6 / 34.1 -> 18.7 / 24.3, 19.9 / 28.1.  Hidden 768,
+// MLP 2048: 66 tiles 13.2 / 15.9 -> 12.7 / 16.7, 14.4 / 18.0; 84 tiles 14.7 / 17.8 -> 13.3 / 16.7, 14.4 / 18.5; 114 tiles
+// 16.8 / 20.0 -> 15.5 / 22.5, 14.7 / 18.8.
 static int gemm_p_width(int n_sm, int form, int T, int dh, int M, int N, int K, int S) {
     // a 128-row tile must not span more frames than the kernel keeps tables for; rotary rows of 64 floats at most
     if (form == FORM_NONE || 127 / T + 2 > GemmPCfg<128, FORM_MLP>::MAX_FR || (form == FORM_QKV && dh > 64)) return 0;
     const int mt = (M + 127) / 128, t128 = mt * ((N + 127) / 128);
     if (form == FORM_RES) {
         if (t128 < (88 * n_sm) / 148) return 0;
-        // 96 columns unless they need a wave more.  128 -> 96 wide, us with launch, K = 4096: 88 -> 121 tiles 27.8 -> 23.4,
-        // 152 -> 209 38.5 -> 36.2, 168 -> 231 40.9 -> 36.3 (K = 1024: 23.0 -> 20.9); a wave more: 112 -> 154 27.9 -> 33.4,
+        // 96 columns unless they need a wave more.  128 -> 96 wide, us with launch, K = 4096: 88 -> 121 tiles 27.5 -> 23.6,
+        // 152 -> 209 38.5 -> 36.2, 168 -> 231 40.0 -> 37.4 (K = 1024: 20.9 -> 20.1); a wave more: 112 -> 154 27.7 -> 33.9,
         // 252 -> 336 48.6 -> 54.8
         const int t96 = mt * ((N + 95) / 96);
         return (t96 + n_sm - 1) / n_sm <= (t128 + n_sm - 1) / n_sm ? 96 : 128;
@@ -233,7 +238,8 @@ static int gemm_p_width(int n_sm, int form, int T, int dh, int M, int N, int K, 
     return best;
 }
 // CTAs of k_gemm_tc that can be resident at once: one per SM, less what clusters cannot use (a cluster lives inside one
-// GPC; on a 148-SM B200 cudaOccupancyMaxActiveClusters gives 148 CTAs for clusters of 1 and 2, 132 for clusters of 4).
+// GPC; on a 148-SM B200 cudaOccupancyMaxActiveClusters gives 148 CTAs for clusters of 1 and 2, 132 for clusters of 4; the
+// formula goes through this one measured point, so that plans, and with them the bits, follow from sizes alone).
 static int gemm_slots(int n_sm, int S) { return S >= 4 ? (n_sm / 4 - 4) * 4 : n_sm; }
 // The narrowest tile whose CTAs fit the machine at once, 0 if none does.
 static int gemm_tc_width(int n_sm, int M, int N, int S) {

@@ -1,6 +1,6 @@
 """The tensor-core attention kernel where its tiles and pages end: pages that its key block does not divide, pages
 shorter than one block, query tiles with one row, head dimension 32, windows of one block and of several splits, more
-items than CTAs, and scores that rise along the keys, so that a row's reference maximum has to be raised."""
+items than CTAs, and scores that rise along the keys, away from the first ones, which are a row's reference."""
 import numpy as np
 import pytest
 
