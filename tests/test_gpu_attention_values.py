@@ -1,6 +1,6 @@
 """Attention on values that a fast softmax can get wrong: NaN in a key, at every place that a key can have among the
 columns that one thread takes together; how exact its probabilities are, for flat and for peaked rows; scores that rise
-beyond what the first ones are a reference for, and scores of -inf."""
+beyond what the first ones are a reference for, scores of -inf, and pages smaller than a tile of keys."""
 import pytest
 
 from paper_2506_01380_b200 import inputs as I
