@@ -14,13 +14,18 @@
 //     cluster barrier CTA r reads rows [r*128/S, (r+1)*128/S) of all S partials
 //     through distributed shared memory, sums them in split order
 //     (deterministic) and runs the epilogue for those rows;
-//   - warp 0 = TMA producer, warp 1 = tensor-memory allocation + UMMA issue,
-//     warps 2-9 = accumulator read-out and epilogue (two warps per TMEM lane
-//     quadrant, each taking half of the columns);
+//   - warps 0 and 10 = TMA producers (activations, weights), warp 1 =
+//     tensor-memory allocation + UMMA issue, warps 2-9 = accumulator read-out and
+//     epilogue (two warps per TMEM lane quadrant, each taking half of the columns).
+//     With one thread for both operands, the weights of the ring's first fill went
+//     out ahead of the activations, 0.7 us on the path of a CTA that starts when its
+//     predecessor is through, and the byte counts were announced between the copies
+//     (one frame of the 310M class 5458 -> 5363 us, of a 64-token model 307 -> 290);
 //   - programmatic dependent launch: barrier set-up, tensor-memory allocation and
 //     the first weight tiles (which never depend on the previous kernel) are
-//     issued before the wait on the predecessor grid; the epilogue's side inputs
-//     (bias, gate, residual, rotary table) are fetched while the UMMAs run;
+//     issued before the wait on the predecessor grid, and what the epilogue needs of
+//     the modulation cache and the descriptor is fetched there too; its other side
+//     inputs (residual, rotary table, row sums) are fetched while the UMMAs run;
 //   - every CTA also pulls a slice of the NEXT GEMM's weights towards L2, so that
 //     the weight stream from HBM runs one kernel ahead of its use.
 // One CTA fills an SM (its operand ring is sized for that): with programmatic
@@ -31,13 +36,14 @@
 #include "nfd_sm100.cuh"
 
 template <int BN> struct GemmCfg {
-    // A ring stage holds KU k-blocks of 64 elements.  A stage costs the producer about 280 clocks of barrier
-    // operations and 40 per TMA instruction whatever its size, an SM takes in up to 120 bytes per clock: with
-    // one 64-element block per stage the producer's own instructions set the pace (128 + 64 rows: 380 clocks per
-    // block, 65 bytes per clock), with two the SM's intake does (220 clocks per block).
-    static constexpr int KU = 2;
+    // A ring stage holds KU k-blocks of 64 elements.  A producer takes about 280 clocks for a stage's barrier operations and
+    // 60 per copy whatever their size, the products of a block 160 to 256: the narrow tiles, whose rings are deep, take two
+    // blocks to a stage, the others one, which comes back sooner.  One frame of the 310M class (QKV 64, out of attention
+    // 32, into the MLP 96, out of it 64 wide), us: all two blocks 5396, all one 5378, one from 96 on 5363, from 64 on 5367;
+    // hidden 768 (32 and 96 wide): 2328, 2346, 2322, 2322.
+    static constexpr int KU = BN <= 64 ? 2 : 1;
     // ring deep enough that one CTA owns an SM
-    static constexpr int STAGES = BN <= 64 ? 4 : 3;
+    static constexpr int STAGES = BN <= 32 ? 5 : (BN <= 64 ? 4 : (BN <= 96 ? 7 : 6));
     static constexpr int A_BYTES = 128 * 128;                  // 128 rows x 64 bf16
     static constexpr int B_BYTES = BN * 128;
     static constexpr int KB_BYTES = A_BYTES + B_BYTES;
@@ -50,8 +56,9 @@ template <int BN> struct GemmCfg {
     static constexpr int TAB_BYTES = 128 * 16 + (BN / 8) * 32 + 128;   // epilogue row and column tables, row -> frame
     static constexpr int SMEM = RING_BYTES + 1024 /*align*/ + 256 /*barriers*/ + 1024 /*row statistics*/ + UV_BYTES +
                                 TAB_BYTES;
-    static constexpr int THREADS = 320;
+    static constexpr int THREADS = 352;
     static constexpr int EPI_THREADS = 256;
+    static constexpr int B_WARP = 10;                          // weight producer
     static constexpr int MAX_S = 4;                            // largest cluster split
     static constexpr int MIN_CTAS = 1;
     static_assert(SMEM <= 232448, "shared memory of a CTA");
@@ -102,7 +109,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
         tma_prefetch_desc(&tmA);
         tma_prefetch_desc(&tmB);
         for (int s = 0; s < G::STAGES; ++s) {
-            mbar_init(full0 + 8 * s, 1);
+            mbar_init(full0 + 8 * s, 2);                     // one arrival per operand
             mbar_init(empty0 + 8 * s, 1);
         }
         mbar_init(accf, 1);
@@ -127,44 +134,41 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
     if constexpr (Epi::kRowStats) uv_f0 = m0 / epi.ln.T;
 
     const int nst = (nkb + G::KU - 1) / G::KU;               // ring stages of this CTA's K range
-    if (warp == 0) {
+    if (warp == 0 || warp >= G::B_WARP) {
+        // ---------------- TMA producers: activations (warp 0), weights ----------------
         if (elect_one()) {
-            const uint32_t ring = smem_u32(smem);
-            // the k-blocks of stage st: KU, fewer in the last one
-            auto load_b = [&](int st, int s) {
-                const int n = nkb - st * G::KU < G::KU ? nkb - st * G::KU : G::KU;
-                mbar_expect_tx(full0 + 8 * s, (uint32_t)n * G::KB_BYTES);
+            const bool is_a = warp == 0;
+            const uint32_t ring = smem_u32(smem) + (is_a ? 0 : G::KU * G::A_BYTES);
+            const CUtensorMap *tm = is_a ? &tmA : &tmB;
+            const uint32_t bytes = is_a ? G::A_BYTES : G::B_BYTES;
+            const int y = is_a ? m0 : n0;
+            // test switch (see nfd_sm100.cuh): leave out the last stage of the activations, so that the wait for it runs out
+            const int skip_last = is_a ? *reinterpret_cast<volatile int *>(status + 2) : 0;
+            const int n_st = nst - (skip_last ? 1 : 0);
+            auto blocks = [&](int st) { return nkb - st * G::KU < G::KU ? nkb - st * G::KU : G::KU; };
+            auto load = [&](int st, int s) {
 #pragma unroll
                 for (int u = 0; u < G::KU; ++u)
-                    if (u < n)
-                        tma_load_2d(ring + s * G::ST_BYTES + G::KU * G::A_BYTES + u * G::B_BYTES, &tmB, full0 + 8 * s,
-                                    (kb0 + st * G::KU + u) * 64, n0);
+                    if (u < blocks(st))
+                        tma_load_2d(ring + s * G::ST_BYTES + u * bytes, tm, full0 + 8 * s, (kb0 + st * G::KU + u) * 64, y);
             };
-            auto load_a = [&](int st, int s) {
-                const int n = nkb - st * G::KU < G::KU ? nkb - st * G::KU : G::KU;
-#pragma unroll
-                for (int u = 0; u < G::KU; ++u)
-                    if (u < n)
-                        tma_load_2d(ring + s * G::ST_BYTES + u * G::A_BYTES, &tmA, full0 + 8 * s,
-                                    (kb0 + st * G::KU + u) * 64, m0);
-            };
-            // weights never depend on the previous kernel: fill the ring's weight halves first
-            const int pre = nst < G::STAGES ? nst : G::STAGES;
-            for (int st = 0; st < pre; ++st) load_b(st, st);
-            // test switch (see nfd_sm100.cuh): leave out the last stage, so that the wait for it runs out
-            const int skip_last = *reinterpret_cast<volatile int *>(status + 2);
-            pdl_wait();
-            NFD_TRACE_MARK(TRK_OTHER + 1);
-            for (int st = 0; st < pre; ++st) {
-                if (skip_last && st == nst - 1) continue;      // its weight half has landed; the stage stays incomplete
-                load_a(st, st);
+            // the ring's first fill: every byte count is announced before the wait, so that the copies follow one another
+            const int pre = n_st < G::STAGES ? n_st : G::STAGES;
+#pragma unroll 1
+            for (int st = 0; st < pre; ++st) mbar_expect_tx(full0 + 8 * st, (uint32_t)blocks(st) * bytes);
+            if (is_a) {
+                pdl_wait();                                    // weights never depend on the previous kernel
+                NFD_TRACE_MARK(TRK_OTHER + 1);
             }
-            for (int st = pre; st < nst; ++st) {
-                if (skip_last && st == nst - 1) break;
-                const int s = st % G::STAGES;
-                if (!mbar_wait(empty0 + 8 * s, ((st / G::STAGES) - 1) & 1, status)) break;
-                load_b(st, s);
-                load_a(st, s);
+#pragma unroll 1
+            for (int st = 0; st < pre; ++st) load(st, st);
+            int s = 0, lap = 0;
+#pragma unroll 1
+            for (int st = G::STAGES; st < n_st; ++st) {
+                if (!mbar_wait(empty0 + 8 * s, lap & 1, status)) break;
+                mbar_expect_tx(full0 + 8 * s, (uint32_t)blocks(st) * bytes);
+                load(st, s);
+                if (++s == G::STAGES) s = 0, ++lap;
             }
         }
     } else if (warp == 1) {
@@ -208,14 +212,14 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
             }
         }
         __syncwarp();
-        pdl_wait();
-        // side inputs of the first items (bias, gate, residual, rotary table), fetched while the UMMAs run
+        // What depends on the pass descriptor and the modulation cache only, both complete before the first GEMM of a pass can
+        // start: fetched before the wait.  (The row sums, the residual stream and the rotary table are the predecessors'.)
 #pragma unroll
         for (int i = 0; i < MAX_ITEMS; ++i) {
             const int it = et + i * G::EPI_THREADS;
             if (it < n_items) {
                 const int m = m0 + r_base + it / CPR, n = n0 + (it % CPR) * 8;
-                if (m < M && n < N) epi.load(m, n, side[i]);
+                if (m < M && n < N) epi.load_early(m, n, side[i]);
             }
         }
         if constexpr (Epi::kTables) {
@@ -228,8 +232,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
         }
         if constexpr (Epi::kRowStats) {
             if (epi.ln.on()) {
-                // folded LayerNorm: (u, v) of the tile's columns for every frame the tile's rows belong to, and
-                // (mean, rstd) of the rows this CTA finishes, from the producer's partial sums
+                // folded LayerNorm: (u, v) of the tile's columns for every frame the tile's rows belong to
                 const int m_last = (m0 + 127 < M ? m0 + 127 : M - 1);
                 const int n_fr = m_last / epi.ln.T - uv_f0 + 1;
                 // layout [frame][pair of columns within a chunk][chunk]: the lanes of a warp, which hold adjacent
@@ -243,6 +246,21 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
                     const int m = m0 + r_base + et;
                     rowfr[r_base + et] = (uint8_t)((m < M ? m : M - 1) / epi.ln.T - uv_f0);
                 }
+            }
+        }
+        pdl_wait();
+        // the other side inputs of the first items, fetched while the UMMAs run
+#pragma unroll
+        for (int i = 0; i < MAX_ITEMS; ++i) {
+            const int it = et + i * G::EPI_THREADS;
+            if (it < n_items) {
+                const int m = m0 + r_base + it / CPR, n = n0 + (it % CPR) * 8;
+                if (m < M && n < N) epi.load(m, n, side[i]);
+            }
+        }
+        if constexpr (Epi::kRowStats) {
+            if (epi.ln.on()) {
+                // (mean, rstd) of the rows this CTA finishes, from the producer's partial sums
                 // 8 lanes per row, 32 rows per sweep; every load is issued before the first sum
                 constexpr int SWEEPS = 128 / (G::EPI_THREADS / 8);
                 const int sub = et & 7;
@@ -303,7 +321,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
     else
         __syncthreads();
     NFD_TRACE_MARK_T(TRK_OTHER + 3, 64);
-    if (warp >= 2) {
+    if (warp >= 2 && warp < G::B_WARP) {
         // Items in batches of MAX_ITEMS: first every side input of the batch is requested, then the items are
         // finished two at a time: all loads of the S partials of the pair (remote ones come through distributed
         // shared memory and take long), the sum in split order, the fused epilogue (8 adjacent columns per item).
@@ -319,7 +337,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
                 if (it >= n_items || mm[i] >= M || nn[i] >= N)
                     mm[i] = -1;
                 else if (i0 > 0)
-                    epi.load(mm[i], nn[i], side[i]);
+                    epi.load_early(mm[i], nn[i], side[i]), epi.load(mm[i], nn[i], side[i]);
                 vmask[i] = __ballot_sync(0xffffffffu, mm[i] >= 0);
             }
 #pragma unroll

@@ -478,9 +478,10 @@ __device__ __forceinline__ uint4 pack_bf16x8(const float *f) {
 // GEMM epilogues.  operator() takes one output row m and two adjacent columns
 // (n, n+1), n even, holding the fp32 accumulators (plain GEMM).  The tensor-core
 // GEMM (bf16 storage only) works on eight adjacent columns n..n+7, n a multiple
-// of 8, 16 bytes at a time, in two steps: load() fetches everything the item
-// needs besides the accumulators (bias, gate, residual, rotary table) into a
-// Side record, so that the fetch can be issued while the UMMAs still run;
+// of 8, 16 bytes at a time, in steps: load_early() and load() fetch everything the
+// item needs besides the accumulators into a Side record, the former what is there
+// before the predecessor grid has ended (bias, gate, scale), the latter the rest
+// (residual, rotary table), so that the fetch can be issued while the UMMAs still run;
 // apply() combines it with the accumulators and stores.  apply() also gets the
 // (mean, rstd) of the item's row and the (u, v) pairs of its 8 columns (in shared
 // memory) when the functor asks for row statistics (kRowStats) and the
@@ -600,8 +601,10 @@ template <typename TS> struct EpiQKV {
         uint4 bias;             // unused with the folded LayerNorm (v carries the bias)
         float4 c01, c23;        // (cos, sin) of four adjacent pairs
     };
-    __device__ __forceinline__ void load(int m, int n, Side &s) const {
+    __device__ __forceinline__ void load_early(int, int n, Side &s) const {
         if (!ln.on()) s.bias = *reinterpret_cast<const uint4 *>(bias + n);
+    }
+    __device__ __forceinline__ void load(int m, int n, Side &s) const {
         const int which = n / D.d, col = n - which * D.d;
         const int e = col % D.dh;
         if (which < 2) {
@@ -684,17 +687,19 @@ template <typename TS> struct EpiGateRes {
         uint4 bias;
         float4 g0, g1, z0, z1, s0, s1;
     };
-    __device__ __forceinline__ void load(int m, int n, Side &s) const {
+    __device__ __forceinline__ void load_early(int m, int n, Side &s) const {
         s.bias = *reinterpret_cast<const uint4 *>(bias + n);
         const int row = sp->fr[m / D.T].cond_row;
         const float4 *g = reinterpret_cast<const float4 *>(gate + (size_t)row * row_stride + n);
-        const float4 *zp = reinterpret_cast<const float4 *>(z + (size_t)m * D.d + n);
         s.g0 = g[0], s.g1 = g[1];
-        s.z0 = zp[0], s.z1 = zp[1];
         if (a_out) {
             const float4 *sc = reinterpret_cast<const float4 *>(scale_next + (size_t)row * row_stride + n);
             s.s0 = sc[0], s.s1 = sc[1];
         }
+    }
+    __device__ __forceinline__ void load(int m, int n, Side &s) const {
+        const float4 *zp = reinterpret_cast<const float4 *>(z + (size_t)m * D.d + n);
+        s.z0 = zp[0], s.z1 = zp[1];
     }
     __device__ __forceinline__ void apply(int m, int n, float *a, const Side &s, float2, const float4 *, int,
                                           unsigned mask, const Row &, const Col &) const {
@@ -754,10 +759,10 @@ template <typename TS> struct EpiGelu {
     struct Side {
         uint4 bias;         // unused with the folded LayerNorm (v carries the bias)
     };
-    __device__ __forceinline__ void load(int m, int n, Side &s) const {
-        (void)m;
+    __device__ __forceinline__ void load_early(int, int n, Side &s) const {
         if (!ln.on()) s.bias = *reinterpret_cast<const uint4 *>(bias + n);
     }
+    __device__ __forceinline__ void load(int, int, Side &) const {}
     __device__ __forceinline__ void apply(int m, int n, float *a, const Side &s, float2 ms, const float4 *uv,
                                           int uv_stride, unsigned, const Row &, const Col &) const {
         if (ln.on())
@@ -803,6 +808,7 @@ template <typename TS> struct EpiFinal {
     struct Side {
         int unused;
     };
+    __device__ __forceinline__ void load_early(int, int, Side &) const {}
     __device__ __forceinline__ void load(int, int, Side &) const {}
     __device__ __forceinline__ void apply(int m, int n, float *a, const Side &, float2, const float4 *, int,
                                           unsigned, const Row &, const Col &) const {
