@@ -1366,9 +1366,8 @@ static bool noalloc_launch_tc(int dev, cudaStream_t st, const StepParams *d_sp, 
     }
     AttnPlan pl;
     attn_blocks(pl, D.T);
-    pl.CH = (D.W + 1) * pl.BPF, pl.MAXSPLIT = 1;
-    const long long n_items = (long long)pl.QT * D.H * n_q;
-    if (!attn_divisors(pl, D.H, n_items, D.W, n_sm[dev])) return false;
+    pl.CH = (D.W + 1) * pl.BPF, pl.MAXSPLIT = 1, pl.SP = D.H * pl.QT;
+    if (!attn_divisors(pl, n_q, D.W, n_sm[dev])) return false;
     return launch_attn_plan(false, 0, enc[dev], n_sm[dev], st, d_sp, D, n_q, 0, pl, (size_t)D.R * D.H, (const bf16 *)q,
                             (const bf16 *)k_pages, (const bf16 *)v_pages, (bf16 *)out, nullptr, nullptr, d_stat) != 0;
 }

@@ -58,9 +58,11 @@
 // issuer run ahead into the next item.  A key range
 // longer than CH blocks is split over several items; each publishes its
 // unnormalised (O, m, l) state in global memory, stored so that a warp writes and reads
-// whole lines, and the warp that finishes last (a counter per half of O and quadrant of a
-// query tile) reads the states and merges them in split order.  CH depends only on the configuration, so
-// a frame's result does not depend on which other frames share its pass.
+// whole lines.  When a CTA is through with all its items, one warp counts it in at each of
+// them (a counter per query tile) and all its warps merge, in split order, those for which
+// it is the last (attn_merge).  CH depends only on the configuration, so
+// a frame's result does not depend on which other frames share its pass.  In a context of
+// several streams some (head, query tile) pairs are not split: attn_split_plan.
 #pragma once
 #include "nfd_sm100.cuh"
 
@@ -70,12 +72,14 @@ struct AttnPlan {
     int QT = 0;          // 128-row query tiles per frame
     int CH = 0;          // key blocks per split
     int MAXSPLIT = 0;    // splits of the longest window
-    FastDiv split_div, qt_div, h_div, ch_div, bpf_div;      // by MAXSPLIT, QT, heads, CH, BPF
+    int WH = 0;          // (head, query tile) pairs of a frame whose key range is not split: the first ones
+    int SP = 0;          // those whose key range is
+    int whole = 0;       // of a launch: items that are not split (frames x WH); they come first
+    FastDiv split_div, qt_div, wh_div, sp_div, ch_div, bpf_div;      // by MAXSPLIT, QT, WH, SP, CH, BPF
 };
 
 // A published state: [16 groups of 4 columns][128 rows] float4, then [2 halves of O][128 rows] (m, l).
 #define ATTN_STATE_BYTES (128 * 64 * 4 + 2 * 128 * 8)
-#define ATTN_COUNTERS 8          // of a query tile: one per half of O and quadrant of its rows
 #define ATTN_CTA_ITEMS 2048      // items of a CTA, at most: each has a byte of shared memory (see attn_finish)
 // Flags that are read when all roles are through: an item is marked, a wait has run out.  (In registers, with a vote at the
 // end, they cost two frames 39.6 -> 41.5 us.)
@@ -94,6 +98,7 @@ template <int KB> struct AttnCfg {
     static constexpr int TM_O = 448;
     static constexpr int SM_WARP0 = 4;                     // first softmax warp
     static constexpr int THREADS = 32 * (SM_WARP0 + 4 * NGRP);
+    static_assert(THREADS == 512, "attn_merge: a warp per quarter of the columns and quadrant of the rows");
     static_assert(KB % 16 == 0 && KB <= 128 && NS * S_STRIDE <= TM_O, "key block");
     static_assert(SMEM <= 232448, "shared memory of a CTA");
 };
@@ -136,17 +141,32 @@ __device__ __forceinline__ unsigned int atomic_inc_acq_rel(unsigned int *p) {
 // One item of the grid.
 struct AttnItem {
     int j, h, qt, split;     // frame of the pass, head, query tile, split
+    int tile;                // number of the query tile among those that are split
     int b0, nb, nsplit;      // key blocks of this split (nb = 0: the frame's window has no such split)
     FrameDesc fr;
+    __device__ __forceinline__ void place(int item, const AttnPlan &pl) {
+        int t;                                                 // (head, query tile) of the frame
+        if (item < pl.whole) {
+            j = pl.wh_div.div(item), t = item - j * pl.WH;
+            split = 0, tile = 0;
+        } else {
+            item -= pl.whole;
+            tile = pl.split_div.div(item), split = item - tile * pl.MAXSPLIT;
+            j = pl.sp_div.div(tile), t = pl.WH + tile - j * pl.SP;
+        }
+        h = pl.qt_div.div(t), qt = t - h * pl.QT;
+    }
     __device__ __forceinline__ void set(int item, const StepParams *sp, const Dims &D, const AttnPlan &pl) {
-        const int a = pl.split_div.div(item), b = pl.qt_div.div(a);
-        split = item - a * pl.MAXSPLIT, qt = a - b * pl.QT;
-        j = pl.h_div.div(b), h = b - j * D.H;
+        place(item, pl);
         fr = sp->fr[j];
         const int nbt = (fr.frame - fr.win_first + 1) * pl.BPF;      // key blocks of this frame's window
-        nsplit = pl.ch_div.div(nbt + pl.CH - 1);
-        b0 = split * pl.CH;
-        nb = min(nbt, b0 + pl.CH) - b0;
+        if (item < pl.whole) {
+            nsplit = 1, b0 = 0, nb = nbt;
+        } else {
+            nsplit = pl.ch_div.div(nbt + pl.CH - 1);
+            b0 = split * pl.CH;
+            nb = min(nbt, b0 + pl.CH) - b0;
+        }
         if (nb < 0) nb = 0;
     }
     // the first item at or after `item` (in steps of the grid) that has blocks; `end` or more: there is none
@@ -159,32 +179,34 @@ struct AttnItem {
     }
 };
 
+// Offsets in a published state of row `trow`: columns 4 g .. 4 g + 3, (m, l) as the warp with half p of the columns wrote it.
+__device__ __forceinline__ uint32_t attn_o_at(int g, int trow) { return (uint32_t)(g * 128 + trow) * 16; }
+__device__ __forceinline__ uint32_t attn_ml_at(int p, int trow) { return 128 * 64 * 4 + (uint32_t)(p * 128 + trow) * 8; }
+// n (a multiple of 8) columns of a result row from column e0 on
+template <int n>
+__device__ __forceinline__ void attn_write(const AttnItem &w, int row, int e0, const float *O, float l, const Dims &D, bf16 *out) {
+    if (row >= D.T || e0 >= D.dh) return;
+    const float inv = 1.0f / l;
+    bf16 *o = out + (size_t)(w.j * D.T + row) * D.d + w.h * D.dh + e0;
+#pragma unroll
+    for (int e = 0; e < n; e += 8) {
+        float t[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) t[u] = O[e + u] * inv;
+        *reinterpret_cast<uint4 *>(o + e) = pack_bf16x8(t);
+    }
+}
+
 // The end of an item for one warp: halves p0 .. p0 + np - 1 (32 columns each) of the 32 rows of its quadrant are read from
-// tensor memory and written out, or published; of the warps that hold a half of a tile's rows in its splits, the one that
-// finishes last merges them in split order.  (A counter per half and quadrant: no barrier of the CTA.)
+// tensor memory and written out, or published (attn_merge_all).
 // m, l: reference and sum of this thread's row.  With `redo` (see AttnShared; a byte per item, a bit per half and
 // quadrant; this is item `num`) a half whose l or O has left fp32 is left alone and marked there; without it, `mask` tells
 // which halves to take.
 static __device__ __forceinline__ void attn_finish(const AttnItem &w, int p0, int np, int mask, uint32_t tO, uint32_t o_free,
                                                    int trow, float m, float l, const Dims &D, const AttnPlan &pl, bf16 *out,
-                                                   float *part_o, unsigned int *counters, uint32_t *redo, int num) {
+                                                   float *part_o, uint32_t *redo, int num) {
     const int lane = threadIdx.x & 31, row = w.qt * 128 + trow;
-    const size_t item_q = ((size_t)w.j * D.H + w.h) * pl.QT + w.qt;
-    uint8_t *states = reinterpret_cast<uint8_t *>(part_o) + item_q * pl.MAXSPLIT * ATTN_STATE_BYTES;
-    auto o_at = [&](int p) { return (uint32_t)(p * 8 * 128 + trow) * 16; };
-    auto ml_at = [&](int p) { return 128 * 64 * 4 + (uint32_t)(p * 128 + trow) * 8; };
-    auto write_part = [&](int p, const float *O, float lt) {
-        if (row >= D.T || p * 32 >= D.dh) return;
-        const float inv = 1.0f / lt;
-        bf16 *o = out + (size_t)(w.j * D.T + row) * D.d + w.h * D.dh + p * 32;
-#pragma unroll
-        for (int e = 0; e < 32; e += 8) {
-            float t[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) t[u] = O[e + u] * inv;
-            *reinterpret_cast<uint4 *>(o + e) = pack_bf16x8(t);
-        }
-    };
+    uint8_t *states = reinterpret_cast<uint8_t *>(part_o) + (size_t)w.tile * pl.MAXSPLIT * ATTN_STATE_BYTES;
 #pragma unroll 1
     for (int p = p0; p < p0 + np; ++p) {
         float O[32];
@@ -205,57 +227,96 @@ static __device__ __forceinline__ void attn_finish(const AttnItem &w, int p0, in
         }
         if (!((mask >> p) & 1)) continue;
         if (w.nsplit == 1) {
-            write_part(p, O, l);
+            attn_write<32>(w, row, 32 * p, O, l, D, out);
         } else {
             uint8_t *st = states + (size_t)w.split * ATTN_STATE_BYTES;
 #pragma unroll
             for (int e = 0; e < 8; ++e)
-                *reinterpret_cast<float4 *>(st + o_at(p) + e * 2048) = make_float4(O[4 * e], O[4 * e + 1], O[4 * e + 2], O[4 * e + 3]);
-            *reinterpret_cast<float2 *>(st + ml_at(p)) = make_float2(m, l);
+                *reinterpret_cast<float4 *>(st + attn_o_at(8 * p + e, trow)) = make_float4(O[4 * e], O[4 * e + 1], O[4 * e + 2], O[4 * e + 3]);
+            *reinterpret_cast<float2 *>(st + attn_ml_at(p, trow)) = make_float2(m, l);
         }
     }
     tc_fence_before();
     __syncwarp();
     if (lane == 0 && o_free) mbar_arrive(o_free);
-    if (w.nsplit == 1) return;
-    unsigned int last = 0;
-    if (lane < np && ((mask >> (p0 + lane)) & 1)) {
-        unsigned int *cnt = counters + item_q * ATTN_COUNTERS + (p0 + lane) * 4 + (trow >> 5);
-        last = atomic_inc_acq_rel(cnt) == (unsigned int)(w.nsplit - 1);
+}
+
+// When a CTA is through with its items: one warp counts it in for each of those that are pieces of a split key range, a lane
+// for an item, and all merge, in split order, those for which it is the last, a warp a quarter of the columns of a quadrant's
+// rows.  Done as each item ended, the fence, the counter and the merge kept one of the softmax groups, and with it the order
+// of the products, for 3.5 us an item.  us, 310M class: four-frame speculation 14400 -> 13940, one frame (an item per CTA)
+// 5380 -> 5358, 220 tokens 4150 -> 4101.  Three states in flight and no more: with four the kernel's spilled registers
+// doubled, on the path of every item (5407, 13880, 4142).
+// The counter of the lane's item, if it has one; `all`: its pieces.
+static __device__ __forceinline__ unsigned int *attn_counter(int item, int n_items, const StepParams *sp, const Dims &D, const AttnPlan &pl,
+                                                             unsigned int *counters, unsigned int &all) {
+    if (item >= n_items) return nullptr;
+    AttnItem w;
+    w.set(item, sp, D, pl);
+    all = w.nsplit;
+    return w.nb > 0 && w.nsplit > 1 ? counters + w.tile : nullptr;
+}
+// Bit i: this CTA is the last of the tile of lane i's item.  (One warp; a barrier has ordered the CTA's states before.)
+static __device__ __forceinline__ uint32_t attn_count(unsigned int *cnt, unsigned int all) {
+    bool last = false;
+    if (cnt) {
+        last = atomic_inc_acq_rel(cnt) == all - 1;
         if (last) *cnt = 0;                                // ready for the next launch
     }
-    last = __ballot_sync(0xffffffffu, last);
-    // the ballot orders control only: this hands what the counting lanes have acquired to the lanes that read the states
-    __syncwarp();
+    return __ballot_sync(0xffffffffu, last);
+}
+// i0: item of bit 0
+static __device__ __forceinline__ void attn_merge(uint32_t last, int i0, const StepParams *sp, const Dims &D, const AttnPlan &pl,
+                                                  bf16 *out, const float *part_o) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int cq = warp >> 2, trow = (warp & 3) * 32 + lane;
+    if (16 * cq >= D.dh) return;
+    AttnItem w;
 #pragma unroll 1
-    for (int p = p0; p < p0 + np; ++p) {
-        if (!((last >> (p - p0)) & 1)) continue;
-        float O[32], lt = 0.f, mx = -INFINITY;
+    for (; last; last &= last - 1) {
+        w.set(i0 + (__ffs(last) - 1) * gridDim.x, sp, D, pl);
+        const uint8_t *st = reinterpret_cast<const uint8_t *>(part_o) + (size_t)w.tile * pl.MAXSPLIT * ATTN_STATE_BYTES;
+        float O[16], lt = 0.f, mx = -INFINITY;
 #pragma unroll
-        for (int e = 0; e < 32; ++e) O[e] = 0.f;
-        // (its own state is read back like the others)
+        for (int e = 0; e < 16; ++e) O[e] = 0.f;
+        // three states at a time, their loads in flight together
 #pragma unroll 1
-        for (int sp = 0; sp < w.nsplit; ++sp) {
-            const uint8_t *st = states + (size_t)sp * ATTN_STATE_BYTES;
-            const float2 ml = __ldcg(reinterpret_cast<const float2 *>(st + ml_at(p)));
-            float4 v[8];
+        for (int s0 = 0; s0 < w.nsplit; s0 += 3, st += 3 * ATTN_STATE_BYTES) {
+            float2 ml[3];
+            float4 v[3][4];
 #pragma unroll
-            for (int e = 0; e < 8; ++e) v[e] = __ldcg(reinterpret_cast<const float4 *>(st + o_at(p) + e * 2048));
+            for (int i = 0; i < 3; ++i) {
+                ml[i] = make_float2(-INFINITY, 0.f);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) v[i][e] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (s0 + i < w.nsplit) {
+                    ml[i] = __ldcg(reinterpret_cast<const float2 *>(st + i * ATTN_STATE_BYTES + attn_ml_at(cq >> 1, trow)));
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        v[i][e] = __ldcg(reinterpret_cast<const float4 *>(st + i * ATTN_STATE_BYTES + attn_o_at(4 * cq + e, trow)));
+                }
+            }
             // every rounding is spelled out: the bits must not depend on which CTA merges
-            const float mb = fmaxf(mx, ml.x);
-            // (a state with nothing but scores of -inf has m = -inf and counts for nothing)
-            const float fo = mx == mb ? 1.0f : ex2_approx(mx - mb), wgt = ml.x == -INFINITY ? 0.f : ex2_approx(ml.x - mb);
-            mx = mb;
-            lt = fmaf(ml.y, wgt, __fmul_rn(lt, fo));
+            const float mb = fmaxf(fmaxf(mx, ml[0].x), fmaxf(ml[1].x, ml[2].x));
+            const float fo = mx == mb ? 1.0f : ex2_approx(mx - mb);
+            mx = mb, lt = __fmul_rn(lt, fo);
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                O[4 * e] = fmaf(v[e].x, wgt, __fmul_rn(O[4 * e], fo));
-                O[4 * e + 1] = fmaf(v[e].y, wgt, __fmul_rn(O[4 * e + 1], fo));
-                O[4 * e + 2] = fmaf(v[e].z, wgt, __fmul_rn(O[4 * e + 2], fo));
-                O[4 * e + 3] = fmaf(v[e].w, wgt, __fmul_rn(O[4 * e + 3], fo));
+            for (int e = 0; e < 16; ++e) O[e] = __fmul_rn(O[e], fo);
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                // (a state with nothing but scores of -inf has m = -inf and counts for nothing)
+                const float wgt = ml[i].x == -INFINITY ? 0.f : ex2_approx(ml[i].x - mb);
+                lt = fmaf(ml[i].y, wgt, lt);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    O[4 * e] = fmaf(v[i][e].x, wgt, O[4 * e]);
+                    O[4 * e + 1] = fmaf(v[i][e].y, wgt, O[4 * e + 1]);
+                    O[4 * e + 2] = fmaf(v[i][e].z, wgt, O[4 * e + 2]);
+                    O[4 * e + 3] = fmaf(v[i][e].w, wgt, O[4 * e + 3]);
+                }
             }
         }
-        write_part(p, O, lt);
+        attn_write<16>(w, w.qt * 128 + trow, 16 * cq, O, lt, D, out);
     }
 }
 
@@ -264,7 +325,7 @@ template <int KB> struct AttnShared {
     using A = AttnCfg<KB>;
     uint32_t q, kv, bars, tmem;
     float *m, *l, *mx;       // [item parity][128], [item parity][group][128], [128] true maxima (times c)
-    uint32_t *redo;          // flags (below), nothing, and a byte per item (see attn_finish)
+    uint32_t *redo;          // flags (below), the items to merge, and a byte per item (see attn_finish)
     __device__ __forceinline__ uint32_t *tmem_slot() const { return redo + 2 + ATTN_CTA_ITEMS / 4 + 2 * (11 + 5 * A::NS); }
     __device__ __forceinline__ AttnShared(uint8_t *raw) {
         uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~(uintptr_t)1023);
@@ -318,7 +379,7 @@ template <int KB>
 __device__ __forceinline__ void attn_items(const AttnShared<KB> &sh, const CUtensorMap &tmQ, const CUtensorMap &tmK,
                                            const CUtensorMap &tmV, const StepParams *sp, const Dims &D, int layer, const AttnPlan &pl,
                                            const AttnItem &w0, int first, int end, int mode, int num, bf16 *out, float *part_o,
-                                           unsigned int *counters, int *status, int test_skip) {
+                                           int *status, int test_skip) {
     using A = AttnCfg<KB>;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t q_full = sh.q_full(), q_empty = sh.q_empty(), o_free = sh.o_free(), k_first = sh.k_first(), s_full = sh.s_full(),
@@ -590,6 +651,7 @@ __device__ __forceinline__ void attn_items(const AttnShared<KB> &sh, const CUten
             const int gl = (n03 + w.nb - 1) % A::NGRP;     // the group of that block
             n03 = gl + 1 == A::NGRP ? 0 : gl + 1;
             AttnItem wn;
+            int was = item;
             item = wn.find(item + gridDim.x, end, sp, D, pl);
             // The group of the last block finishes the item while the others are on the next one; groups 0 and 1 share the
             // CTA's last item.
@@ -618,8 +680,11 @@ __device__ __forceinline__ void attn_items(const AttnShared<KB> &sh, const CUten
                         mask = (marks & 1) | ((marks >> 3) & 2);
                         if (l == 0.f) m = -INFINITY;
                     }
+                    // (worked out again: kept through the loop they would cost registers that it needs)
+                    asm volatile("" : "+r"(was));
+                    w.place(was, pl);
                     attn_finish(w, fin ? g : 0, fin ? 1 : 2, mask, tO, fin ? 0u : o_free, trow, m, l, D, pl, out,
-                                part_o, counters, mode == RD_FIRST && ok ? sh.redo : nullptr, it - 1);
+                                part_o, mode == RD_FIRST && ok ? sh.redo : nullptr, it - 1);
                 }
             }
             w = wn;
@@ -633,8 +698,7 @@ __device__ __forceinline__ void attn_items(const AttnShared<KB> &sh, const CUten
 template <int KB>
 static __device__ __noinline__ void attn_again(const AttnShared<KB> sh, const CUtensorMap &tmQ, const CUtensorMap &tmK,
                                                const CUtensorMap &tmV, const StepParams *sp, const Dims &D, int layer,
-                                               const AttnPlan &pl, int n_items, bf16 *out, float *part_o, unsigned int *counters,
-                                               int *status) {
+                                               const AttnPlan &pl, int n_items, bf16 *out, float *part_o, int *status) {
     using A = AttnCfg<KB>;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = (warp - A::SM_WARP0) >> 2, quad = warp & 3;
     AttnItem w;
@@ -649,14 +713,14 @@ static __device__ __noinline__ void attn_again(const AttnShared<KB> sh, const CU
             if (threadIdx.x == 0) sh.inval_bars(), sh.init_bars();
             __syncthreads();
             tc_fence_after();
-            attn_items<KB>(sh, tmQ, tmK, tmV, sp, D, layer, pl, w, item, item + 1, mode, num, out, part_o, counters, status, 0);
+            attn_items<KB>(sh, tmQ, tmK, tmV, sp, D, layer, pl, w, item, item + 1, mode, num, out, part_o, status, 0);
             tc_fence_before();
             __syncthreads();
         }
         // (the second walk writes its rows in any case)
         if (mode <= RD_AGAIN && warp >= A::SM_WARP0 && g < 2)
             attn_finish(w, g, 1, (marks >> quad & 1) | (marks >> quad >> 3 & 2), sh.tmem + A::TM_O + ((uint32_t)(quad * 32) << 16), 0u,
-                        quad * 32 + lane, 0.f, NAN, D, pl, out, part_o, counters, nullptr, 0);
+                        quad * 32 + lane, 0.f, NAN, D, pl, out, part_o, nullptr, 0);
     }
 }
 
@@ -693,13 +757,29 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
     tc_fence_after();
     sh.tmem = *sh.tmem_slot();
 
-    attn_items<KB>(sh, tmQ, tmK, tmV, sp, D, layer, pl, w0, blockIdx.x, n_items, RD_FIRST, 0, out, part_o, counters, status,
-                   test_skip);
+    attn_items<KB>(sh, tmQ, tmK, tmV, sp, D, layer, pl, w0, blockIdx.x, n_items, RD_FIRST, 0, out, part_o, status, test_skip);
     NFD_TRACE_MARK_T(TRK_OTHER + 16, 128);
+    unsigned int *cnt = nullptr, all = 0;
+    if (warp == 2 && pl.MAXSPLIT > 1) cnt = attn_counter(blockIdx.x + lane * gridDim.x, n_items, sp, D, pl, counters, all);
     tc_fence_before();
     __syncthreads();
-    if (sh.redo[0] & ATTN_MARKED)
-        attn_again<KB>(sh, tmQ, tmK, tmV, sp, D, layer, pl, n_items, out, part_o, counters, status);
+    if (sh.redo[0] & ATTN_MARKED) {
+        attn_again<KB>(sh, tmQ, tmK, tmV, sp, D, layer, pl, n_items, out, part_o, status);
+        __syncthreads();                                   // (it writes states too)
+    }
+    if (pl.MAXSPLIT > 1) {
+#pragma unroll 1
+        for (int i0 = blockIdx.x; i0 < n_items; i0 += 32 * gridDim.x) {
+            if (warp == 2) {
+                if (i0 != blockIdx.x) cnt = attn_counter(i0 + lane * gridDim.x, n_items, sp, D, pl, counters, all);
+                const uint32_t last = attn_count(cnt, all);
+                if (lane == 0) sh.redo[1] = last;
+            }
+            __syncthreads();                               // what that warp has acquired is handed to the others
+            attn_merge(sh.redo[1], i0, sp, D, pl, out, part_o);
+            if (i0 + 32 * gridDim.x < n_items) __syncthreads();
+        }
+    }
     if (warp == 1) tmem_dealloc(sh.tmem, A::TMEM_COLS);
     NFD_TRACE_END(TRK_ATTN);
 }

@@ -3,9 +3,11 @@
 // nfd_api.cu.  fast_gemm / fast_attention return false when they do not handle
 // a case; the caller then launches the plain kernels.
 #pragma once
+#include <algorithm>
 #include <map>
 #include <tuple>
 #include <utility>
+#include <vector>
 
 #include "nfd_sm100.cuh"
 #include "nfd_gemm_tc.cuh"
@@ -24,7 +26,7 @@ struct FastState {
     size_t a_rows = 0;     // rows of every activation buffer (NFD_MAX_PASS_FRAMES * T)
     AttnPlan plan;         // KB == 0: tensor-core attention not available for this shape
     float *part_o = nullptr;           // per-split states of the attention kernel: [query tile][split] x ATTN_STATE_BYTES
-    unsigned int *attn_counters = nullptr;   // ATTN_COUNTERS per (frame, head, query tile); zero between launches
+    unsigned int *attn_counters = nullptr;   // one per query tile; zero between launches
     size_t cache_pages = 0;            // (stream, layer, ring slot, head) pages of T rows
     std::map<std::tuple<const void *, int, int, int>, CUtensorMap> maps;   // (ptr, rows, cols, box_rows)
 };
@@ -41,11 +43,45 @@ static void attn_blocks(AttnPlan &pl, int T) {
 }
 // The plan's divisors; false where a dividend is too large for them (n * d has to stay below 2^32) or a CTA would get more
 // items than it keeps account of.
-static bool attn_divisors(AttnPlan &pl, int H, long long n_items, int W, int n_sm) {
-    pl.split_div.set(pl.MAXSPLIT), pl.qt_div.set(pl.QT), pl.h_div.set(H), pl.ch_div.set(pl.CH), pl.bpf_div.set(pl.BPF);
+static bool attn_divisors(AttnPlan &pl, int n_frames, int W, int n_sm) {
+    pl.split_div.set(pl.MAXSPLIT), pl.qt_div.set(pl.QT), pl.ch_div.set(pl.CH), pl.bpf_div.set(pl.BPF);
+    pl.wh_div.set(pl.WH > 0 ? pl.WH : 1), pl.sp_div.set(pl.SP > 0 ? pl.SP : 1);
     const long long nb = ((long long)W + 1) * pl.BPF + pl.CH, big = 0x100000000ll;
-    const int d_item = pl.QT > H ? (pl.QT > pl.MAXSPLIT ? pl.QT : pl.MAXSPLIT) : (H > pl.MAXSPLIT ? H : pl.MAXSPLIT);
+    const long long n_items = n_frames * (pl.WH + (long long)pl.SP * pl.MAXSPLIT);
+    const int tiles = pl.WH + pl.SP, d_item = tiles > pl.MAXSPLIT ? tiles : pl.MAXSPLIT;
     return n_items <= (long long)ATTN_CTA_ITEMS * n_sm && n_items * d_item < big && nb < 0x7fffffffll && nb * (pl.CH > pl.BPF ? pl.CH : pl.BPF) < big;
+}
+// How the key ranges of a frame's `tiles` (head, query tile) pairs are split.  By the configuration alone (the longest
+// window, as many frames as there are streams), never by the pass: the order of the sums must not depend on it.
+//   One stream: all of them, into as many pieces as fill the SMs once.
+//   Several: the items are dealt out to the CTAs in order, and whole windows leave a last round in which most SMs idle (16 heads
+// x 3 query tiles x 8 streams = 384 items on 148 SMs: two rounds and six tenths of one, at the price of three).  Splitting all
+// of them finely costs a state of 33 KB each; so the first WH are left whole and the others split, for the least blocks on the
+// busiest CTA, a whole item counted a block more than it has and a piece two and a half (start, publication, merge).
+static void attn_split_plan(AttnPlan &pl, int tiles, int n_streams, int n_blocks, int n_sm) {
+    auto pieces = [&](int k) { pl.CH = (n_blocks + k - 1) / k, pl.MAXSPLIT = (n_blocks + pl.CH - 1) / pl.CH; };
+    pl.WH = 0, pl.SP = tiles;
+    const int items = n_streams * tiles;
+    if (n_streams == 1) return pieces(n_sm / items > 1 ? n_sm / items : 1);
+    float best = 1e30f;
+    int best_k = 1, best_wh = tiles;
+    std::vector<float> load(n_sm);
+    for (int k = 1; k <= 8 && k <= n_blocks; ++k) {
+        pieces(k);
+        for (int wh = k == 1 ? tiles : 0; wh <= (k == 1 ? tiles : tiles - 1); ++wh) {
+            const int nw = n_streams * wh, n = nw + n_streams * (tiles - wh) * pl.MAXSPLIT, grid = n < n_sm ? n : n_sm;
+            std::fill(load.begin(), load.end(), 0.f);
+            float most = 0.f;
+            for (int i = 0; i < n; ++i) {
+                const int b0 = i < nw ? 0 : (i - nw) % pl.MAXSPLIT * pl.CH;
+                load[i % grid] += i < nw ? n_blocks + 1.f : (n_blocks - b0 < pl.CH ? n_blocks - b0 : pl.CH) + 2.5f;
+                if (load[i % grid] > most) most = load[i % grid];
+            }
+            if (most < best) best = most, best_k = k, best_wh = wh;
+        }
+    }
+    pieces(best_k);
+    pl.WH = best_wh, pl.SP = tiles - best_wh;
 }
 static PFN_encodeTiled get_encode_fn() {
     void *fn = nullptr;
@@ -79,22 +115,15 @@ static int fast_create(FastState &fs, const Dims &D, bool bf16_mode, cudaStream_
     fs.cache_pages = (size_t)D.n_streams * D.L * D.R * D.H;
     if ((D.dh == 64 || D.dh == 32) && fs.cache_pages < 0x7fffffffull) {
         attn_blocks(pl, D.T);
-        // split the longest window (a frame sees at most W + 1 pages) so that streams x heads x query tiles x
-        // splits fills the SMs once: a context made for several streams is run with batched passes, which bring
-        // enough (frame, head, query tile) items by themselves, and long unsplit key ranges amortise the
-        // start and the merge of a CTA.  The split depends on the configuration only, never on the pass.
-        const int items_per_pass = D.n_streams * D.H * pl.QT;
-        const int target = fs.n_sm / items_per_pass > 1 ? fs.n_sm / items_per_pass : 1;
-        pl.CH = ((D.W + 1) * pl.BPF + target - 1) / target;
-        pl.MAXSPLIT = ((D.W + 1) * pl.BPF + pl.CH - 1) / pl.CH;
-        if (attn_divisors(pl, D.H, (long long)NFD_MAX_PASS_FRAMES * D.H * pl.QT * pl.MAXSPLIT, D.W, fs.n_sm)) {
-            if (pl.MAXSPLIT > 1) {
+        attn_split_plan(pl, D.H * pl.QT, D.n_streams, (D.W + 1) * pl.BPF, fs.n_sm);
+        if (attn_divisors(pl, NFD_MAX_PASS_FRAMES, D.W, fs.n_sm)) {
+            if (pl.SP > 0 && pl.MAXSPLIT > 1) {
                 // (the largest pass of this context: per stream a speculation and the deferred frames of the last one)
                 const int nf_max = D.n_streams * (D.R - D.W);
-                const size_t tiles = (size_t)(nf_max < NFD_MAX_PASS_FRAMES ? nf_max : NFD_MAX_PASS_FRAMES) * D.H * pl.QT;
+                const size_t tiles = (size_t)(nf_max < NFD_MAX_PASS_FRAMES ? nf_max : NFD_MAX_PASS_FRAMES) * pl.SP;
                 if (cudaMalloc((void **)&fs.part_o, tiles * pl.MAXSPLIT * (size_t)ATTN_STATE_BYTES) != cudaSuccess ||
-                    cudaMalloc((void **)&fs.attn_counters, tiles * ATTN_COUNTERS * sizeof(unsigned int)) != cudaSuccess ||
-                    cudaMemset(fs.attn_counters, 0, tiles * ATTN_COUNTERS * sizeof(unsigned int)) != cudaSuccess) {
+                    cudaMalloc((void **)&fs.attn_counters, tiles * sizeof(unsigned int)) != cudaSuccess ||
+                    cudaMemset(fs.attn_counters, 0, tiles * sizeof(unsigned int)) != cudaSuccess) {
                     cudaGetLastError();
                     return NFD_E_NOMEM;
                 }
@@ -388,7 +417,7 @@ static bool fast_gemm(bool enabled, FastState &fs, cudaStream_t st, const TS *A,
 
 template <int KB>
 static int launch_attn_tc(bool early, int test_skip, PFN_encodeTiled encode, int n_sm, cudaStream_t st, const StepParams *sp, const Dims &D, int nf,
-                          int layer, const AttnPlan &pl, size_t pages, const bf16 *q, const bf16 *kc, const bf16 *vc,
+                          int layer, AttnPlan pl, size_t pages, const bf16 *q, const bf16 *kc, const bf16 *vc,
                           bf16 *out, float *part_o, unsigned int *counters, int *status) {
     using A = AttnCfg<KB>;
     auto kern = k_attn_tc<KB>;
@@ -397,7 +426,8 @@ static int launch_attn_tc(bool early, int test_skip, PFN_encodeTiled encode, int
     if (!encode_map_3d(encode, &mq, q, D.H, nf * D.T, D.dh, 128) || !encode_map_3d(encode, &mk, kc, pages, D.T, D.dh, KB) ||
         !encode_map_3d(encode, &mv, vc, pages, D.T, D.dh, KB))
         return 0;
-    const int n_items = pl.MAXSPLIT * pl.QT * D.H * nf;
+    pl.whole = nf * pl.WH;
+    const int n_items = pl.whole + nf * pl.SP * pl.MAXSPLIT;
     dim3 grid(n_items < n_sm ? n_items : n_sm);
     cudaError_t e = launch_kernel(early, kern, grid, dim3(A::THREADS), (size_t)A::SMEM, st, 1, mq, mk, mv, sp, D, layer, pl, n_items,
                                   out, part_o, counters, status, test_skip);

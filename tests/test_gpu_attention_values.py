@@ -74,6 +74,25 @@ def test_bf16_result_is_as_exact_as_its_own_rounding(heads, dh, T, n_kv, n_q, wi
         assert g.status() == 0
 
 
+@pytest.mark.parametrize("streams,heads,T,window,n_kv,n_q", [
+    (4, 16, 336, 16, 17, 8),         # 35 of 48 (head, query tile) pairs whole, 13 in three pieces
+    (8, 16, 336, 32, 20, 3),         # 37 whole, 11 in five pieces of which the window fills three and a bit
+    (3, 12, 220, 9, 12, 2),          # all in two pieces
+    (2, 4, 64, 16, 17, 8)])          # all in six pieces, the last one shorter
+def test_windows_whole_and_in_pieces(streams, heads, T, window, n_kv, n_q):
+    """Contexts of several streams split the key ranges of some (head, query tile) pairs and not those of others."""
+    from paper_2506_01380_b200 import nfd as N
+    q, k, v, _ = _pages(heads, 64, T, n_kv, n_q, seed=T + streams)
+    ref = _exact(q, k, v, n_q, window)
+    cfg = I.make_cfg("nfd310m", n_layers=1, d_model=heads * 64, n_heads=heads, head_dim=64, d_mlp=256, latent_h=T // 2,
+                     latent_w=8, patch=2, ctx_frames=window, max_spec=8, n_streams=streams)
+    g = N.NFD(cfg, I.make_weights(cfg, 0))
+    rows = lambda x: x.permute(1, 0, 2, 3).reshape(heads, n_kv * T, 64).contiguous()
+    for _ in range(2):               # (the counters of the pieces are at rest after a call)
+        assert _rel(g.attention(q, rows(k), rows(v), n_q, n_kv, window), ref) <= 1.02 * _rel(ref.bfloat16(), ref)
+    assert g.status() == 0
+
+
 def _rising(heads, dh, T, n_kv, n_q, seed, nats, v_scale=1.0):
     """Scores that rise by `nats` from the first page to the last, evenly: q has 8 in one column, and k there what it takes.
     The first rows of q take no part in it."""
