@@ -425,6 +425,11 @@ template <typename TS> static void enqueue_body(nfd_ctx *c, int nf, int kind) {
         EpiFinal<TS> ef{sp, (const TS *)c->b_out, D};
         launch_gemm<TS>(c, (const TS *)c->hbuf, (const TS *)c->w_out, M, D.P, d, ef);
     }
+    if (c->h_sp.post.kind) {
+        // (frames that ride along have no output: the grid is for all of them, the kernel has the number of elements)
+        c->cls = CLS_SAMPLER;
+        PLAUNCH(c, k_sampler_step, (int)(((size_t)nf * c->frame_elems() + 255) / 256), 256, 0, sp);
+    }
 }
 
 static void enqueue_body_any(nfd_ctx *c, int nf, int kind) {
@@ -461,7 +466,7 @@ static int run_pass_inner(nfd_ctx *c) {
     }
     // (no conditioning kernels when all pairs are cached)
     const int key = kind * 64 + nf + (c->fast ? 0 : 4096) + (c->h_sp.nc > 0 ? 0 : 8192) + (c->fuse_ln ? 0 : 16384) +
-                    (c->l2_prefetch ? 0 : 32768) + (c->kv_prefetch ? 0 : 65536);
+                    (c->l2_prefetch ? 0 : 32768) + (c->kv_prefetch ? 0 : 65536) + (c->h_sp.post.kind ? 131072 : 0);
     auto it = c->graphs.find(key);
     if (it == c->graphs.end()) {
         GraphEntry ge;
@@ -520,6 +525,7 @@ struct PassInputs {
     const float *x_a[2] = {nullptr, nullptr}, *x_b[2] = {nullptr, nullptr};
     float alpha[2] = {0.f, 0.f}, beta[2] = {0.f, 0.f};
     float *v_out = nullptr;
+    PostStep post = {};          // the sampler's step behind the pass, if any
 };
 
 // Fill c->h_sp for a pass over the given frames.  Nothing is changed if it fails.
@@ -540,6 +546,7 @@ static int build_pass_frames(nfd_ctx *c, const std::vector<PassFrame> &fr, int k
     p.kind = kind;
     for (int s = 0; s < 2; ++s) p.x_a[s] = in.x_a[s], p.x_b[s] = in.x_b[s], p.alpha[s] = in.alpha[s], p.beta[s] = in.beta[s];
     p.v_out = in.v_out;
+    p.post = in.post;
     int nc = 0;
     for (int j = 0; j < nf; ++j) {
         const PassFrame &pf = fr[j];
@@ -580,7 +587,7 @@ static int build_pass_frames(nfd_ctx *c, const std::vector<PassFrame> &fr, int k
 //   actions: per stream (per_frame_actions = false) or per frame.
 static int build_pass(nfd_ctx *c, int n, const int *streams, int k, int offset, const float *t, const int *actions,
                       bool per_frame_actions, int kind, const float *x_a, float alpha, const float *x_b, float beta,
-                      float *v_out) {
+                      float *v_out, const PostStep &post = PostStep()) {
     const nfd_cfg &g = c->cfg;
     if (n < 1 || k < 1 || offset < 0 || offset + k > g.max_spec) return NFD_E_RANGE;
     if ((long long)n * k > NFD_MAX_PASS_FRAMES) return NFD_E_RANGE;
@@ -602,7 +609,7 @@ static int build_pass(nfd_ctx *c, int n, const int *streams, int k, int offset, 
             fr.push_back(f);
         }
     PassInputs in;
-    in.x_a[0] = x_a, in.x_b[0] = x_b, in.alpha[0] = alpha, in.beta[0] = beta, in.v_out = v_out;
+    in.x_a[0] = x_a, in.x_b[0] = x_b, in.alpha[0] = alpha, in.beta[0] = beta, in.v_out = v_out, in.post = post;
     return build_pass_frames(c, fr, kind, in);
 }
 
@@ -940,6 +947,15 @@ int nfd_speculate_batched(nfd_ctx *c, int n, const int *streams, int k, const in
         const double t = sn / (sn + cs);
         const double alpha = sqrt(t * t + (1 - t) * (1 - t)) / sd;
         for (int i = 0; i < n; ++i) tv[i] = (float)t;
+        // clean estimate sigma_d (x_in - t v), then re-noise to the next timestep
+        PostStep post = {};
+        post.kind = 1, post.x = c->xp, post.v = c->vbuf, post.x0 = x0_out, post.n = (long long)ne;
+        post.a = (float)(sd * alpha), post.b = (float)(-sd * t);
+        if (s + 1 < S) {
+            const double tpn = 0.5 * M_PI * (double)(S - s - 1) / (double)S;
+            post.z = noise + (size_t)(s + 1) * ne;
+            post.c = (float)cos(tpn), post.s = (float)(sin(tpn) * sd);
+        }
         if (s == 0 && carry) {
             // one block-causal pass: per stream its deferred frames (K/V only), then the k new frames
             std::vector<PassFrame> fr;
@@ -958,26 +974,15 @@ int nfd_speculate_batched(nfd_ctx *c, int n, const int *streams, int k, const in
             float t_fm;
             commit_coeffs(c, &t_fm, &in.alpha[1], &in.beta[1]);
             in.x_a[1] = c->pend_x0, in.x_b[1] = c->pend_cz;
-            in.x_a[0] = c->xp, in.alpha[0] = (float)alpha, in.v_out = c->vbuf;
+            in.x_a[0] = c->xp, in.alpha[0] = (float)alpha, in.v_out = c->vbuf, in.post = post;
             RET(build_pass_frames(c, fr, 0, in));
             RET(run_pass(c));
             for (int i = 0; i < n; ++i) c->n_pending[streams[i]] = 0;
         } else {
             RET(build_pass(c, n, streams, k, 0, tv.data(), actions, false, 0, c->xp, (float)alpha, nullptr, 0.f,
-                           c->vbuf));
+                           c->vbuf, post));
             RET(run_pass(c));
         }
-        // clean estimate sigma_d (x_in - t v), then re-noise to the next timestep
-        const float *z = nullptr;
-        double cn = 0, sn_next = 0;
-        if (s + 1 < S) {
-            const double tpn = 0.5 * M_PI * (double)(S - s - 1) / (double)S;
-            z = noise + (size_t)(s + 1) * ne;
-            cn = cos(tpn), sn_next = sin(tpn) * sd;
-        }
-        c->cls = CLS_SAMPLER;
-        PLAUNCH(c, k_sampler_post, eg, 256, 0, c->xp, (const float *)c->vbuf, z, x0_out, (float)(sd * alpha),
-                (float)(-sd * t), (float)cn, (float)sn_next, ne);
     }
     CK(take_launch_err(c));
     if (!c->lazy) {
@@ -1027,8 +1032,6 @@ int nfd_sample_dpmpp(nfd_ctx *c, int stream, int k, int action, int n_evals, con
     for (int i = 1; i <= M; ++i) {
         const double tp = tgrid(i - 1), tn = tgrid(i);
         const float tf = (float)tp;
-        RET(build_pass(c, 1, &stream, k, 0, &tf, &action, false, 0, c->xp, 1.0f, nullptr, 0.f, c->vbuf));
-        RET(run_pass(c));
         const double a = tn / tp;
         const double b = (1.0 - tn) - (1.0 - tp) * tn / tp;
         double cc = 0.0;
@@ -1036,9 +1039,11 @@ int nfd_sample_dpmpp(nfd_ctx *c, int stream, int k, int action, int n_evals, con
             const double tpp = tgrid(i - 2);
             cc = (lam(tn) - lam(tp)) / (2.0 * (lam(tp) - lam(tpp)));
         }
-        c->cls = CLS_SAMPLER;
-        PLAUNCH(c, k_dpmpp_update, eg, 256, 0, c->xp, (const float *)c->vbuf, c->x0_prev, tf, (float)a, (float)b,
-                (float)cc, i == M ? x0_out : (float *)nullptr, c->cfg.sigma_d, ne);
+        PostStep post = {};
+        post.kind = 2, post.x = c->xp, post.v = c->vbuf, post.x0 = i == M ? x0_out : nullptr, post.x0_prev = c->x0_prev;
+        post.a = (float)a, post.b = (float)b, post.c = (float)cc, post.t = tf, post.scale = c->cfg.sigma_d, post.n = (long long)ne;
+        RET(build_pass(c, 1, &stream, k, 0, &tf, &action, false, 0, c->xp, 1.0f, nullptr, 0.f, c->vbuf, post));
+        RET(run_pass(c));
     }
     CK(take_launch_err(c));
     std::vector<int> fa(k, action);

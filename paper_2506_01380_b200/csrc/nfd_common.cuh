@@ -37,6 +37,19 @@ struct CondDesc {
     int slot;        // cache slot the result goes to
 };
 
+// The sampler's step at the end of a denoising pass (Section 4.1), if there is one: see k_sampler_step.
+struct PostStep {
+    int kind;               // 0 none, 1 few-step sampler, 2 DPM-Solver++
+    float a, b, c, s;       // coefficients
+    float t, scale;         // (DPM-Solver++)
+    float *x;               // the sampler's state
+    const float *v;         // the pass's velocity
+    const float *z;         // noise for the next step, or NULL
+    float *x0;              // clean estimate (DPM-Solver++: the result, last step only, or NULL)
+    float *x0_prev;         // (DPM-Solver++)
+    long long n;            // elements
+};
+
 // Everything that changes from pass to pass.  Written to device memory by the
 // first kernel of every pass so that a captured graph can be replayed with new
 // values (cache position, timestep, action, I/O pointers).
@@ -52,6 +65,7 @@ struct StepParams {
     const float *x_b[2];    // may be NULL
     float alpha[2], beta[2];
     float *v_out;           // [frames with out_index >= 0, C,H,W]
+    PostStep post;
     FrameDesc fr[NFD_MAX_PASS_FRAMES];
     CondDesc cd[NFD_MAX_PASS_FRAMES];
 };
