@@ -53,7 +53,9 @@ static bool attn_divisors(AttnPlan &pl, int n_frames, int W, int n_sm) {
 }
 // How the key ranges of a frame's `tiles` (head, query tile) pairs are split.  By the configuration alone (the longest
 // window, as many frames as there are streams), never by the pass: the order of the sums must not depend on it.
-//   One stream: all of them, into as many pieces as fill the SMs once.
+//   One stream: all of them, into at most as many pieces as fill the SMs once, and no more than pay: a block takes about 0.65
+// us (of 112 keys; its columns and 24 count), publishing and counting 2.5, the merge 0.25 per piece.  (A frame of a model of 2 layers,
+// 4 heads, 64 tokens: behind four frames five pieces of a block 286 us, one of five 270; behind 30 frames 31 pieces 443, six 300.)
 //   Several: the items are dealt out to the CTAs in order, and whole windows leave a last round in which most SMs idle (16 heads
 // x 3 query tiles x 8 streams = 384 items on 148 SMs: two rounds and six tenths of one, at the price of three).  Splitting all
 // of them finely costs a state of 33 KB each; so the first WH are left whole and the others split, for the least blocks on the
@@ -62,9 +64,16 @@ static void attn_split_plan(AttnPlan &pl, int tiles, int n_streams, int n_blocks
     auto pieces = [&](int k) { pl.CH = (n_blocks + k - 1) / k, pl.MAXSPLIT = (n_blocks + pl.CH - 1) / pl.CH; };
     pl.WH = 0, pl.SP = tiles;
     const int items = n_streams * tiles;
-    if (n_streams == 1) return pieces(n_sm / items > 1 ? n_sm / items : 1);
     float best = 1e30f;
     int best_k = 1, best_wh = tiles;
+    if (n_streams == 1) {
+        for (int k = 1; k <= n_blocks && (k == 1 || k * items <= n_sm); ++k) {
+            pieces(k);
+            const float t = pl.CH * 0.65f * (pl.KB + 24) / 136.f + (k > 1 ? 2.5f + 0.25f * k : 0.f);
+            if (t < best) best = t, best_k = k;
+        }
+        return pieces(best_k);
+    }
     std::vector<float> load(n_sm);
     for (int k = 1; k <= 8 && k <= n_blocks; ++k) {
         pieces(k);
