@@ -7,6 +7,7 @@
 
 #include <map>
 #include <new>
+#include <type_traits>
 #include <vector>
 
 #include "nfd_kernels.cuh"
@@ -305,6 +306,16 @@ static void launch_gemm(nfd_ctx *c, const TS *A, const TS *Wt, int M, int N, int
 }
 
 // `early`: see launch_attn_plan; set inside a pass, where the QKV projection comes before.
+// `launch` with the instance of k_attn_rows for the head dimension, and its grid.
+template <typename TS, typename F> static void launch_attn_rows(int n_sm, const Dims &D, int nf, F launch) {
+    const int nq = attn_rows_q(D, nf, n_sm);
+    const dim3 grid((D.T + nq - 1) / nq, D.H, nf);
+    switch (D.dh) {
+        case 32: return nq == 8 ? launch(k_attn_rows<TS, 32, 8>, grid) : launch(k_attn_rows<TS, 32, 16>, grid);
+        case 64: return nq == 8 ? launch(k_attn_rows<TS, 64, 8>, grid) : launch(k_attn_rows<TS, 64, 16>, grid);
+        default: return nq == 8 ? launch(k_attn_rows<TS, 128, 8>, grid) : launch(k_attn_rows<TS, 128, 16>, grid);
+    }
+}
 template <typename TS> static void launch_attention(nfd_ctx *c, int nf, int layer, bool early, int test_skip = 0) {
     const Dims &D = c->D;
     c->cls = CLS_ATTN;
@@ -316,16 +327,10 @@ template <typename TS> static void launch_attention(nfd_ctx *c, int nf, int laye
         c->launches += n_fast;
         return;
     }
-    const dim3 grid((D.T + ATTN_ROWS_Q - 1) / ATTN_ROWS_Q, D.H, nf);
-    if (D.dh == 32)
-        PLAUNCH(c, (k_attn_rows<TS, 32>), grid, 256, 0, (const StepParams *)c->d_sp, D, layer, (const TS *)c->qbuf,
-                (const TS *)c->kc, (const TS *)c->vc, (TS *)c->abuf);
-    else if (D.dh == 64)
-        PLAUNCH(c, (k_attn_rows<TS, 64>), grid, 256, 0, (const StepParams *)c->d_sp, D, layer, (const TS *)c->qbuf,
-                (const TS *)c->kc, (const TS *)c->vc, (TS *)c->abuf);
-    else
-        PLAUNCH(c, (k_attn_rows<TS, 128>), grid, 256, 0, (const StepParams *)c->d_sp, D, layer, (const TS *)c->qbuf,
-                (const TS *)c->kc, (const TS *)c->vc, (TS *)c->abuf);
+    launch_attn_rows<TS>(c->fs.n_sm, D, nf, [&](auto kern, dim3 grid) {
+        PLAUNCH(c, kern, grid, 256, 0, (const StepParams *)c->d_sp, D, layer, (const TS *)c->qbuf, (const TS *)c->kc, (const TS *)c->vc,
+                (TS *)c->abuf);
+    });
 }
 
 // Conditioning kernels for the c->h_sp.nc (time, action) pairs that the pass found missing in the
@@ -1340,41 +1345,42 @@ static_assert(sizeof(StepParams) <= NFD_NOALLOC_STATUS_OFFSET, "pass descriptor 
 static void *g_noalloc_dev_ptr[NFD_NOALLOC_MAX_DEVICES] = {nullptr};
 
 template <typename TS>
-static int noalloc_launch(cudaStream_t st, const StepParams *d_sp, const Dims &D, int n_q, const void *q,
+static int noalloc_launch(cudaStream_t st, int n_sm, const StepParams *d_sp, const Dims &D, int n_q, const void *q,
                           const void *k_pages, const void *v_pages, void *out) {
-    const dim3 grid((D.T + ATTN_ROWS_Q - 1) / ATTN_ROWS_Q, D.H, n_q);
-    if (D.dh == 32)
-        k_attn_rows<TS, 32><<<grid, 256, 0, st>>>(d_sp, D, 0, (const TS *)q, (const TS *)k_pages, (const TS *)v_pages, (TS *)out);
-    else if (D.dh == 64)
-        k_attn_rows<TS, 64><<<grid, 256, 0, st>>>(d_sp, D, 0, (const TS *)q, (const TS *)k_pages, (const TS *)v_pages, (TS *)out);
-    else
-        k_attn_rows<TS, 128><<<grid, 256, 0, st>>>(d_sp, D, 0, (const TS *)q, (const TS *)k_pages, (const TS *)v_pages, (TS *)out);
+    launch_attn_rows<TS>(n_sm, D, n_q, [&](auto kern, dim3 grid) {
+        kern<<<grid, 256, 0, st>>>(d_sp, D, 0, (const TS *)q, (const TS *)k_pages, (const TS *)v_pages, (TS *)out);
+    });
     CK(cudaGetLastError());
     return NFD_OK;
 }
 
-// The tensor-core kernel on the caller's pages, key ranges unsplit (a split would need memory for its states).
+// The tensor-core kernel on the caller's pages.
 // Returns false where it does not handle the case.
-static bool noalloc_launch_tc(int dev, cudaStream_t st, const StepParams *d_sp, int *d_stat, const Dims &D, int n_q,
+static bool noalloc_launch_tc(int dev, int n_sm, cudaStream_t st, const StepParams *d_sp, int *d_stat, const Dims &D, int n_q,
                               const void *q, const void *k_pages, const void *v_pages, void *out) {
     static PFN_encodeTiled enc[NFD_NOALLOC_MAX_DEVICES];
-    static int n_sm[NFD_NOALLOC_MAX_DEVICES];
     if (D.dh != 64 && D.dh != 32) return false;
     if (!enc[dev]) {
         // looked up once per device, like the array's address
         PFN_encodeTiled e = get_encode_fn();
-        if (!e || cudaDeviceGetAttribute(&n_sm[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-            cudaGetLastError();
-            return false;
-        }
+        if (!e) return false;
         enc[dev] = e;
     }
     AttnPlan pl;
     attn_blocks(pl, D.T);
-    pl.CH = (D.W + 1) * pl.BPF, pl.MAXSPLIT = 1, pl.SP = D.H * pl.QT;
-    if (!attn_divisors(pl, n_q, D.W, n_sm[dev])) return false;
-    return launch_attn_plan(false, 0, enc[dev], n_sm[dev], st, d_sp, D, n_q, 0, pl, (size_t)D.R * D.H, (const bf16 *)q,
-                            (const bf16 *)k_pages, (const bf16 *)v_pages, (bf16 *)out, nullptr, nullptr, d_stat) != 0;
+    pl.SP = D.H * pl.QT;
+    attn_own_plan(pl, n_q * pl.SP, (D.W < D.R ? D.W + 1 : D.R) * pl.BPF, n_sm);
+    if (!attn_divisors(pl, n_q, D.W, n_sm)) return false;
+    auto go = [&](auto kb) {
+        return launch_attn_own<decltype(kb)::value>(enc[dev], n_sm, st, d_sp, n_q, D, pl, (size_t)D.R * D.H, (const bf16 *)q,
+                                                    (const bf16 *)k_pages, (const bf16 *)v_pages, (bf16 *)out, d_stat);
+    };
+    switch (pl.KB) {
+        case 128: return go(std::integral_constant<int, 128>());
+        case 112: return go(std::integral_constant<int, 112>());
+        case 96: return go(std::integral_constant<int, 96>());
+        default: return go(std::integral_constant<int, 64>());
+    }
 }
 
 extern "C" int nfd_attention_noalloc(const void *q, const void *k_pages, const void *v_pages, int dtype, int n_heads,
@@ -1400,13 +1406,16 @@ extern "C" int nfd_attention_noalloc(const void *q, const void *k_pages, const v
     int dev = -1;
     CK(cudaGetDevice(&dev));
     if (dev < 0 || dev >= NFD_NOALLOC_MAX_DEVICES) return NFD_E_RANGE;
+    static int n_sms[NFD_NOALLOC_MAX_DEVICES];
     if (!g_noalloc_dev_ptr[dev]) {
         // one-time set-up for the current device: turn the symbol into a device address
         void *p = nullptr;
+        CK(cudaDeviceGetAttribute(&n_sms[dev], cudaDevAttrMultiProcessorCount, dev));
         CK(cudaGetSymbolAddress(&p, g_noalloc_scratch));
         if (!p) return NFD_E_CUDA;
         g_noalloc_dev_ptr[dev] = p;
     }
+    const int n_sm = n_sms[dev];
     StepParams *d_sp = (StepParams *)g_noalloc_dev_ptr[dev];
     // the descriptor check of k_set_params records a failure in a status word; it lives in the same array
     int *d_stat = (int *)((unsigned char *)g_noalloc_dev_ptr[dev] + NFD_NOALLOC_STATUS_OFFSET);
@@ -1433,8 +1442,8 @@ extern "C" int nfd_attention_noalloc(const void *q, const void *k_pages, const v
     // the descriptor is rewritten in full on every call; nothing of the previous call survives
     k_set_params<<<1, 256, 0, st>>>(p, d_sp, lim, d_stat);
     CK(cudaGetLastError());
-    if (dtype == NFD_DTYPE_BF16 && noalloc_launch_tc(dev, st, d_sp, d_stat, D, n_q_frames, q, k_pages, v_pages, out))
+    if (dtype == NFD_DTYPE_BF16 && noalloc_launch_tc(dev, n_sm, st, d_sp, d_stat, D, n_q_frames, q, k_pages, v_pages, out))
         return NFD_OK;
-    if (dtype == NFD_DTYPE_BF16) return noalloc_launch<bf16>(st, d_sp, D, n_q_frames, q, k_pages, v_pages, out);
-    return noalloc_launch<float>(st, d_sp, D, n_q_frames, q, k_pages, v_pages, out);
+    if (dtype == NFD_DTYPE_BF16) return noalloc_launch<bf16>(st, n_sm, d_sp, D, n_q_frames, q, k_pages, v_pages, out);
+    return noalloc_launch<float>(st, n_sm, d_sp, D, n_q_frames, q, k_pages, v_pages, out);
 }

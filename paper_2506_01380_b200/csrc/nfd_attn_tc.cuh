@@ -93,6 +93,7 @@ template <int KB> struct AttnCfg {
     static constexpr int KV_BYTES = KB * 128;              // one K (or V) block
     static constexpr int ML_BYTES = (2 * (1 + NGRP) + 1) * 128 * 4;   // m of every row, l of every row and group, two items; maxima
     static constexpr int SMEM = 2 * Q_BYTES + 2 * NS * KV_BYTES + ML_BYTES + 8 + ATTN_CTA_ITEMS + 256 + 1024;
+    static constexpr int STATE_AT = (SMEM + 127) / 128 * 128;              // k_attn_own: the CTA's state, behind the rest
     static constexpr int TMEM_COLS = 512;
     static constexpr int S_STRIDE = KB <= 112 ? 112 : 128; // S accumulators from column 0, O at column 448
     static constexpr int TM_O = 448;
@@ -202,11 +203,13 @@ __device__ __forceinline__ void attn_write(const AttnItem &w, int row, int e0, c
 // m, l: reference and sum of this thread's row.  With `redo` (see AttnShared; a byte per item, a bit per half and
 // quadrant; this is item `num`) a half whose l or O has left fp32 is left alone and marked there; without it, `mask` tells
 // which halves to take.
+template <bool OWN>
 static __device__ __forceinline__ void attn_finish(const AttnItem &w, int p0, int np, int mask, uint32_t tO, uint32_t o_free,
                                                    int trow, float m, float l, const Dims &D, const AttnPlan &pl, bf16 *out,
                                                    float *part_o, uint32_t *redo, int num) {
     const int lane = threadIdx.x & 31, row = w.qt * 128 + trow;
-    uint8_t *states = reinterpret_cast<uint8_t *>(part_o) + (size_t)w.tile * pl.MAXSPLIT * ATTN_STATE_BYTES;
+    // OWN: the state goes to the CTA's own shared memory, for its cluster
+    uint8_t *state = reinterpret_cast<uint8_t *>(part_o) + (OWN ? 0 : ((size_t)w.tile * pl.MAXSPLIT + w.split) * ATTN_STATE_BYTES);
 #pragma unroll 1
     for (int p = p0; p < p0 + np; ++p) {
         float O[32];
@@ -229,11 +232,10 @@ static __device__ __forceinline__ void attn_finish(const AttnItem &w, int p0, in
         if (w.nsplit == 1) {
             attn_write<32>(w, row, 32 * p, O, l, D, out);
         } else {
-            uint8_t *st = states + (size_t)w.split * ATTN_STATE_BYTES;
 #pragma unroll
             for (int e = 0; e < 8; ++e)
-                *reinterpret_cast<float4 *>(st + attn_o_at(8 * p + e, trow)) = make_float4(O[4 * e], O[4 * e + 1], O[4 * e + 2], O[4 * e + 3]);
-            *reinterpret_cast<float2 *>(st + attn_ml_at(p, trow)) = make_float2(m, l);
+                *reinterpret_cast<float4 *>(state + attn_o_at(8 * p + e, trow)) = make_float4(O[4 * e], O[4 * e + 1], O[4 * e + 2], O[4 * e + 3]);
+            *reinterpret_cast<float2 *>(state + attn_ml_at(p, trow)) = make_float2(m, l);
         }
     }
     tc_fence_before();
@@ -375,7 +377,7 @@ enum { RD_FIRST, RD_MAX, RD_AGAIN };
 
 // The CTA's items first, first + gridDim.x, ... below end (w0 is the first one); `num`: number of the item in sh.redo, not for
 // RD_FIRST.
-template <int KB>
+template <int KB, bool OWN>
 __device__ __forceinline__ void attn_items(const AttnShared<KB> &sh, const CUtensorMap &tmQ, const CUtensorMap &tmK,
                                            const CUtensorMap &tmV, const StepParams *sp, const Dims &D, int layer, const AttnPlan &pl,
                                            const AttnItem &w0, int first, int end, int mode, int num, bf16 *out, float *part_o,
@@ -683,7 +685,7 @@ __device__ __forceinline__ void attn_items(const AttnShared<KB> &sh, const CUten
                     // (worked out again: kept through the loop they would cost registers that it needs)
                     asm volatile("" : "+r"(was));
                     w.place(was, pl);
-                    attn_finish(w, fin ? g : 0, fin ? 1 : 2, mask, tO, fin ? 0u : o_free, trow, m, l, D, pl, out,
+                    attn_finish<OWN>(w, fin ? g : 0, fin ? 1 : 2, mask, tO, fin ? 0u : o_free, trow, m, l, D, pl, out,
                                 part_o, mode == RD_FIRST && ok ? sh.redo : nullptr, it - 1);
                 }
             }
@@ -695,7 +697,7 @@ __device__ __forceinline__ void attn_items(const AttnShared<KB> &sh, const CUten
 
 // The items with marked rows once more, each twice.  Not inlined: the first walk's code is as if this were not there.
 // After a wait that has run out the marked rows are NaN (and counted: the tile's other splits may be waited for).
-template <int KB>
+template <int KB, bool OWN>
 static __device__ __noinline__ void attn_again(const AttnShared<KB> sh, const CUtensorMap &tmQ, const CUtensorMap &tmK,
                                                const CUtensorMap &tmV, const StepParams *sp, const Dims &D, int layer,
                                                const AttnPlan &pl, int n_items, bf16 *out, float *part_o, int *status) {
@@ -713,15 +715,36 @@ static __device__ __noinline__ void attn_again(const AttnShared<KB> sh, const CU
             if (threadIdx.x == 0) sh.inval_bars(), sh.init_bars();
             __syncthreads();
             tc_fence_after();
-            attn_items<KB>(sh, tmQ, tmK, tmV, sp, D, layer, pl, w, item, item + 1, mode, num, out, part_o, status, 0);
+            attn_items<KB, OWN>(sh, tmQ, tmK, tmV, sp, D, layer, pl, w, item, item + 1, mode, num, out, part_o, status, 0);
             tc_fence_before();
             __syncthreads();
         }
         // (the second walk writes its rows in any case)
         if (mode <= RD_AGAIN && warp >= A::SM_WARP0 && g < 2)
-            attn_finish(w, g, 1, (marks >> quad & 1) | (marks >> quad >> 3 & 2), sh.tmem + A::TM_O + ((uint32_t)(quad * 32) << 16), 0u,
+            attn_finish<OWN>(w, g, 1, (marks >> quad & 1) | (marks >> quad >> 3 & 2), sh.tmem + A::TM_O + ((uint32_t)(quad * 32) << 16), 0u,
                         quad * 32 + lane, 0.f, NAN, D, pl, out, part_o, nullptr, 0);
     }
+}
+
+template <int KB>
+__device__ __forceinline__ void attn_set_up(AttnShared<KB> &sh, const CUtensorMap &tmQ, const CUtensorMap &tmK, const CUtensorMap &tmV) {
+    using A = AttnCfg<KB>;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (warp == 0 && lane == 0) {
+        tma_prefetch_desc(&tmQ);
+        tma_prefetch_desc(&tmK);
+        tma_prefetch_desc(&tmV);
+        sh.init_bars();
+    }
+    for (int i = threadIdx.x; i < 2 + ATTN_CTA_ITEMS / 4; i += A::THREADS) sh.redo[i] = 0;
+    if (warp == 1) {
+        tmem_alloc(smem_u32(sh.tmem_slot()), A::TMEM_COLS);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    sh.tmem = *sh.tmem_slot();
 }
 
 template <int KB>
@@ -741,30 +764,15 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
     AttnItem w0;
     w0.set(blockIdx.x, sp, D, pl);
 
-    if (warp == 0 && lane == 0) {
-        tma_prefetch_desc(&tmQ);
-        tma_prefetch_desc(&tmK);
-        tma_prefetch_desc(&tmV);
-        sh.init_bars();
-    }
-    for (int i = threadIdx.x; i < 2 + ATTN_CTA_ITEMS / 4; i += A::THREADS) sh.redo[i] = 0;
-    if (warp == 1) {
-        tmem_alloc(smem_u32(sh.tmem_slot()), A::TMEM_COLS);
-        tmem_relinquish();
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    sh.tmem = *sh.tmem_slot();
-
-    attn_items<KB>(sh, tmQ, tmK, tmV, sp, D, layer, pl, w0, blockIdx.x, n_items, RD_FIRST, 0, out, part_o, status, test_skip);
+    attn_set_up<KB>(sh, tmQ, tmK, tmV);
+    attn_items<KB, false>(sh, tmQ, tmK, tmV, sp, D, layer, pl, w0, blockIdx.x, n_items, RD_FIRST, 0, out, part_o, status, test_skip);
     NFD_TRACE_MARK_T(TRK_OTHER + 16, 128);
     unsigned int *cnt = nullptr, all = 0;
     if (warp == 2 && pl.MAXSPLIT > 1) cnt = attn_counter(blockIdx.x + lane * gridDim.x, n_items, sp, D, pl, counters, all);
     tc_fence_before();
     __syncthreads();
     if (sh.redo[0] & ATTN_MARKED) {
-        attn_again<KB>(sh, tmQ, tmK, tmV, sp, D, layer, pl, n_items, out, part_o, status);
+        attn_again<KB, false>(sh, tmQ, tmK, tmV, sp, D, layer, pl, n_items, out, part_o, status);
         __syncthreads();                                   // (it writes states too)
     }
     if (pl.MAXSPLIT > 1) {
@@ -782,4 +790,68 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
     }
     if (warp == 1) tmem_dealloc(sh.tmem, A::TMEM_COLS);
     NFD_TRACE_END(TRK_ATTN);
+}
+
+// The caller's pages (nfd_attention_noalloc), for which there is no memory for states: the pieces of a split key range are the
+// CTAs of a cluster.  Each leaves its state in its own shared memory, and after a cluster barrier they merge them through
+// distributed shared memory, in split order, each CTA some quarters of the columns.  Without a split the grid is persistent,
+// as in k_attn_tc.
+// Measured, 16 heads x 64, 336 queries behind 16 frames of 336 (48 query tiles), us with both launches of the call: one CTA to a
+// tile 43.1, two 30.8.  (Three would want 48 clusters, and the machine holds 45.)
+template <int KB>
+__global__ void __launch_bounds__(AttnCfg<KB>::THREADS, 1)
+k_attn_own(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
+           const __grid_constant__ CUtensorMap tmV, const StepParams *sp, const __grid_constant__ Dims D,
+           const __grid_constant__ AttnPlan pl, int n_items, bf16 *out, int *status) {
+    using A = AttnCfg<KB>;
+    extern __shared__ uint8_t smem_raw[];
+    AttnShared<KB> sh(smem_raw);
+    float *state = reinterpret_cast<float *>(smem_raw + A::STATE_AT);
+    AttnItem w0;
+    w0.set(blockIdx.x, sp, D, pl);
+    attn_set_up<KB>(sh, tmQ, tmK, tmV);
+    // (with a split a CTA has one item)
+    const int end = pl.MAXSPLIT > 1 ? (int)blockIdx.x + 1 : n_items;
+    attn_items<KB, true>(sh, tmQ, tmK, tmV, sp, D, 0, pl, w0, blockIdx.x, end, RD_FIRST, 0, out, state, status, 0);
+    tc_fence_before();
+    __syncthreads();
+    if (sh.redo[0] & ATTN_MARKED) attn_again<KB, true>(sh, tmQ, tmK, tmV, sp, D, 0, pl, end, out, state, status);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (pl.MAXSPLIT > 1) {
+        __syncwarp();
+        cluster_sync_all();                                // every state of the cluster is in place
+        w0.set(blockIdx.x, sp, D, pl);
+        const int cq = warp >> 2, trow = (warp & 3) * 32 + lane;
+        if (w0.nsplit > 1 && w0.split < w0.nsplit && cq % w0.nsplit == w0.split && 16 * cq < D.dh) {
+            const uint32_t st = smem_u32(state);
+            float O[16], lt = 0.f, mx = -INFINITY;
+#pragma unroll
+            for (int e = 0; e < 16; ++e) O[e] = 0.f;
+#pragma unroll 1
+            for (int s = 0; s < w0.nsplit; ++s) {
+                const float2 ml = ld_cluster_f2(cluster_map(st + attn_ml_at(cq >> 1, trow), s));
+                float4 v[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) v[e] = ld_cluster_f4(cluster_map(st + attn_o_at(4 * cq + e, trow), s));
+                const float mb = fmaxf(mx, ml.x);
+                // (a state with nothing but scores of -inf has m = -inf and counts for nothing)
+                const float fo = mx == mb ? 1.0f : ex2_approx(mx - mb), wgt = ml.x == -INFINITY ? 0.f : ex2_approx(ml.x - mb);
+                mx = mb, lt = fmaf(ml.y, wgt, __fmul_rn(lt, fo));
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    O[4 * e] = fmaf(v[e].x, wgt, __fmul_rn(O[4 * e], fo));
+                    O[4 * e + 1] = fmaf(v[e].y, wgt, __fmul_rn(O[4 * e + 1], fo));
+                    O[4 * e + 2] = fmaf(v[e].z, wgt, __fmul_rn(O[4 * e + 2], fo));
+                    O[4 * e + 3] = fmaf(v[e].w, wgt, __fmul_rn(O[4 * e + 3], fo));
+                }
+            }
+            attn_write<16>(w0, w0.qt * 128 + trow, 16 * cq, O, lt, D, out);
+        }
+        __syncwarp();
+        cluster_arrive_relaxed();                          // no CTA leaves while a peer may still read its state
+        cluster_wait();
+    } else {
+        __syncthreads();
+    }
+    if (warp == 1) tmem_dealloc(sh.tmem, A::TMEM_COLS);
 }

@@ -51,6 +51,21 @@ static bool attn_divisors(AttnPlan &pl, int n_frames, int W, int n_sm) {
     const int tiles = pl.WH + pl.SP, d_item = tiles > pl.MAXSPLIT ? tiles : pl.MAXSPLIT;
     return n_items <= (long long)ATTN_CTA_ITEMS * n_sm && n_items * d_item < big && nb < 0x7fffffffll && nb * (pl.CH > pl.BPF ? pl.CH : pl.BPF) < big;
 }
+// Pieces of the key range of a call on the caller's pages: as many as pay (as in attn_split_plan; the merge is through
+// distributed shared memory) and as clusters of that size fit the machine at once.  On a 148-SM B200 clusters of 1, 2, 3, 4, 5,
+// 6, 8 hold 148, 148, 135, 132, 130, 132, 120 CTAs (cudaOccupancyMaxActiveClusters); from 3 on four clusters less than the SMs
+// would make is within that.
+static void attn_own_plan(AttnPlan &pl, int tiles, int n_blocks, int n_sm) {
+    float best = 1e30f;
+    int best_k = 1;
+    for (int k = 1; k <= 8 && k <= n_blocks; ++k) {
+        const int clusters = k <= 2 ? n_sm / k : n_sm / k - 4, ch = (n_blocks + k - 1) / k;
+        if (k > 1 && (tiles > clusters || (n_blocks + ch - 1) / ch != k)) continue;
+        const float t = ch * 0.65f * (pl.KB + 24) / 136.f + (k > 1 ? 1.5f + 0.2f * k : 0.f);
+        if (t < best) best = t, best_k = k;
+    }
+    pl.CH = (n_blocks + best_k - 1) / best_k, pl.MAXSPLIT = best_k;
+}
 // How the key ranges of a frame's `tiles` (head, query tile) pairs are split.  By the configuration alone (the longest
 // window, as many frames as there are streams), never by the pass: the order of the sums must not depend on it.
 //   One stream: all of them, into at most as many pieces as fill the SMs once, and no more than pay: a block takes about 0.65
@@ -446,6 +461,30 @@ static int launch_attn_tc(bool early, int test_skip, PFN_encodeTiled encode, int
         return 0;
     }
     return 1;
+}
+
+// The caller's pages: see k_attn_own.
+template <int KB>
+static bool launch_attn_own(PFN_encodeTiled encode, int n_sm, cudaStream_t st, const StepParams *sp, int nf, const Dims &D, const AttnPlan &pl,
+                            size_t pages, const bf16 *q, const bf16 *kc, const bf16 *vc, bf16 *out, int *status) {
+    using A = AttnCfg<KB>;
+    auto kern = k_attn_own<KB>;
+    constexpr int smem = A::STATE_AT + ATTN_STATE_BYTES;
+    static_assert(smem <= 232448, "shared memory of a CTA");
+    if (!allow_smem(kern, smem)) return false;
+    CUtensorMap mq, mk, mv;
+    if (!encode_map_3d(encode, &mq, q, D.H, nf * D.T, D.dh, 128) || !encode_map_3d(encode, &mk, kc, pages, D.T, D.dh, KB) ||
+        !encode_map_3d(encode, &mv, vc, pages, D.T, D.dh, KB))
+        return false;
+    const int n_items = nf * pl.SP * pl.MAXSPLIT;
+    const dim3 grid(pl.MAXSPLIT > 1 || n_items < n_sm ? n_items : n_sm);
+    const cudaError_t e = launch_kernel(false, kern, grid, dim3(A::THREADS), (size_t)smem, st, pl.MAXSPLIT, mq, mk, mv, sp, D, pl, n_items, out, status);
+    if (e != cudaSuccess) {
+        fprintf(stderr, "libnfd: tensor-core attention launch failed: %s\n", cudaGetErrorString(e));
+        cudaGetLastError();
+        return false;
+    }
+    return true;
 }
 
 // Attention of a pass by plan `pl` over `pages` (stream, layer, ring slot, head) pages of K and V.  `early`: the kernel may

@@ -887,7 +887,7 @@ __global__ void __launch_bounds__(256) k_gemm_simple(const StepParams *sp, int T
 
 // ---------------------------------------------------------------------------
 // Block-wise causal attention (Section 3.1) on the fp32 pipes: fp32 storage, bf16
-// with head dimension 128, and the "fast = 0" path.  A CTA takes 16 queries of one
+// with head dimension 128, and the "fast = 0" path.  A CTA takes 16 or 8 queries of one
 // (frame, head); its eight warps take the 32-key tiles of the query frame's window
 // in turn, page by page, so that the mask is a page range and never a matrix, each
 // with an online softmax of its own, merged at the end.
@@ -897,13 +897,15 @@ __global__ void __launch_bounds__(256) k_gemm_simple(const StepParams *sp, int T
 // broadcasts), in O += P V a lane owns DH/32 columns (V rows are read coalesced, P is
 // a broadcast); no sum over lanes is taken until the end, and the maximum over lanes
 // only where a tile raises it.  (One warp per query with a sum over lanes per key, as
-// it was: 139 us for 6 heads x 32, 2 x 77 queries, 462 keys in fp32.)
+// it was: 139 us for 6 heads x 32, 2 x 77 queries, 462 keys in fp32.)  A tile is a chain of loads: a batch of eight
+// 16-byte words of K and of up to 16 rows of V is in flight together, and where CTAs of 16 queries leave half of the SMs
+// idle they take 8 (that case 24.6 -> 20.5 us, 8 heads x 128, 100 queries, 1000 keys 84 -> 56).
 // ---------------------------------------------------------------------------
-#define ATTN_ROWS_Q 16
-template <typename TS, int DH>
+template <typename TS, int DH, int NQ>
 __global__ void __launch_bounds__(256) k_attn_rows(const StepParams *sp, Dims D, int layer, const TS *q, const TS *kc,
                                                    const TS *vc, TS *out) {
-    constexpr int R = DH / 32, NQ = ATTN_ROWS_Q, PS = NQ + 4, NV = WVec<TS>::N;
+    constexpr int R = DH / 32, PS = NQ + 4, NV = WVec<TS>::N;
+    constexpr int UK = DH / NV < 8 ? DH / NV : 8, UV = R == 1 ? 16 : (R == 2 ? 8 : 4);     // loads in flight together: of K, rows of V
     __shared__ __align__(16) float s_q[NQ][DH];
     __shared__ __align__(16) float s_p[8][32 * PS];              // P of a tile: [key][query]; later O of a column slice
     __shared__ float s_m[8][NQ], s_l[8][NQ];
@@ -945,7 +947,7 @@ __global__ void __launch_bounds__(256) k_attn_rows(const StepParams *sp, Dims D,
         float s[NQ];
 #pragma unroll
         for (int i = 0; i < NQ; ++i) s[i] = 0.f;
-#pragma unroll 2
+#pragma unroll UK
         for (int e = 0; e < DH; e += NV) {
             float kf[NV];
             WVec<TS>::load(krow + e, kf);
@@ -980,7 +982,7 @@ __global__ void __launch_bounds__(256) k_attn_rows(const StepParams *sp, Dims D,
         for (int x = 0; x < np; ++x) {
             const TS *vrow = vc + page_at(x) + lane;
             const float *px = pw + x * per * PS;
-#pragma unroll 4
+#pragma unroll UV
             for (int kk = 0; kk < per; ++kk) {
                 float v[R];
 #pragma unroll
@@ -1025,6 +1027,8 @@ __global__ void __launch_bounds__(256) k_attn_rows(const StepParams *sp, Dims D,
         }
     }
 }
+// Queries per CTA: 16, or 8 where CTAs of 16 leave half of the SMs idle (a row's bits are the same).
+static int attn_rows_q(const Dims &D, int nf, int n_sm) { return 2ll * ((D.T + 15) / 16) * D.H * nf <= n_sm ? 8 : 16; }
 
 // ---------------------------------------------------------------------------
 // Sampler glue (Section 4.1): elementwise.

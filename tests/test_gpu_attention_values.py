@@ -195,3 +195,18 @@ def test_small_pages_on_the_fp32_pipes(T, dtype, dh, tol):
     q, k, v, out = _pages(3, dh, T, 37, 2, seed=T, dtype=dtype)
     for window in (36, 5, 0):
         assert _rel(N.attention_noalloc(q, k, v, 2, window, out), _exact(q, k, v, 2, window)) <= tol
+
+
+@pytest.mark.parametrize("nats", [0, 30])          # (30 nats a page: items are walked again)
+@pytest.mark.parametrize("heads,T,dh,n_kv,n_q,window", [
+    (16, 336, 64, 17, 1, 16),        # two pieces of 26 and 25 blocks
+    (2, 100, 32, 9, 3, 8),           # pages of one masked block, head dimension 32
+    (2, 64, 64, 8, 8, 8),            # windows of one to eight blocks: some have fewer pieces than the cluster has CTAs
+    (1, 336, 64, 17, 1, 16)])        # eight pieces, the last one shorter
+def test_pieces_as_the_ctas_of_a_cluster(heads, T, dh, n_kv, n_q, window, nats):
+    import torch
+    from paper_2506_01380_b200 import nfd as N
+    q, k, v, out = _rising(heads, dh, T, n_kv, n_q, seed=T, nats=nats * n_kv) if nats else _pages(heads, dh, T, n_kv, n_q, seed=T)
+    ref = _exact(q, k, v, n_q, window)
+    got = N.attention_noalloc(q, k, v, n_q, window, out.fill_(float("nan")))
+    assert _rel(got, ref) <= 1.02 * _rel(ref.to(torch.bfloat16), ref)
