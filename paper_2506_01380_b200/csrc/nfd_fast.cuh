@@ -274,6 +274,11 @@ static int gemm_p_width(int n_sm, int form, int T, int dh, int M, int N, int K, 
         const int t96 = mt * ((N + 95) / 96);
         return (t96 + n_sm - 1) / n_sm <= (t128 + n_sm - 1) / n_sm ? 96 : 128;
     }
+    // Into the MLP, where k_gemm_tc would take 96 columns in one wave (its epilogue, GELU or gate behind a staging tile, is the
+    // longer half of it): from 100 CTAs on k_gemm_p in the same tiles.  One frame, us: 310M class (129 tiles) 5350 -> 5332,
+    // hidden 768 with a gated MLP (129) 2315 -> 2297; 86 tiles (220 tokens) 4203 -> 4211, 12 tiles (64 tokens) 299 -> 307.
+    const int t96 = mt * ((N + 95) / 96);
+    if (form == FORM_MLP && S == 1 && t96 <= n_sm && t96 >= (100 * n_sm) / 148 && mt * ((N + 63) / 64) > n_sm) return 96;
     if (t128 < (100 * n_sm) / 148) return 0;
     if (S > 1) return 128;
     // microseconds: a base and a wave, fitted to K = 768, 1024 and 1536 (within 2 us up to ten waves)
@@ -410,6 +415,9 @@ static bool launch_gemm_p_any(FastState &fs, cudaStream_t st, const bf16 *A, con
                                    : launch_gemm_p<96, Epi, false>(fs, st, A, Wt, M, N, K, S, epi, pf);
     }
     if (S > 1) return launch_gemm_p<128, Epi, true>(fs, st, A, Wt, M, N, K, S, epi, pf);
+    if constexpr (Epi::kForm == FORM_MLP) {
+        if (BN == 96) return launch_gemm_p<96, Epi, false>(fs, st, A, Wt, M, N, K, S, epi, pf);
+    }
     if constexpr (Epi::kForm != FORM_RES) {
         if (BN == 256) return launch_gemm_p<256, Epi, false>(fs, st, A, Wt, M, N, K, S, epi, pf);
         if (BN == 192) return launch_gemm_p<192, Epi, false>(fs, st, A, Wt, M, N, K, S, epi, pf);

@@ -28,7 +28,7 @@ template <int BN, int FORM> struct GemmPCfg {
     static constexpr int A_BYTES = 128 * 128, B_BYTES = BN * 128, ST_BYTES = A_BYTES + B_BYTES;
     // a stage (64 elements of K) comes back about 1200 clocks after it was asked for: the ring holds about what the
     // products use in that time
-    static constexpr int STAGES = BN <= 96 ? 5 : (BN <= 128 ? (FORM == FORM_MLP ? 5 : 4) : (BN <= 192 && FORM == FORM_MLP ? 4 : 3));
+    static constexpr int STAGES = BN <= 96 ? (FORM == FORM_MLP ? 6 : 5) : (BN <= 128 ? (FORM == FORM_MLP ? 5 : 4) : (BN <= 192 && FORM == FORM_MLP ? 4 : 3));
     static constexpr int RING_BYTES = STAGES * ST_BYTES;
     static constexpr int PARTS = BN == 96 ? 3 : 2;             // epilogue warps per tensor-memory lane quadrant
     static constexpr int EPI_WARP0 = 4, EPI_WARPS = 4 * PARTS;

@@ -31,6 +31,12 @@ def test_tiles_of_three_groups_per_warp(streams, k):
     _batched_equals_single(1024, (48, 28), streams, k, 0, 1024, 16, 1, passes=40)
 
 
+@pytest.mark.parametrize("hw,act,dm,fuse_ln", [((48, 28), 0, 4096, 1), ((46, 30), 1, 2052, 1), ((48, 28), 0, 4100, 0)])
+def test_mlp_of_a_single_frame_in_one_wave(hw, act, dm, fuse_ln):
+    """4096 to 4104 columns: 43 tiles 96 wide, the last one 64 to 80, by three row blocks; the batched pass has wider ones."""
+    _batched_equals_single(768, hw, 4, 2, act, dm, 12, fuse_ln)
+
+
 def _batched_equals_single(d, hw, streams, k, act, dm, heads, fuse_ln, passes=1):
     import torch
     from paper_2506_01380_b200.nfd import NFD
