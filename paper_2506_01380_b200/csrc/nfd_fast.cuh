@@ -3,11 +3,9 @@
 // nfd_api.cu.  fast_gemm / fast_attention return false when they do not handle
 // a case; the caller then launches the plain kernels.
 #pragma once
-#include <algorithm>
 #include <map>
 #include <tuple>
 #include <utility>
-#include <vector>
 
 #include "nfd_sm100.cuh"
 #include "nfd_gemm_tc.cuh"
@@ -89,17 +87,17 @@ static void attn_split_plan(AttnPlan &pl, int tiles, int n_streams, int n_blocks
         }
         return pieces(best_k);
     }
-    std::vector<float> load(n_sm);
     for (int k = 1; k <= 8 && k <= n_blocks; ++k) {
         pieces(k);
         for (int wh = k == 1 ? tiles : 0; wh <= (k == 1 ? tiles : tiles - 1); ++wh) {
             const int nw = n_streams * wh, n = nw + n_streams * (tiles - wh) * pl.MAXSPLIT, grid = n < n_sm ? n : n_sm;
-            std::fill(load.begin(), load.end(), 0.f);
+            // the CTAs before, between and behind those with a whole item and with an item more than others
             float most = 0.f;
-            for (int i = 0; i < n; ++i) {
-                const int b0 = i < nw ? 0 : (i - nw) % pl.MAXSPLIT * pl.CH;
-                load[i % grid] += i < nw ? n_blocks + 1.f : (n_blocks - b0 < pl.CH ? n_blocks - b0 : pl.CH) + 2.5f;
-                if (load[i % grid] > most) most = load[i % grid];
+            const int at[3] = {0, nw % grid, n % grid};
+            for (int c : at) {
+                const int w = nw / grid + (c < nw % grid), all = n / grid + (c < n % grid);
+                const float t = w * (n_blocks + 1.f) + (all - w) * (pl.CH + 2.5f);
+                if (t > most) most = t;
             }
             if (most < best) best = most, best_k = k, best_wh = wh;
         }
