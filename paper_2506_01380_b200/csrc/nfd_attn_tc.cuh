@@ -93,7 +93,8 @@ template <int KB> struct AttnCfg {
     static constexpr int KV_BYTES = KB * 128;              // one K (or V) block
     static constexpr int ML_BYTES = (2 * (1 + NGRP) + 1) * 128 * 4;   // m of every row, l of every row and group, two items; maxima
     static constexpr int SMEM = 2 * Q_BYTES + 2 * NS * KV_BYTES + ML_BYTES + 8 + ATTN_CTA_ITEMS + 256 + 1024;
-    static constexpr int STATE_AT = (SMEM + 127) / 128 * 128;              // k_attn_own: the CTA's state, behind the rest
+    // k_attn_own: the CTA's state, behind the rest, from the 1024-byte boundary that AttnShared starts at
+    static constexpr int STATE_AT = (SMEM - 1024 + 127) / 128 * 128, OWN_SMEM = 1024 + STATE_AT + ATTN_STATE_BYTES;
     static constexpr int TMEM_COLS = 512;
     static constexpr int S_STRIDE = KB <= 112 ? 112 : 128; // S accumulators from column 0, O at column 448
     static constexpr int TM_O = 448;
@@ -101,7 +102,8 @@ template <int KB> struct AttnCfg {
     static constexpr int THREADS = 32 * (SM_WARP0 + 4 * NGRP);
     static_assert(THREADS == 512, "attn_merge: a warp per quarter of the columns and quadrant of the rows");
     static_assert(KB % 16 == 0 && KB <= 128 && NS * S_STRIDE <= TM_O, "key block");
-    static_assert(SMEM <= 232448, "shared memory of a CTA");
+    static_assert(SMEM <= 232448 && OWN_SMEM <= 232448, "shared memory of a CTA");
+    static_assert(STATE_AT % 16 == 0 && ATTN_STATE_BYTES % 16 == 0, "states are read and written in 16-byte words");
 };
 
 __host__ __device__ constexpr uint32_t umma_idesc_bf16_bmn(int M, int N) {
@@ -325,12 +327,13 @@ static __device__ __forceinline__ void attn_merge(uint32_t last, int i0, const S
 // The shared memory of a CTA, and its tensor memory.
 template <int KB> struct AttnShared {
     using A = AttnCfg<KB>;
+    uint8_t *base;           // 1024-byte boundary
     uint32_t q, kv, bars, tmem;
     float *m, *l, *mx;       // [item parity][128], [item parity][group][128], [128] true maxima (times c)
     uint32_t *redo;          // flags (below), the items to merge, and a byte per item (see attn_finish)
     __device__ __forceinline__ uint32_t *tmem_slot() const { return redo + 2 + ATTN_CTA_ITEMS / 4 + 2 * (11 + 5 * A::NS); }
     __device__ __forceinline__ AttnShared(uint8_t *raw) {
-        uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~(uintptr_t)1023);
+        uint8_t *smem = base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~(uintptr_t)1023);
         q = smem_u32(smem), kv = q + 2 * A::Q_BYTES, tmem = 0;
         m = reinterpret_cast<float *>(smem + 2 * A::Q_BYTES + 2 * A::NS * A::KV_BYTES), l = m + 2 * 128;
         mx = l + 2 * A::NGRP * 128, redo = reinterpret_cast<uint32_t *>(mx + 128);
@@ -806,7 +809,7 @@ k_attn_own(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     using A = AttnCfg<KB>;
     extern __shared__ uint8_t smem_raw[];
     AttnShared<KB> sh(smem_raw);
-    float *state = reinterpret_cast<float *>(smem_raw + A::STATE_AT);
+    float *state = reinterpret_cast<float *>(sh.base + A::STATE_AT);
     AttnItem w0;
     w0.set(blockIdx.x, sp, D, pl);
     attn_set_up<KB>(sh, tmQ, tmK, tmV);
@@ -848,8 +851,9 @@ k_attn_own(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             attn_write<16>(w0, w0.qt * 128 + trow, 16 * cq, O, lt, D, out);
         }
         __syncwarp();
-        cluster_arrive_relaxed();                          // no CTA leaves while a peer may still read its state
-        cluster_wait();
+        // No CTA leaves while a peer may still read its state.  (With release: lanes of rows beyond the frame's have nothing that
+        // waits for what they read, and their loads must be over too.)
+        cluster_sync_all();
     } else {
         __syncthreads();
     }

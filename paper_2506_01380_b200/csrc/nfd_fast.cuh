@@ -475,8 +475,7 @@ static bool launch_attn_own(PFN_encodeTiled encode, int n_sm, cudaStream_t st, c
                             size_t pages, const bf16 *q, const bf16 *kc, const bf16 *vc, bf16 *out, int *status) {
     using A = AttnCfg<KB>;
     auto kern = k_attn_own<KB>;
-    constexpr int smem = A::STATE_AT + ATTN_STATE_BYTES;
-    static_assert(smem <= 232448, "shared memory of a CTA");
+    constexpr int smem = A::OWN_SMEM;
     if (!allow_smem(kern, smem)) return false;
     CUtensorMap mq, mk, mv;
     if (!encode_map_3d(encode, &mq, q, D.H, nf * D.T, D.dh, 128) || !encode_map_3d(encode, &mk, kc, pages, D.T, D.dh, KB) ||

@@ -1,0 +1,32 @@
+"""Rules of order that the kernels rely on and that no result shows while they are broken, checked in the sources."""
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2506_01380_b200", "csrc")
+
+
+def _kernels(name):
+    """{kernel: body} of a source file, comments removed."""
+    text = open(os.path.join(CSRC, name)).read()
+    text = re.sub(r"//[^\n]*", "", text)
+    out = {}
+    for m in re.finditer(r"__global__\s+void\b", text):
+        i = text.index("{", m.end())
+        head, depth, j = text[m.end():i], 0, i
+        while True:
+            depth += {"{": 1, "}": -1}.get(text[j], 0)
+            j += 1
+            if depth == 0:
+                break
+        out[re.search(r"\b(k_\w+)\s*\(", head).group(1)] = text[i:j]
+    return out
+
+
+def test_cluster_pieces_are_read_before_their_cta_may_leave():
+    """The states of k_attn_own's pieces are read from peers' shared memory, by some lanes without any use for the value: the
+    barrier behind the reads has to order them.  The state starts where 16-byte words may: at the rounded base."""
+    body = _kernels("nfd_attn_tc.cuh")["k_attn_own"]
+    reads = [m.start() for m in re.finditer(r"ld_cluster_f[24]\(", body)]
+    after = body[max(reads):]
+    assert "cluster_sync_all()" in after and "cluster_arrive_relaxed" not in after
+    assert re.search(r"state = reinterpret_cast<float \*>\(sh\.base \+ A::STATE_AT\)", body)
