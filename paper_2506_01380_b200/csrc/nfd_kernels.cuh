@@ -897,15 +897,20 @@ __global__ void __launch_bounds__(256) k_gemm_simple(const StepParams *sp, int T
 // broadcasts), in O += P V a lane owns DH/32 columns (V rows are read coalesced, P is
 // a broadcast); no sum over lanes is taken until the end, and the maximum over lanes
 // only where a tile raises it.  (One warp per query with a sum over lanes per key, as
-// it was: 139 us for 6 heads x 32, 2 x 77 queries, 462 keys in fp32.)  A tile is a chain of loads: a batch of eight
-// 16-byte words of K and of up to 16 rows of V is in flight together, and where CTAs of 16 queries leave half of the SMs
-// idle they take 8 (that case 24.6 -> 20.5 us, 8 heads x 128, 100 queries, 1000 keys 84 -> 56).
+// it was: 139 us for 6 heads x 32, 2 x 77 queries, 462 keys in fp32.)  A tile is a chain of loads: a batch of up to
+// eight 16-byte words of K and of up to 16 rows of V is in flight together, and where CTAs of 16 queries leave half of the SMs
+// idle they take 8 (that case 24.6 -> 20.5 us, 8 heads x 128, 100 queries, 1000 keys 84 -> 56).  Where such batches leave one
+// CTA to an SM they are smaller: us with large ones and as they are, 4 heads x 32 in fp32, 8 x 336 queries behind 32 frames 977
+// -> 890, 8 x 77 queries 129 -> 99; in bf16 16 heads x 64, 4 x 336 queries behind 16 frames 1714 -> 1295.
 // ---------------------------------------------------------------------------
 template <typename TS, int DH, int NQ>
 __global__ void __launch_bounds__(256) k_attn_rows(const StepParams *sp, Dims D, int layer, const TS *q, const TS *kc,
                                                    const TS *vc, TS *out) {
     constexpr int R = DH / 32, PS = NQ + 4, NV = WVec<TS>::N;
-    constexpr int UK = DH / NV < 8 ? DH / NV : 8, UV = R == 1 ? 16 : (R == 2 ? 8 : 4);     // loads in flight together: of K, rows of V
+    // Loads in flight together: words of K, rows of V.  Few where more of them would take the registers of the SM's second CTA
+    // (128 a thread: 16 queries, head dimension 32, and 64 in bf16, whose words of K are 8 elements).
+    constexpr bool FEW = NQ == 16 && (R == 1 || (R == 2 && NV == 8));
+    constexpr int UK = FEW ? 2 : (DH / NV < 8 ? DH / NV : 8), UV = FEW ? 4 : (R == 1 ? 16 : (R == 2 ? 8 : 4));
     __shared__ __align__(16) float s_q[NQ][DH];
     __shared__ __align__(16) float s_p[8][32 * PS];              // P of a tile: [key][query]; later O of a column slice
     __shared__ float s_m[8][NQ], s_l[8][NQ];

@@ -1,0 +1,53 @@
+"""Which kernel a call runs, and whether it fills the SMs as its rule of dispatch says (launch records of the profiler)."""
+import json
+
+import pytest
+
+from paper_2506_01380_b200 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+
+def _launches(call, tmp_path):
+    """[(kernel name, registers per thread, CTAs, threads)] of the launches that `call` makes."""
+    import torch
+    call()
+    torch.cuda.synchronize()
+    with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CPU, torch.profiler.ProfilerActivity.CUDA]) as p:
+        call()
+        torch.cuda.synchronize()
+    p.export_chrome_trace(str(tmp_path / "t.json"))
+    events = [e for e in json.load(open(tmp_path / "t.json"))["traceEvents"] if e.get("cat") == "kernel"]
+    if not events:
+        pytest.skip("the profiler gives no launch records here")
+    return [(e["name"], e["args"]["registers per thread"], e["args"]["grid"][0] * e["args"]["grid"][1] * e["args"]["grid"][2],
+             e["args"]["block"][0]) for e in sorted(events, key=lambda e: e["ts"])]
+
+
+def _pages(dtype, heads, dh, T, n_q, n_kv):
+    import torch
+    tdt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    zeros = lambda *s: torch.zeros(*s, device="cuda", dtype=tdt)
+    return zeros(heads, n_q * T, dh), zeros(n_kv, heads, T, dh), zeros(n_q * T, heads * dh)
+
+
+@pytest.mark.parametrize("dtype,heads,dh", [("fp32", 4, 32), ("bf16", 12, 32), ("bf16", 16, 64)])
+def test_many_queries_on_the_fp32_pipes_leave_room_for_a_second_cta(dtype, heads, dh, tmp_path):
+    """CTAs of 16 queries, 256 threads: two to an SM, 128 registers a thread, for head dimension 32 and for 64 in bf16 (the
+    plain path of a bf16 context).  With one CTA to an SM these calls took up to a third longer."""
+    from paper_2506_01380_b200 import nfd as N
+    T, n_q = 336, 4
+    if dtype == "fp32":
+        q, k, out = _pages(dtype, heads, dh, T, n_q, 6)
+        call = lambda: N.attention_noalloc(q, k, k, n_q, 2, out)
+    else:
+        rope = dict(rope_t=16, rope_h=24, rope_w=24) if dh == 64 else dict(rope_t=8, rope_h=12, rope_w=12)
+        cfg = I.make_cfg("nfd310m", n_layers=1, d_model=heads * dh, n_heads=heads, head_dim=dh, d_mlp=256, ctx_frames=2, **rope)
+        g = N.NFD(cfg, I.make_weights(cfg, 0))
+        g.set_option("fast", 0)
+        q, k, out = _pages(dtype, heads, dh, T, n_q, 6)
+        rows = k.permute(1, 0, 2, 3).reshape(heads, 6 * T, dh).contiguous()
+        call = lambda: g.attention(q, rows, rows, n_q, 6, 2, out=out)
+    run = [x for x in _launches(call, tmp_path) if "k_attn_rows" in x[0]]
+    assert len(run) == 1 and f"{dh}, 16>" in run[0][0] and run[0][2] == heads * n_q * T // 16 and run[0][3] == 256
+    assert run[0][1] <= 128, run
