@@ -1354,7 +1354,7 @@ static int noalloc_launch(cudaStream_t st, int n_sm, const StepParams *d_sp, con
     return NFD_OK;
 }
 
-// The tensor-core kernel on the caller's pages.
+// The tensor-core kernels on the caller's pages.
 // Returns false where it does not handle the case.
 static bool noalloc_launch_tc(int dev, int n_sm, cudaStream_t st, const StepParams *d_sp, int *d_stat, const Dims &D, int n_q,
                               const void *q, const void *k_pages, const void *v_pages, void *out) {
@@ -1371,8 +1371,11 @@ static bool noalloc_launch_tc(int dev, int n_sm, cudaStream_t st, const StepPara
     pl.SP = D.H * pl.QT;
     attn_own_plan(pl, n_q * pl.SP, (D.W < D.R ? D.W + 1 : D.R) * pl.BPF, n_sm);
     if (!attn_divisors(pl, n_q, D.W, n_sm)) return false;
+    if (pl.MAXSPLIT == 1)
+        return launch_attn_plan(false, 0, enc[dev], n_sm, st, d_sp, D, n_q, 0, pl, (size_t)D.R * D.H, (const bf16 *)q,
+                                (const bf16 *)k_pages, (const bf16 *)v_pages, (bf16 *)out, nullptr, nullptr, d_stat) != 0;
     auto go = [&](auto kb) {
-        return launch_attn_own<decltype(kb)::value>(enc[dev], n_sm, st, d_sp, n_q, D, pl, (size_t)D.R * D.H, (const bf16 *)q,
+        return launch_attn_own<decltype(kb)::value>(enc[dev], st, d_sp, n_q, D, pl, (size_t)D.R * D.H, (const bf16 *)q,
                                                     (const bf16 *)k_pages, (const bf16 *)v_pages, (bf16 *)out, d_stat);
     };
     switch (pl.KB) {

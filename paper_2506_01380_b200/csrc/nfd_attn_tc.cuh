@@ -796,16 +796,16 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
 }
 
 // The caller's pages (nfd_attention_noalloc), for which there is no memory for states: the pieces of a split key range are the
-// CTAs of a cluster.  Each leaves its state in its own shared memory, and after a cluster barrier they merge them through
-// distributed shared memory, in split order, each CTA some quarters of the columns.  Without a split the grid is persistent,
-// as in k_attn_tc.
+// CTAs of a cluster, an item each.  Each leaves its state in its own shared memory, and after a cluster barrier they merge them
+// through distributed shared memory, in split order, each CTA some quarters of the columns.  Without a split k_attn_tc takes the
+// call (run as clusters of one here: 4 heads x 32, 8 x 336 queries behind 32 frames 72.6 -> 74.5 us, 16 x 64 200.0 -> 202.5).
 // Measured, 16 heads x 64, 336 queries behind 16 frames of 336 (48 query tiles), us with both launches of the call: one CTA to a
 // tile 43.1, two 30.8.  (Three would want 48 clusters, and the machine holds 45.)
 template <int KB>
 __global__ void __launch_bounds__(AttnCfg<KB>::THREADS, 1)
 k_attn_own(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
            const __grid_constant__ CUtensorMap tmV, const StepParams *sp, const __grid_constant__ Dims D,
-           const __grid_constant__ AttnPlan pl, int n_items, bf16 *out, int *status) {
+           const __grid_constant__ AttnPlan pl, bf16 *out, int *status) {
     using A = AttnCfg<KB>;
     extern __shared__ uint8_t smem_raw[];
     AttnShared<KB> sh(smem_raw);
@@ -813,49 +813,44 @@ k_attn_own(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     AttnItem w0;
     w0.set(blockIdx.x, sp, D, pl);
     attn_set_up<KB>(sh, tmQ, tmK, tmV);
-    // (with a split a CTA has one item)
-    const int end = pl.MAXSPLIT > 1 ? (int)blockIdx.x + 1 : n_items;
+    const int end = blockIdx.x + 1;
     attn_items<KB, true>(sh, tmQ, tmK, tmV, sp, D, 0, pl, w0, blockIdx.x, end, RD_FIRST, 0, out, state, status, 0);
     tc_fence_before();
     __syncthreads();
     if (sh.redo[0] & ATTN_MARKED) attn_again<KB, true>(sh, tmQ, tmK, tmV, sp, D, 0, pl, end, out, state, status);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (pl.MAXSPLIT > 1) {
-        __syncwarp();
-        cluster_sync_all();                                // every state of the cluster is in place
-        w0.set(blockIdx.x, sp, D, pl);
-        const int cq = warp >> 2, trow = (warp & 3) * 32 + lane;
-        if (w0.nsplit > 1 && w0.split < w0.nsplit && cq % w0.nsplit == w0.split && 16 * cq < D.dh) {
-            const uint32_t st = smem_u32(state);
-            float O[16], lt = 0.f, mx = -INFINITY;
+    __syncwarp();
+    cluster_sync_all();                                    // every state of the cluster is in place
+    w0.set(blockIdx.x, sp, D, pl);
+    const int cq = warp >> 2, trow = (warp & 3) * 32 + lane;
+    if (w0.nsplit > 1 && w0.split < w0.nsplit && cq % w0.nsplit == w0.split && 16 * cq < D.dh) {
+        const uint32_t st = smem_u32(state);
+        float O[16], lt = 0.f, mx = -INFINITY;
 #pragma unroll
-            for (int e = 0; e < 16; ++e) O[e] = 0.f;
+        for (int e = 0; e < 16; ++e) O[e] = 0.f;
 #pragma unroll 1
-            for (int s = 0; s < w0.nsplit; ++s) {
-                const float2 ml = ld_cluster_f2(cluster_map(st + attn_ml_at(cq >> 1, trow), s));
-                float4 v[4];
+        for (int s = 0; s < w0.nsplit; ++s) {
+            const float2 ml = ld_cluster_f2(cluster_map(st + attn_ml_at(cq >> 1, trow), s));
+            float4 v[4];
 #pragma unroll
-                for (int e = 0; e < 4; ++e) v[e] = ld_cluster_f4(cluster_map(st + attn_o_at(4 * cq + e, trow), s));
-                const float mb = fmaxf(mx, ml.x);
-                // (a state with nothing but scores of -inf has m = -inf and counts for nothing)
-                const float fo = mx == mb ? 1.0f : ex2_approx(mx - mb), wgt = ml.x == -INFINITY ? 0.f : ex2_approx(ml.x - mb);
-                mx = mb, lt = fmaf(ml.y, wgt, __fmul_rn(lt, fo));
+            for (int e = 0; e < 4; ++e) v[e] = ld_cluster_f4(cluster_map(st + attn_o_at(4 * cq + e, trow), s));
+            const float mb = fmaxf(mx, ml.x);
+            // (a state with nothing but scores of -inf has m = -inf and counts for nothing)
+            const float fo = mx == mb ? 1.0f : ex2_approx(mx - mb), wgt = ml.x == -INFINITY ? 0.f : ex2_approx(ml.x - mb);
+            mx = mb, lt = fmaf(ml.y, wgt, __fmul_rn(lt, fo));
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    O[4 * e] = fmaf(v[e].x, wgt, __fmul_rn(O[4 * e], fo));
-                    O[4 * e + 1] = fmaf(v[e].y, wgt, __fmul_rn(O[4 * e + 1], fo));
-                    O[4 * e + 2] = fmaf(v[e].z, wgt, __fmul_rn(O[4 * e + 2], fo));
-                    O[4 * e + 3] = fmaf(v[e].w, wgt, __fmul_rn(O[4 * e + 3], fo));
-                }
+            for (int e = 0; e < 4; ++e) {
+                O[4 * e] = fmaf(v[e].x, wgt, __fmul_rn(O[4 * e], fo));
+                O[4 * e + 1] = fmaf(v[e].y, wgt, __fmul_rn(O[4 * e + 1], fo));
+                O[4 * e + 2] = fmaf(v[e].z, wgt, __fmul_rn(O[4 * e + 2], fo));
+                O[4 * e + 3] = fmaf(v[e].w, wgt, __fmul_rn(O[4 * e + 3], fo));
             }
-            attn_write<16>(w0, w0.qt * 128 + trow, 16 * cq, O, lt, D, out);
         }
-        __syncwarp();
-        // No CTA leaves while a peer may still read its state.  (With release: lanes of rows beyond the frame's have nothing that
-        // waits for what they read, and their loads must be over too.)
-        cluster_sync_all();
-    } else {
-        __syncthreads();
+        attn_write<16>(w0, w0.qt * 128 + trow, 16 * cq, O, lt, D, out);
     }
+    __syncwarp();
+    // No CTA leaves while a peer may still read its state.  (With release: lanes of rows beyond the frame's have nothing that
+    // waits for what they read, and their loads must be over too.)
+    cluster_sync_all();
     if (warp == 1) tmem_dealloc(sh.tmem, A::TMEM_COLS);
 }

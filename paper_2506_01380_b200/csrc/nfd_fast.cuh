@@ -469,9 +469,9 @@ static int launch_attn_tc(bool early, int test_skip, PFN_encodeTiled encode, int
     return 1;
 }
 
-// The caller's pages: see k_attn_own.
+// Split key ranges of the caller's pages: see k_attn_own.
 template <int KB>
-static bool launch_attn_own(PFN_encodeTiled encode, int n_sm, cudaStream_t st, const StepParams *sp, int nf, const Dims &D, const AttnPlan &pl,
+static bool launch_attn_own(PFN_encodeTiled encode, cudaStream_t st, const StepParams *sp, int nf, const Dims &D, const AttnPlan &pl,
                             size_t pages, const bf16 *q, const bf16 *kc, const bf16 *vc, bf16 *out, int *status) {
     using A = AttnCfg<KB>;
     auto kern = k_attn_own<KB>;
@@ -481,9 +481,8 @@ static bool launch_attn_own(PFN_encodeTiled encode, int n_sm, cudaStream_t st, c
     if (!encode_map_3d(encode, &mq, q, D.H, nf * D.T, D.dh, 128) || !encode_map_3d(encode, &mk, kc, pages, D.T, D.dh, KB) ||
         !encode_map_3d(encode, &mv, vc, pages, D.T, D.dh, KB))
         return false;
-    const int n_items = nf * pl.SP * pl.MAXSPLIT;
-    const dim3 grid(pl.MAXSPLIT > 1 || n_items < n_sm ? n_items : n_sm);
-    const cudaError_t e = launch_kernel(false, kern, grid, dim3(A::THREADS), (size_t)smem, st, pl.MAXSPLIT, mq, mk, mv, sp, D, pl, n_items, out, status);
+    const cudaError_t e = launch_kernel(false, kern, dim3(nf * pl.SP * pl.MAXSPLIT), dim3(A::THREADS), (size_t)smem, st, pl.MAXSPLIT, mq, mk,
+                                        mv, sp, D, pl, out, status);
     if (e != cudaSuccess) {
         fprintf(stderr, "libnfd: tensor-core attention launch failed: %s\n", cudaGetErrorString(e));
         cudaGetLastError();

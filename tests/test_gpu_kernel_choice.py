@@ -51,3 +51,14 @@ def test_many_queries_on_the_fp32_pipes_leave_room_for_a_second_cta(dtype, heads
     run = [x for x in _launches(call, tmp_path) if "k_attn_rows" in x[0]]
     assert len(run) == 1 and f"{dh}, 16>" in run[0][0] and run[0][2] == heads * n_q * T // 16 and run[0][3] == 256
     assert run[0][1] <= 128, run
+
+
+@pytest.mark.parametrize("heads,dh,T,n_q,n_kv,window,kernel", [
+    (16, 64, 336, 1, 17, 16, "k_attn_own"),       # 48 query tiles, 51 blocks: two pieces
+    (16, 64, 336, 4, 12, 8, "k_attn_tc"),         # 192 query tiles: whole
+    (4, 32, 77, 1, 5, 4, "k_attn_tc")])           # five blocks: a merge would take longer
+def test_split_windows_of_the_caller_as_clusters_whole_ones_on_the_persistent_kernel(heads, dh, T, n_q, n_kv, window, kernel, tmp_path):
+    from paper_2506_01380_b200 import nfd as N
+    q, k, out = _pages("bf16", heads, dh, T, n_q, n_kv)
+    run = _launches(lambda: N.attention_noalloc(q, k, k, n_q, window, out), tmp_path)
+    assert len(run) == 2 and "k_set_params" in run[0][0] and kernel + "<" in run[1][0], run
