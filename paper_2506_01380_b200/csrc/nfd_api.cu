@@ -1339,10 +1339,9 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[NFD_NOALLOC_SCR
 #define NFD_NOALLOC_STATUS_OFFSET 3072       // four status ints behind the descriptor
 static_assert(sizeof(StepParams) <= NFD_NOALLOC_STATUS_OFFSET, "pass descriptor must fit the static scratch");
 
-#define NFD_NOALLOC_MAX_DEVICES 64
 // Device address of g_noalloc_scratch per device ordinal.  In host code the
 // symbol itself is only a stand-in, so its address is looked up once per device.
-static void *g_noalloc_dev_ptr[NFD_NOALLOC_MAX_DEVICES] = {nullptr};
+static void *g_noalloc_dev_ptr[NFD_MAX_DEVICES] = {nullptr};
 
 template <typename TS>
 static int noalloc_launch(cudaStream_t st, int n_sm, const StepParams *d_sp, const Dims &D, int n_q, const void *q,
@@ -1358,7 +1357,7 @@ static int noalloc_launch(cudaStream_t st, int n_sm, const StepParams *d_sp, con
 // Returns false where it does not handle the case.
 static bool noalloc_launch_tc(int dev, int n_sm, cudaStream_t st, const StepParams *d_sp, int *d_stat, const Dims &D, int n_q,
                               const void *q, const void *k_pages, const void *v_pages, void *out) {
-    static PFN_encodeTiled enc[NFD_NOALLOC_MAX_DEVICES];
+    static PFN_encodeTiled enc[NFD_MAX_DEVICES];
     if (D.dh != 64 && D.dh != 32) return false;
     if (!enc[dev]) {
         // looked up once per device, like the array's address
@@ -1369,14 +1368,16 @@ static bool noalloc_launch_tc(int dev, int n_sm, cudaStream_t st, const StepPara
     AttnPlan pl;
     attn_blocks(pl, D.T);
     pl.SP = D.H * pl.QT;
-    attn_own_plan(pl, n_q * pl.SP, (D.W < D.R ? D.W + 1 : D.R) * pl.BPF, n_sm);
-    if (!attn_divisors(pl, n_q, D.W, n_sm)) return false;
-    if (pl.MAXSPLIT == 1)
-        return launch_attn_plan(false, 0, enc[dev], n_sm, st, d_sp, D, n_q, 0, pl, (size_t)D.R * D.H, (const bf16 *)q,
-                                (const bf16 *)k_pages, (const bf16 *)v_pages, (bf16 *)out, nullptr, nullptr, d_stat) != 0;
+    const int n_blocks = (D.W < D.R ? D.W + 1 : D.R) * pl.BPF;
     auto go = [&](auto kb) {
-        return launch_attn_own<decltype(kb)::value>(enc[dev], st, d_sp, n_q, D, pl, (size_t)D.R * D.H, (const bf16 *)q,
-                                                    (const bf16 *)k_pages, (const bf16 *)v_pages, (bf16 *)out, d_stat);
+        constexpr int KB = decltype(kb)::value;
+        attn_own_plan(pl, n_q * pl.SP, n_blocks, [&](int k) { return attn_own_clusters<KB>(dev, k); });
+        if (!attn_divisors(pl, n_q, D.W, n_sm)) return false;
+        if (pl.MAXSPLIT == 1)
+            return launch_attn_plan(false, 0, enc[dev], n_sm, st, d_sp, D, n_q, 0, pl, (size_t)D.R * D.H, (const bf16 *)q,
+                                    (const bf16 *)k_pages, (const bf16 *)v_pages, (bf16 *)out, nullptr, nullptr, d_stat) != 0;
+        return launch_attn_own<KB>(enc[dev], st, d_sp, n_q, D, pl, (size_t)D.R * D.H, (const bf16 *)q, (const bf16 *)k_pages,
+                                   (const bf16 *)v_pages, (bf16 *)out, d_stat);
     };
     switch (pl.KB) {
         case 128: return go(std::integral_constant<int, 128>());
@@ -1408,8 +1409,8 @@ extern "C" int nfd_attention_noalloc(const void *q, const void *k_pages, const v
     cudaStream_t st = (cudaStream_t)cuda_stream;
     int dev = -1;
     CK(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= NFD_NOALLOC_MAX_DEVICES) return NFD_E_RANGE;
-    static int n_sms[NFD_NOALLOC_MAX_DEVICES];
+    if (dev < 0 || dev >= NFD_MAX_DEVICES) return NFD_E_RANGE;
+    static int n_sms[NFD_MAX_DEVICES];
     if (!g_noalloc_dev_ptr[dev]) {
         // one-time set-up for the current device: turn the symbol into a device address
         void *p = nullptr;

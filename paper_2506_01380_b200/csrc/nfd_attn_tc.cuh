@@ -66,21 +66,8 @@
 #pragma once
 #include "nfd_sm100.cuh"
 
-struct AttnPlan {
-    int KB = 0;          // keys per block
-    int BPF = 0;         // blocks per frame page
-    int QT = 0;          // 128-row query tiles per frame
-    int CH = 0;          // key blocks per split
-    int MAXSPLIT = 0;    // splits of the longest window
-    int WH = 0;          // (head, query tile) pairs of a frame whose key range is not split: the first ones
-    int SP = 0;          // those whose key range is
-    int whole = 0;       // of a launch: items that are not split (frames x WH); they come first
-    FastDiv split_div, qt_div, wh_div, sp_div, ch_div, bpf_div;      // by MAXSPLIT, QT, WH, SP, CH, BPF
-};
-
 // A published state: [16 groups of 4 columns][128 rows] float4, then [2 halves of O][128 rows] (m, l).
 #define ATTN_STATE_BYTES (128 * 64 * 4 + 2 * 128 * 8)
-#define ATTN_CTA_ITEMS 2048      // items of a CTA, at most: each has a byte of shared memory (see attn_finish)
 // Flags that are read when all roles are through: an item is marked, a wait has run out.  (In registers, with a vote at the
 // end, they cost two frames 39.6 -> 41.5 us.)
 #define ATTN_MARKED 1u

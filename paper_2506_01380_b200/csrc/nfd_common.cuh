@@ -5,6 +5,7 @@
 #include <float.h>
 #include <stdint.h>
 #include "nfd.h"
+#include "nfd_attn_plan.h"
 
 typedef __nv_bfloat16 bf16;
 
@@ -19,14 +20,6 @@ struct FrameDesc {
     int src_index;   // frame slot inside that input set
     int out_index;   // frame slot of v_out this frame's velocity goes to, or -1 (no output wanted)
     int win_slot;    // ring slot of win_first (win_first % R)
-};
-
-// Division by a number that is fixed at launch, as a multiplication: exact for n < 2^32 / d.  An integer division
-// costs over a hundred clocks and takes the special-function unit.
-struct FastDiv {
-    unsigned int d = 1, m = 0;       // m = ceil(2^32 / d); d = 1: m = 0
-    void set(unsigned int v) { d = v, m = v > 1 ? (unsigned int)((0x100000000ull + v - 1) / v) : 0; }
-    __device__ __forceinline__ int div(int n) const { return m ? (int)__umulhi((unsigned int)n, m) : n; }
 };
 
 // One (FM time, action) pair whose modulation this pass has to compute: the pairs

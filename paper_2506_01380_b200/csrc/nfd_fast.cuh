@@ -3,6 +3,7 @@
 // nfd_api.cu.  fast_gemm / fast_attention return false when they do not handle
 // a case; the caller then launches the plain kernels.
 #pragma once
+#include <atomic>
 #include <map>
 #include <tuple>
 #include <utility>
@@ -11,6 +12,8 @@
 #include "nfd_gemm_tc.cuh"
 #include "nfd_gemm_p.cuh"
 #include "nfd_attn_tc.cuh"
+
+#define NFD_MAX_DEVICES 64       // devices of a process that the allocation-free call knows
 
 typedef CUresult (*PFN_encodeTiled)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
                                     const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
@@ -29,82 +32,6 @@ struct FastState {
     std::map<std::tuple<const void *, int, int, int>, CUtensorMap> maps;   // (ptr, rows, cols, box_rows)
 };
 
-// Key block, blocks per page and query tiles for pages of T tokens: the block that walks a page in the least time, a
-// block costing its columns (padded ones included) plus a fixed part of about 24 columns (barriers and hand-overs).
-static void attn_blocks(AttnPlan &pl, int T) {
-    const int kbs[4] = {128, 112, 96, 64};
-    for (int kb : kbs) {
-        const int bpf = (T + kb - 1) / kb;
-        if (!pl.KB || bpf * (kb + 24) < pl.BPF * (pl.KB + 24)) pl.KB = kb, pl.BPF = bpf;
-    }
-    pl.QT = (T + 127) / 128;
-}
-// The plan's divisors; false where a dividend is too large for them (n * d has to stay below 2^32) or a CTA would get more
-// items than it keeps account of.
-static bool attn_divisors(AttnPlan &pl, int n_frames, int W, int n_sm) {
-    pl.split_div.set(pl.MAXSPLIT), pl.qt_div.set(pl.QT), pl.ch_div.set(pl.CH), pl.bpf_div.set(pl.BPF);
-    pl.wh_div.set(pl.WH > 0 ? pl.WH : 1), pl.sp_div.set(pl.SP > 0 ? pl.SP : 1);
-    const long long nb = ((long long)W + 1) * pl.BPF + pl.CH, big = 0x100000000ll;
-    const long long n_items = n_frames * (pl.WH + (long long)pl.SP * pl.MAXSPLIT);
-    const int tiles = pl.WH + pl.SP, d_item = tiles > pl.MAXSPLIT ? tiles : pl.MAXSPLIT;
-    return n_items <= (long long)ATTN_CTA_ITEMS * n_sm && n_items * d_item < big && nb < 0x7fffffffll && nb * (pl.CH > pl.BPF ? pl.CH : pl.BPF) < big;
-}
-// Pieces of the key range of a call on the caller's pages: as many as pay (as in attn_split_plan; the merge is through
-// distributed shared memory) and as clusters of that size fit the machine at once.  On a 148-SM B200 clusters of 1, 2, 3, 4, 5,
-// 6, 8 hold 148, 148, 135, 132, 130, 132, 120 CTAs (cudaOccupancyMaxActiveClusters); from 3 on four clusters less than the SMs
-// would make is within that.
-static void attn_own_plan(AttnPlan &pl, int tiles, int n_blocks, int n_sm) {
-    float best = 1e30f;
-    int best_k = 1;
-    for (int k = 1; k <= 8 && k <= n_blocks; ++k) {
-        const int clusters = k <= 2 ? n_sm / k : n_sm / k - 4, ch = (n_blocks + k - 1) / k;
-        if (k > 1 && (tiles > clusters || (n_blocks + ch - 1) / ch != k)) continue;
-        const float t = ch * 0.65f * (pl.KB + 24) / 136.f + (k > 1 ? 1.5f + 0.2f * k : 0.f);
-        if (t < best) best = t, best_k = k;
-    }
-    pl.CH = (n_blocks + best_k - 1) / best_k, pl.MAXSPLIT = best_k;
-}
-// How the key ranges of a frame's `tiles` (head, query tile) pairs are split.  By the configuration alone (the longest
-// window, as many frames as there are streams), never by the pass: the order of the sums must not depend on it.
-//   One stream: all of them, into at most as many pieces as fill the SMs once, and no more than pay: a block takes about 0.65
-// us (of 112 keys; its columns and 24 count), publishing and counting 2.5, the merge 0.25 per piece.  (A frame of a model of 2 layers,
-// 4 heads, 64 tokens: behind four frames five pieces of a block 286 us, one of five 270; behind 30 frames 31 pieces 443, six 300.)
-//   Several: the items are dealt out to the CTAs in order, and whole windows leave a last round in which most SMs idle (16 heads
-// x 3 query tiles x 8 streams = 384 items on 148 SMs: two rounds and six tenths of one, at the price of three).  Splitting all
-// of them finely costs a state of 33 KB each; so the first WH are left whole and the others split, for the least blocks on the
-// busiest CTA, a whole item counted a block more than it has and a piece two and a half (start, publication, merge).
-static void attn_split_plan(AttnPlan &pl, int tiles, int n_streams, int n_blocks, int n_sm) {
-    auto pieces = [&](int k) { pl.CH = (n_blocks + k - 1) / k, pl.MAXSPLIT = (n_blocks + pl.CH - 1) / pl.CH; };
-    pl.WH = 0, pl.SP = tiles;
-    const int items = n_streams * tiles;
-    float best = 1e30f;
-    int best_k = 1, best_wh = tiles;
-    if (n_streams == 1) {
-        for (int k = 1; k <= n_blocks && (k == 1 || k * items <= n_sm); ++k) {
-            pieces(k);
-            const float t = pl.CH * 0.65f * (pl.KB + 24) / 136.f + (k > 1 ? 2.5f + 0.25f * k : 0.f);
-            if (t < best) best = t, best_k = k;
-        }
-        return pieces(best_k);
-    }
-    for (int k = 1; k <= 8 && k <= n_blocks; ++k) {
-        pieces(k);
-        for (int wh = k == 1 ? tiles : 0; wh <= (k == 1 ? tiles : tiles - 1); ++wh) {
-            const int nw = n_streams * wh, n = nw + n_streams * (tiles - wh) * pl.MAXSPLIT, grid = n < n_sm ? n : n_sm;
-            // the CTAs before, between and behind those with a whole item and with an item more than others
-            float most = 0.f;
-            const int at[3] = {0, nw % grid, n % grid};
-            for (int c : at) {
-                const int w = nw / grid + (c < nw % grid), all = n / grid + (c < n % grid);
-                const float t = w * (n_blocks + 1.f) + (all - w) * (pl.CH + 2.5f);
-                if (t > most) most = t;
-            }
-            if (most < best) best = most, best_k = k, best_wh = wh;
-        }
-    }
-    pieces(best_k);
-    pl.WH = best_wh, pl.SP = tiles - best_wh;
-}
 static PFN_encodeTiled get_encode_fn() {
     void *fn = nullptr;
     cudaDriverEntryPointQueryResult qres;
@@ -469,6 +396,26 @@ static int launch_attn_tc(bool early, int test_skip, PFN_encodeTiled encode, int
     return 1;
 }
 
+// Clusters of k CTAs of k_attn_own that device `dev`, the current one, holds at once (0: it runs none).  Asked for once.
+template <int KB> static int attn_own_clusters(int dev, int k) {
+    static std::atomic<int> known[NFD_MAX_DEVICES][9];                     // and one
+    int n = known[dev][k].load(std::memory_order_relaxed);
+    if (n) return n - 1;
+    using A = AttnCfg<KB>;
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3(k), cfg.blockDim = dim3(A::THREADS), cfg.dynamicSmemBytes = A::OWN_SMEM;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)k, attr.val.clusterDim.y = 1, attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr, cfg.numAttrs = 1;
+    if (!allow_smem(k_attn_own<KB>, A::OWN_SMEM) || cudaOccupancyMaxActiveClusters(&n, k_attn_own<KB>, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        n = 0;
+    }
+    known[dev][k].store(n + 1, std::memory_order_relaxed);
+    return n;
+}
 // Split key ranges of the caller's pages: see k_attn_own.
 template <int KB>
 static bool launch_attn_own(PFN_encodeTiled encode, cudaStream_t st, const StepParams *sp, int nf, const Dims &D, const AttnPlan &pl,
