@@ -317,6 +317,8 @@ int nfd_warm_modulation(nfd_ctx *ctx);
  * nfd_attention all of K), so that
  * the consumer's wait for it expires (NFD_E_TIMEOUT); "test_wait_limit_us" n:
  * bounded waits give up after n microseconds instead of 0.4 s (0 = default).
+ * "test_noalloc" n, for the calling thread's next nfd_attention_noalloc: 1 K does
+ * not come, and every wait behind it expires; 2 the launch as clusters is refused.
  * Returns NFD_E_RANGE for unknown names. */
 int nfd_set_option(nfd_ctx *ctx, const char *name, int value);
 

@@ -621,6 +621,9 @@ static int build_pass(nfd_ctx *c, int n, const int *streams, int k, int offset, 
 // ---------------------------------------------------------------------------
 // C ABI
 // ---------------------------------------------------------------------------
+// Test switch "test_noalloc" of nfd_set_option, for this thread's next nfd_attention_noalloc: NFD_TEST_SKIP, NFD_TEST_REFUSE.
+static thread_local int t_noalloc_test = 0;
+
 extern "C" {
 
 const char *nfd_strerror(int code) {
@@ -1293,6 +1296,10 @@ int nfd_set_option(nfd_ctx *c, const char *name, int value) {
         c->test_fail_launch = value != 0;
         return NFD_OK;
     }
+    if (!strcmp(name, "test_noalloc")) {
+        t_noalloc_test = value;
+        return NFD_OK;
+    }
     if (!strcmp(name, "test_corrupt_desc")) {
         c->test_corrupt_desc = value != 0;
         return NFD_OK;
@@ -1355,7 +1362,7 @@ static int noalloc_launch(cudaStream_t st, int n_sm, const StepParams *d_sp, con
 
 // The tensor-core kernels on the caller's pages.
 // Returns false where it does not handle the case.
-static bool noalloc_launch_tc(int dev, int n_sm, cudaStream_t st, const StepParams *d_sp, int *d_stat, const Dims &D, int n_q,
+static bool noalloc_launch_tc(int test, int dev, int n_sm, cudaStream_t st, const StepParams *d_sp, int *d_stat, const Dims &D, int n_q,
                               const void *q, const void *k_pages, const void *v_pages, void *out) {
     static PFN_encodeTiled enc[NFD_MAX_DEVICES];
     if (D.dh != 64 && D.dh != 32) return false;
@@ -1372,12 +1379,17 @@ static bool noalloc_launch_tc(int dev, int n_sm, cudaStream_t st, const StepPara
     auto go = [&](auto kb) {
         constexpr int KB = decltype(kb)::value;
         attn_own_plan(pl, n_q * pl.SP, n_blocks, [&](int k) { return attn_own_clusters<KB>(dev, k); });
-        if (!attn_divisors(pl, n_q, D.W, n_sm)) return false;
-        if (pl.MAXSPLIT == 1)
-            return launch_attn_plan(false, 0, enc[dev], n_sm, st, d_sp, D, n_q, 0, pl, (size_t)D.R * D.H, (const bf16 *)q,
-                                    (const bf16 *)k_pages, (const bf16 *)v_pages, (bf16 *)out, nullptr, nullptr, d_stat) != 0;
-        return launch_attn_own<KB>(enc[dev], st, d_sp, n_q, D, pl, (size_t)D.R * D.H, (const bf16 *)q, (const bf16 *)k_pages,
-                                   (const bf16 *)v_pages, (bf16 *)out, d_stat);
+        if (pl.MAXSPLIT > 1) {
+            if (attn_divisors(pl, n_q, D.W, n_sm) &&
+                launch_attn_own<KB>(test, enc[dev], st, d_sp, n_q, D, pl, (size_t)D.R * D.H, (const bf16 *)q, (const bf16 *)k_pages,
+                                    (const bf16 *)v_pages, (bf16 *)out, d_stat))
+                return true;
+            // clusters are refused (a part of a machine): the windows stay whole
+            pl.CH = n_blocks, pl.MAXSPLIT = 1;
+        }
+        return attn_divisors(pl, n_q, D.W, n_sm) &&
+               launch_attn_plan(false, test & NFD_TEST_SKIP, enc[dev], n_sm, st, d_sp, D, n_q, 0, pl, (size_t)D.R * D.H, (const bf16 *)q,
+                                (const bf16 *)k_pages, (const bf16 *)v_pages, (bf16 *)out, nullptr, nullptr, d_stat) != 0;
     };
     switch (pl.KB) {
         case 128: return go(std::integral_constant<int, 128>());
@@ -1407,6 +1419,8 @@ extern "C" int nfd_attention_noalloc(const void *q, const void *k_pages, const v
     const long long warps_ll = rows_ll * n_heads;
     if (rows_ll > 0x7fffffffLL / 4 || (warps_ll + 3) / 4 > 0x7fffffffLL) return NFD_E_RANGE;
     cudaStream_t st = (cudaStream_t)cuda_stream;
+    const int test = t_noalloc_test;
+    t_noalloc_test = 0;
     int dev = -1;
     CK(cudaGetDevice(&dev));
     if (dev < 0 || dev >= NFD_MAX_DEVICES) return NFD_E_RANGE;
@@ -1446,7 +1460,7 @@ extern "C" int nfd_attention_noalloc(const void *q, const void *k_pages, const v
     // the descriptor is rewritten in full on every call; nothing of the previous call survives
     k_set_params<<<1, 256, 0, st>>>(p, d_sp, lim, d_stat);
     CK(cudaGetLastError());
-    if (dtype == NFD_DTYPE_BF16 && noalloc_launch_tc(dev, n_sm, st, d_sp, d_stat, D, n_q_frames, q, k_pages, v_pages, out))
+    if (dtype == NFD_DTYPE_BF16 && noalloc_launch_tc(test, dev, n_sm, st, d_sp, d_stat, D, n_q_frames, q, k_pages, v_pages, out))
         return NFD_OK;
     if (dtype == NFD_DTYPE_BF16) return noalloc_launch<bf16>(st, n_sm, d_sp, D, n_q_frames, q, k_pages, v_pages, out);
     return noalloc_launch<float>(st, n_sm, d_sp, D, n_q_frames, q, k_pages, v_pages, out);

@@ -792,7 +792,7 @@ template <int KB>
 __global__ void __launch_bounds__(AttnCfg<KB>::THREADS, 1)
 k_attn_own(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
            const __grid_constant__ CUtensorMap tmV, const StepParams *sp, const __grid_constant__ Dims D,
-           const __grid_constant__ AttnPlan pl, bf16 *out, int *status) {
+           const __grid_constant__ AttnPlan pl, bf16 *out, int *status, int test_skip) {
     using A = AttnCfg<KB>;
     extern __shared__ uint8_t smem_raw[];
     AttnShared<KB> sh(smem_raw);
@@ -801,7 +801,7 @@ k_attn_own(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     w0.set(blockIdx.x, sp, D, pl);
     attn_set_up<KB>(sh, tmQ, tmK, tmV);
     const int end = blockIdx.x + 1;
-    attn_items<KB, true>(sh, tmQ, tmK, tmV, sp, D, 0, pl, w0, blockIdx.x, end, RD_FIRST, 0, out, state, status, 0);
+    attn_items<KB, true>(sh, tmQ, tmK, tmV, sp, D, 0, pl, w0, blockIdx.x, end, RD_FIRST, 0, out, state, status, test_skip);
     tc_fence_before();
     __syncthreads();
     if (sh.redo[0] & ATTN_MARKED) attn_again<KB, true>(sh, tmQ, tmK, tmV, sp, D, 0, pl, end, out, state, status);

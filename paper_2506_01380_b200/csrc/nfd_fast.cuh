@@ -416,9 +416,11 @@ template <int KB> static int attn_own_clusters(int dev, int k) {
     known[dev][k].store(n + 1, std::memory_order_relaxed);
     return n;
 }
+// Test switches of the allocation-free call: K does not come, the launch of clusters is refused.
+enum { NFD_TEST_SKIP = 1, NFD_TEST_REFUSE = 2 };
 // Split key ranges of the caller's pages: see k_attn_own.
 template <int KB>
-static bool launch_attn_own(PFN_encodeTiled encode, cudaStream_t st, const StepParams *sp, int nf, const Dims &D, const AttnPlan &pl,
+static bool launch_attn_own(int test, PFN_encodeTiled encode, cudaStream_t st, const StepParams *sp, int nf, const Dims &D, const AttnPlan &pl,
                             size_t pages, const bf16 *q, const bf16 *kc, const bf16 *vc, bf16 *out, int *status) {
     using A = AttnCfg<KB>;
     auto kern = k_attn_own<KB>;
@@ -428,14 +430,11 @@ static bool launch_attn_own(PFN_encodeTiled encode, cudaStream_t st, const StepP
     if (!encode_map_3d(encode, &mq, q, D.H, nf * D.T, D.dh, 128) || !encode_map_3d(encode, &mk, kc, pages, D.T, D.dh, KB) ||
         !encode_map_3d(encode, &mv, vc, pages, D.T, D.dh, KB))
         return false;
-    const cudaError_t e = launch_kernel(false, kern, dim3(nf * pl.SP * pl.MAXSPLIT), dim3(A::THREADS), (size_t)smem, st, pl.MAXSPLIT, mq, mk,
-                                        mv, sp, D, pl, out, status);
-    if (e != cudaSuccess) {
-        fprintf(stderr, "libnfd: tensor-core attention launch failed: %s\n", cudaGetErrorString(e));
-        cudaGetLastError();
-        return false;
-    }
-    return true;
+    // (test switch: a cluster size that the runtime refuses)
+    const cudaError_t e = launch_kernel(false, kern, dim3(nf * pl.SP * pl.MAXSPLIT), dim3(A::THREADS), (size_t)smem, st,
+                                        test & NFD_TEST_REFUSE ? 64 : pl.MAXSPLIT, mq, mk, mv, sp, D, pl, out, status, test & NFD_TEST_SKIP);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e == cudaSuccess;
 }
 
 // Attention of a pass by plan `pl` over `pages` (stream, layer, ring slot, head) pages of K and V.  `early`: the kernel may

@@ -133,3 +133,50 @@ def test_expired_wait_in_attention_leaves_nan(streams, n_q):
     assert g.status() == E_TIMEOUT
     _in_time(g)
     assert torch.equal(g.attention(q, k, v, n_q, 20, 16), ref) and g.status() == 0
+
+
+def _caller_pages(heads, T, n_kv, seed=5):
+    import torch
+    q, k, v = [torch.as_tensor(a).cuda().bfloat16() for a in I.make_qkv(heads, 64, T, n_kv * T, seed=seed)]
+    pages = lambda x: x.view(heads, n_kv, T, 64).permute(1, 0, 2, 3).contiguous()
+    return q, pages(k), pages(v)
+
+
+def _any_context():
+    from paper_2506_01380_b200.nfd import NFD
+    cfg = I.make_cfg("tiny_bf16")
+    return NFD(cfg, I.make_weights(cfg, 0))
+
+
+def test_refused_clusters_leave_the_windows_whole():
+    """Where the runtime refuses the launch as clusters the call stays on the tensor cores, its windows whole: the bits of a
+    call whose windows the plan leaves whole (78 query tiles), head by head, which neither the merge of two pieces nor the
+    kernel on the fp32 pipes gives."""
+    import torch
+    from paper_2506_01380_b200 import nfd as N
+    g, T, n_kv = _any_context(), 336, 17
+    q, k, v = _caller_pages(26, T, n_kv)
+    whole = N.attention_noalloc(q, k, v, 1, 16, torch.empty(T, 26 * 64, device="cuda", dtype=torch.bfloat16))
+    q, k, v = q[:16].contiguous(), k[:, :16].contiguous(), v[:, :16].contiguous()
+    call = lambda: N.attention_noalloc(q, k, v, 1, 16, torch.full((T, 16 * 64), float("nan"), device="cuda", dtype=torch.bfloat16))
+    split = call()
+    g.set_option("test_noalloc", 2)
+    refused = call()
+    assert torch.equal(refused, whole[:, :16 * 64]) and not torch.equal(refused, split)
+    assert torch.equal(call(), split)                # one call only
+
+
+@pytest.mark.parametrize("heads,T", [(16, 336), (1, 336), (3, 100), (26, 336)])    # 2, 8 and 6 pieces, whole windows
+def test_expired_wait_in_the_allocation_free_call_leaves_nan(heads, T):
+    """K does not come: every wait behind it gives up (after 0.4 s), the rows are NaN, the CTAs of the clusters all leave, and
+    the next call computes as ever."""
+    import torch
+    from paper_2506_01380_b200 import nfd as N
+    g = _any_context()
+    q, k, v = _caller_pages(heads, T, 17)
+    call = lambda: N.attention_noalloc(q, k, v, 1, 16, torch.zeros(T, heads * 64, device="cuda", dtype=torch.bfloat16))
+    ref = call()
+    assert torch.isfinite(ref).all()
+    g.set_option("test_noalloc", 1)
+    assert torch.isnan(call()).all()
+    assert torch.equal(call(), ref)
