@@ -134,9 +134,10 @@ __device__ __forceinline__ void nfd_trace_flush(int kind, unsigned long long t0,
         if (at < NFD_TRACE_CAP) g_trace[at].t0 = g_trace[at].t1 = marks[i], g_trace[at].kind = i, g_trace[at].sm = (int)sm;
     }
 }
+// (of the CTA, for marks in functions that a kernel calls too)
+__shared__ unsigned long long nfd_marks_[NFD_TRACE_MARKS];
 #define NFD_TRACE_T0()                                               \
     const unsigned long long nfd_t0_ = nfd_trace_now();              \
-    __shared__ unsigned long long nfd_marks_[NFD_TRACE_MARKS];       \
     if (threadIdx.x < NFD_TRACE_MARKS) nfd_marks_[threadIdx.x] = 0
 #define NFD_TRACE_END(kind)                          \
     do {                                             \

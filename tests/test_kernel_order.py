@@ -30,3 +30,12 @@ def test_cluster_pieces_are_read_before_their_cta_may_leave():
     after = body[max(reads):]
     assert "cluster_sync_all()" in after and "cluster_arrive_relaxed" not in after
     assert re.search(r"state = reinterpret_cast<float \*>\(sh\.base \+ A::STATE_AT\)", body)
+
+
+def test_marks_of_the_timeline_may_be_taken_in_functions():
+    """The timeline's marks (builds with -DNFD_TRACE) are taken in functions that a kernel calls as well: their array belongs
+    to the file and not to the kernel that opens its record, or such a build does not compile."""
+    common = open(os.path.join(CSRC, "nfd_common.cuh")).read()
+    t0 = re.search(r"#define NFD_TRACE_T0\(\)((?:[^\n]*\\\n)*[^\n]*)", common).group(1)
+    assert "nfd_marks_" in t0 and "__shared__" not in t0
+    assert re.search(r"^__shared__ unsigned long long nfd_marks_\[", common, re.M)
