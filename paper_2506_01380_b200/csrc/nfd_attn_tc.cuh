@@ -236,7 +236,8 @@ static __device__ __forceinline__ void attn_finish(const AttnItem &w, int p0, in
 // for an item, and all merge, in split order, those for which it is the last, a warp a quarter of the columns of a quadrant's
 // rows.  Done as each item ended, the fence, the counter and the merge kept one of the softmax groups, and with it the order
 // of the products, for 3.5 us an item.  us, 310M class: four-frame speculation 14400 -> 13940, one frame (an item per CTA)
-// 5380 -> 5358, 220 tokens 4150 -> 4101.  Three states in flight and no more: with four the kernel's spilled registers
+// 5380 -> 5358, 220 tokens 4150 -> 4101.  What the merge needs of an item comes through shared memory: read from the descriptor
+// once more, behind the barrier, it cost launches of one item to a CTA 0.2 to 0.5 us.  Three states in flight and no more: with four the kernel's spilled registers
 // doubled, on the path of every item (5407, 13880, 4142).
 // The counter of the lane's item, if it has one; `all`: its pieces.
 static __device__ __forceinline__ unsigned int *attn_counter(int item, int n_items, const StepParams *sp, const Dims &D, const AttnPlan &pl,
@@ -256,8 +257,8 @@ static __device__ __forceinline__ uint32_t attn_count(unsigned int *cnt, unsigne
     }
     return __ballot_sync(0xffffffffu, last);
 }
-// i0: item of bit 0
-static __device__ __forceinline__ void attn_merge(uint32_t last, int i0, const StepParams *sp, const Dims &D, const AttnPlan &pl,
+// i0: item of bit 0; pieces: of the tile of each bit's item
+static __device__ __forceinline__ void attn_merge(uint32_t last, int i0, const uint32_t *pieces, const Dims &D, const AttnPlan &pl,
                                                   bf16 *out, const float *part_o) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int cq = warp >> 2, trow = (warp & 3) * 32 + lane;
@@ -265,7 +266,9 @@ static __device__ __forceinline__ void attn_merge(uint32_t last, int i0, const S
     AttnItem w;
 #pragma unroll 1
     for (; last; last &= last - 1) {
-        w.set(i0 + (__ffs(last) - 1) * gridDim.x, sp, D, pl);
+        const int bit = __ffs(last) - 1;
+        w.place(i0 + bit * gridDim.x, pl);
+        w.nsplit = pieces[bit];
         const uint8_t *st = reinterpret_cast<const uint8_t *>(part_o) + (size_t)w.tile * pl.MAXSPLIT * ATTN_STATE_BYTES;
         float O[16], lt = 0.f, mx = -INFINITY;
 #pragma unroll
@@ -649,6 +652,10 @@ __device__ __forceinline__ void attn_items(const AttnShared<KB> &sh, const CUten
             // CTA's last item.
             const bool fin = item >= end;
             if (fin ? g < 2 : g == gl) {
+                // (The item worked out again: kept through the loop it would cost registers that it needs.  Ahead of the waits:
+                // behind them it held back the next item's products, 0.1 us an item.)
+                asm volatile("" : "+r"(was));
+                w.place(was, pl);
                 ok = ok && mbar_wait(l_full + 8 * ip, iph, status);
                 const float *sl = s_l + ip * A::NGRP * 128 + trow;
                 float l = (sl[0] + sl[128]) + sl[256];
@@ -672,9 +679,6 @@ __device__ __forceinline__ void attn_items(const AttnShared<KB> &sh, const CUten
                         mask = (marks & 1) | ((marks >> 3) & 2);
                         if (l == 0.f) m = -INFINITY;
                     }
-                    // (worked out again: kept through the loop they would cost registers that it needs)
-                    asm volatile("" : "+r"(was));
-                    w.place(was, pl);
                     attn_finish<OWN>(w, fin ? g : 0, fin ? 1 : 2, mask, tO, fin ? 0u : o_free, trow, m, l, D, pl, out,
                                 part_o, mode == RD_FIRST && ok ? sh.redo : nullptr, it - 1);
                 }
@@ -772,9 +776,10 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
                 if (i0 != blockIdx.x) cnt = attn_counter(i0 + lane * gridDim.x, n_items, sp, D, pl, counters, all);
                 const uint32_t last = attn_count(cnt, all);
                 if (lane == 0) sh.redo[1] = last;
+                sh.redo[2 + lane] = all;                   // (the marks have been seen to)
             }
             __syncthreads();                               // what that warp has acquired is handed to the others
-            attn_merge(sh.redo[1], i0, sp, D, pl, out, part_o);
+            attn_merge(sh.redo[1], i0, sh.redo + 2, D, pl, out, part_o);
             if (i0 + 32 * gridDim.x < n_items) __syncthreads();
         }
     }
