@@ -222,30 +222,22 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
                 if (m < M && n < N) epi.load_early(m, n, side[i]);
             }
         }
+        // (Into registers, and stored when the loads that the wait holds back have been issued: with the stores here those loads
+        // went out a global latency later, 0.1 to 0.3 us of the QKV projection where its main loop is short.)
+        typename Epi::Row row_e{};
+        typename Epi::Col col_e{};
+        float4 uv_e = make_float4(0.f, 0.f, 0.f, 0.f);
+        int n_uv = 0;                                        // pairs of columns that (u, v) is fetched for
         if constexpr (Epi::kTables) {
-            // where the rows and the column chunks of this CTA's slice go
-            if (et < rows_per && m0 + r_base + et < M)
-                *reinterpret_cast<typename Epi::Row *>(tab_raw + (r_base + et) * 16) = epi.row_info(m0 + r_base + et);
-            if (et >= 128 && et < 128 + CPR && n0 + (et - 128) * 8 < N)
-                *reinterpret_cast<typename Epi::Col *>(tab_raw + 128 * 16 + (et - 128) * 32) =
-                    epi.col_info(n0 + (et - 128) * 8);
+            if (et < rows_per && m0 + r_base + et < M) row_e = epi.row_info(m0 + r_base + et);
+            if (et >= 128 && et < 128 + CPR && n0 + (et - 128) * 8 < N) col_e = epi.col_info(n0 + (et - 128) * 8);
         }
         if constexpr (Epi::kRowStats) {
             if (epi.ln.on()) {
                 // folded LayerNorm: (u, v) of the tile's columns for every frame the tile's rows belong to
                 const int m_last = (m0 + 127 < M ? m0 + 127 : M - 1);
-                const int n_fr = m_last / epi.ln.T - uv_f0 + 1;
-                // layout [frame][pair of columns within a chunk][chunk]: the lanes of a warp, which hold adjacent
-                // chunks, read adjacent 16-byte words
-                for (int idx = et; idx < n_fr * (BN / 2); idx += G::EPI_THREADS) {
-                    const int fr = idx / (BN / 2), c2 = idx - fr * (BN / 2);
-                    if (n0 + 2 * c2 < N)
-                        uvs[(fr * 4 + (c2 & 3)) * CPR + (c2 >> 2)] = epi.ln.uv_pair(uv_f0 + fr, n0 + 2 * c2);
-                }
-                if (et < rows_per) {
-                    const int m = m0 + r_base + et;
-                    rowfr[r_base + et] = (uint8_t)((m < M ? m : M - 1) / epi.ln.T - uv_f0);
-                }
+                n_uv = (m_last / epi.ln.T - uv_f0 + 1) * (BN / 2);
+                if (et < n_uv && n0 + 2 * (et % (BN / 2)) < N) uv_e = epi.ln.uv_pair(uv_f0 + et / (BN / 2), n0 + 2 * (et % (BN / 2)));
             }
         }
         pdl_wait();
@@ -272,6 +264,17 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
 #pragma unroll
                     for (int u = 0; u < 4; ++u) pv[w][u] = epi.ln.part(m, sub + 8 * u);
                 }
+                if (et < rows_per) {
+                    const int m = m0 + r_base + et;
+                    rowfr[r_base + et] = (uint8_t)((m < M ? m : M - 1) / epi.ln.T - uv_f0);
+                }
+                // layout [frame][pair of columns within a chunk][chunk]: the lanes of a warp, which hold adjacent
+                // chunks, read adjacent 16-byte words
+                for (int idx = et; idx < n_uv; idx += G::EPI_THREADS) {
+                    const int fr = idx / (BN / 2), c2 = idx - fr * (BN / 2);
+                    if (n0 + 2 * c2 < N)
+                        uvs[(fr * 4 + (c2 & 3)) * CPR + (c2 >> 2)] = idx == et ? uv_e : epi.ln.uv_pair(uv_f0 + fr, n0 + 2 * c2);
+                }
 #pragma unroll
                 for (int w = 0; w < SWEEPS; ++w) {
                     const int r = (et >> 3) + w * (G::EPI_THREADS / 8);
@@ -293,6 +296,12 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
                     if (sub == 0 && r < rows_per) rowstat[r_base + r] = epi.ln.finish(s1, s2);
                 }
             }
+        }
+        if constexpr (Epi::kTables) {
+            // where the rows and the column chunks of this CTA's slice go
+            if (et < rows_per && m0 + r_base + et < M) *reinterpret_cast<typename Epi::Row *>(tab_raw + (r_base + et) * 16) = row_e;
+            if (et >= 128 && et < 128 + CPR && n0 + (et - 128) * 8 < N)
+                *reinterpret_cast<typename Epi::Col *>(tab_raw + 128 * 16 + (et - 128) * 32) = col_e;
         }
         // partial accumulator: tensor memory -> this CTA's staging tile (the ring is free by now)
         const int quad = warp & 3;                           // TMEM lane quadrant this warp may read

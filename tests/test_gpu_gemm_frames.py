@@ -18,6 +18,7 @@ pytestmark = pytest.mark.gpu
     ((40, 22), 4, 3, 0, 3072, 12, 1),       # 220 tokens: frames end inside tiles and inside a warp's 32 rows
     ((16, 16), 8, 4, 1, 2048, 12, 1),       # 64 tokens: three frames in a tile
     ((46, 30), 4, 2, 0, 3072, 24, 1),       # 345 tokens, head dimension 32
+    ((8, 6), 4, 4, 0, 4096, 12, 1),         # 12 tokens: eleven frames in a tile, more (u, v) pairs than epilogue threads
 ])
 def test_batched_pass_equals_single_frames(hw, streams, k, act, dm, heads, fuse_ln):
     _batched_equals_single(768, hw, streams, k, act, dm, heads, fuse_ln)
