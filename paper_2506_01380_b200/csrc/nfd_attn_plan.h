@@ -31,9 +31,65 @@ struct AttnPlan {
     int MAXSPLIT = 0;    // splits of the longest window
     int WH = 0;          // (head, query tile) pairs of a frame whose key range is not split: the first ones
     int SP = 0;          // those whose key range is
-    int whole = 0;       // of a launch: items that are not split (frames x WH); they come first
+    int NB = 0;          // key blocks of the longest window (with WH)
     FastDiv split_div, qt_div, wh_div, sp_div, ch_div, bpf_div;      // by MAXSPLIT, QT, WH, SP, CH, BPF
+    // of a launch (attn_deal)
+    int grid = 0, n_items = 0;       // CTAs, items
+    int whole = 0, pieces = 0;       // items that are not split, and that are
+    int wq = 0, wr = 0;              // whole / grid, whole % grid
+    int first = 0, fq = 0, fr = 0;   // pieces that the CTAs from wr on get before all get some; that by grid - wr, and what is left
+    int rq = 0, rr = 0;              // the other pieces by grid, and what is left
+    NFD_HD bool dealt() const { return whole > 0; }
 };
+
+// An item of a launch: one of the `whole` ones, (frame, head, query tile) that are not split, and behind them the pieces,
+// (frame, head, query tile, split).  Without whole ones CTA c takes the items c, c + grid, ...  With both, a CTA takes its
+// whole ones in turn; then the pieces go first to the CTAs that have a whole item fewer than others, about as many as take the time
+// of one (a piece six blocks more than it has, where several follow one another), then to all in turn.  (Dealt on in turn behind the
+// whole ones, pieces went to CTAs that had one while others stood idle.  A context for 8 streams of 16 heads x 3 query tiles behind 32
+// frames, 4 layers, us of a pass with whole windows, with pieces in turn, as it is: two streams 470, 533, 467; three 505, 566,
+// 540; five 890, 1065, 956; six 1017, 1083, 1019; eight 1460, 1388, 1393.)
+static inline void attn_deal(AttnPlan &pl, int frames, int n_sm) {
+    pl.whole = frames * pl.WH, pl.pieces = frames * pl.SP * pl.MAXSPLIT;
+    pl.n_items = pl.whole + pl.pieces;
+    pl.grid = pl.n_items < n_sm ? pl.n_items : n_sm;
+    pl.wq = pl.whole / pl.grid, pl.wr = pl.whole % pl.grid;
+    const int behind = pl.grid - pl.wr, each = pl.whole ? (pl.NB + 1) / (pl.CH + 6) : 0;
+    pl.first = pl.pieces < each * behind ? pl.pieces : each * behind;
+    pl.fq = pl.first / behind, pl.fr = pl.first % behind;
+    pl.rq = (pl.pieces - pl.first) / pl.grid, pl.rr = (pl.pieces - pl.first) % pl.grid;
+}
+// Item n of CTA c, and their number.
+NFD_HD int attn_dealt(int c, int n, const AttnPlan &pl) {
+    const int m = n - pl.wq - (c < pl.wr);
+    if (m < 0) return c + n * pl.grid;
+    const int b = pl.grid - pl.wr, o = c < pl.wr ? c + b : c - pl.wr;      // place of the CTA in a round of pieces
+    const int own = c < pl.wr ? 0 : pl.fq + (o < pl.fr);
+    return pl.whole + (m < own ? o + m * b : pl.first + o + (m - own) * pl.grid);
+}
+NFD_HD int attn_dealt_count(int c, const AttnPlan &pl) {
+    const int o = c < pl.wr ? c + pl.grid - pl.wr : c - pl.wr;
+    return pl.wq + (c < pl.wr) + (c < pl.wr ? 0 : pl.fq + (o < pl.fr)) + pl.rq + (o < pl.rr);
+}
+// What an item is: frame j of the pass, (head, query tile) t of it, split; number of its query tile among those that are split.
+struct AttnPlace {
+    int j, t, split, tile;
+    bool whole;
+};
+template <bool DEALT> NFD_HD AttnPlace attn_place(int item, const AttnPlan &pl) {
+    AttnPlace p;
+    p.whole = DEALT && item < pl.whole;
+    if (p.whole) {
+        p.j = pl.wh_div.div(item), p.t = item - p.j * pl.WH;
+        p.split = p.tile = 0;
+    } else {
+        if (DEALT) item -= pl.whole;
+        p.tile = pl.split_div.div(item), p.split = item - p.tile * pl.MAXSPLIT;
+        p.j = pl.sp_div.div(p.tile), p.t = p.tile - p.j * pl.SP;
+        if (DEALT) p.t += pl.WH;
+    }
+    return p;
+}
 
 // Key block, blocks per page and query tiles for pages of T tokens: the block that walks a page in the least time, a
 // block costing its columns (padded ones included) plus a fixed part of about 24 columns (barriers and hand-overs).
@@ -53,7 +109,8 @@ static bool attn_divisors(AttnPlan &pl, int n_frames, int W, int n_sm) {
     const long long nb = ((long long)W + 1) * pl.BPF + pl.CH, big = 0x100000000ll;
     const long long n_items = n_frames * (pl.WH + (long long)pl.SP * pl.MAXSPLIT);
     const int tiles = pl.WH + pl.SP, d_item = tiles > pl.MAXSPLIT ? tiles : pl.MAXSPLIT;
-    return n_items <= (long long)ATTN_CTA_ITEMS * n_sm && n_items * d_item < big && nb < 0x7fffffffll && nb * (pl.CH > pl.BPF ? pl.CH : pl.BPF) < big;
+    // (a CTA may get ten items more than its share: attn_deal)
+    return n_items <= (long long)(ATTN_CTA_ITEMS - 16) * n_sm && n_items * d_item < big && nb < 0x7fffffffll && nb * (pl.CH > pl.BPF ? pl.CH : pl.BPF) < big;
 }
 // Pieces of the key range of a call on the caller's pages: as many as pay (as in attn_split_plan; the merge is through
 // distributed shared memory) and as clusters of that size fit the machine at once.  clusters(k): clusters of k CTAs that it
@@ -70,21 +127,35 @@ template <typename F> static void attn_own_plan(AttnPlan &pl, int tiles, int n_b
     }
     pl.CH = (n_blocks + best_k - 1) / best_k, pl.MAXSPLIT = best_k;
 }
+// Time of a pass of `frames` frames as attn_deal gives them out, in key blocks of the busiest CTA: a whole item counts a block
+// more than it has, a piece two and a half (start, publication, merge).
+static inline float attn_pass_blocks(const AttnPlan &plan, int frames, int n_sm) {
+    AttnPlan pl = plan;
+    attn_deal(pl, frames, n_sm);
+    const float w = pl.NB + 1.f, p = pl.CH + 2.5f;
+    auto second = [&](int o) { return pl.rq + (o < pl.rr); };
+    float most = pl.wr ? (pl.wq + 1) * w + second(pl.grid - pl.wr) * p : 0.f;
+    const float a = pl.wq * w + (pl.fq + (pl.fr > 0) + second(0)) * p, b = pl.wq * w + (pl.fq + second(pl.fr)) * p;
+    if (a > most) most = a;
+    return b > most ? b : most;
+}
 // How the key ranges of a frame's `tiles` (head, query tile) pairs are split.  By the configuration alone (the longest
 // window, as many frames as there are streams), never by the pass: the order of the sums must not depend on it.
-//   One stream: all of them, into at most as many pieces as fill the SMs once, and no more than pay: a block takes about 0.65
-// us (of 112 keys; its columns and 24 count), publishing and counting 2.5, the merge 0.25 per piece.  (A frame of a model of 2 layers,
-// 4 heads, 64 tokens: behind four frames five pieces of a block 286 us, one of five 270; behind 30 frames 31 pieces 443, six 300.)
-//   Several: the items are dealt out to the CTAs in order, and whole windows leave a last round in which most SMs idle (16 heads
+//   One stream: all of them, into at most as many pieces as fill the SMs once, and
+// no more than pay: a block takes about 0.65 us (of 112 keys; its columns and 24 count), publishing and counting 2.5, the merge
+// 0.25 per piece.  (A frame of a model of 2 layers, 4 heads, 64 tokens: behind four frames five pieces of a block 286 us, one of
+// five 270; behind 30 frames 31 pieces 443, eight 300.)
+//   Else whole windows, dealt out to the CTAs, may leave a last round in which most SMs idle (16 heads
 // x 3 query tiles x 8 streams = 384 items on 148 SMs: two rounds and six tenths of one, at the price of three).  Splitting all
-// of them finely costs a state of 33 KB each; so the first WH are left whole and the others split, for the least blocks on the
-// busiest CTA, a whole item counted a block more than it has and a piece two and a half (start, publication, merge).
+// of them finely costs a state of 33 KB each; so the first WH are left whole and the others split, for the least time of a pass
+// with a frame of every stream; but by no plan that makes a pass with fewer frames, when not all streams are used, take an eighth
+// longer than whole windows would.
 static void attn_split_plan(AttnPlan &pl, int tiles, int n_streams, int n_blocks, int n_sm) {
     auto pieces = [&](int k) { pl.CH = (n_blocks + k - 1) / k, pl.MAXSPLIT = (n_blocks + pl.CH - 1) / pl.CH; };
-    pl.WH = 0, pl.SP = tiles;
-    const int items = n_streams * tiles;
+    pl.WH = 0, pl.SP = tiles, pl.NB = n_blocks;
+    const long long items = (long long)n_streams * tiles;
     float best = 1e30f;
-    int best_k = 1, best_wh = tiles;
+    int best_k = 1;
     if (n_streams == 1) {
         for (int k = 1; k <= n_blocks && (k == 1 || k * items <= n_sm); ++k) {
             pieces(k);
@@ -93,19 +164,20 @@ static void attn_split_plan(AttnPlan &pl, int tiles, int n_streams, int n_blocks
         }
         return pieces(best_k);
     }
-    for (int k = 1; k <= 8 && k <= n_blocks; ++k) {
+    const int full = n_streams < 32 ? n_streams : 32;      // frames of a pass, at most
+    auto whole = [&](int f) { return (float)(((long long)f * tiles + n_sm - 1) / n_sm) * (n_blocks + 1.f); };
+    best = whole(full);
+    int best_wh = 0;                                       // (none is split: MAXSPLIT 1)
+    const int step = tiles > 256 ? tiles / 256 : 1;
+    for (int k = 2; k <= 8 && k <= n_blocks; ++k) {
         pieces(k);
-        for (int wh = k == 1 ? tiles : 0; wh <= (k == 1 ? tiles : tiles - 1); ++wh) {
-            const int nw = n_streams * wh, n = nw + n_streams * (tiles - wh) * pl.MAXSPLIT, grid = n < n_sm ? n : n_sm;
-            // the CTAs before, between and behind those with a whole item and with an item more than others
-            float most = 0.f;
-            const int at[3] = {0, nw % grid, n % grid};
-            for (int c : at) {
-                const int w = nw / grid + (c < nw % grid), all = n / grid + (c < n % grid);
-                const float t = w * (n_blocks + 1.f) + (all - w) * (pl.CH + 2.5f);
-                if (t > most) most = t;
-            }
-            if (most < best) best = most, best_k = k, best_wh = wh;
+        for (int wh = 0; wh < tiles; wh += step) {
+            pl.WH = wh, pl.SP = tiles - wh;
+            const float t = attn_pass_blocks(pl, full, n_sm);
+            if (t >= best) continue;
+            bool good = true;
+            for (int f = 1; f < full && good; ++f) good = attn_pass_blocks(pl, f, n_sm) <= 1.13f * whole(f);
+            if (good) best = t, best_k = k, best_wh = wh;
         }
     }
     pieces(best_k);

@@ -54,7 +54,7 @@
 // Tried and worse: sixteen softmax warps with half a row each (178 -> 201: the fixed part of a block doubles); four epilogue
 // warps beside the groups (96 registers a thread: four frames 60, but 2 us more on every short launch).
 //
-// The grid is persistent: a CTA takes items blockIdx.x, + gridDim.x, ...; producers and
+// The grid is persistent: a CTA takes items blockIdx.x, + gridDim.x, ..., or those that attn_deal gives it; producers and
 // issuer run ahead into the next item.  A key range
 // longer than CH blocks is split over several items; each publishes its
 // unnormalised (O, m, l) state in global memory, stored so that a warp writes and reads
@@ -80,8 +80,9 @@ template <int KB> struct AttnCfg {
     static constexpr int KV_BYTES = KB * 128;              // one K (or V) block
     static constexpr int ML_BYTES = (2 * (1 + NGRP) + 1) * 128 * 4;   // m of every row, l of every row and group, two items; maxima
     static constexpr int SMEM = 2 * Q_BYTES + 2 * NS * KV_BYTES + ML_BYTES + 8 + ATTN_CTA_ITEMS + 256 + 1024;
-    // k_attn_own: the CTA's state, behind the rest, from the 1024-byte boundary that AttnShared starts at
-    static constexpr int STATE_AT = (SMEM - 1024 + 127) / 128 * 128, OWN_SMEM = 1024 + STATE_AT + ATTN_STATE_BYTES;
+    // behind the rest, from the 1024-byte boundary that AttnShared starts at: the CTA's state (k_attn_own), or its items
+    static constexpr int STATE_AT = (SMEM - 1024 + 127) / 128 * 128, OWN_SMEM = 1024 + STATE_AT + ATTN_STATE_BYTES,
+                         DEALT_SMEM = 1024 + STATE_AT + 4 * ATTN_CTA_ITEMS;
     static constexpr int TMEM_COLS = 512;
     static constexpr int S_STRIDE = KB <= 112 ? 112 : 128; // S accumulators from column 0, O at column 448
     static constexpr int TM_O = 448;
@@ -89,7 +90,7 @@ template <int KB> struct AttnCfg {
     static constexpr int THREADS = 32 * (SM_WARP0 + 4 * NGRP);
     static_assert(THREADS == 512, "attn_merge: a warp per quarter of the columns and quadrant of the rows");
     static_assert(KB % 16 == 0 && KB <= 128 && NS * S_STRIDE <= TM_O, "key block");
-    static_assert(SMEM <= 232448 && OWN_SMEM <= 232448, "shared memory of a CTA");
+    static_assert(SMEM <= 232448 && OWN_SMEM <= 232448 && DEALT_SMEM <= 232448, "shared memory of a CTA");
     static_assert(STATE_AT % 16 == 0 && ATTN_STATE_BYTES % 16 == 0, "states are read and written in 16-byte words");
 };
 
@@ -128,29 +129,26 @@ __device__ __forceinline__ unsigned int atomic_inc_acq_rel(unsigned int *p) {
     return v;
 }
 
-// One item of the grid.
+// One item of the grid.  A CTA's items are numbered from attn_first<DEALT>() on in steps of attn_step<DEALT>(): by themselves, or, in a
+// launch that deals them out, by their places in a table of the CTA's.
+template <bool DEALT> __device__ __forceinline__ int attn_first() { return DEALT ? 0 : blockIdx.x; }
+template <bool DEALT> __device__ __forceinline__ int attn_step() { return DEALT ? 1 : gridDim.x; }
 struct AttnItem {
     int j, h, qt, split;     // frame of the pass, head, query tile, split
     int tile;                // number of the query tile among those that are split
     int b0, nb, nsplit;      // key blocks of this split (nb = 0: the frame's window has no such split)
     FrameDesc fr;
-    __device__ __forceinline__ void place(int item, const AttnPlan &pl) {
-        int t;                                                 // (head, query tile) of the frame
-        if (item < pl.whole) {
-            j = pl.wh_div.div(item), t = item - j * pl.WH;
-            split = 0, tile = 0;
-        } else {
-            item -= pl.whole;
-            tile = pl.split_div.div(item), split = item - tile * pl.MAXSPLIT;
-            j = pl.sp_div.div(tile), t = pl.WH + tile - j * pl.SP;
-        }
-        h = pl.qt_div.div(t), qt = t - h * pl.QT;
+    template <bool DEALT> __device__ __forceinline__ bool place(int item, const AttnPlan &pl) {
+        const AttnPlace p = attn_place<DEALT>(item, pl);
+        j = p.j, split = p.split, tile = p.tile;
+        h = pl.qt_div.div(p.t), qt = p.t - h * pl.QT;
+        return p.whole;
     }
-    __device__ __forceinline__ void set(int item, const StepParams *sp, const Dims &D, const AttnPlan &pl) {
-        place(item, pl);
+    template <bool DEALT> __device__ __forceinline__ void set(int item, const StepParams *sp, const Dims &D, const AttnPlan &pl) {
+        const bool whole = place<DEALT>(item, pl);
         fr = sp->fr[j];
         const int nbt = (fr.frame - fr.win_first + 1) * pl.BPF;      // key blocks of this frame's window
-        if (item < pl.whole) {
+        if (whole) {
             nsplit = 1, b0 = 0, nb = nbt;
         } else {
             nsplit = pl.ch_div.div(nbt + pl.CH - 1);
@@ -159,13 +157,14 @@ struct AttnItem {
         }
         if (nb < 0) nb = 0;
     }
-    // the first item at or after `item` (in steps of the grid) that has blocks; `end` or more: there is none
-    __device__ __forceinline__ int find(int item, int end, const StepParams *sp, const Dims &D, const AttnPlan &pl) {
-        for (; item < end; item += gridDim.x) {
-            set(item, sp, D, pl);
+    // the first item at or after `num` (in steps) that has blocks; `end` or more: there is none
+    template <bool DEALT>
+    __device__ __forceinline__ int find(int num, int end, const int *tab, const StepParams *sp, const Dims &D, const AttnPlan &pl) {
+        for (; num < end; num += attn_step<DEALT>()) {
+            set<DEALT>(DEALT ? tab[num] : num, sp, D, pl);
             if (nb > 0) break;
         }
-        return item;
+        return num;
     }
 };
 
@@ -240,11 +239,12 @@ static __device__ __forceinline__ void attn_finish(const AttnItem &w, int p0, in
 // once more, behind the barrier, it cost launches of one item to a CTA 0.2 to 0.5 us.  Three states in flight and no more: with four the kernel's spilled registers
 // doubled, on the path of every item (5407, 13880, 4142).
 // The counter of the lane's item, if it has one; `all`: its pieces.
-static __device__ __forceinline__ unsigned int *attn_counter(int item, int n_items, const StepParams *sp, const Dims &D, const AttnPlan &pl,
-                                                             unsigned int *counters, unsigned int &all) {
-    if (item >= n_items) return nullptr;
+template <bool DEALT>
+static __device__ __forceinline__ unsigned int *attn_counter(int num, int end, const int *tab, const StepParams *sp, const Dims &D,
+                                                             const AttnPlan &pl, unsigned int *counters, unsigned int &all) {
+    if (num >= end) return nullptr;
     AttnItem w;
-    w.set(item, sp, D, pl);
+    w.set<DEALT>(DEALT ? tab[num] : num, sp, D, pl);
     all = w.nsplit;
     return w.nb > 0 && w.nsplit > 1 ? counters + w.tile : nullptr;
 }
@@ -258,8 +258,9 @@ static __device__ __forceinline__ uint32_t attn_count(unsigned int *cnt, unsigne
     return __ballot_sync(0xffffffffu, last);
 }
 // i0: item of bit 0; pieces: of the tile of each bit's item
-static __device__ __forceinline__ void attn_merge(uint32_t last, int i0, const uint32_t *pieces, const Dims &D, const AttnPlan &pl,
-                                                  bf16 *out, const float *part_o) {
+template <bool DEALT>
+static __device__ __forceinline__ void attn_merge(uint32_t last, int i0, const int *tab, const uint32_t *pieces, const Dims &D,
+                                                  const AttnPlan &pl, bf16 *out, const float *part_o) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int cq = warp >> 2, trow = (warp & 3) * 32 + lane;
     if (16 * cq >= D.dh) return;
@@ -267,7 +268,8 @@ static __device__ __forceinline__ void attn_merge(uint32_t last, int i0, const u
 #pragma unroll 1
     for (; last; last &= last - 1) {
         const int bit = __ffs(last) - 1;
-        w.place(i0 + bit * gridDim.x, pl);
+        const int num = i0 + bit * attn_step<DEALT>();
+        w.place<DEALT>(DEALT ? tab[num] : num, pl);
         w.nsplit = pieces[bit];
         const uint8_t *st = reinterpret_cast<const uint8_t *>(part_o) + (size_t)w.tile * pl.MAXSPLIT * ATTN_STATE_BYTES;
         float O[16], lt = 0.f, mx = -INFINITY;
@@ -320,6 +322,7 @@ template <int KB> struct AttnShared {
     uint8_t *base;           // 1024-byte boundary
     uint32_t q, kv, bars, tmem;
     float *m, *l, *mx;       // [item parity][128], [item parity][group][128], [128] true maxima (times c)
+    int *tab;                // [ATTN_CTA_ITEMS] the CTA's items, where they are dealt out
     uint32_t *redo;          // flags (below), the items to merge, and a byte per item (see attn_finish)
     __device__ __forceinline__ uint32_t *tmem_slot() const { return redo + 2 + ATTN_CTA_ITEMS / 4 + 2 * (11 + 5 * A::NS); }
     __device__ __forceinline__ AttnShared(uint8_t *raw) {
@@ -328,6 +331,7 @@ template <int KB> struct AttnShared {
         m = reinterpret_cast<float *>(smem + 2 * A::Q_BYTES + 2 * A::NS * A::KV_BYTES), l = m + 2 * 128;
         mx = l + 2 * A::NGRP * 128, redo = reinterpret_cast<uint32_t *>(mx + 128);
         bars = smem_u32(redo + 2 + ATTN_CTA_ITEMS / 4);
+        tab = reinterpret_cast<int *>(smem + A::STATE_AT);
     }
     // barriers (K of blocks 0 .. NS-1 arrives on k_first, V(n) and K(n + NS) on kv_full)
     __device__ __forceinline__ uint32_t q_full() const { return bars; }
@@ -368,9 +372,9 @@ template <int KB> struct AttnShared {
 // counts: P and O are not looked at); the results with these as m.
 enum { RD_FIRST, RD_MAX, RD_AGAIN };
 
-// The CTA's items first, first + gridDim.x, ... below end (w0 is the first one); `num`: number of the item in sh.redo, not for
+// The CTA's items from number `first` on, below end (w0 is the first one); `num`: number of the item in sh.redo, not for
 // RD_FIRST.
-template <int KB, bool OWN>
+template <int KB, bool OWN, bool DEALT>
 __device__ __forceinline__ void attn_items(const AttnShared<KB> &sh, const CUtensorMap &tmQ, const CUtensorMap &tmK,
                                            const CUtensorMap &tmV, const StepParams *sp, const Dims &D, int layer, const AttnPlan &pl,
                                            const AttnItem &w0, int first, int end, int mode, int num, bf16 *out, float *part_o,
@@ -397,8 +401,8 @@ __device__ __forceinline__ void attn_items(const AttnShared<KB> &sh, const CUten
             if (is_k && test_skip) ok = false;             // test switch: no K comes, and every wait behind it runs out
             int st = 0, lap = 0;                           // ring stage of the next block, how often the ring was filled
             AttnItem w = w0;
-            for (int item = first; item < end && ok; item += gridDim.x) {
-                if (item != first) w.set(item, sp, D, pl);
+            for (int item = first; item < end && ok; item += attn_step<DEALT>()) {
+                if (item != first) w.set<DEALT>(DEALT ? sh.tab[item] : item, sp, D, pl);
                 const int f = pl.bpf_div.div(w.b0);
                 int kb = w.b0 - f * pl.BPF;
                 int left = w.fr.first_new - (w.fr.win_first + f);      // frames until the pages that this pass writes
@@ -445,7 +449,7 @@ __device__ __forceinline__ void attn_items(const AttnShared<KB> &sh, const CUten
             // later ones: this thread's registers and instruction fetches are on every block's path.)
             AttnItem ws = w0, w = w0;
             int item_s = first, it_s = -1, left_s = 0;            // item whose Q was asked for last; items before S's; S to come
-            int item = first - gridDim.x, it = 0, left = 0;            // the same for P V
+            int item = first - attn_step<DEALT>(), it = 0, left = 0;            // the same for P V
             int st_s = 0, lap_s = 0, st = 0, lap = 0;
             int ahead = A::NS;                             // S to issue before the first P V
             auto load_q = [&](int qs) {                    // Q of item ws
@@ -453,7 +457,7 @@ __device__ __forceinline__ void attn_items(const AttnShared<KB> &sh, const CUten
                 tma_load_3d(sQ + qs * A::Q_BYTES, &tmQ, q_full + 8 * qs, 0, ws.j * D.T + ws.qt * 128, ws.h);
             };
             pdl_wait();
-            if (ws.nb == 0) item_s = ws.find(item_s + gridDim.x, end, sp, D, pl);
+            if (ws.nb == 0) item_s = ws.find<DEALT>(item_s + attn_step<DEALT>(), end, sh.tab, sp, D, pl);
             if (item_s < end) load_q(0);
             while (ok) {
                 if (ahead > 0) {
@@ -461,7 +465,7 @@ __device__ __forceinline__ void attn_items(const AttnShared<KB> &sh, const CUten
                 } else {
                     uint32_t acc = 1;
                     if (left == 0) {
-                        item = w.find(item + gridDim.x, end, sp, D, pl);
+                        item = w.find<DEALT>(item + attn_step<DEALT>(), end, sh.tab, sp, D, pl);
                         if (item >= end) break;
                         left = w.nb, acc = 0;
                         if (it > 0) ok = mbar_wait(o_free, (it - 1) & 1, status);          // O of the last item has been read
@@ -488,7 +492,7 @@ __device__ __forceinline__ void attn_items(const AttnShared<KB> &sh, const CUten
                     if (item_s >= end) continue;
                     ++it_s, left_s = ws.nb;
                     ok = mbar_wait(q_full + 8 * (it_s & 1), (it_s >> 1) & 1, status);
-                    item_s = ws.find(item_s + gridDim.x, end, sp, D, pl);
+                    item_s = ws.find<DEALT>(item_s + attn_step<DEALT>(), end, sh.tab, sp, D, pl);
                     if (ok && item_s < end) {              // Q of the item after it
                         if (it_s >= 1) ok = ok && mbar_wait(q_empty + 8 * ((it_s + 1) & 1), ((it_s - 1) >> 1) & 1, status);
                         if (ok) load_q((it_s + 1) & 1);    // (no copy is begun after a wait has run out)
@@ -526,7 +530,7 @@ __device__ __forceinline__ void attn_items(const AttnShared<KB> &sh, const CUten
         const uint32_t tO = tmem + A::TM_O + lane_off;
         AttnItem w = w0;
         int item = first;
-        if (w.nb == 0) item = w.find(item + gridDim.x, end, sp, D, pl);
+        if (w.nb == 0) item = w.find<DEALT>(item + attn_step<DEALT>(), end, sh.tab, sp, D, pl);
         while (item < end) {
             const int ip = it & 1, iph = (it >> 1) & 1;    // item parity: which m and l, phase of their barriers
             const int r = g >= n03 ? g - n03 : g - n03 + A::NGRP;      // this group's blocks: b % 3 == r
@@ -647,7 +651,7 @@ __device__ __forceinline__ void attn_items(const AttnShared<KB> &sh, const CUten
             n03 = gl + 1 == A::NGRP ? 0 : gl + 1;
             AttnItem wn;
             int was = item;
-            item = wn.find(item + gridDim.x, end, sp, D, pl);
+            item = wn.find<DEALT>(item + attn_step<DEALT>(), end, sh.tab, sp, D, pl);
             // The group of the last block finishes the item while the others are on the next one; groups 0 and 1 share the
             // CTA's last item.
             const bool fin = item >= end;
@@ -655,7 +659,7 @@ __device__ __forceinline__ void attn_items(const AttnShared<KB> &sh, const CUten
                 // (The item worked out again: kept through the loop it would cost registers that it needs.  Ahead of the waits:
                 // behind them it held back the next item's products, 0.1 us an item.)
                 asm volatile("" : "+r"(was));
-                w.place(was, pl);
+                w.place<DEALT>(DEALT ? sh.tab[was] : was, pl);
                 ok = ok && mbar_wait(l_full + 8 * ip, iph, status);
                 const float *sl = s_l + ip * A::NGRP * 128 + trow;
                 float l = (sl[0] + sl[128]) + sl[256];
@@ -691,15 +695,15 @@ __device__ __forceinline__ void attn_items(const AttnShared<KB> &sh, const CUten
 
 // The items with marked rows once more, each twice.  Not inlined: the first walk's code is as if this were not there.
 // After a wait that has run out the marked rows are NaN (and counted: the tile's other splits may be waited for).
-template <int KB, bool OWN>
+template <int KB, bool OWN, bool DEALT>
 static __device__ __noinline__ void attn_again(const AttnShared<KB> sh, const CUtensorMap &tmQ, const CUtensorMap &tmK,
                                                const CUtensorMap &tmV, const StepParams *sp, const Dims &D, int layer,
-                                               const AttnPlan &pl, int n_items, bf16 *out, float *part_o, int *status) {
+                                               const AttnPlan &pl, int end, bf16 *out, float *part_o, int *status) {
     using A = AttnCfg<KB>;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = (warp - A::SM_WARP0) >> 2, quad = warp & 3;
     AttnItem w;
     int num = 0;                                           // items with blocks so far
-    for (int item = blockIdx.x; (item = w.find(item, n_items, sp, D, pl)) < n_items; item += gridDim.x, ++num) {
+    for (int item = attn_first<DEALT>(); (item = w.find<DEALT>(item, end, sh.tab, sp, D, pl)) < end; item += attn_step<DEALT>(), ++num) {
         const uint32_t marks = (sh.redo[2 + (num >> 2)] >> (8 * (num & 3))) & 255;
         if (!marks) continue;
         int mode = RD_MAX;
@@ -709,7 +713,7 @@ static __device__ __noinline__ void attn_again(const AttnShared<KB> sh, const CU
             if (threadIdx.x == 0) sh.inval_bars(), sh.init_bars();
             __syncthreads();
             tc_fence_after();
-            attn_items<KB, OWN>(sh, tmQ, tmK, tmV, sp, D, layer, pl, w, item, item + 1, mode, num, out, part_o, status, 0);
+            attn_items<KB, OWN, DEALT>(sh, tmQ, tmK, tmV, sp, D, layer, pl, w, item, item + 1, mode, num, out, part_o, status, 0);
             tc_fence_before();
             __syncthreads();
         }
@@ -741,49 +745,50 @@ __device__ __forceinline__ void attn_set_up(AttnShared<KB> &sh, const CUtensorMa
     sh.tmem = *sh.tmem_slot();
 }
 
-template <int KB>
+template <int KB, bool DEALT>
 __global__ void __launch_bounds__(AttnCfg<KB>::THREADS, 1)
 k_attn_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
           const __grid_constant__ CUtensorMap tmV, const StepParams *sp, const __grid_constant__ Dims D, int layer,
-          const __grid_constant__ AttnPlan pl, int n_items, bf16 *out, float *part_o, unsigned int *counters, int *status,
-          int test_skip) {
-    using A = AttnCfg<KB>;
+          const __grid_constant__ AttnPlan pl, bf16 *out, float *part_o, unsigned int *counters, int *status, int test_skip) {
     extern __shared__ uint8_t smem_raw[];
     NFD_TRACE_T0();
     AttnShared<KB> sh(smem_raw);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int first = attn_first<DEALT>(), step = attn_step<DEALT>(), end = DEALT ? attn_dealt_count(blockIdx.x, pl) : pl.n_items;
     // The first item's descriptor: its loads are in flight during the set-up.  (In a pass the descriptor was written by the
     // first kernel, for whose end the kernels between have waited; where its writer is this kernel's predecessor, the launch
     // is in plain stream order.)
     AttnItem w0;
-    w0.set(blockIdx.x, sp, D, pl);
+    w0.set<DEALT>(DEALT ? attn_dealt(blockIdx.x, 0, pl) : blockIdx.x, sp, D, pl);
+    if (DEALT)
+        for (int n = threadIdx.x; n < end; n += AttnCfg<KB>::THREADS) sh.tab[n] = attn_dealt(blockIdx.x, n, pl);
 
     attn_set_up<KB>(sh, tmQ, tmK, tmV);
-    attn_items<KB, false>(sh, tmQ, tmK, tmV, sp, D, layer, pl, w0, blockIdx.x, n_items, RD_FIRST, 0, out, part_o, status, test_skip);
+    attn_items<KB, false, DEALT>(sh, tmQ, tmK, tmV, sp, D, layer, pl, w0, first, end, RD_FIRST, 0, out, part_o, status, test_skip);
     NFD_TRACE_MARK_T(TRK_OTHER + 16, 128);
     unsigned int *cnt = nullptr, all = 0;
-    if (warp == 2 && pl.MAXSPLIT > 1) cnt = attn_counter(blockIdx.x + lane * gridDim.x, n_items, sp, D, pl, counters, all);
+    if (warp == 2 && pl.MAXSPLIT > 1) cnt = attn_counter<DEALT>(first + lane * step, end, sh.tab, sp, D, pl, counters, all);
     tc_fence_before();
     __syncthreads();
     if (sh.redo[0] & ATTN_MARKED) {
-        attn_again<KB, false>(sh, tmQ, tmK, tmV, sp, D, layer, pl, n_items, out, part_o, status);
+        attn_again<KB, false, DEALT>(sh, tmQ, tmK, tmV, sp, D, layer, pl, end, out, part_o, status);
         __syncthreads();                                   // (it writes states too)
     }
     if (pl.MAXSPLIT > 1) {
 #pragma unroll 1
-        for (int i0 = blockIdx.x; i0 < n_items; i0 += 32 * gridDim.x) {
+        for (int i0 = first; i0 < end; i0 += 32 * step) {
             if (warp == 2) {
-                if (i0 != blockIdx.x) cnt = attn_counter(i0 + lane * gridDim.x, n_items, sp, D, pl, counters, all);
+                if (i0 != first) cnt = attn_counter<DEALT>(i0 + lane * step, end, sh.tab, sp, D, pl, counters, all);
                 const uint32_t last = attn_count(cnt, all);
                 if (lane == 0) sh.redo[1] = last;
                 sh.redo[2 + lane] = all;                   // (the marks have been seen to)
             }
             __syncthreads();                               // what that warp has acquired is handed to the others
-            attn_merge(sh.redo[1], i0, sh.redo + 2, D, pl, out, part_o);
-            if (i0 + 32 * gridDim.x < n_items) __syncthreads();
+            attn_merge<DEALT>(sh.redo[1], i0, sh.tab, sh.redo + 2, D, pl, out, part_o);
+            if (i0 + 32 * step < end) __syncthreads();
         }
     }
-    if (warp == 1) tmem_dealloc(sh.tmem, A::TMEM_COLS);
+    if (warp == 1) tmem_dealloc(sh.tmem, AttnCfg<KB>::TMEM_COLS);
     NFD_TRACE_END(TRK_ATTN);
 }
 
@@ -803,17 +808,17 @@ k_attn_own(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     AttnShared<KB> sh(smem_raw);
     float *state = reinterpret_cast<float *>(sh.base + A::STATE_AT);
     AttnItem w0;
-    w0.set(blockIdx.x, sp, D, pl);
+    w0.set<false>(blockIdx.x, sp, D, pl);
     attn_set_up<KB>(sh, tmQ, tmK, tmV);
     const int end = blockIdx.x + 1;
-    attn_items<KB, true>(sh, tmQ, tmK, tmV, sp, D, 0, pl, w0, blockIdx.x, end, RD_FIRST, 0, out, state, status, test_skip);
+    attn_items<KB, true, false>(sh, tmQ, tmK, tmV, sp, D, 0, pl, w0, blockIdx.x, end, RD_FIRST, 0, out, state, status, test_skip);
     tc_fence_before();
     __syncthreads();
-    if (sh.redo[0] & ATTN_MARKED) attn_again<KB, true>(sh, tmQ, tmK, tmV, sp, D, 0, pl, end, out, state, status);
+    if (sh.redo[0] & ATTN_MARKED) attn_again<KB, true, false>(sh, tmQ, tmK, tmV, sp, D, 0, pl, end, out, state, status);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     __syncwarp();
     cluster_sync_all();                                    // every state of the cluster is in place
-    w0.set(blockIdx.x, sp, D, pl);
+    w0.set<false>(blockIdx.x, sp, D, pl);
     const int cq = warp >> 2, trow = (warp & 3) * 32 + lane;
     if (w0.nsplit > 1 && w0.split < w0.nsplit && cq % w0.nsplit == w0.split && 16 * cq < D.dh) {
         const uint32_t st = smem_u32(state);

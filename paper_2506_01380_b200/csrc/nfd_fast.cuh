@@ -6,6 +6,7 @@
 #include <atomic>
 #include <map>
 #include <tuple>
+#include <type_traits>
 #include <utility>
 
 #include "nfd_sm100.cuh"
@@ -372,22 +373,19 @@ static bool fast_gemm(bool enabled, FastState &fs, cudaStream_t st, const TS *A,
     }
 }
 
-template <int KB>
+template <int KB, bool DEALT>
 static int launch_attn_tc(bool early, int test_skip, PFN_encodeTiled encode, int n_sm, cudaStream_t st, const StepParams *sp, const Dims &D, int nf,
-                          int layer, AttnPlan pl, size_t pages, const bf16 *q, const bf16 *kc, const bf16 *vc,
+                          int layer, const AttnPlan &pl, size_t pages, const bf16 *q, const bf16 *kc, const bf16 *vc,
                           bf16 *out, float *part_o, unsigned int *counters, int *status) {
     using A = AttnCfg<KB>;
-    auto kern = k_attn_tc<KB>;
-    if (!allow_smem(kern, A::SMEM)) return 0;
+    auto kern = k_attn_tc<KB, DEALT>;
+    constexpr int smem = DEALT ? A::DEALT_SMEM : A::SMEM;
+    if (!allow_smem(kern, smem)) return 0;
     CUtensorMap mq, mk, mv;
     if (!encode_map_3d(encode, &mq, q, D.H, nf * D.T, D.dh, 128) || !encode_map_3d(encode, &mk, kc, pages, D.T, D.dh, KB) ||
         !encode_map_3d(encode, &mv, vc, pages, D.T, D.dh, KB))
         return 0;
-    pl.whole = nf * pl.WH;
-    const int n_items = pl.whole + nf * pl.SP * pl.MAXSPLIT;
-    dim3 grid(n_items < n_sm ? n_items : n_sm);
-    cudaError_t e = launch_kernel(early, kern, grid, dim3(A::THREADS), (size_t)A::SMEM, st, 1, mq, mk, mv, sp, D, layer, pl, n_items,
-                                  out, part_o, counters, status, test_skip);
+    cudaError_t e = launch_kernel(early, kern, dim3(pl.grid), dim3(A::THREADS), (size_t)smem, st, 1, mq, mk, mv, sp, D, layer, pl, out, part_o, counters, status, test_skip);
     if (e != cudaSuccess) {
         fprintf(stderr, "libnfd: tensor-core attention launch failed: %s\n", cudaGetErrorString(e));
         cudaGetLastError();
@@ -420,7 +418,7 @@ template <int KB> static int attn_own_clusters(int dev, int k) {
 enum { NFD_TEST_SKIP = 1, NFD_TEST_REFUSE = 2 };
 // Split key ranges of the caller's pages: see k_attn_own.
 template <int KB>
-static bool launch_attn_own(int test, PFN_encodeTiled encode, cudaStream_t st, const StepParams *sp, int nf, const Dims &D, const AttnPlan &pl,
+static bool launch_attn_own(int test, PFN_encodeTiled encode, cudaStream_t st, const StepParams *sp, int nf, const Dims &D, AttnPlan pl,
                             size_t pages, const bf16 *q, const bf16 *kc, const bf16 *vc, bf16 *out, int *status) {
     using A = AttnCfg<KB>;
     auto kern = k_attn_own<KB>;
@@ -430,8 +428,9 @@ static bool launch_attn_own(int test, PFN_encodeTiled encode, cudaStream_t st, c
     if (!encode_map_3d(encode, &mq, q, D.H, nf * D.T, D.dh, 128) || !encode_map_3d(encode, &mk, kc, pages, D.T, D.dh, KB) ||
         !encode_map_3d(encode, &mv, vc, pages, D.T, D.dh, KB))
         return false;
+    attn_deal(pl, nf, 0x7fffffff);                         // an item to a CTA
     // (test switch: a cluster size that the runtime refuses)
-    const cudaError_t e = launch_kernel(false, kern, dim3(nf * pl.SP * pl.MAXSPLIT), dim3(A::THREADS), (size_t)smem, st,
+    const cudaError_t e = launch_kernel(false, kern, dim3(pl.grid), dim3(A::THREADS), (size_t)smem, st,
                                         test & NFD_TEST_REFUSE ? 64 : pl.MAXSPLIT, mq, mk, mv, sp, D, pl, out, status, test & NFD_TEST_SKIP);
     if (e != cudaSuccess) cudaGetLastError();
     return e == cudaSuccess;
@@ -441,14 +440,22 @@ static bool launch_attn_own(int test, PFN_encodeTiled encode, cudaStream_t st, c
 // start before its predecessor ends.  It reads the pass descriptor, and pages that the pass does not write, without waiting
 // for the predecessor: that must not be the kernel that writes them.  `test_skip`: the test switch of nfd_sm100.cuh.
 static int launch_attn_plan(bool early, int test_skip, PFN_encodeTiled encode, int n_sm, cudaStream_t st, const StepParams *sp, const Dims &D, int nf,
-                            int layer, const AttnPlan &pl, size_t pages, const bf16 *q, const bf16 *kc, const bf16 *vc,
+                            int layer, AttnPlan pl, size_t pages, const bf16 *q, const bf16 *kc, const bf16 *vc,
                             bf16 *out, float *part_o, unsigned int *counters, int *status) {
-    switch (pl.KB) {
-        case 128: return launch_attn_tc<128>(early, test_skip, encode, n_sm, st, sp, D, nf, layer, pl, pages, q, kc, vc, out, part_o, counters, status);
-        case 112: return launch_attn_tc<112>(early, test_skip, encode, n_sm, st, sp, D, nf, layer, pl, pages, q, kc, vc, out, part_o, counters, status);
-        case 96: return launch_attn_tc<96>(early, test_skip, encode, n_sm, st, sp, D, nf, layer, pl, pages, q, kc, vc, out, part_o, counters, status);
-        default: return launch_attn_tc<64>(early, test_skip, encode, n_sm, st, sp, D, nf, layer, pl, pages, q, kc, vc, out, part_o, counters, status);
-    }
+    attn_deal(pl, nf, n_sm);
+    auto go = [&](auto kb, auto dealt) {
+        return launch_attn_tc<decltype(kb)::value, decltype(dealt)::value>(early, test_skip, encode, n_sm, st, sp, D, nf, layer, pl, pages, q, kc,
+                                                                           vc, out, part_o, counters, status);
+    };
+    auto width = [&](auto dealt) {
+        switch (pl.KB) {
+            case 128: return go(std::integral_constant<int, 128>(), dealt);
+            case 112: return go(std::integral_constant<int, 112>(), dealt);
+            case 96: return go(std::integral_constant<int, 96>(), dealt);
+            default: return go(std::integral_constant<int, 64>(), dealt);
+        }
+    };
+    return pl.dealt() ? width(std::true_type()) : width(std::false_type());
 }
 
 // Returns the number of kernels launched (0: not handled, use the plain kernel).

@@ -15,6 +15,44 @@ extern "C" void own_plan(int T, int tiles, int n_blocks, const int *clusters, in
     attn_own_plan(pl, tiles, n_blocks, [&](int k) { return clusters[k]; });
     out[0] = pl.MAXSPLIT, out[1] = pl.CH;
 }
+// The plan of a configuration.
+extern "C" int context_plan(int T, int heads, int n_streams, int window, int n_sm, int *out) {
+    AttnPlan pl;
+    attn_blocks(pl, T);
+    const int n_blocks = (window + 1) * pl.BPF;
+    attn_split_plan(pl, heads * pl.QT, n_streams, n_blocks, n_sm);
+    if (!attn_divisors(pl, 32, window, n_sm)) return 0;
+    out[0] = pl.WH, out[1] = pl.SP, out[2] = pl.MAXSPLIT, out[3] = pl.CH, out[4] = n_blocks, out[5] = pl.BPF, out[6] = pl.QT;
+    return 1;
+}
+// Every item of a pass of `frames` frames, whose windows are full: seen[(frame, tile) * MAXSPLIT + split] counts it, load[c] is
+// the time of CTA c in half blocks (a whole item a block more than it has, a piece two and a half), `most` that of the busiest one
+// by the closed form; the largest number of items of a CTA, -1 where an item is out of range.
+extern "C" int deal(int T, int heads, int n_streams, int window, int n_sm, int frames, int *seen, int *load, float *most) {
+    AttnPlan pl;
+    attn_blocks(pl, T);
+    const int n_blocks = (window + 1) * pl.BPF, tiles = heads * pl.QT;
+    attn_split_plan(pl, tiles, n_streams, n_blocks, n_sm);
+    if (!attn_divisors(pl, 32, window, n_sm)) return -2;
+    attn_deal(pl, frames, n_sm);
+    int items = 0;
+    for (int c = 0; c < pl.grid; ++c) {
+        const int n = pl.dealt() ? attn_dealt_count(c, pl) : (pl.n_items - c + pl.grid - 1) / pl.grid;
+        for (int i = 0; i < n; ++i) {
+            const int item = pl.dealt() ? attn_dealt(c, i, pl) : c + i * pl.grid;
+            if (item < 0 || item >= pl.n_items) return -1;
+            const AttnPlace p = pl.dealt() ? attn_place<true>(item, pl) : attn_place<false>(item, pl);
+            if (p.j < 0 || p.j >= frames || p.t < 0 || p.t >= tiles || p.split < 0 || p.split >= pl.MAXSPLIT) return -1;
+            if (p.whole != (p.t < pl.WH) || (!p.whole && p.tile != p.j * pl.SP + p.t - pl.WH)) return -1;
+            ++seen[(p.j * tiles + p.t) * pl.MAXSPLIT + p.split];
+            load[c] += p.whole || pl.MAXSPLIT == 1 ? 2 * (n_blocks + 1) : 2 * pl.CH + 5;
+        }
+        if (n > items) items = n;
+        if (n < 1) return -1;
+    }
+    *most = attn_pass_blocks(pl, frames, n_sm);
+    return items;
+}
 """
 
 
@@ -44,3 +82,40 @@ def test_clusters_of_the_caller_s_pages_fit_the_machine(lib, T):
                 assert 1 <= k <= n_blocks and (k - 1) * ch < n_blocks <= k * ch
     lib.own_plan(40, 16, 33, (C.c_int * 9)(*B200), out)
     assert out[0] not in (7, 8)          # 16 clusters of either do not fit
+
+
+SHAPES = [(336, 16, 32), (336, 16, 16), (336, 24, 16), (336, 12, 16), (220, 12, 9), (220, 16, 16), (390, 24, 8), (64, 4, 32),
+          (96, 24, 8), (336, 3, 31)]                        # tokens, heads, window
+
+
+@pytest.mark.parametrize("T,heads,window", SHAPES)
+def test_every_item_is_dealt_out_once_and_partial_batches_lose_little(lib, T, heads, window):
+    """Passes of 1 to 32 frames in contexts of 1 to 9 streams: every piece of every query tile comes up once, the busiest CTA is as
+    busy as the plan's closed form says, and where not all streams have a frame in the pass it has at most an eighth more to do
+    than with whole windows.  (Pieces dealt on in turn behind the whole items: up to 1.6 times as much.)"""
+    info, most = (C.c_int * 7)(), C.c_float()
+    for n_sm in (148, 132, 20):
+        for streams in range(1, 10):
+            assert lib.context_plan(T, heads, streams, window, n_sm, info)
+            wh, sp, k, ch, n_blocks, bpf, qt = info
+            tiles = heads * qt
+            assert wh + sp == tiles and (k - 1) * ch < n_blocks <= k * ch
+            for frames in sorted({1, 2, 3, 4, 5, 6, 7, 8, streams, 2 * streams, 16, 31, 32}):
+                seen, load = (C.c_int * (frames * tiles * k))(), (C.c_int * n_sm)()
+                items = lib.deal(T, heads, streams, window, n_sm, frames, seen, load, C.byref(most))
+                assert 0 < items <= 2048
+                want = [1 if t >= wh or s == 0 else 0 for _ in range(frames) for t in range(tiles) for s in range(k)]
+                assert list(seen) == want, (n_sm, streams, frames)
+                busy = max(load) / 2
+                assert k == 1 or abs(busy - most.value) < 1e-3
+                if wh and frames <= streams:
+                    whole = -(-frames * tiles // n_sm) * (n_blocks + 1)
+                    assert busy <= 1.13 * whole, (n_sm, streams, frames, busy, whole)
+
+
+def test_configuration_whose_pieces_are_counted_in_two_sweeps(lib):
+    """32 heads, 336 tokens, four streams behind 12 frames, 32 frames in a pass: some CTA has more than the 32 items that one sweep of
+    a warp counts (its values are checked on the GPU)."""
+    frames, tiles, k = 32, 96, 3
+    seen, load, most = (C.c_int * (frames * tiles * k))(), (C.c_int * 148)(), C.c_float()
+    assert lib.deal(336, 32, 4, 12, 148, frames, seen, load, C.byref(most)) > 32
