@@ -141,10 +141,11 @@ static inline float attn_pass_blocks(const AttnPlan &plan, int frames, int n_sm)
 }
 // How the key ranges of a frame's `tiles` (head, query tile) pairs are split.  By the configuration alone (the longest
 // window, as many frames as there are streams), never by the pass: the order of the sums must not depend on it.
-//   One stream: all of them, into at most as many pieces as fill the SMs once, and
+//   Where a frame of every stream leaves half of the SMs idle, all of them, into at most as many pieces as fill the SMs once, and
 // no more than pay: a block takes about 0.65 us (of 112 keys; its columns and 24 count), publishing and counting 2.5, the merge
 // 0.25 per piece.  (A frame of a model of 2 layers, 4 heads, 64 tokens: behind four frames five pieces of a block 286 us, one of
-// five 270; behind 30 frames 31 pieces 443, eight 300.)
+// five 270; behind 30 frames 31 pieces 443, eight 300; two streams of 4 heads x 32 behind 1000 frames, eight pieces a tile 766,
+// eighteen 619.)
 //   Else whole windows, dealt out to the CTAs, may leave a last round in which most SMs idle (16 heads
 // x 3 query tiles x 8 streams = 384 items on 148 SMs: two rounds and six tenths of one, at the price of three).  Splitting all
 // of them finely costs a state of 33 KB each; so the first WH are left whole and the others split, for the least time of a pass
@@ -156,7 +157,7 @@ static void attn_split_plan(AttnPlan &pl, int tiles, int n_streams, int n_blocks
     const long long items = (long long)n_streams * tiles;
     float best = 1e30f;
     int best_k = 1;
-    if (n_streams == 1) {
+    if (n_streams == 1 || 2 * items <= n_sm) {
         for (int k = 1; k <= n_blocks && (k == 1 || k * items <= n_sm); ++k) {
             pieces(k);
             const float t = pl.CH * 0.65f * (pl.KB + 24) / 136.f + (k > 1 ? 2.5f + 0.25f * k : 0.f);

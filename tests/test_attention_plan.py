@@ -113,6 +113,15 @@ def test_every_item_is_dealt_out_once_and_partial_batches_lose_little(lib, T, he
                     assert busy <= 1.13 * whole, (n_sm, streams, frames, busy, whole)
 
 
+@pytest.mark.parametrize("T,heads,streams,window", [(64, 4, 2, 1000), (128, 2, 3, 400), (64, 4, 4, 200), (64, 4, 1, 1000)])
+def test_long_windows_of_few_heads_fill_the_machine(lib, T, heads, streams, window):
+    """With a few query tiles to a frame and hundreds of blocks to a window the pieces of a frame of every stream fill more than
+    half of the SMs.  (At most eight pieces a tile: 64 to 128 CTAs, windows up to 2.2 times as long.)"""
+    info = (C.c_int * 7)()
+    assert lib.context_plan(T, heads, streams, window, 148, info)
+    assert 74 < info[1] * info[2] * streams <= 148 and info[0] == 0
+
+
 def test_configuration_whose_pieces_are_counted_in_two_sweeps(lib):
     """32 heads, 336 tokens, four streams behind 12 frames, 32 frames in a pass: some CTA has more than the 32 items that one sweep of
     a warp counts (its values are checked on the GPU)."""
