@@ -8,16 +8,20 @@ from paper_2506_01380_b200 import inputs as I
 pytestmark = pytest.mark.gpu
 
 
-def _launches(call, tmp_path):
-    """[(kernel name, registers per thread, CTAs, threads)] of the launches that `call` makes."""
+def _events(call, tmp_path):
     import torch
-    call()
     torch.cuda.synchronize()
     with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CPU, torch.profiler.ProfilerActivity.CUDA]) as p:
         call()
         torch.cuda.synchronize()
     p.export_chrome_trace(str(tmp_path / "t.json"))
-    events = [e for e in json.load(open(tmp_path / "t.json"))["traceEvents"] if e.get("cat") == "kernel"]
+    return json.load(open(tmp_path / "t.json"))["traceEvents"]
+
+
+def _launches(call, tmp_path):
+    """[(kernel name, registers per thread, CTAs, threads)] of the launches that `call` makes."""
+    call()
+    events = [e for e in _events(call, tmp_path) if e.get("cat") == "kernel"]
     if not events:
         pytest.skip("the profiler gives no launch records here")
     return [(e["name"], e["args"]["registers per thread"], e["args"]["grid"][0] * e["args"]["grid"][1] * e["args"]["grid"][2],
@@ -62,3 +66,59 @@ def test_split_windows_of_the_caller_as_clusters_whole_ones_on_the_persistent_ke
     q, k, out = _pages("bf16", heads, dh, T, n_q, n_kv)
     run = _launches(lambda: N.attention_noalloc(q, k, k, n_q, window, out), tmp_path)
     assert len(run) == 2 and "k_set_params" in run[0][0] and kernel + "<" in run[1][0], run
+
+
+def test_a_pass_has_one_graph_for_velocities_and_samplers(tmp_path):
+    """The first velocity asked for behind a generation, and the first undistilled sample, replay the generation's graphs."""
+    import torch
+    from paper_2506_01380_b200 import nfd as N
+    cfg = I.make_cfg("tiny_bf16")
+    g = N.NFD(cfg, I.make_weights(cfg, 0))
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(1)
+    noise = torch.randn(cfg["n_steps"], 1, *I.frame_shape(cfg), generator=gen, device="cuda")
+    x, v = noise[0].contiguous(), torch.empty_like(noise[0])
+    g.set_option("lazy_commit", 0)
+
+    def made(call):
+        return [e["name"] for e in _events(call, tmp_path) if "GraphInstantiate" in e.get("name", "")]
+
+    if not made(lambda: g.speculate(1, 1, noise)):
+        pytest.skip("the profiler gives no records of graphs here")
+    g.rollback(1)
+    g.speculate(1, 1, noise)                         # the modulation is cached now: graphs without conditioning
+    g.rollback(1)
+    for _ in range(2):                               # with conditioning and without
+        assert not made(lambda: g.denoise_step(x, 0.77, 1, out=v))
+    assert not made(lambda: g.sample_dpmpp(1, 1, x, n_evals=3))
+
+
+@pytest.mark.parametrize("model", ["tiny_bf16", "tiny"])
+def test_velocities_and_samples_in_turn(model):
+    """The sampler's step is switched on and off in the one graph of a pass: a program that asks for velocities, generations and
+    undistilled samples in turn gets what launches without graphs give."""
+    import torch
+    from paper_2506_01380_b200 import nfd as N
+    cfg = I.make_cfg(model)
+    w = I.make_weights(cfg, 3, "stress")
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(2)
+    noise = [torch.randn(cfg["n_steps"], 2, *I.frame_shape(cfg), generator=gen, device="cuda") for _ in range(3)]
+    outs = []
+    for graph in (1, 0):
+        g = N.NFD(cfg, w)
+        g.set_option("graph", graph)
+        out = []
+        for i, n in enumerate(noise):
+            out.append(g.denoise_step(n[0].contiguous(), 0.4 + 0.1 * i, 1))
+            out.append(g.speculate(2, i, n))
+            g.rollback(1)
+            out.append(g.denoise_step(n[1].contiguous(), 0.9, 2))
+            out.append(g.denoise_step(n[2].contiguous(), 0.9, 2))
+            out.append(g.sample_dpmpp(2, i, n[0].contiguous(), n_evals=4))
+            g.rollback(0)
+        out.append(torch.tensor([g.kv_hash() % 2 ** 40], device="cuda"))
+        assert g.status() == 0
+        outs.append(out)
+    for a, b in zip(*outs):
+        assert torch.equal(a, b)
