@@ -24,7 +24,7 @@ struct FastState {
     bool ready = false;
     PFN_encodeTiled encode = nullptr;
     int *d_status = nullptr;
-    int n_sm = 148, dh = 0;
+    int n_sm = 0, dh = 0;
     size_t a_rows = 0;     // rows of every activation buffer (NFD_MAX_PASS_FRAMES * T)
     AttnPlan plan;         // KB == 0: tensor-core attention not available for this shape
     float *part_o = nullptr;           // per-split states of the attention kernel: [query tile][split] x ATTN_STATE_BYTES
@@ -49,6 +49,11 @@ static int fast_create(FastState &fs, const Dims &D, bool bf16_mode, cudaStream_
     fs.ready = false;
     fs.d_status = d_status;
     fs.a_rows = (size_t)NFD_MAX_PASS_FRAMES * D.T, fs.dh = D.dh;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&fs.n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+        cudaGetLastError();
+        return NFD_E_CUDA;
+    }
     if (!bf16_mode) return NFD_OK;
     fs.encode = get_encode_fn();
     if (!fs.encode) {
@@ -56,9 +61,6 @@ static int fast_create(FastState &fs, const Dims &D, bool bf16_mode, cudaStream_
         fprintf(stderr, "libnfd: the driver does not provide cuTensorMapEncodeTiled; a bf16 context needs it\n");
         return NFD_E_CUDA;
     }
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&fs.n_sm, cudaDevAttrMultiProcessorCount, dev);
     fs.ready = true;
     // attention plan: any number of tokens per frame, head dimension 64 or 32
     AttnPlan pl;

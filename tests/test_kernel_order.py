@@ -39,3 +39,12 @@ def test_marks_of_the_timeline_may_be_taken_in_functions():
     t0 = re.search(r"#define NFD_TRACE_T0\(\)((?:[^\n]*\\\n)*[^\n]*)", common).group(1)
     assert "nfd_marks_" in t0 and "__shared__" not in t0
     assert re.search(r"^__shared__ unsigned long long nfd_marks_\[", common, re.M)
+
+
+def test_plans_go_by_the_device_and_not_by_one_machine():
+    """The number of SMs that a context's launches go by is asked of the device, in fp32 contexts too, and has no default that could
+    pass for one."""
+    text = open(os.path.join(CSRC, "nfd_fast.cuh")).read()
+    assert re.search(r"int n_sm = 0\b", text)
+    create = text[text.index("static int fast_create("):]
+    assert create.index("cudaDevAttrMultiProcessorCount") < create.index("if (!bf16_mode) return")
