@@ -268,7 +268,11 @@ static void prof_mark(nfd_ctx *c, bool stop) {
 
 // Kernels of a forward pass: launched with programmatic stream serialisation, so
 // that each one's prologue overlaps the tail of its predecessor.  Every such
-// kernel calls pdl_wait() before it touches global memory.
+// kernel calls pdl_wait() before it touches what a kernel before it writes; except
+// that the projections and the attention read the pass descriptor, the former the
+// modulation cache, the latter pages of earlier passes without.  These are complete:
+// k_set_params releases nobody early, and everything between it and the first
+// projection releases its dependents after its own wait.
 #define PLAUNCH(c, kern, grid, block, smem, ...)                                                    \
     do {                                                                                            \
         prof_mark((c), false);                                                                      \

@@ -265,6 +265,8 @@ static bool launch_gemm_tc_sc(FastState &fs, cudaStream_t st, const bf16 *A, con
     const CUtensorMap *mb = get_map_2d(fs, Wt, N, K, BN);
     if (!ma || !mb) return false;
     dim3 grid(((N + BN - 1) / BN) * S, (M + 127) / 128);
+    // Always early: in a pass the kernels before the first projection release their dependents after their own wait, so that
+    // the descriptor and the modulation cache, which this one reads before its wait, are complete.
     cudaError_t e = launch_pdl(kern, grid, dim3(G::THREADS), (size_t)G::SMEM, st, S, *ma, *mb, M, N, K, S, epi, pf,
                                fs.d_status);
     if (e != cudaSuccess) {

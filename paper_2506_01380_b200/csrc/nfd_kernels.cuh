@@ -269,6 +269,8 @@ __global__ void __launch_bounds__(256) k_modw(const StepParams *sp, const TS *co
 // With a_out set (folded LayerNorm, see the GEMM epilogues below; d a multiple of
 // 32) it also writes the first layer's GEMM operand z*(1+scale) and the row-sum
 // partials of z per 32 columns.
+// It waits for its predecessor before it releases its dependents: the projections
+// behind it read the descriptor and the modulation cache before they wait.
 // ---------------------------------------------------------------------------
 #define PE_TOK 8
 template <typename TS>
@@ -363,7 +365,7 @@ __global__ void __launch_bounds__(256) k_patch_embed(const StepParams *sp, Dims 
 // ---------------------------------------------------------------------------
 // adaLN: out = norm(z) * (1 + scale_f) + shift_f, one warp per token.  Rows of
 // up to 1024 elements are held in registers (one read of z); longer rows are
-// re-read from L1/L2.
+// re-read from L1/L2.  Its dependents are released after its wait, as in k_patch_embed.
 // ---------------------------------------------------------------------------
 template <typename TS> __device__ __forceinline__ void store4(TS *o, float a, float b, float c, float d);
 template <> __device__ __forceinline__ void store4<float>(float *o, float a, float b, float c, float d) {

@@ -48,3 +48,16 @@ def test_plans_go_by_the_device_and_not_by_one_machine():
     assert re.search(r"int n_sm = 0\b", text)
     create = text[text.index("static int fast_create("):]
     assert create.index("cudaDevAttrMultiProcessorCount") < create.index("if (!bf16_mode) return")
+
+
+def test_the_descriptor_and_the_modulation_are_complete_when_a_projection_starts():
+    """The projections read both before their grid wait.  So the descriptor's writer releases nobody early, and every kernel up to
+    the first projection of a pass waits before it releases its dependents."""
+    kernels = _kernels("nfd_kernels.cuh")
+    assert "pdl_launch()" not in kernels["k_set_params"]
+    for name in ("k_temb", "k_gemv", "k_modw", "k_patch_embed", "k_adaln"):
+        body = kernels[name]
+        assert body.count("pdl_wait()") == body.count("pdl_launch()") == 1, name
+        assert body.index("pdl_wait()") < body.index("pdl_launch()"), name
+        # nobody leaves, and with it releases its dependents, before the wait
+        assert "return" not in body[:body.index("pdl_wait()")], name
