@@ -112,17 +112,20 @@ static bool attn_divisors(AttnPlan &pl, int n_frames, int W, int n_sm) {
     // (a CTA may get ten items more than its share: attn_deal)
     return n_items <= (long long)(ATTN_CTA_ITEMS - 16) * n_sm && n_items * d_item < big && nb < 0x7fffffffll && nb * (pl.CH > pl.BPF ? pl.CH : pl.BPF) < big;
 }
-// Pieces of the key range of a call on the caller's pages: as many as pay (as in attn_split_plan; the merge is through
-// distributed shared memory) and as clusters of that size fit the machine at once.  clusters(k): clusters of k CTAs that it
-// holds.  (Clusters of 1 to 8 are 148, 74, 45, 33, 26, 22, 15, 15 on a 148-SM B200, which no formula gives: by SMs / k - 4 there
-// would be 17 of seven, and 2 heads x 64, 8 x 40 queries behind 32 frames, 16 query tiles, took 25.3 -> 27.2 us in two rounds of them.)
+// Pieces of the key range of a call on the caller's pages: as many as pay (as in attn_split_plan; starting a cluster and the merge
+// through distributed shared memory take 2 us and 0.2 per piece) and as clusters of that size fit the machine at once.  Head
+// dimension 64, us of whole windows and in pieces, on the device: 30 heads x 40 tokens, 8 blocks of 64 keys 10.8, 11.3, 12 blocks
+// 12.6, 11.8; 8 x 96 tokens, 6 blocks of 96 10.7, 11.2, 10 blocks 12.7, 11.9; 8 x 336, 12 blocks of 112 15.3, 13.1.
+// clusters(k): clusters of k CTAs that the machine holds.  (Clusters of 1 to 8 are 148, 74, 45, 33, 26, 22, 15, 15 on a 148-SM B200,
+// which no formula gives: by SMs / k - 4 there would be 17 of seven, and 2 heads x 64, 8 x 40 queries behind 32 frames, 16 query
+// tiles, took 25.3 -> 27.2 us in two rounds of them.)
 template <typename F> static void attn_own_plan(AttnPlan &pl, int tiles, int n_blocks, F clusters) {
     float best = 1e30f;
     int best_k = 1;
     for (int k = 1; k <= 8 && k <= n_blocks; ++k) {
         const int ch = (n_blocks + k - 1) / k;
         if (k > 1 && ((n_blocks + ch - 1) / ch != k || tiles > clusters(k))) continue;
-        const float t = ch * 0.65f * (pl.KB + 24) / 136.f + (k > 1 ? 1.5f + 0.2f * k : 0.f);
+        const float t = ch * 0.65f * (pl.KB + 24) / 136.f + (k > 1 ? 2.0f + 0.2f * k : 0.f);
         if (t < best) best = t, best_k = k;
     }
     pl.CH = (n_blocks + best_k - 1) / best_k, pl.MAXSPLIT = best_k;

@@ -80,6 +80,10 @@ def test_clusters_of_the_caller_s_pages_fit_the_machine(lib, T):
                 k, ch = out
                 assert k == 1 or tiles <= machine[k], (machine, tiles, n_blocks, k)
                 assert 1 <= k <= n_blocks and (k - 1) * ch < n_blocks <= k * ch
+    # windows that are too short for a merge stay whole: 6 blocks of 96 keys, 8 and 9 of 64; not 8 and 10
+    for tokens, n_blocks, split in ((96, 6, False), (40, 8, False), (40, 9, False), (96, 8, True), (40, 10, True)):
+        lib.own_plan(tokens, 8, n_blocks, (C.c_int * 9)(*B200), out)
+        assert (out[0] > 1) == split, (tokens, n_blocks)
     lib.own_plan(40, 16, 33, (C.c_int * 9)(*B200), out)
     assert out[0] not in (7, 8)          # 16 clusters of either do not fit
 
