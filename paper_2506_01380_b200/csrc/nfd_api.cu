@@ -313,7 +313,6 @@ static void launch_gemm(nfd_ctx *c, const TS *A, const TS *Wt, int M, int N, int
     PLAUNCH(c, (k_gemm_simple<TS, Epi>), grid, 256, 0, (const StepParams *)c->d_sp, c->D.T, A, Wt, N, K, epi);
 }
 
-// `early`: see launch_attn_plan; set inside a pass, where the QKV projection comes before.
 // `launch` with the instance of k_attn_rows for the head dimension, and its grid.
 template <typename TS, typename F> static void launch_attn_rows(int n_sm, const Dims &D, int nf, F launch) {
     const int nq = attn_rows_q(D, nf, n_sm);
@@ -324,6 +323,7 @@ template <typename TS, typename F> static void launch_attn_rows(int n_sm, const 
         default: return nq == 8 ? launch(k_attn_rows<TS, 128, 8>, grid) : launch(k_attn_rows<TS, 128, 16>, grid);
     }
 }
+// `early`: see launch_attn_plan; set inside a pass, where the QKV projection comes before.
 template <typename TS> static void launch_attention(nfd_ctx *c, int nf, int layer, bool early, int test_skip = 0) {
     const Dims &D = c->D;
     c->cls = CLS_ATTN;

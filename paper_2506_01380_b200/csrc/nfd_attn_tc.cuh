@@ -43,11 +43,11 @@
 // 128 x 112 block on the special-function unit) and the one issuer (18 products, 29 to 60 clocks each, and their barriers); a
 // block takes about 1300 clocks.  Registers and code size count: spilled registers are cold local memory, about 1 us on the
 // path of a short item, and a cold code path costs as much.
-// Measured, 16 heads x 64 on one B200 (events around a launch), one, two and four frames of 336 tokens behind 16 and eight
-// streams behind 32: 25.0, 40.8, 71.8, 210 us (580 TFLOP/s).  How it came there, with P rounded to bf16 and a quarter of the
-// exponentials by a polynomial on the FMA pipe: one frame 28.4 with one thread for all loads, one for all products and a
+// Measured, 16 heads x 64 on one B200 (events around a launch), one, two and four frames of 336 tokens behind 16: 25.0, 39.3,
+// 65.6 us (25.0, 40.8, 71.8 with pieces merged as their items end).  How it came there, with P rounded to bf16 and a quarter of
+// the exponentials by a polynomial on the FMA pipe: one frame 28.4 with one thread for all loads, one for all products and a
 // maximum pass over S; 25.0 with the threads split and no maximum pass; 23.0 with three groups; 22.5 with items that overlap
-// and the issuer's loop in one copy (then 35.2, 61 and 165 for the others).  The polynomial's range reduction saturated,
+// and the issuer's loop in one copy (then 35.2, 61 and, eight streams behind 32 frames, 165 for the others).  The polynomial's range reduction saturated,
 // which gave the score NaN a probability of nought; with every exponential the special-function unit's 23.0, 37.3, 64.2, 181.
 // With P as two numbers the polynomial gains nothing (24.9, 39.4, 69.5, 210 with an eighth of the exponentials, 25.0, 39.9,
 // 70.2, 207 without).  Pages of 220 tokens behind nine frames: 17 us (plain kernel: 800).
@@ -187,7 +187,7 @@ __device__ __forceinline__ void attn_write(const AttnItem &w, int row, int e0, c
 }
 
 // The end of an item for one warp: halves p0 .. p0 + np - 1 (32 columns each) of the 32 rows of its quadrant are read from
-// tensor memory and written out, or published (attn_merge_all).
+// tensor memory and written out, or published (attn_merge).
 // m, l: reference and sum of this thread's row.  With `redo` (see AttnShared; a byte per item, a bit per half and
 // quadrant; this is item `num`) a half whose l or O has left fp32 is left alone and marked there; without it, `mask` tells
 // which halves to take.
@@ -234,8 +234,8 @@ static __device__ __forceinline__ void attn_finish(const AttnItem &w, int p0, in
 // When a CTA is through with its items: one warp counts it in for each of those that are pieces of a split key range, a lane
 // for an item, and all merge, in split order, those for which it is the last, a warp a quarter of the columns of a quadrant's
 // rows.  Done as each item ended, the fence, the counter and the merge kept one of the softmax groups, and with it the order
-// of the products, for 3.5 us an item.  us, 310M class: four-frame speculation 14400 -> 13940, one frame (an item per CTA)
-// 5380 -> 5358, 220 tokens 4150 -> 4101.  What the merge needs of an item comes through shared memory: read from the descriptor
+// of the products, for 3.5 us an item (310M class, four frames behind 16: 70.7 -> 65.6 us a launch; one frame, an item to a CTA, 25.0
+// both ways).  What the merge needs of an item comes through shared memory: read from the descriptor
 // once more, behind the barrier, it cost launches of one item to a CTA 0.2 to 0.5 us.  Three states in flight and no more: with four the kernel's spilled registers
 // doubled, on the path of every item (5407, 13880, 4142).
 // The counter of the lane's item, if it has one; `all`: its pieces.

@@ -1,4 +1,5 @@
-// Persistent tensor-core GEMM for passes of several frames (bf16 operands, fp32 accumulation in tensor memory).
+// Persistent tensor-core GEMM for passes of several frames, and for one frame's projection into the MLP (bf16 operands, fp32
+// accumulation in tensor memory).
 //
 //   C[M,N] = A[M,K] * Wt[N,K]^T  followed by the row form of a fused epilogue functor.
 //

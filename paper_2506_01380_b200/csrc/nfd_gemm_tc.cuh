@@ -38,9 +38,9 @@
 template <int BN> struct GemmCfg {
     // A ring stage holds KU k-blocks of 64 elements.  A producer takes about 280 clocks for a stage's barrier operations and
     // 60 per copy whatever their size, the products of a block 160 to 256: the narrow tiles, whose rings are deep, take two
-    // blocks to a stage, the others one, which comes back sooner.  One frame of the 310M class (QKV 64, out of attention
-    // 32, into the MLP 96, out of it 64 wide), us: all two blocks 5396, all one 5378, one from 96 on 5363, from 64 on 5367;
-    // hidden 768 (32 and 96 wide): 2328, 2346, 2322, 2322.
+    // blocks to a stage, the others one, which comes back sooner.  All two blocks -> one block from 96 wide on, 4 layers, us:
+    // two frames of 336 tokens, out of the MLP 96 wide with K in two, 261.4 -> 258.7, hidden 1536 354.1 -> 351.1; 220 tokens, three
+    // frames 275.2 -> 272.8; 390 tokens, three frames 419.2 -> 411.6; one frame (64 and 32 wide) the same.
     static constexpr int KU = BN <= 64 ? 2 : 1;
     // ring deep enough that one CTA owns an SM
     static constexpr int STAGES = BN <= 32 ? 5 : (BN <= 64 ? 4 : (BN <= 96 ? 7 : 6));
