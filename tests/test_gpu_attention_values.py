@@ -131,11 +131,14 @@ def test_scores_that_rise_beyond_the_reference(heads, T, streams, n_kv, n_q, win
     assert _rel(N.attention_noalloc(q, k, v, n_q, window, out), ref) <= limit
 
 
-def test_rising_scores_over_a_long_window():
-    """The same with 1200 frames in the window of the allocation-free call, one CTA to a query tile."""
+@pytest.mark.parametrize("heads,n_kv", [
+    (2, 1201),          # 6 query tiles: eight pieces each, 451 blocks and fewer to a CTA
+    (26, 301)])         # 78, more than clusters of two fit: one CTA to a tile, 903 blocks
+def test_rising_scores_over_a_long_window(heads, n_kv):
+    """The same with hundreds of frames in the window of the allocation-free call, in pieces and whole."""
     import torch
     from paper_2506_01380_b200 import nfd as N
-    heads, T, n_kv = 2, 336, 1201
+    T = 336
     q, k, v, out = _rising(heads, 64, T, n_kv, 1, seed=1, nats=400)
     got = N.attention_noalloc(q, k, v, 1, n_kv, out)
     ref = torch.cat([_exact(q[h:h + 1], k[:, h:h + 1], v[:, h:h + 1], 1, n_kv) for h in range(heads)], dim=1)
@@ -239,3 +242,20 @@ def test_a_frame_s_bits_do_not_depend_on_the_batch(streams, heads, hw, window, u
             both = g.denoise_step_batched(list(range(n)), x[:n].contiguous(), [0.6] * n, list(range(n)))
             assert torch.isfinite(both).all() and torch.equal(both, torch.stack(one[:n]))
     assert g.status() == 0
+
+
+@pytest.mark.parametrize("T", [5, 33, 77])
+@pytest.mark.parametrize("dtype,dh,tol", [("fp32", 32, 1e-5), ("fp32", 64, 1e-5), ("fp32", 128, 1e-5), ("bf16", 128, 4e-3)])
+def test_sixteen_queries_to_a_cta_on_the_fp32_pipes(T, dtype, dh, tol):
+    """With 60 heads CTAs take 16 queries (a last one with fewer), with 3 of them 8: a row's bits are the same.  Pages of 5 tokens
+    are several to a tile.  The tolerances of the small pages above."""
+    import torch
+    from paper_2506_01380_b200 import nfd as N
+    n_kv, n_q = 11, 2
+    q, k, v, out = _pages(60, dh, T, n_kv, n_q, seed=T + dh, dtype=dtype)
+    few = torch.empty(n_q * T, 3 * dh, device="cuda", dtype=out.dtype)
+    for window in (10, 3):
+        N.attention_noalloc(q, k, v, n_q, window, out)
+        assert _rel(out, _exact(q, k, v, n_q, window)) <= tol
+        N.attention_noalloc(q[:3].contiguous(), k[:, :3].contiguous(), v[:, :3].contiguous(), n_q, window, few)
+        assert torch.equal(few, out[:, :3 * dh])

@@ -5,7 +5,7 @@ import pytest
 
 from paper_2506_01380_b200 import inputs as I
 
-pytestmark = pytest.mark.gpu
+pytestmark = [pytest.mark.gpu, pytest.mark.filterwarnings("ignore:.*Profiler clears events")]
 
 
 def _events(call, tmp_path):
