@@ -225,12 +225,13 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
         // (Into registers, and stored when the loads that the wait holds back have been issued: with the stores here those loads
         // went out a global latency later, 0.1 to 0.3 us of the QKV projection where its main loop is short.)
         typename Epi::Row row_e{};
-        typename Epi::Col col_e{};
         float4 uv_e = make_float4(0.f, 0.f, 0.f, 0.f);
         int n_uv = 0;                                        // pairs of columns that (u, v) is fetched for
         if constexpr (Epi::kTables) {
+            // where the rows and the column chunks of this CTA's slice go
             if (et < rows_per && m0 + r_base + et < M) row_e = epi.row_info(m0 + r_base + et);
-            if (et >= 128 && et < 128 + CPR && n0 + (et - 128) * 8 < N) col_e = epi.col_info(n0 + (et - 128) * 8);
+            if (et >= 128 && et < 128 + CPR && n0 + (et - 128) * 8 < N)
+                *reinterpret_cast<typename Epi::Col *>(tab_raw + 128 * 16 + (et - 128) * 32) = epi.col_info(n0 + (et - 128) * 8);
         }
         if constexpr (Epi::kRowStats) {
             if (epi.ln.on()) {
@@ -238,6 +239,10 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
                 const int m_last = (m0 + 127 < M ? m0 + 127 : M - 1);
                 n_uv = (m_last / epi.ln.T - uv_f0 + 1) * (BN / 2);
                 if (et < n_uv && n0 + 2 * (et % (BN / 2)) < N) uv_e = epi.ln.uv_pair(uv_f0 + et / (BN / 2), n0 + 2 * (et % (BN / 2)));
+                if (et < rows_per) {
+                    const int m = m0 + r_base + et;
+                    rowfr[r_base + et] = (uint8_t)((m < M ? m : M - 1) / epi.ln.T - uv_f0);
+                }
             }
         }
         pdl_wait();
@@ -263,10 +268,6 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
                     const int m = (r < rows_per && m0 + r_base + r < M) ? m0 + r_base + r : -1;
 #pragma unroll
                     for (int u = 0; u < 4; ++u) pv[w][u] = epi.ln.part(m, sub + 8 * u);
-                }
-                if (et < rows_per) {
-                    const int m = m0 + r_base + et;
-                    rowfr[r_base + et] = (uint8_t)((m < M ? m : M - 1) / epi.ln.T - uv_f0);
                 }
                 // layout [frame][pair of columns within a chunk][chunk]: the lanes of a warp, which hold adjacent
                 // chunks, read adjacent 16-byte words
@@ -298,10 +299,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
             }
         }
         if constexpr (Epi::kTables) {
-            // where the rows and the column chunks of this CTA's slice go
             if (et < rows_per && m0 + r_base + et < M) *reinterpret_cast<typename Epi::Row *>(tab_raw + (r_base + et) * 16) = row_e;
-            if (et >= 128 && et < 128 + CPR && n0 + (et - 128) * 8 < N)
-                *reinterpret_cast<typename Epi::Col *>(tab_raw + 128 * 16 + (et - 128) * 32) = col_e;
         }
         // partial accumulator: tensor memory -> this CTA's staging tile (the ring is free by now)
         const int quad = warp & 3;                           // TMEM lane quadrant this warp may read
