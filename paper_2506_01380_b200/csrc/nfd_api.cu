@@ -317,10 +317,18 @@ static void launch_gemm(nfd_ctx *c, const TS *A, const TS *Wt, int M, int N, int
 template <typename TS, typename F> static void launch_attn_rows(int n_sm, const Dims &D, int nf, F launch) {
     const int nq = attn_rows_q(D, nf, n_sm);
     const dim3 grid((D.T + nq - 1) / nq, D.H, nf);
+    auto go = [&](auto dh) {
+        constexpr int DH = decltype(dh)::value;
+        if (nq == 8) return launch(k_attn_rows<TS, DH, 8, false>, grid);
+        if constexpr (attn_rows_wide<TS, DH>()) {
+            if (attn_rows_few(D, nf, n_sm)) return launch(k_attn_rows<TS, DH, 16, true>, grid);
+        }
+        return launch(k_attn_rows<TS, DH, 16, false>, grid);
+    };
     switch (D.dh) {
-        case 32: return nq == 8 ? launch(k_attn_rows<TS, 32, 8>, grid) : launch(k_attn_rows<TS, 32, 16>, grid);
-        case 64: return nq == 8 ? launch(k_attn_rows<TS, 64, 8>, grid) : launch(k_attn_rows<TS, 64, 16>, grid);
-        default: return nq == 8 ? launch(k_attn_rows<TS, 128, 8>, grid) : launch(k_attn_rows<TS, 128, 16>, grid);
+        case 32: return go(std::integral_constant<int, 32>());
+        case 64: return go(std::integral_constant<int, 64>());
+        default: return go(std::integral_constant<int, 128>());
     }
 }
 // `early`: see launch_attn_plan; set inside a pass, where the QKV projection comes before.

@@ -901,17 +901,14 @@ __global__ void __launch_bounds__(256) k_gemm_simple(const StepParams *sp, int T
 // only where a tile raises it.  (One warp per query with a sum over lanes per key, as
 // it was: 139 us for 6 heads x 32, 2 x 77 queries, 462 keys in fp32.)  A tile is a chain of loads: a batch of up to
 // eight 16-byte words of K and of up to 16 rows of V is in flight together, and where CTAs of 16 queries leave half of the SMs
-// idle they take 8 (that case 24.6 -> 20.5 us, 8 heads x 128, 100 queries, 1000 keys 84 -> 56).  Where such batches leave one
-// CTA to an SM they are smaller: us with large ones and as they are, 4 heads x 32 in fp32, 8 x 336 queries behind 32 frames 977
-// -> 890, 8 x 77 queries 129 -> 99; in bf16 16 heads x 64, 4 x 336 queries behind 16 frames 1714 -> 1295.
+// idle they take 8 (that case 24.6 -> 20.5 us, 8 heads x 128, 100 queries, 1000 keys 84 -> 56).  FEW: smaller batches, which leave
+// the registers for a second CTA on the SM; see attn_rows_few.
 // ---------------------------------------------------------------------------
-template <typename TS, int DH, int NQ>
+template <typename TS, int DH, int NQ, bool FEW>
 __global__ void __launch_bounds__(256) k_attn_rows(const StepParams *sp, Dims D, int layer, const TS *q, const TS *kc,
                                                    const TS *vc, TS *out) {
     constexpr int R = DH / 32, PS = NQ + 4, NV = WVec<TS>::N;
-    // Loads in flight together: words of K, rows of V.  Few where more of them would take the registers of the SM's second CTA
-    // (128 a thread: 16 queries, head dimension 32, and 64 in bf16, whose words of K are 8 elements).
-    constexpr bool FEW = NQ == 16 && (R == 1 || (R == 2 && NV == 8));
+    // loads in flight together: words of K, rows of V
     constexpr int UK = FEW ? 2 : (DH / NV < 8 ? DH / NV : 8), UV = FEW ? 4 : (R == 1 ? 16 : (R == 2 ? 8 : 4));
     __shared__ __align__(16) float s_q[NQ][DH];
     __shared__ __align__(16) float s_p[8][32 * PS];              // P of a tile: [key][query]; later O of a column slice
@@ -1036,6 +1033,12 @@ __global__ void __launch_bounds__(256) k_attn_rows(const StepParams *sp, Dims D,
 }
 // Queries per CTA: 16, or 8 where CTAs of 16 leave half of the SMs idle (a row's bits are the same).
 static int attn_rows_q(const Dims &D, int nf, int n_sm) { return 2ll * ((D.T + 15) / 16) * D.H * nf <= n_sm ? 8 : 16; }
+// Small batches of loads: where there are more CTAs than SMs, and the instance with large ones has more than 128 registers a thread
+// and so one CTA to an SM (16 queries, head dimension 32, and 64 in bf16, whose words of K are 8 elements).  us with large and with small
+// batches, 4 heads x 32 in fp32: 84 CTAs 114 and 132, 96 CTAs 50 and 57, 112 CTAs 143 and 160; 160 CTAs 129 and 99, 168 CTAs 389 and 341,
+// 672 CTAs 977 and 890.  In bf16 4 heads x 64, 84 CTAs 187 and 196, 16 x 64, 112 CTAs 83 and 87, 192 CTAs 92 and 68, 1344 CTAs 1714 and 1294.
+template <typename TS, int DH> constexpr bool attn_rows_wide() { return DH == 32 || (DH == 64 && WVec<TS>::N == 8); }
+static bool attn_rows_few(const Dims &D, int nf, int n_sm) { return (long long)((D.T + 15) / 16) * D.H * nf > n_sm; }
 
 // ---------------------------------------------------------------------------
 // Sampler glue (Section 4.1): elementwise.

@@ -53,8 +53,18 @@ def test_many_queries_on_the_fp32_pipes_leave_room_for_a_second_cta(dtype, heads
         rows = k.permute(1, 0, 2, 3).reshape(heads, 6 * T, dh).contiguous()
         call = lambda: g.attention(q, rows, rows, n_q, 6, 2, out=out)
     run = [x for x in _launches(call, tmp_path) if "k_attn_rows" in x[0]]
-    assert len(run) == 1 and f"{dh}, 16>" in run[0][0] and run[0][2] == heads * n_q * T // 16 and run[0][3] == 256
+    assert len(run) == 1 and f"{dh}, 16, true>" in run[0][0] and run[0][2] == heads * n_q * T // 16 and run[0][3] == 256
     assert run[0][1] <= 128, run
+
+
+@pytest.mark.parametrize("heads,T,n_q,instance", [
+    (4, 40, 2, "8, false"), (4, 40, 8, "16, false"), (4, 77, 8, "16, true")])      # 24, 96 and 160 CTAs of 16 queries
+def test_loads_in_flight_on_the_fp32_pipes_go_by_the_number_of_ctas(heads, T, n_q, instance, tmp_path):
+    """Up to an SM's one CTA each, large batches of loads; beyond, small ones and room for a second."""
+    from paper_2506_01380_b200 import nfd as N
+    q, k, out = _pages("fp32", heads, 32, T, n_q, 9)
+    run = [x for x in _launches(lambda: N.attention_noalloc(q, k, k, n_q, 2, out), tmp_path) if "k_attn_rows" in x[0]]
+    assert len(run) == 1 and f"<float, 32, {instance}>" in run[0][0], run
 
 
 @pytest.mark.parametrize("heads,dh,T,n_q,n_kv,window,kernel", [
