@@ -23,12 +23,15 @@ def _kernels(name):
 
 
 def test_cluster_pieces_are_read_before_their_cta_may_leave():
-    """The states of k_attn_own's pieces are read from peers' shared memory, by some lanes without any use for the value: the
-    barrier behind the reads has to order them.  The state starts where 16-byte words may: at the rounded base."""
+    """The states of k_attn_own's pieces are read from peers' shared memory, and the barrier behind that orders nothing: every value
+    that is read has to go into a result that is stored, or the read may be under way when the peer leaves.  So rows without a
+    result read nothing.  The state starts where 16-byte words may: at the rounded base."""
     body = _kernels("nfd_attn_tc.cuh")["k_attn_own"]
     reads = [m.start() for m in re.finditer(r"ld_cluster_f[24]\(", body)]
-    after = body[max(reads):]
-    assert "cluster_sync_all()" in after and "cluster_arrive_relaxed" not in after
+    guard = body.rindex("if (w0.nsplit > 1", 0, min(reads))
+    condition = body[guard:body.index("{", guard)]
+    assert "w0.qt * 128 + trow < D.T" in condition and "16 * cq < D.dh" in condition
+    assert body.index("attn_write<16>(", max(reads)) < body.index("cluster_", max(reads) + 40)
     assert re.search(r"state = reinterpret_cast<float \*>\(sh\.base \+ A::STATE_AT\)", body)
 
 
