@@ -109,8 +109,9 @@ static bool attn_divisors(AttnPlan &pl, int n_frames, int W, int n_sm) {
     const long long nb = ((long long)W + 1) * pl.BPF + pl.CH, big = 0x100000000ll;
     const long long n_items = n_frames * (pl.WH + (long long)pl.SP * pl.MAXSPLIT);
     const int tiles = pl.WH + pl.SP, d_item = tiles > pl.MAXSPLIT ? tiles : pl.MAXSPLIT;
-    // (a CTA may get ten items more than its share: attn_deal)
-    return n_items <= (long long)(ATTN_CTA_ITEMS - 16) * n_sm && n_items * d_item < big && nb < 0x7fffffffll && nb * (pl.CH > pl.BPF ? pl.CH : pl.BPF) < big;
+    // (with whole items and pieces a CTA may get ten items more than its share: attn_deal)
+    const int cta_items = pl.WH > 0 ? ATTN_CTA_ITEMS - 16 : ATTN_CTA_ITEMS;
+    return n_items <= (long long)cta_items * n_sm && n_items * d_item < big && nb < 0x7fffffffll && nb * (pl.CH > pl.BPF ? pl.CH : pl.BPF) < big;
 }
 // Pieces of the key range of a call on the caller's pages: as many as pay (as in attn_split_plan; starting a cluster and the merge
 // through distributed shared memory take 2 us and 0.2 per piece) and as clusters of that size fit the machine at once.  Head

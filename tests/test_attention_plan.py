@@ -132,3 +132,9 @@ def test_configuration_whose_pieces_are_counted_in_two_sweeps(lib):
     frames, tiles, k = 32, 96, 3
     seen, load, most = (C.c_int * (frames * tiles * k))(), (C.c_int * 148)(), C.c_float()
     assert lib.deal(336, 32, 4, 12, 148, frames, seen, load, C.byref(most)) > 32
+
+
+@pytest.mark.parametrize("heads,taken", [(9398, True), (9472, True), (9473, False)])
+def test_items_of_one_kind_fill_a_cta_s_account(lib, heads, taken):
+    """32 frames x heads x one query tile, whole windows: 2048 items to each of 148 CTAs are taken."""
+    assert lib.context_plan(128, heads, 1, 1, 148, (C.c_int * 7)()) == taken
