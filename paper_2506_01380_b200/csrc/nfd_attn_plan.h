@@ -47,8 +47,8 @@ struct AttnPlan {
 // whole ones in turn; then the pieces go first to the CTAs that have a whole item fewer than others, about as many as take the time
 // of one (a piece six blocks more than it has, where several follow one another), then to all in turn.  (Dealt on in turn behind the
 // whole ones, pieces went to CTAs that had one while others stood idle.  A context for 8 streams of 16 heads x 3 query tiles behind 32
-// frames, 4 layers, us of a pass with whole windows, with pieces in turn, as it is: two streams 470, 533, 467; three 505, 566,
-// 540; five 890, 1065, 956; six 1017, 1083, 1019; eight 1460, 1388, 1393.)
+// frames, 4 layers, us of a pass with whole windows, with pieces in turn, as it is: two streams 470, 530, 465; three 505, 584,
+// 583; five 890, 1011, 923; six 1017, 1133, 1091; eight 1460, 1407, 1379.)
 static inline void attn_deal(AttnPlan &pl, int frames, int n_sm) {
     pl.whole = frames * pl.WH, pl.pieces = frames * pl.SP * pl.MAXSPLIT;
     pl.n_items = pl.whole + pl.pieces;
@@ -131,58 +131,47 @@ template <typename F> static void attn_own_plan(AttnPlan &pl, int tiles, int n_b
     }
     pl.CH = (n_blocks + best_k - 1) / best_k, pl.MAXSPLIT = best_k;
 }
-// Time of a pass of `frames` frames as attn_deal gives them out, in key blocks of the busiest CTA: a whole item counts a block
-// more than it has, a piece two and a half (start, publication, merge).
-static inline float attn_pass_blocks(const AttnPlan &plan, int frames, int n_sm) {
-    AttnPlan pl = plan;
-    attn_deal(pl, frames, n_sm);
-    const float w = pl.NB + 1.f, p = pl.CH + 2.5f;
-    auto second = [&](int o) { return pl.rq + (o < pl.rr); };
-    float most = pl.wr ? (pl.wq + 1) * w + second(pl.grid - pl.wr) * p : 0.f;
-    const float a = pl.wq * w + (pl.fq + (pl.fr > 0) + second(0)) * p, b = pl.wq * w + (pl.fq + second(pl.fr)) * p;
-    if (a > most) most = a;
-    return b > most ? b : most;
-}
 // How the key ranges of a frame's `tiles` (head, query tile) pairs are split.  By the configuration alone (the longest
 // window, as many frames as there are streams), never by the pass: the order of the sums must not depend on it.
-//   Where a frame of every stream leaves half of the SMs idle, all of them, into at most as many pieces as fill the SMs once, and
-// no more than pay: a block takes about 0.65 us (of 112 keys; its columns and 24 count), publishing and counting 2.5, the merge
-// 0.25 per piece.  (A frame of a model of 2 layers, 4 heads, 64 tokens: behind four frames five pieces of a block 286 us, one of
-// five 270; behind 30 frames 31 pieces 443, eight 300; two streams of 4 heads x 32 behind 1000 frames, eight pieces a tile 766,
-// eighteen 619.)
-//   Else whole windows, dealt out to the CTAs, may leave a last round in which most SMs idle (16 heads
+//   One stream: all of them, into at most as many pieces as fill the SMs once, and no more than pay: a block takes about 0.65 us
+// (of 112 keys; its columns and 24 count), publishing and counting 2.5, the merge 0.25 per piece.  (A frame of a model of 2 layers,
+// 4 heads, 64 tokens: behind four frames five pieces of a block 286 us, one of five 270; behind 30 frames 31 pieces 443, eight 300.)
+//   Several: whole windows, dealt out to the CTAs, may leave a last round in which most SMs idle (16 heads
 // x 3 query tiles x 8 streams = 384 items on 148 SMs: two rounds and six tenths of one, at the price of three).  Splitting all
-// of them finely costs a state of 33 KB each; so the first WH are left whole and the others split, for the least time of a pass
-// with a frame of every stream; but by no plan that makes a pass with fewer frames, when not all streams are used, take an eighth
-// longer than whole windows would.
+// of them finely costs a state of 33 KB each; so the first WH are left whole and the others split, for the least blocks on the
+// busiest CTA of a pass with a frame of every stream, a whole item counted a block more than it has and a piece two and a half (start,
+// publication, merge).  Eight pieces to a window are looked at; where that is the best, of all windows, half of the SMs idle all the
+// same and a piece has more than sixteen blocks, as long as starting and merging it take, the rule for one stream holds (two streams of
+// 4 heads x 32 behind 1000 frames, eight pieces a tile 766 us a frame step, eighteen 619).
+//   A pass with fewer frames than streams may take longer than with whole windows (see attn_deal for both sides): a plan that
+// did not let it would be another order of the sums.
 static void attn_split_plan(AttnPlan &pl, int tiles, int n_streams, int n_blocks, int n_sm) {
     auto pieces = [&](int k) { pl.CH = (n_blocks + k - 1) / k, pl.MAXSPLIT = (n_blocks + pl.CH - 1) / pl.CH; };
     pl.WH = 0, pl.SP = tiles, pl.NB = n_blocks;
     const long long items = (long long)n_streams * tiles;
     float best = 1e30f;
-    int best_k = 1;
-    if (n_streams == 1 || 2 * items <= n_sm) {
-        for (int k = 1; k <= n_blocks && (k == 1 || k * items <= n_sm); ++k) {
+    int best_k = 1, best_wh = 0;
+    for (int k = 1; n_streams > 1 && k <= 8 && k <= n_blocks; ++k) {
+        pieces(k);
+        for (int wh = k == 1 ? tiles : 0; wh <= (k == 1 ? tiles : tiles - 1); ++wh) {
+            const int nw = n_streams * wh, n = nw + n_streams * (tiles - wh) * pl.MAXSPLIT, grid = n < n_sm ? n : n_sm;
+            // the CTAs before, between and behind those with a whole item and with an item more than others
+            float most = 0.f;
+            const int at[3] = {0, nw % grid, n % grid};
+            for (int c : at) {
+                const int w = nw / grid + (c < nw % grid), all = n / grid + (c < n % grid);
+                const float t = w * (n_blocks + 1.f) + (all - w) * (pl.CH + 2.5f);
+                if (t > most) most = t;
+            }
+            if (most < best) best = most, best_k = k, best_wh = k == 1 ? 0 : wh;      // (none is split: MAXSPLIT 1)
+        }
+    }
+    if (n_streams == 1 || (best_k == 8 && best_wh == 0 && 16 * items <= n_sm && n_blocks > 128)) {
+        best = 1e30f;
+        for (int k = n_streams == 1 ? 1 : 8; k <= n_blocks && (k == 1 || k * items <= n_sm); ++k) {
             pieces(k);
             const float t = pl.CH * 0.65f * (pl.KB + 24) / 136.f + (k > 1 ? 2.5f + 0.25f * k : 0.f);
             if (t < best) best = t, best_k = k;
-        }
-        return pieces(best_k);
-    }
-    const int full = n_streams < 32 ? n_streams : 32;      // frames of a pass, at most
-    auto whole = [&](int f) { return (float)(((long long)f * tiles + n_sm - 1) / n_sm) * (n_blocks + 1.f); };
-    best = whole(full);
-    int best_wh = 0;                                       // (none is split: MAXSPLIT 1)
-    const int step = tiles > 256 ? tiles / 256 : 1;
-    for (int k = 2; k <= 8 && k <= n_blocks; ++k) {
-        pieces(k);
-        for (int wh = 0; wh < tiles; wh += step) {
-            pl.WH = wh, pl.SP = tiles - wh;
-            const float t = attn_pass_blocks(pl, full, n_sm);
-            if (t >= best) continue;
-            bool good = true;
-            for (int f = 1; f < full && good; ++f) good = attn_pass_blocks(pl, f, n_sm) <= 1.13f * whole(f);
-            if (good) best = t, best_k = k, best_wh = wh;
         }
     }
     pieces(best_k);

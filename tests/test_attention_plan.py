@@ -26,9 +26,9 @@ extern "C" int context_plan(int T, int heads, int n_streams, int window, int n_s
     return 1;
 }
 // Every item of a pass of `frames` frames, whose windows are full: seen[(frame, tile) * MAXSPLIT + split] counts it, load[c] is
-// the time of CTA c in half blocks (a whole item a block more than it has, a piece two and a half), `most` that of the busiest one
-// by the closed form; the largest number of items of a CTA, -1 where an item is out of range.
-extern "C" int deal(int T, int heads, int n_streams, int window, int n_sm, int frames, int *seen, int *load, float *most) {
+// the time of CTA c in half blocks (a whole item a block more than it has, a piece two and a half), turn[c] the same where the pieces
+// follow the whole items in turn; the largest number of items of a CTA, -1 where an item is out of range.
+extern "C" int deal(int T, int heads, int n_streams, int window, int n_sm, int frames, int *seen, int *load, int *turn) {
     AttnPlan pl;
     attn_blocks(pl, T);
     const int n_blocks = (window + 1) * pl.BPF, tiles = heads * pl.QT;
@@ -50,7 +50,8 @@ extern "C" int deal(int T, int heads, int n_streams, int window, int n_sm, int f
         if (n > items) items = n;
         if (n < 1) return -1;
     }
-    *most = attn_pass_blocks(pl, frames, n_sm);
+    for (int i = 0; i < pl.n_items; ++i)
+        turn[i % pl.grid] += i < pl.whole || pl.MAXSPLIT == 1 ? 2 * (n_blocks + 1) : 2 * pl.CH + 5;
     return items;
 }
 """
@@ -93,11 +94,11 @@ SHAPES = [(336, 16, 32), (336, 16, 16), (336, 24, 16), (336, 12, 16), (220, 12, 
 
 
 @pytest.mark.parametrize("T,heads,window", SHAPES)
-def test_every_item_is_dealt_out_once_and_partial_batches_lose_little(lib, T, heads, window):
-    """Passes of 1 to 32 frames in contexts of 1 to 9 streams: every piece of every query tile comes up once, the busiest CTA is as
-    busy as the plan's closed form says, and where not all streams have a frame in the pass it has at most an eighth more to do
-    than with whole windows.  (Pieces dealt on in turn behind the whole items: up to 1.6 times as much.)"""
-    info, most = (C.c_int * 7)(), C.c_float()
+def test_every_item_is_dealt_out_once_and_no_cta_is_busier_than_in_turn(lib, T, heads, window):
+    """Passes of 1 to 32 frames in contexts of 1 to 9 streams: every piece of every query tile comes up once, and the busiest CTA of
+    a pass of no more frames than streams has no more to do than with the pieces dealt on in turn behind the whole items, half a
+    piece aside."""
+    info = (C.c_int * 7)()
     for n_sm in (148, 132, 20):
         for streams in range(1, 10):
             assert lib.context_plan(T, heads, streams, window, n_sm, info)
@@ -105,16 +106,40 @@ def test_every_item_is_dealt_out_once_and_partial_batches_lose_little(lib, T, he
             tiles = heads * qt
             assert wh + sp == tiles and (k - 1) * ch < n_blocks <= k * ch
             for frames in sorted({1, 2, 3, 4, 5, 6, 7, 8, streams, 2 * streams, 16, 31, 32}):
-                seen, load = (C.c_int * (frames * tiles * k))(), (C.c_int * n_sm)()
-                items = lib.deal(T, heads, streams, window, n_sm, frames, seen, load, C.byref(most))
+                seen, load, turn = (C.c_int * (frames * tiles * k))(), (C.c_int * n_sm)(), (C.c_int * n_sm)()
+                items = lib.deal(T, heads, streams, window, n_sm, frames, seen, load, turn)
                 assert 0 < items <= 2048
                 want = [1 if t >= wh or s == 0 else 0 for _ in range(frames) for t in range(tiles) for s in range(k)]
                 assert list(seen) == want, (n_sm, streams, frames)
-                busy = max(load) / 2
-                assert k == 1 or abs(busy - most.value) < 1e-3
-                if wh and frames <= streams:
-                    whole = -(-frames * tiles // n_sm) * (n_blocks + 1)
-                    assert busy <= 1.13 * whole, (n_sm, streams, frames, busy, whole)
+                assert sum(load) == sum(turn)
+                if frames <= streams:
+                    assert max(load) <= max(turn) + ch, (n_sm, streams, frames)
+
+
+def _start_plan(tiles, streams, n_blocks, n_sm):
+    """The split of several streams as it was chosen at first, from its definition: (whole pairs, blocks of a piece)."""
+    best = None
+    for k in range(1, min(8, n_blocks) + 1):
+        ch = -(-n_blocks // k)
+        split = -(-n_blocks // ch)
+        for wh in [tiles] if k == 1 else range(tiles):
+            nw = streams * wh
+            n = nw + streams * (tiles - wh) * split
+            grid = min(n, n_sm)
+            most = max(w * (n_blocks + 1) + (n // grid + (c < n % grid) - w) * (ch + 2.5)
+                       for c in (0, nw % grid, n % grid) for w in [nw // grid + (c < nw % grid)])
+            if best is None or most < best[0]:
+                best = (most, 0 if k == 1 else wh, ch)
+    return best[1:]
+
+
+@pytest.mark.parametrize("T,heads,window", SHAPES)
+def test_order_of_the_sums_of_several_streams(lib, T, heads, window):
+    """The plan decides in which order a frame's sums are taken: windows of up to 33 frames keep the one they have."""
+    info = (C.c_int * 7)()
+    for streams in range(2, 10):
+        assert lib.context_plan(T, heads, streams, window, 148, info)
+        assert (info[0], info[3]) == _start_plan(heads * info[6], streams, info[4], 148)
 
 
 @pytest.mark.parametrize("T,heads,streams,window", [(64, 4, 2, 1000), (128, 2, 3, 400), (64, 4, 4, 200), (64, 4, 1, 1000)])
@@ -129,9 +154,10 @@ def test_long_windows_of_few_heads_fill_the_machine(lib, T, heads, streams, wind
 def test_configuration_whose_pieces_are_counted_in_two_sweeps(lib):
     """32 heads, 336 tokens, four streams behind 12 frames, 32 frames in a pass: some CTA has more than the 32 items that one sweep of
     a warp counts (its values are checked on the GPU)."""
-    frames, tiles, k = 32, 96, 3
-    seen, load, most = (C.c_int * (frames * tiles * k))(), (C.c_int * 148)(), C.c_float()
-    assert lib.deal(336, 32, 4, 12, 148, frames, seen, load, C.byref(most)) > 32
+    frames, info = 32, (C.c_int * 7)()
+    assert lib.context_plan(336, 32, 4, 12, 148, info) and info[2] > 1
+    seen, load, turn = (C.c_int * (frames * 96 * info[2]))(), (C.c_int * 148)(), (C.c_int * 148)()
+    assert lib.deal(336, 32, 4, 12, 148, frames, seen, load, turn) > 32
 
 
 @pytest.mark.parametrize("heads,taken", [(9398, True), (9472, True), (9473, False)])

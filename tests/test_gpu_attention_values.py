@@ -216,10 +216,10 @@ def test_pieces_as_the_ctas_of_a_cluster(heads, T, dh, n_kv, n_q, window, nats):
 
 
 @pytest.mark.parametrize("streams,heads,hw,window,used,k", [
-    (8, 16, (48, 28), 32, (2, 5), 1),        # 33 of 48 (head, query tile) pairs whole: batches that leave CTAs without a whole window
-    (5, 16, (48, 28), 16, (3, 5), 2),        # 26 of 48, two frames a stream
+    (8, 16, (48, 28), 32, (2, 5), 1),        # 37 of 48 (head, query tile) pairs whole: batches that leave CTAs without a whole window
+    (5, 16, (48, 28), 16, (3, 5), 2),        # 28 of 48, two frames a stream
     (4, 12, (40, 22), 9, (4,), 8),           # every pair in three pieces: 72 items a frame, 32 frames
-    (4, 32, (48, 28), 12, (4,), 8)])         # 66 of 96, 32 frames: more than 32 items to a CTA, counted in two sweeps
+    (4, 32, (48, 28), 12, (4,), 8)])         # 70 of 96, 32 frames: more than 32 items to a CTA, counted in two sweeps
 def test_a_frame_s_bits_do_not_depend_on_the_batch(streams, heads, hw, window, used, k):
     """Contexts of several streams deal whole windows and pieces out to the CTAs by the number of frames in the pass; a frame's
     bits are those that it has alone."""
